@@ -38,7 +38,7 @@ GRID_TEMPLATES = 8000
 # an ncu capture of one launch on 8 templates (its summary is kept with the profiles;
 # the reads of a_r, b_r grow with the templates of a launch).  None once the kernel
 # changes.
-SEGPAIR_DRAM_BYTES_PER_TEMPLATE = (1.790227e9 + 46.770432e6) / 8
+SEGPAIR_DRAM_BYTES_PER_TEMPLATE = (2.040888e9 + 63.628800e6) / 8
 SM_COUNT = 152
 FP32_LANES = 128
 # days of the 120-day band in the bounded CPU samples (both CPU legs use the same sample)
@@ -113,16 +113,38 @@ def fp32_peak(cc, clk):
                      + (f" (measured {measured:.2f})" if measured else ""))
 
 
+def output_cosets(info, bf16):
+    """Whether the two-pass path sums its pair products at the output bins: segments longer
+    than 4096 samples stored in BF16.  Every other plan sums them on the lag grid."""
+    return bf16 and info["N_s"] > 4096 and info["L"] == 4096 and info["N_s"] % 4 == 0
+
+
 def spectrum_kernel_name(info, bf16=False):
     """The two-pass path's spectrum + pair-sum kernel(s) for this plan's geometry (the
     event pair of the plan's kernel timing brackets all of them)."""
-    if info["L"] == 4096 and info["N_s"] % 16 == 0 and info["R"] <= 1:
-        if info["N_s"] <= 4096:
-            return "segpair_tma_kernel"
-        if bf16:   # folded segments: the persistent kernel's shared memory holds a BF16 stage
-            return ("fold64_kernel + segpair_tma_kernel" if info["C"] == 64
-                    else "fold_kernel + segpair_tma_kernel")
-    return "segpair_grouped_kernel" if info["L"] <= 2048 else "segpair_kernel"
+    if output_cosets(info, bf16):
+        return ("fold64_kernel + segpair_tma_kernel" if info["C"] == 64
+                else "fold_cosets_kernel + segpair_tma_kernel")
+    return "fold_kernel + corr_kernel" if info["N_s"] > 4096 else "corr_kernel"
+
+
+def spectrum_flops(info, Q, bf16=False):
+    """Operations per template of that kernel: on the lag grid of G points (the power of two
+    of at least 2 N_s, or 2 ceil(N_s / 4096) x 4096 for longer segments) 5 G log2 G per
+    (weight, detector, segment) and per grid point and (weight, segment) the products of two
+    detectors (4) and of two segments (2 to sum the detectors, 8); at the output bins those of
+    algorithmic_costs."""
+    if output_cosets(info, bf16):
+        c = algorithmic_costs(info, Q, 1)
+        return c["fft_flops"] + c["pair_flops"]
+    N_s, M = info["N_s"], info["M"]
+    G = 8192 * -(-N_s // 4096) if N_s > 4096 else 1 << (2 * N_s - 1).bit_length()
+    return 2 * Q * M * 5.0 * G * math.log2(G) + 2 * M * G * (4.0 + (10.0 if info["R"] else 0.0))
+
+
+def path_flops(info, Q, D, learned):
+    """Whole two-pass path: resampling plus the spectrum kernel's operations."""
+    return algorithmic_costs(info, Q, 1, D, learned)["interp_flops"] + spectrum_flops(info, Q)
 
 
 # ---------------------------------------------------------------------------
@@ -585,7 +607,7 @@ def run_gpu(args):
         # the fused path the one-pass kernel (all flops).  Against the FP32-ALU roofline
         # from the SM count, FP32 lanes and the maximum SM clock.
         if path == cc.PATH_TWO_PASS:
-            kname, kflops = spectrum_kernel_name(info, long_lag), costs["fft_flops"] + costs["pair_flops"]
+            kname, kflops = spectrum_kernel_name(info, long_lag), spectrum_flops(info, Q, long_lag)
         else:
             kname, kflops = "fused_kernel", costs["total_flops"]
         achieved = kflops * B * args.steps / (fused_ms / 1e3) / 1e12
@@ -593,7 +615,7 @@ def run_gpu(args):
         other_ms = max(0.0, 1e3 * elapsed - fused_ms) / (B * args.steps)
         traffic = None
         if path == cc.PATH_TWO_PASS and SEGPAIR_DRAM_BYTES_PER_TEMPLATE is not None and fused_launches \
-                and not long_lag and kname == "segpair_tma_kernel" and not learned and args.pair_mode == "unordered":
+                and not long_lag and kname == "corr_kernel" and not learned and args.pair_mode == "unordered":
             traffic = SEGPAIR_DRAM_BYTES_PER_TEMPLATE * B * args.steps / fused_launches
         # the staged stage kernels are HBM-bound: algorithmic bytes (input read once,
         # output written once) over their event-timed duration, against the measured copy peak
@@ -700,10 +722,9 @@ def variant_stencils(args, ds, x, tm_host, plan, peak):
     with cc.CrossCorrPlan(ds.cfg, ds.dets, interp=cc.INTERP_LEARNED) as lp:
         for name, pl, learned in (("exact_d8", plan, False), ("learned", lp, True)):
             ms, kms, _ = _time_search(pl, x, tm, steps=2)
-            kfl = algorithmic_costs(pl.info, pl.Q, 1, ds.cfg.D, learned)
             res[name] = {"value": B * pl.N_f / (ms / 1e3), "unit": UNIT, "ms_per_template": ms / B,
                          "other_kernels_ms_per_template": (ms - kms) / B,
-                         "spectrum_frac": (kfl["fft_flops"] + kfl["pair_flops"]) * B / (kms / 1e3) / 1e12 / peak}
+                         "spectrum_frac": spectrum_flops(pl.info, pl.Q) * B / (kms / 1e3) / 1e12 / peak}
     # accuracy: noiseless injection, the injected template and three grid neighbours
     dn = synth.o1_band(seed=1002, noise=False)
     inj = dn.injection
@@ -749,10 +770,9 @@ def variant_long_lag(args, peak):
     res = {"templates": B}
     with cc.CrossCorrPlan(dl.cfg, dl.dets, store=cc.STORE_BF16) as pl:
         ms, kms, _ = _time_search(pl, x, tm, steps=2)
-        kfl = algorithmic_costs(pl.info, pl.Q, 1, dl.cfg.D, False)
         res.update({"value": B * pl.N_f / (ms / 1e3), "unit": UNIT, "ms_per_template": ms / B,
                     "kernel": spectrum_kernel_name(pl.info, True),
-                    "spectrum_frac": (kfl["fft_flops"] + kfl["pair_flops"]) * B / (kms / 1e3) / 1e12 / peak,
+                    "spectrum_frac": spectrum_flops(pl.info, pl.Q, True) * B / (kms / 1e3) / 1e12 / peak,
                     "spectrum_share": kms / ms, "N_f": pl.N_f, "N_FFT": pl.info["N_FFT"]})
         inj = dl.injection
         two = torch.from_numpy(np.array([[inj.a_p, inj.T_asc, inj.P, 0.0, 0.0],
@@ -791,7 +811,7 @@ def variant_multiband(args, peak, scale=0.05):
     e1.record(stream)
     torch.cuda.synchronize()
     sec = e0.elapsed_time(e1) / 1000.0 / 2
-    flops = sum(algorithmic_costs(p.info, p.Q, tm.shape[0], cfg.D, False)["total_flops"]
+    flops = sum(path_flops(p.info, p.Q, cfg.D, False) * tm.shape[0]
                 for p, (cfg, _, _, tm) in zip(mb.plans, bands))
     res = {"template_scale": scale, "templates": int(sum(t.shape[0] for (_, _, _, t) in bands)),
            "value": mb.units / sec, "unit": UNIT, "ms_per_step": 1e3 * sec,
@@ -862,8 +882,7 @@ def run_multiband(args):
     # algorithmic flops of the whole graph (every kernel), over the graph's time
     flops = 0.0
     for p, (cfg, dets, x, tm) in zip(mb.plans, bands):
-        c = algorithmic_costs(p.info, p.Q, tm.shape[0], cfg.D, learned)
-        flops += c["total_flops"]
+        flops += path_flops(p.info, p.Q, cfg.D, learned) * tm.shape[0]
     achieved = flops * args.steps / elapsed / 1e12
     peak, peak_kind = fp32_peak(cc, clk)
     # e2e: every band's series and templates copied in from pinned memory, rho copied out
@@ -894,7 +913,7 @@ def run_multiband(args):
                    # per band, from the autotuner's timing of its first 64 templates: coset
                    # length, ms per template, fraction of the FP32 peak (algorithmic flops)
                    "bands": [{"L": int(pl.info["L"]), "ms_per_template": round(t["ms"] / min(64, tt.shape[0]), 4),
-                              "frac": round(algorithmic_costs(pl.info, pl.Q, 1, cf.D, learned)["total_flops"]
+                              "frac": round(path_flops(pl.info, pl.Q, cf.D, learned)
                                             / (t["ms"] / min(64, tt.shape[0]) * 1e-3) / (peak * 1e12), 3)}
                              for pl, t, tt, (cf, _, _, _) in zip(mb.plans, mb.tuning, mb.templates, bands)],
                    "interp": "learned 8-tap" if learned else "windowed sinc, 17 taps",

@@ -252,12 +252,15 @@ cc_status crosscorr_search_noalloc(cc_plan* plan, const void* const* x_dev, cons
  *                     each segment into shared memory and transforms it on chip; needs
  *                     a few MB of workspace (FP32 storage, coset length <= 4096);
  *   CC_PATH_TWO_PASS  a_r, b_r of a template batch written to HBM in the plan's
- *                     storage type (up to 24 GB of workspace), then one CTA per
- *                     (coset, weight) transforms each segment and folds it into the
- *                     pair sum on chip (Q <= 2, R <= 1, not CC_PAIRS_CROSS_ONLY, coset
- *                     length >= 64, output bins in the lower half of each coset); for
- *                     coset length 4096 with whole segments this is a persistent kernel
- *                     fed by TMA bulk copies (see crosscorr_plan_check);
+ *                     storage type (up to 24 GB of workspace), then every segment is
+ *                     transformed on chip at the G >= 2 N_s frequencies that determine the
+ *                     products of two segments, the products are summed there, and one
+ *                     transform per template takes the sums to the output bins (Q <= 2,
+ *                     R <= 1, not CC_PAIRS_CROSS_ONLY, coset length >= 64, output bins in the
+ *                     lower half of each coset); a persistent kernel fed by TMA bulk copies
+ *                     where rows are whole 16-byte pieces (see crosscorr_plan_check).
+ *                     Segments longer than 4096 samples stored in BF16 are transformed at
+ *                     the output bins instead;
  *   CC_PATH_STAGED    the three stage kernels with spectra in HBM (any plan). */
 enum { CC_PATH_AUTO = 0, CC_PATH_FUSED = 1, CC_PATH_TWO_PASS = 2, CC_PATH_STAGED = 3 };
 
@@ -287,11 +290,10 @@ typedef struct {
     int32_t chunk_waves;      /* fused and two-pass: split each template's segments into
                                  chunks until the launch has about this many CTA waves
                                  (0: 4 for fused, 40 for two-pass) */
-    int32_t transform_len;    /* two-pass, segments of at most 4096 samples: 0 takes the
-                                 plan's coset length (the power of two covering a segment),
-                                 4096 the persistent kernel's 4096-point coset transforms
-                                 with the segment zero-padded (needs N_FFT >= 4096: fewer
-                                 cosets, more transform work, a faster kernel) */
+    int32_t transform_len;    /* two-pass, segments of at most 1024 samples: 0 takes the
+                                 shortest transform (the power of two of at least twice the
+                                 segment), 4096 one 4096-point transform per segment
+                                 (needs N_FFT >= 4096) */
 } cc_tuning;
 cc_status crosscorr_plan_set_tuning(cc_plan* plan, const cc_tuning* tuning);
 

@@ -140,6 +140,10 @@ struct cc_plan {
     int search_path = CC_PATH_AUTO;           // crosscorr_plan_set_path
     cc_tuning tuning = {0, 0, 0};             // crosscorr_plan_set_tuning
     int kbar_span4 = 0;                       // largest transform position of a bin, 4096-point cosets
+    // two-pass search, lag grid: coset and pass twiddles [C][272] of the plan's grid and of one
+    // coset, roots of its transform length and of 4096 (plan-owned)
+    const float2 *corr_twk = nullptr, *corr_twk1 = nullptr, *corr_twL = nullptr, *corr_tw4096 = nullptr;
+    const float4 *corr_tw8 = nullptr, *corr_tw8_1 = nullptr;   // [C][256][2] last-pass powers (corr.cuh)
     int* segfft_ctr = nullptr;                // [C4] unit counters of the staged segment FFT (plan-owned)
     bool ws_external = false;                 // ws is caller memory (crosscorr_plan_set_workspace)
     // diagnostic event pairs around fused-kernel launches (crosscorr_plan_set_kernel_timing)
@@ -621,6 +625,16 @@ __device__ __forceinline__ SampleWeights sample_weights(const DevParams& p, int 
 __device__ __forceinline__ float2 twiddle_N(uint64_t j, uint64_t N) {
     float s, c;
     sincospif(-2.0f * (float)j / (float)N, &s, &c);
+    return make_float2(c, s);
+}
+
+// exp(-2 pi i e / G) for any integer e and G < 2^24, the angle reduced to half a turn.
+__device__ __forceinline__ float2 unit_root(int64_t e, int64_t G) {
+    int64_t r = e % G;
+    if (r < 0) r += G;
+    if (2 * r > G) r -= G;
+    float s, c;
+    sincospif(-2.0f * (float)r / (float)G, &s, &c);
     return make_float2(c, s);
 }
 

@@ -1,0 +1,519 @@
+// Two-pass search: the resampling kernel writes the weighted source-frame series a_r, b_r of
+// a template batch to HBM; corr_kernel forms every segment's spectrum on the lag grid and
+// sums the pair products there (corr_kernel.cuh says why that grid is enough); this file
+// turns those sums into rho at the output bins:
+//
+//   corr_lags_kernel   sums the partial rows of a template, inverse transform per coset to
+//                      lags, and the template's normalisation;
+//   corr_merge_kernel  the lag sequence from the cosets (more than two cosets only);
+//   corr_rho_kernel    one coset of the N_FFT-point output transform of the lag sequence,
+//                      normalised at the output bins.
+//
+// With a(l) and b(l) the inverse transforms of A and B, the pair sum at bin k is
+//   rho_raw(k) = Re sum_(n = 0)^(2 N_s - 1) h(n) W_N^(k n),
+//   h(0) = a(0), h(n) = 2 a(n) [n < N_s] + conj(b(N_s - n)) [n >= 1]
+// (a(-l) = conj(a(l)) because A is real; a pair of consecutive segments carries the phase
+// W_N^(-k N_s) of their distance; b counts twice with every ordered pair).  Per template the
+// three take about 0.1 % of the operations of the segment transforms at the 120-day band.
+#include <algorithm>
+
+#include "corr.cuh"
+#include "segpair.cuh"
+
+namespace cc {
+
+cc_status launch_resample(cc_plan* plan, const cc_template* t_dev, int64_t n_t, void* ab, float* norm,
+                          cudaStream_t st, const KnotRec* kn = nullptr, int64_t nkn = 0, int write_inactive = 0,
+                          uint8_t* act = nullptr, int t_pad = 0);
+cc_status launch_knots(cc_plan* plan, const cc_template* t_dev, int64_t n_t, KnotRec* kn, cudaStream_t st,
+                       int* zero_word = nullptr);
+cc_status launch_norm(cc_plan* plan, const float* norm, int64_t n_t, double* Dws, cudaStream_t st);
+cc_status launch_pair_finalize(cc_plan* plan, const float* raw, const double* Dws, int n_rows, int64_t n_t,
+                               float* rho, cudaStream_t st);
+int64_t fold_count(const cc_plan* plan);
+cc_status launch_fold(cc_plan* plan, int64_t n_t, const void* ab, const uint8_t* act, int t_pad, float2* z,
+                      cudaStream_t st);
+
+CC_CORR_INST(extern, 128)
+CC_CORR_INST(extern, 256)
+CC_CORR_INST(extern, 512)
+CC_CORR_INST(extern, 1024)
+CC_CORR_INST(extern, 2048)
+CC_CORR_INST(extern, 4096)
+CC_CORR_INST_FULL(extern)
+
+constexpr size_t TWO_PASS_WS_BUDGET = (size_t)24 << 30;   // a_r, b_r (and folded rows) of one template batch
+constexpr int LAG_THREADS = 256;
+constexpr int ROW_BLOCK = 32;        // partial rows summed by one block of corr_rows_kernel
+
+// What the kernels after corr_kernel need.
+struct LagArgs {
+    const float* raw;       // [n_t][n_rows][planes][G]
+    float2* U;              // [n_t][planes > 1 ? 2 : 1][C][L]: per coset the inverse transform of A and B
+    float2* h;              // [n_t][n_lags] (C > 2)
+    const float2* twL;      // exp(-2 pi i j / L)
+    const float4* norm;     // [n_t][Q][M]
+    double* D;              // [n_t]
+    int64_t M;
+    int L, log2L, C, planes, n_rows, n_lags, N_s, Q, R, pair_mode;
+};
+
+// Sum of ROW_BLOCK partial rows (few templates have many): out [n_t][gridDim.y][len].
+__global__ void __launch_bounds__(LAG_THREADS)
+corr_rows_kernel(const float* __restrict__ raw, int n_rows, int64_t len, float* __restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * LAG_THREADS + threadIdx.x, t = blockIdx.z;
+    if (i >= len) return;
+    const int r0 = blockIdx.y * ROW_BLOCK, r1 = min(n_rows, r0 + ROW_BLOCK);
+    const float* p = raw + (size_t)t * n_rows * len + i;
+    float s = 0.f, cp = 0.f;
+#pragma unroll 8
+    for (int r = r0; r < r1; ++r) kahan_add(s, cp, __ldg(p + (size_t)r * len));
+    out[((size_t)t * gridDim.y + blockIdx.y) * len + i] = s;
+}
+
+__device__ __forceinline__ double norm_pair(float4 a, float4 b) {
+    return (double)a.x * b.x + (double)a.y * b.y + 2.0 * (double)a.z * b.z;
+}
+
+// grid: x = coset c (x = C, y = 0: the normalisation D of template z), y = A or B, z = template.
+__global__ void __launch_bounds__(LAG_THREADS)
+corr_lags_kernel(const LagArgs q) {
+    extern __shared__ __align__(16) float2 buf[];
+    const int c = blockIdx.x, ser = blockIdx.y;
+    const size_t t = blockIdx.z;
+    if (c == q.C) {   // sum over the pair set of A_i A_j + B_i B_j + 2 C_i C_j
+        if (ser) return;
+        __shared__ double red[LAG_THREADS / 32];
+        const float4* nt = q.norm + t * q.Q * q.M;
+        double acc = 0.0;
+        for (int64_t idx = threadIdx.x; idx < q.Q * q.M; idx += LAG_THREADS) {
+            const int Y = (int)(idx / q.M);
+            const int64_t K = idx - Y * q.M;
+            const float4 nY = nt[Y * q.M + K];
+            double s = 0.0;
+            for (int X = 0; X < Y; ++X) s += norm_pair(nt[X * q.M + K], nY);
+            if (q.R > 0 && K > 0)
+                for (int X = 0; X < q.Q; ++X) s += norm_pair(nt[X * q.M + K - 1], nY);
+            if (q.pair_mode == CC_PAIRS_ALL_ORDERED) s = 2.0 * s + norm_pair(nY, nY);
+            acc += s;
+        }
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < LAG_THREADS / 32; ++w) s += red[w];
+            q.D[t] = s;
+        }
+        return;
+    }
+    const size_t G = (size_t)q.C * q.L;
+    const float* p0 = q.raw + t * q.n_rows * q.planes * G + (size_t)c * q.L;
+    // the inverse transform as the conjugate of the forward one of the conjugate
+    for (int m = threadIdx.x; m < q.L; m += LAG_THREADS) {
+        float re = 0.f, cr = 0.f, im = 0.f, ci = 0.f;
+        const float* p = p0 + m;
+        if (ser == 0) {
+#pragma unroll 4
+            for (int r = 0; r < q.n_rows; ++r) kahan_add(re, cr, __ldg(p + (size_t)r * q.planes * G));
+        } else {
+#pragma unroll 4
+            for (int r = 0; r < q.n_rows; ++r) {
+                kahan_add(re, cr, __ldg(p + ((size_t)r * q.planes + 1) * G));
+                kahan_add(im, ci, __ldg(p + ((size_t)r * q.planes + 2) * G));
+            }
+        }
+        buf[m] = make_float2(re, -im);
+    }
+    __syncthreads();
+    const float2* res = fft_stockham(buf, buf + q.L, q.L, q.log2L, q.twL);
+    const float sc = 1.0f / (float)G;
+    float2* o = q.U + ((t * (q.planes > 1 ? 2 : 1) + ser) * q.C + c) * q.L;
+    for (int m = threadIdx.x; m < q.L; m += LAG_THREADS) o[m] = make_float2(res[m].x * sc, -res[m].y * sc);
+}
+
+// sum_c W_G^(-c l) u_c(l mod L): the inverse transform at lag l from those of the cosets
+__device__ __forceinline__ float2 lag_value(const float2* __restrict__ u, int C, int L, int l) {
+    float2 v = __ldg(u + (l & (L - 1)));
+    for (int c = 1; c < C; ++c) {
+        const float2 w = unit_root(-(int64_t)c * l, (int64_t)C * L);
+        v = cadd(v, cmul(__ldg(u + (size_t)c * L + (l & (L - 1))), w));
+    }
+    return v;
+}
+
+__device__ __forceinline__ float2 lag_h(const LagArgs& q, size_t t, int n) {
+    const int G = q.C * q.L;
+    const float2* u = q.U + t * (q.planes > 1 ? 2 : 1) * G;
+    float2 h = make_float2(0.f, 0.f);
+    if (n < q.N_s) {
+        const float2 a = lag_value(u, q.C, q.L, n);
+        h = n > 0 ? cscale(a, 2.f) : a;
+    }
+    if (q.planes > 1 && n > 0) {
+        const int l = q.N_s - n;
+        const float2 b = lag_value(u + G, q.C, q.L, l < 0 ? l + G : l);
+        const float f = q.pair_mode == CC_PAIRS_ALL_ORDERED ? 2.f : 1.f;
+        h = make_float2(fmaf(f, b.x, h.x), fmaf(-f, b.y, h.y));
+    }
+    return h;
+}
+
+__global__ void __launch_bounds__(LAG_THREADS)
+corr_merge_kernel(const LagArgs q) {
+    const int n = blockIdx.x * LAG_THREADS + threadIdx.x;
+    const size_t t = blockIdx.y;
+    if (n < q.n_lags) q.h[t * q.n_lags + n] = lag_h(q, t, n);
+}
+
+// Output bins b0 + c + C m (the plan's coset lists), one coset per block: position p takes
+// sum_f h(p + f L) W_N^((b0 + c)(p + f L)), an L-point transform gives the bins.
+// grid: x = coset, y = template.
+__global__ void __launch_bounds__(LAG_THREADS)
+corr_rho_kernel(const LagArgs q, int L, int log2L, const float2* __restrict__ twL, int64_t N_FFT, int64_t b0,
+                const int* __restrict__ off, const int* __restrict__ ck, const int* __restrict__ cm, int64_t N_f,
+                float* __restrict__ rho) {
+    extern __shared__ __align__(16) float2 buf[];
+    const int c = blockIdx.x;
+    const size_t t = blockIdx.y;
+    const uint64_t N = (uint64_t)N_FFT, mask = N - 1;
+    const uint64_t bc = ((uint64_t)b0 + (uint64_t)c) & mask;
+    for (int pos = threadIdx.x; pos < L; pos += LAG_THREADS) {
+        float2 acc = make_float2(0.f, 0.f);
+        for (int n = pos; n < q.n_lags; n += L) {
+            const float2 h = q.h ? __ldg(q.h + t * q.n_lags + n) : lag_h(q, t, n);
+            acc = cadd(acc, cmul(h, twiddle_N((bc * (uint64_t)n) & mask, N)));
+        }
+        buf[pos] = acc;
+    }
+    __syncthreads();
+    const float2* res = fft_stockham(buf, buf + L, L, log2L, twL);
+    const double D = q.D[t];
+    const double sc = D > 0.0 ? 1.4142135623730951 / sqrt(D) : 0.0;
+    const int e = __ldg(off + c + 1);
+    for (int i = __ldg(off + c) + threadIdx.x; i < e; i += LAG_THREADS)
+        rho[t * N_f + __ldg(ck + i)] = D > 0.0 ? (float)((double)res[__ldg(cm + i)].x * sc) : 0.f;
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
+static size_t al128(size_t b) { return (b + 127) & ~(size_t)127; }
+
+struct CorrLayout {
+    int L, C, T, half, folded, bf16_rows, planes, n_rows, n_blocks, n_lags;
+    int64_t G, t_pad;
+    CorrArgs a;
+    // workspace pieces of a batch, bytes
+    size_t ab, z, norm, act, D, raw, rows2, U, h, kn, total;
+};
+
+// Whether the plan takes the two-pass kernels by name (CC_PATH_TWO_PASS): Q <= 2, R <= 1, no
+// cross-only pair set, coset length 64..4096, every bin in the lower half of its coset.
+bool two_pass_supported(const cc_plan* plan) {
+    const DevParams& p = plan->dp;
+    if (p.Q > 2 || p.R > 1 || p.pair_mode == CC_PAIRS_CROSS_ONLY) return false;
+    if (p.L < 64 || p.L > 4096 || plan->N_f < 1) return false;
+    return 2 * ((plan->kbar.back() - plan->k0) / p.C) < p.L;
+}
+
+static int sm_count() {
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+// Grid, shared memory, chunk split and workspace of a batch of n_t templates.
+static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
+    const DevParams& p = plan->dp;
+    const bool padded = plan->tuning.transform_len == CORR_POINTS && p.L < CORR_POINTS;
+    y->folded = p.N_s > CORR_POINTS;
+    y->half = 2 * p.N_s <= CORR_POINTS;
+    y->L = y->half && !padded ? 2 * p.L : CORR_POINTS;
+    y->C = y->folded ? 2 * (int)fold_count(plan) : y->half ? 1 : 2;
+    y->T = CORR_POINTS / y->L;
+    y->G = (int64_t)y->C * y->L;
+    y->planes = p.R > 0 ? 3 : 1;
+    y->n_lags = (int)(p.R > 0 ? 2 * p.N_s : p.N_s);
+    y->bf16_rows = !y->folded && p.store == CC_STORE_BF16;
+    y->t_pad = (n_t + 15) & ~(int64_t)15;
+    const int esz = y->bf16_rows ? 4 : 8;
+    CorrArgs& a = y->a;
+    a = CorrArgs{};
+    a.n_in = y->folded ? CORR_POINTS : (int)p.N_s;
+    a.row_bytes = (uint32_t)(a.n_in * esz);
+    a.row_stride = (uint32_t)((y->half ? y->L / 2 : y->L) * esz);   // whole inputs, zero beyond the samples
+    a.tma = a.row_bytes % 16 == 0;   // bulk copies: rows of whole 16-byte pieces start on 16-byte boundaries
+    const size_t buf = (size_t)y->T * padded_len(y->L) * sizeof(float2);
+    size_t o = al128((size_t)y->T * a.row_stride);
+    a.off_y = (uint32_t)o;
+    o = al128(o + buf);
+    a.off_z = (uint32_t)o;
+    o = al128(o + buf);
+    a.off_act = (uint32_t)o;
+    o += (CORR_MAX_CHUNK + 1) * sizeof(uint32_t);
+    a.off_bar = (uint32_t)o;
+    a.smem = (uint32_t)(o + 16);
+    // Chunks of segments: units are equal, handed out one by one to two CTAs per SM, each
+    // rereads its first segment's predecessor (R = 1) and writes one row (about the traffic of
+    // another segment): the count with the least ceil(units / slots) (length + overhead), at
+    // most M / (4 R + 1) chunks; with cc_tuning.chunk_waves, that many units per slot.
+    const int64_t slots = (int64_t)CORR_CTAS_PER_SM * sm_count();
+    const int64_t per_chunk = (2 * n_t + y->T - 1) / y->T * y->C;
+    const int64_t minch = (p.M + CORR_MAX_CHUNK - 1) / CORR_MAX_CHUNK;
+    const int64_t maxch = std::max<int64_t>(minch, p.M / (4 * p.R + 1));
+    int64_t nch = minch;
+    if (plan->tuning.chunk_waves > 0) {
+        nch = std::max(minch, std::min<int64_t>(maxch, (plan->tuning.chunk_waves * slots + per_chunk - 1) / per_chunk));
+    } else {
+        const int64_t most = std::max(minch, std::min<int64_t>(maxch, (32 * slots + per_chunk - 1) / per_chunk));
+        int64_t best = -1;
+        for (int64_t n = minch; n <= most; n += 1 + n / 16) {
+            const int64_t len = (p.M + n - 1) / n, waves = (per_chunk * ((p.M + len - 1) / len) + slots - 1) / slots;
+            const int64_t cost = waves * (len + p.R + 1);
+            if (best < 0 || cost < best) {
+                best = cost;
+                nch = n;
+            }
+        }
+    }
+    a.chunk_len = (int)((p.M + nch - 1) / nch);
+    a.n_chunks = (int)((p.M + a.chunk_len - 1) / a.chunk_len);
+    y->n_rows = 2 * a.n_chunks;
+    y->n_blocks = y->n_rows > ROW_BLOCK ? (y->n_rows + ROW_BLOCK - 1) / ROW_BLOCK : 0;
+    const size_t b = (size_t)n_t;
+    y->ab = al256(b * plan->Q * 2 * plan->N_tau * (plan->cfg.store == CC_STORE_BF16 ? 4 : 8));
+    y->z = y->folded ? al256(b * plan->Q * 2 * plan->M * y->G * esz) : 0;
+    y->norm = al256(b * plan->Q * plan->M * sizeof(float4));
+    y->act = al256((size_t)2 * plan->M * y->t_pad);
+    y->D = al256(b * sizeof(double));
+    y->raw = al256(b * y->n_rows * y->planes * y->G * sizeof(float));
+    y->rows2 = al256(b * y->n_blocks * y->planes * y->G * sizeof(float));
+    y->U = al256(b * (y->planes > 1 ? 2 : 1) * y->G * sizeof(float2));
+    y->h = y->C > 2 ? al256(b * y->n_lags * sizeof(float2)) : 0;
+    y->kn = al256(b * plan->Q * knot_rows(plan) * sizeof(KnotRec));
+    y->total = y->ab + y->z + y->norm + y->act + y->D + y->raw + y->rows2 + y->U + y->h + y->kn + 256;
+}
+
+// Templates per batch: as many as the budget of a_r, b_r and folded rows holds.
+static int64_t two_pass_batch(const cc_plan* plan, int64_t n_t) {
+    const size_t per = (size_t)plan->Q * 2 * plan->N_tau * (plan->cfg.store == CC_STORE_BF16 ? 4 : 8) +
+                       (plan->N_s > CORR_POINTS ? (size_t)plan->Q * 2 * plan->M * 2 * fold_count(plan) * CORR_POINTS * 8
+                                                : 0);
+    const int64_t b = plan->tuning.batch_templates > 0 ? plan->tuning.batch_templates
+                                                       : (int64_t)std::max<size_t>(1, TWO_PASS_WS_BUDGET / per);
+    return std::max<int64_t>(1, std::min<int64_t>({b, n_t, 65535}));
+}
+
+// Folded segments in BF16 (segpair_tma.cu): batch, chunks and workspace.
+struct FoldedLayout {
+    int64_t batch, chunk_len;
+    int n_chunks;
+    size_t ab, z, norm, D, raw, kn, total;
+};
+
+static void folded_chunks(const cc_plan* plan, int64_t n_t, FoldedLayout* y) {
+    const int64_t nch = segpair_tma_chunks(plan, n_t);
+    y->chunk_len = (plan->M + nch - 1) / nch;
+    y->n_chunks = (int)((plan->M + y->chunk_len - 1) / y->chunk_len);
+}
+
+static void folded_layout(const cc_plan* plan, int64_t n_t, FoldedLayout* y) {
+    const size_t ab = (size_t)plan->Q * 2 * plan->N_tau * 4, z = segpair_tma_fold_bytes(plan);
+    const int64_t want = plan->tuning.batch_templates > 0 ? plan->tuning.batch_templates
+                                                          : (int64_t)std::max<size_t>(1, TWO_PASS_WS_BUDGET / (ab + z));
+    y->batch = std::max<int64_t>(1, std::min<int64_t>({want, n_t, 65535}));
+    folded_chunks(plan, y->batch, y);
+    const size_t b = (size_t)y->batch;
+    y->ab = al256(ab * b);
+    y->z = al256(z * b);
+    y->norm = al256(b * plan->Q * plan->M * sizeof(float4));
+    y->D = al256(b * sizeof(double));
+    y->raw = al256(b * 2 * y->n_chunks * plan->N_f * sizeof(float));
+    y->kn = al256(b * plan->Q * knot_rows(plan) * sizeof(KnotRec));
+    y->total = y->ab + y->z + y->norm + y->D + y->raw + y->kn + al256((size_t)plan->dp.C4 * sizeof(int));
+}
+
+static cc_status search_folded_bf16(cc_plan* plan, const cc_template* t_dev, int64_t n_t, float* rho, cudaStream_t st) {
+    FoldedLayout y;
+    folded_layout(plan, n_t, &y);
+    cc_status s = ensure_workspace(plan, y.total);
+    if (s != CC_OK) return s;
+    char* w = (char*)plan->ws;
+    void* ab = w;
+    void* z = w += y.ab;
+    float* norm = (float*)(w += y.z);
+    double* D = (double*)(w += y.norm);
+    float* raw = (float*)(w += y.D);
+    KnotRec* kn = (KnotRec*)(w += y.raw);
+    int* counters = (int*)(w += y.kn);
+    for (int64_t t0 = 0; t0 < n_t; t0 += y.batch) {
+        const int64_t nb = std::min(y.batch, n_t - t0);
+        FoldedLayout b = y;
+        folded_chunks(plan, nb, &b);   // chunking for this batch size (workspace sized for the largest)
+        if (b.n_chunks > y.n_chunks) b = y;
+        if ((s = launch_knots(plan, t_dev + t0, nb, kn, st)) != CC_OK) return s;
+        if ((s = launch_resample(plan, t_dev + t0, nb, ab, norm, st, kn, knot_rows(plan))) != CC_OK) return s;
+        if ((s = launch_norm(plan, norm, nb, D, st)) != CC_OK) return s;
+        cudaEvent_t ev0, ev1;
+        timing_pair(plan, &ev0, &ev1);
+        if (ev0) cudaEventRecord(ev0, st);
+        s = launch_fold_bf16(plan, nb, ab, (const float4*)norm, z, st);
+        if (s == CC_OK) s = launch_segpair_tma(plan, b.n_chunks, b.chunk_len, nb, z, (const float4*)norm, raw, counters, st);
+        if (ev1) cudaEventRecord(ev1, st);
+        if (s != CC_OK) return s;
+        if ((s = launch_pair_finalize(plan, raw, D, 2 * b.n_chunks, nb, rho + t0 * plan->N_f, st)) != CC_OK) return s;
+    }
+    return CC_OK;
+}
+
+size_t two_pass_workspace_bytes(const cc_plan* plan, int64_t n_t) {
+    if (n_t < 1) return 0;
+    if (segpair_tma_supported(plan)) {
+        FoldedLayout y;
+        folded_layout(plan, n_t, &y);
+        return y.total;
+    }
+    const int64_t b = two_pass_batch(plan, n_t);
+    CorrLayout y;
+    corr_layout(plan, b, &y);
+    size_t bytes = y.total;
+    if (n_t % b) {   // the last batch may split its segments into more chunks
+        corr_layout(plan, n_t % b, &y);
+        bytes = std::max(bytes, y.total);
+    }
+    return bytes;
+}
+
+template <bool BF16, bool LAG>
+static cudaError_t launch_corr_l(const CorrLayout& y, int sms, cudaStream_t st) {
+    if (!y.half) return launch_corr_t<4096, BF16, LAG, false>(y.a, sms, st);
+    switch (y.L) {
+        case 128: return launch_corr_t<128, BF16, LAG, true>(y.a, sms, st);
+        case 256: return launch_corr_t<256, BF16, LAG, true>(y.a, sms, st);
+        case 512: return launch_corr_t<512, BF16, LAG, true>(y.a, sms, st);
+        case 1024: return launch_corr_t<1024, BF16, LAG, true>(y.a, sms, st);
+        case 2048: return launch_corr_t<2048, BF16, LAG, true>(y.a, sms, st);
+        case 4096: return launch_corr_t<4096, BF16, LAG, true>(y.a, sms, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+static cudaError_t launch_corr(const CorrLayout& y, cudaStream_t st) {
+    const int sms = sm_count();
+    if (y.bf16_rows) return y.planes > 1 ? launch_corr_l<true, true>(y, sms, st) : launch_corr_l<true, false>(y, sms, st);
+    return y.planes > 1 ? launch_corr_l<false, true>(y, sms, st) : launch_corr_l<false, false>(y, sms, st);
+}
+
+cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, float* rho, cudaStream_t st) {
+    if (segpair_tma_supported(plan)) return search_folded_bf16(plan, t_dev, n_t, rho, st);
+    const DevParams& p = plan->dp;
+    const int64_t batch = two_pass_batch(plan, n_t);
+    cc_status s = ensure_workspace(plan, two_pass_workspace_bytes(plan, n_t));
+    if (s != CC_OK) return s;
+    cudaError_t e;
+    for (int64_t t0 = 0; t0 < n_t; t0 += batch) {
+        const int64_t nb = std::min(batch, n_t - t0);
+        CorrLayout y;
+        corr_layout(plan, nb, &y);
+        const int64_t units = (2 * nb + y.T - 1) / y.T * y.C * y.a.n_chunks;
+        if (units > 0x7fffffff) return fail(CC_ERR_UNSUPPORTED, "too many work units in one launch");
+        char* w = (char*)plan->ws;
+        auto take = [&](size_t bytes) {
+            char* r = w;
+            w += bytes;
+            return r;
+        };
+        void* ab = take(y.ab);
+        void* z = take(y.z);
+        float* norm = (float*)take(y.norm);
+        uint8_t* act = (uint8_t*)take(y.act);
+        double* D = (double*)take(y.D);
+        float* raw = (float*)take(y.raw);
+        float* rows2 = (float*)take(y.rows2);
+        float2* U = (float2*)take(y.U);
+        float2* h = (float2*)take(y.h);
+        KnotRec* kn = (KnotRec*)take(y.kn);
+        int* ctr = (int*)take(256);
+        if ((s = launch_knots(plan, t_dev + t0, nb, kn, st, ctr)) != CC_OK) return s;
+        if ((s = launch_resample(plan, t_dev + t0, nb, ab, norm, st, kn, knot_rows(plan), 0, act, (int)y.t_pad)) != CC_OK)
+            return s;
+        cudaEvent_t ev0, ev1;
+        timing_pair(plan, &ev0, &ev1);
+        if (ev0) cudaEventRecord(ev0, st);
+        if (y.folded && (s = launch_fold(plan, nb, ab, act, (int)y.t_pad, (float2*)z, st)) != CC_OK) {
+            if (ev1) cudaEventRecord(ev1, st);
+            return s;
+        }
+        CorrArgs& a = y.a;
+        a.src = y.folded ? z : ab;
+        a.act = act;
+        a.raw = raw;
+        a.ctr = ctr;
+        a.err = p.err;
+        a.twk = y.C == 1 ? plan->corr_twk1 : plan->corr_twk;
+        a.tw8 = y.C == 1 ? plan->corr_tw8_1 : plan->corr_tw8;
+        a.twL = y.L == CORR_POINTS ? plan->corr_tw4096 : plan->corr_twL;
+        a.N_s = p.N_s;
+        a.M = (int)p.M;
+        a.N_tau = p.N_tau;
+        a.n_t = (int)nb;
+        a.t_pad = (int)y.t_pad;
+        a.Q = p.Q;
+        a.C = y.C;
+        a.units = (int)units;
+        a.folded = y.folded;
+        a.all_ordered = p.pair_mode == CC_PAIRS_ALL_ORDERED;
+        a.wait_test = p.wait_test;
+        e = launch_corr(y, st);
+        count_launch();
+        if (ev1) cudaEventRecord(ev1, st);
+        if (e != cudaSuccess) return cuda_fail(e, "pair products launch");
+        LagArgs q;
+        q.raw = raw;
+        q.n_rows = y.n_rows;
+        if (y.n_blocks) {
+            const int64_t len = y.planes * y.G;
+            corr_rows_kernel<<<dim3((unsigned)launch_blocks_for(len, LAG_THREADS), (unsigned)y.n_blocks, (unsigned)nb),
+                               LAG_THREADS, 0, st>>>(raw, y.n_rows, len, rows2);
+            count_launch();
+            q.raw = rows2;
+            q.n_rows = y.n_blocks;
+        }
+        q.U = U;
+        q.h = y.C > 2 ? h : nullptr;
+        q.twL = a.twL;
+        q.norm = (const float4*)norm;
+        q.D = D;
+        q.M = p.M;
+        q.L = y.L;
+        q.log2L = 0;
+        while ((1 << q.log2L) < y.L) ++q.log2L;
+        q.C = y.C;
+        q.planes = y.planes;
+        q.n_lags = y.n_lags;
+        q.N_s = (int)p.N_s;
+        q.Q = p.Q;
+        q.R = (int)p.R;
+        q.pair_mode = p.pair_mode;
+        const size_t sm1 = (size_t)2 * y.L * sizeof(float2), sm2 = (size_t)2 * p.L * sizeof(float2);
+        const int big = (int)(2 * CORR_POINTS * sizeof(float2));
+        if ((e = cudaFuncSetAttribute(corr_lags_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(corr_rho_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess)
+            return cuda_fail(e, "lag kernels smem attribute");
+        corr_lags_kernel<<<dim3((unsigned)(y.C + 1), y.planes > 1 ? 2u : 1u, (unsigned)nb), LAG_THREADS, sm1, st>>>(q);
+        count_launch();
+        if (y.C > 2) {
+            corr_merge_kernel<<<dim3((unsigned)launch_blocks_for(y.n_lags, LAG_THREADS), (unsigned)nb), LAG_THREADS, 0, st>>>(q);
+            count_launch();
+        }
+        corr_rho_kernel<<<dim3((unsigned)p.C, (unsigned)nb), LAG_THREADS, sm2, st>>>(
+            q, p.L, p.log2L, p.twL, p.N_FFT, p.b0, p.coset_off, p.coset_k, p.coset_m, p.N_f, rho + t0 * plan->N_f);
+        count_launch();
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "lag kernels launch");
+    }
+    return CC_OK;
+}
+
+}  // namespace cc

@@ -1,0 +1,471 @@
+// Spectra and pair products of the two-pass search on the lag grid.
+//
+// The pair sum rho_raw(f) = Re sum_P conj(F_K(f)) F_L(f) (Sec. III B 1, Eq.
+// final-formatted-rho) is the Fourier transform of a correlation that lives on a bounded
+// set of lags: a product of two N_s-sample segments has 2 N_s - 1 of them.  So the products
+// need only be known at G >= 2 N_s - 1 equally spaced frequencies omega_j = 2 pi j / G;
+// their sums over segments, an inverse transform to lags and one transform per template to
+// the N_FFT-point output grid (corr.cu) give rho at every output bin, the same value as
+// products taken bin by bin (an exact identity; the rounding differs).  Per segment that is
+// a transform of G = 8192 points for N_s = 3600 instead of the N_FFT = 32768 output grid.
+//
+// With T_K(j) the transform of segment K from its own first sample on, S_K the sum over
+// detectors, the kernel accumulates over segments, per template and weight,
+//   A(j) = sum_K Re(conj(T1_K) T0_K)   (|S_K|^2 with every ordered pair), real,
+//   B(j) = sum_K conj(S_K) S_(K-1)     (R = 1), complex,
+// each in compensated FP32.
+//
+// A CTA of 256 threads holds 4096 points, 16 per thread: T = 4096 / L transforms of L
+// points, each one (template, weight) series (L = 4096: one).  G = L for N_s <= 2048
+// (HALF: the upper half of the transform's input is zero); G = C L with cosets c (frequency
+// j = C m + c, one work unit each) for longer segments, C = 2 up to 4096 samples, folded
+// rows beyond that.
+//
+//   * persistent CTAs, two per SM, take units (series group, chunk of segments, coset) from
+//     one counter; the cosets of a unit are neighbours, so their CTAs read the same rows
+//     from L2.  A unit is computed by one CTA in a fixed order: repeated runs give the same
+//     bits;
+//   * the rows of the next (detector, segment) arrive by cp.async.bulk (TMA) on an mbarrier
+//     under the current transform's later passes (16-byte rows; otherwise by 8- or 4-byte
+//     cp.async);
+//   * the running sums, their compensations and S_(K-1) -- 128 words per thread -- live in
+//     tensor memory, 32 columns per group of four bins, read and written by
+//     tcgen05.ld/st once per segment: registers hold only the transform (16 points), and
+//     detector 0's spectrum, so two CTAs of 128 registers fit an SM without spills;
+//   * twiddles as in the staged kernel: the coset factor of sample s = t + 256 r is split
+//     between a factor per r (first pass) and the table of the second and the powers of the
+//     last pass.
+//
+// What bounds it (L = 4096): the FP32 pipe and the shared-memory exchanges of the two inner
+// passes, each about 1500 cycles per 4096-point transform and SM.
+//
+// Waits are bounded (about one second): a wait that runs out sets bit 0 of the plan's error
+// word; the CTA agrees on it at the next barrier, waits for its copies in flight, frees its
+// tensor memory and returns.
+#pragma once
+
+#include "corr.cuh"
+#include "tma.cuh"
+
+namespace cc {
+
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(slot)), "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_free(uint32_t addr, uint32_t cols) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(cols) : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+#define CC_R8(v, o) "+f"(v[o]), "+f"(v[o + 1]), "+f"(v[o + 2]), "+f"(v[o + 3]), "+f"(v[o + 4]), "+f"(v[o + 5]), "+f"(v[o + 6]), "+f"(v[o + 7])
+#define CC_W8(v, o) "=f"(v[o]), "=f"(v[o + 1]), "=f"(v[o + 2]), "=f"(v[o + 3]), "=f"(v[o + 4]), "=f"(v[o + 5]), "=f"(v[o + 6]), "=f"(v[o + 7])
+#define CC_I8(v, o) "f"(v[o]), "f"(v[o + 1]), "f"(v[o + 2]), "f"(v[o + 3]), "f"(v[o + 4]), "f"(v[o + 5]), "f"(v[o + 6]), "f"(v[o + 7])
+
+// 32 (8) columns of this thread's lane into registers, complete on return, and back.  The
+// wait takes the loaded values as operands, so that no use of them moves above it.
+__device__ __forceinline__ void tmem_ld(float (&v)[32], uint32_t a) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                 : CC_W8(v, 0), CC_W8(v, 8), CC_W8(v, 16), CC_W8(v, 24) : "r"(a) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : CC_R8(v, 0), CC_R8(v, 8), CC_R8(v, 16) :: "memory");
+    asm volatile("" : CC_R8(v, 24) :: "memory");
+}
+__device__ __forceinline__ void tmem_st(uint32_t a, const float (&v)[32]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+                 "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
+                 :: "r"(a), CC_I8(v, 0), CC_I8(v, 8), CC_I8(v, 16), CC_I8(v, 24) : "memory");
+}
+__device__ __forceinline__ void tmem_ld(float (&v)[8], uint32_t a) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : CC_W8(v, 0) : "r"(a) : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : CC_R8(v, 0) :: "memory");
+}
+__device__ __forceinline__ void tmem_st(uint32_t a, const float (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" :: "r"(a), CC_I8(v, 0) : "memory");
+}
+
+// Shape of the transforms of L points.
+template <int LT>
+struct CorrShape {
+    static constexpr int L = LT;
+    static constexpr int T = CORR_POINTS / L;            // transforms per CTA
+    static constexpr int GT = L / 16;                    // threads per transform
+    static constexpr int PL = padded_len(L);
+    static constexpr bool PASS2 = L >= 512;              // a radix-16 pass with NS = 16
+    static constexpr int RL = PASS2 ? L / 256 : L / 16;  // radix of the last pass
+    static constexpr int NSL = L / RL;                   // its butterflies
+    static constexpr int BPT = 16 / RL;                  // of them per thread
+    static constexpr int TA = T > 1 ? T / 2 : 1;         // templates of a series group
+    static_assert(T * GT == CORR_THREADS && NSL == GT * BPT, "16 points per thread in every pass");
+};
+
+// Compensated sums of two FP32 values in paired operations (the same rounding as kahan_add
+// on each): y = v - c, t = s + y, c = (t - s) - y.
+__device__ __forceinline__ void kahan2(float2& s, float2& c, float2 v) {
+    const float2 y = csub(v, c), t = cadd(s, y);
+    c = csub(csub(t, s), y);
+    s = t;
+}
+
+// The TA activity bytes (0 or 1) at p, aligned to TA, of which the first `valid` count, as bits.
+template <int TA>
+__device__ __forceinline__ uint32_t act_bits(const uint8_t* p, int valid) {
+    uint32_t b = 0;
+#pragma unroll
+    for (int i = 0; i < TA; ++i)
+        if (i < valid) b |= (uint32_t)__ldg(p + i) << i;
+    return b;
+}
+
+template <int LT, bool BF16, bool LAG, bool HALF>
+__global__ void __launch_bounds__(CORR_THREADS, CORR_CTAS_PER_SM)
+corr_kernel(const CorrArgs q) {
+    using S = CorrShape<LT>;
+    constexpr int L = S::L, T = S::T, GT = S::GT, PL = S::PL, RL = S::RL, NSL = S::NSL, BPT = S::BPT, TA = S::TA;
+    constexpr int W = LAG ? 32 : 8;                  // tensor-memory words per group of four bins
+    constexpr uint32_t COLS = LAG ? 256 : 64;        // two warps of a lane quarter, four groups each
+    constexpr uint32_t ESZ = BF16 ? 4 : 8;
+    constexpr int PLANES = LAG ? 3 : 1;
+    extern __shared__ __align__(128) unsigned char sm[];
+    unsigned char* stage = sm;
+    uint64_t* bar = (uint64_t*)(sm + q.off_bar);
+    __shared__ int s_unit;
+    __shared__ uint32_t s_tmem;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int g = tid / GT, j = tid % GT;
+    float2* Y = (float2*)(sm + q.off_y) + g * PL;
+    float2* Z = (float2*)(sm + q.off_z) + g * PL;
+    uint32_t* aw = (uint32_t*)(sm + q.off_act);      // per segment of the chunk: activity bits
+    const int C = q.C, M = q.M;
+    const size_t act_x = (size_t)M * q.t_pad;        // bytes of one detector's activity
+
+    if (warp == 0) tmem_alloc(&s_tmem, COLS);
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    // the stage's rows end in zeros up to the transform's input length; no copy reaches them
+    for (int s = q.n_in + j; s < (HALF ? L / 2 : L); s += GT) {
+        if constexpr (BF16) ((uint32_t*)(stage + g * q.row_stride))[s] = 0u;
+        else ((float2*)(stage + g * q.row_stride))[s] = make_float2(0.f, 0.f);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tm_base = s_tmem;
+    const uint32_t tm = tm_base + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * (COLS / 2);
+    const uint32_t own_bit = T > 1 ? 1u << (g >> 1) : 1u;
+    uint32_t phase = 0;
+    bool first_unit = true;
+    bool failed = false;
+
+    for (;;) {
+        if (tid == 0) s_unit = atomicAdd(q.ctr, 1);
+        __syncthreads();
+        const int u = s_unit;
+        if (u >= q.units) break;
+        const int c = u % C, v0 = u / C;
+        const int chunk = v0 % q.n_chunks, sg = v0 / q.n_chunks;
+        const int Ka = chunk * q.chunk_len;
+        const int Kb = min(M, Ka + q.chunk_len);
+        const int Kl = LAG ? max(0, Ka - 1) : Ka;
+        // this thread's series: template t, weight w
+        const int ser = sg * T + g;
+        const int t = ser >> 1, w = ser & 1;
+        const bool valid = t < q.n_t;
+        // activity of the chunk's segments: bit i, template i of the group has weight of
+        // detector 0; bit 16 + i, of the last detector
+        {
+            const int t0 = (sg * T) >> 1, nvalid = min(TA, q.n_t - t0);
+            for (int K = Kl + tid; K < Kb; K += CORR_THREADS) {
+                const uint8_t* p = q.act + (size_t)K * q.t_pad + t0;
+                uint32_t b = act_bits<TA>(p + act_x, nvalid) << 16;
+                if (q.Q > 1) b |= act_bits<TA>(p, nvalid);
+                aw[K - Kl] = b;
+            }
+        }
+        __syncthreads();
+        // the transform after (K, X) in unit order; X = -1 starts at segment K
+        auto next_after = [&](int K, int X, int& nK, int& nX) -> bool {
+            if (X == 0 && q.Q > 1 && (aw[K - Kl] >> 16)) {
+                nK = K;
+                nX = q.Q - 1;
+                return true;
+            }
+            for (int k = X < 0 ? K : K + 1; k < Kb; ++k) {
+                const uint32_t b = aw[k - Kl];
+                if (b) {
+                    nK = k;
+                    nX = (b & 0xffffu) ? 0 : q.Q - 1;
+                    return true;
+                }
+            }
+            return false;
+        };
+        auto row = [&](int K, int X, int tt, int ww) -> const char* {
+            const size_t el = q.folded ? (((((size_t)tt * q.Q + X) * 2 + ww) * M + K) * C + c) * L
+                                       : (((size_t)tt * q.Q + X) * 2 + ww) * q.N_tau + (size_t)K * q.N_s;
+            return (const char*)q.src + el * ESZ;
+        };
+        // copy of the group's rows of the transform after (K, X) into the stage, after a
+        // barrier that ends every read of it.  Rows of a template without weight there are
+        // not copied (nor read).
+        auto issue_after = [&](int K, int X) {
+            int nK, nX;
+            if (q.tma) {
+                if (T == 1) {
+                    if (tid == 0 && next_after(K, X, nK, nX)) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        mbar_arrive_expect_tx(bar, q.row_bytes);
+                        tma_load_1d(stage, row(nK, nX, t, w), q.row_bytes, bar);
+                    }
+                } else if (warp == 0 && next_after(K, X, nK, nX)) {
+                    const int s2 = sg * T + lane, tt = s2 >> 1;
+                    const uint32_t b = aw[nK - Kl] >> (nX == q.Q - 1 ? 16 : 0);
+                    const bool on = lane < T && ((b >> (lane >> 1)) & 1u);
+                    const int n = __popc(__ballot_sync(0xffffffffu, on));
+                    if (lane == 0) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        mbar_arrive_expect_tx(bar, (uint32_t)n * q.row_bytes);
+                    }
+                    __syncwarp();
+                    if (on) tma_load_1d(stage + lane * q.row_stride, row(nK, nX, tt, s2 & 1), q.row_bytes, bar);
+                }
+            } else {
+                if (next_after(K, X, nK, nX) && ((aw[nK - Kl] >> (nX == q.Q - 1 ? 16 : 0)) & own_bit)) {
+                    const char* src = row(nK, nX, t, w);
+                    unsigned char* dst = stage + g * q.row_stride;
+                    for (int s = j; s < q.n_in; s += GT) cp_async<ESZ>(dst + s * ESZ, src + s * ESZ);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            }
+        };
+
+        {   // zero sums
+            float z[W];
+#pragma unroll
+            for (int i = 0; i < W; ++i) z[i] = 0.f;
+#pragma unroll
+            for (int gi = 0; gi < 4; ++gi) tmem_st(tm + gi * W, z);
+        }
+        // last pass of L = 4096: e, 2 e, 4 e and 8 e-th powers of W_G^(c + C tid)
+        const float4* __restrict__ tw8 = q.tw8 + ((size_t)c * CORR_THREADS + j) * 2;
+        const float2* __restrict__ twk = q.twk + (size_t)c * 272;
+
+        if (!(q.wait_test && first_unit)) issue_after(Kl, -1);
+        first_unit = false;
+        bool prev_zero = true;
+        int parity = 0;
+
+        for (int K = Kl; K < Kb; ++K) {
+            const uint32_t bits = aw[K - Kl];
+            if (!bits) {
+                prev_zero = true;
+                continue;
+            }
+            const bool a0 = (bits & 0xffffu) != 0, al = (bits >> 16) != 0;
+            float2 v[16], f0[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = make_float2(0.f, 0.f);
+#pragma unroll 1
+            for (int pass = a0 ? 0 : 1; pass < (al ? 2 : 1); ++pass) {
+                if (pass == 1) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) f0[e] = v[e];   // detector 0's spectrum (zero without weight)
+                }
+                bool ok = true;
+                if (q.tma) {
+                    ok = mbar_wait(bar, phase);
+                    phase ^= 1;
+                } else {
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    __syncthreads();
+                }
+                // first pass: sample s = j + r GT of the segment
+                const unsigned char* st = stage + g * q.row_stride;
+#pragma unroll
+                for (int r = 0; r < (HALF ? 8 : 16); ++r) {
+                    if constexpr (BF16) v[r] = __bfloat1622float2(((const __nv_bfloat162*)st)[j + r * GT]);
+                    else v[r] = ((const float2*)st)[j + r * GT];
+                }
+                if (T > 1 && !((pass == 0 ? bits : bits >> 16) & own_bit)) {   // no weight: the row was not copied
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) v[r] = make_float2(0.f, 0.f);
+                }
+                // buffers alternate between transforms when there is no second pass
+                float2* buf = S::PASS2 || parity == 0 ? Y : Z;
+                parity ^= 1;
+                if constexpr (HALF) {
+                    dft16_in8(v);
+                } else {
+                    if (c > 0) {
+#pragma unroll
+                        for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(twk + r));
+                    }
+                    dft16(v);
+                }
+                {
+                    float2* d = buf + 17 * j;   // padi(16 j + r)
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) d[r] = v[r];
+                }
+                // every thread has read the stage and written its outputs; all agree on a failed wait
+                if (__syncthreads_or(!ok)) {
+                    failed = true;
+                    break;
+                }
+                issue_after(K, pass == 0 && q.Q > 1 ? 0 : q.Q - 1);
+                const float2* src = buf;
+                if constexpr (S::PASS2) {
+                    const int k = j & 15;
+                    const float2* s = Y + padi(j);
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) v[r] = s[r * pstride<S::PASS2 ? GT : 16>()];
+#pragma unroll
+                    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(twk + 16 + r * 16 + k));
+                    dft16(v);
+                    float2* d = Z + padi((j - k) * 16 + k);
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) d[r * pstride<16>()] = v[r];
+                    __syncthreads();
+                    src = Z;
+                }
+                // last pass into registers: butterfly b = j + GT i leaves outputs m = b + NSL r
+                // in v[i RL + r]
+                if constexpr (L == 4096) {
+                    const float2* s = src + padi(j);
+                    const float4 p0 = __ldg(tw8), p1 = __ldg(tw8 + 1);
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) v[r] = s[r * pstride<256>()];
+                    const float2 b1 = make_float2(p0.x, p0.y), b2 = make_float2(p0.z, p0.w);
+                    const float2 b4 = make_float2(p1.x, p1.y), b8 = make_float2(p1.z, p1.w);
+                    const float2 b3 = cmul(b2, b1), b12 = cmul(b8, b4);
+                    v[1] = cmul(v[1], b1);
+                    v[2] = cmul(v[2], b2);
+                    v[3] = cmul(v[3], b3);
+                    v[4] = cmul(v[4], b4);
+                    v[5] = cmul(v[5], cmul(b4, b1));
+                    v[6] = cmul(v[6], cmul(b4, b2));
+                    v[7] = cmul(v[7], cmul(b4, b3));
+                    v[8] = cmul(v[8], b8);
+                    v[9] = cmul(v[9], cmul(b8, b1));
+                    v[10] = cmul(v[10], cmul(b8, b2));
+                    v[11] = cmul(v[11], cmul(b8, b3));
+                    v[12] = cmul(v[12], b12);
+                    v[13] = cmul(v[13], cmul(b12, b1));
+                    v[14] = cmul(v[14], cmul(b12, b2));
+                    v[15] = cmul(v[15], cmul(b12, b3));
+                    dft16(v);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < BPT; ++i) {
+                        const int b = j + GT * i;
+                        const float2* s = src + padi(b);
+                        float2 x[16];
+#pragma unroll
+                        for (int r = 0; r < RL; ++r) x[r] = s[r * pstride<NSL>()];
+                        apply_twiddles<RL>(x, q.twL, b, L - 1);
+                        dft_r<RL>(x);
+#pragma unroll
+                        for (int r = 0; r < RL; ++r) v[i * RL + r] = x[r];
+                    }
+                }
+            }
+            if (failed) break;
+            if (!al) {   // the last detector has no weight
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    f0[e] = v[e];
+                    v[e] = make_float2(0.f, 0.f);
+                }
+            }
+            // pair terms of segment K
+            const bool acc_on = !LAG || K >= Ka;
+            tmem_wait_st();
+#pragma unroll
+            for (int gi = 0; gi < 4; ++gi) {
+                float z[W];
+                tmem_ld(z, tm + gi * W);   // A[4], its compensation[4]; B[4] re im, compensation, S of segment K - 1
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int e = 4 * gi + 2 * h;
+                    const float2 S0 = cadd(f0[e], v[e]), S1 = cadd(f0[e + 1], v[e + 1]);
+                    if (acc_on) {
+                        const float2 d = q.all_ordered ? make_float2(redot(S0, S0), redot(S1, S1))
+                                                       : make_float2(redot(v[e], f0[e]), redot(v[e + 1], f0[e + 1]));
+                        float2 s = make_float2(z[2 * h], z[2 * h + 1]), cp = make_float2(z[4 + 2 * h], z[5 + 2 * h]);
+                        kahan2(s, cp, d);
+                        z[2 * h] = s.x;
+                        z[2 * h + 1] = s.y;
+                        z[4 + 2 * h] = cp.x;
+                        z[5 + 2 * h] = cp.y;
+                    }
+                    if constexpr (LAG) {
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            float* zb = z + 8 + 6 * (2 * h + i);
+                            const float2 Sk = i == 0 ? S0 : S1;
+                            if (acc_on && !prev_zero) {
+                                const float2 d = make_float2(fmaf(Sk.x, zb[4], Sk.y * zb[5]), fmaf(Sk.x, zb[5], -Sk.y * zb[4]));
+                                float2 s = make_float2(zb[0], zb[1]), cp = make_float2(zb[2], zb[3]);
+                                kahan2(s, cp, d);
+                                zb[0] = s.x;
+                                zb[1] = s.y;
+                                zb[2] = cp.x;
+                                zb[3] = cp.y;
+                            }
+                            zb[4] = Sk.x;
+                            zb[5] = Sk.y;
+                        }
+                    }
+                }
+                tmem_st(tm + gi * W, z);
+            }
+            prev_zero = false;
+        }
+        if (failed) break;
+        // the unit's sums to its row
+        tmem_wait_st();
+        float* out = q.raw + (((size_t)t * 2 * q.n_chunks + (size_t)w * q.n_chunks + chunk) * PLANES * C + c) * L;
+        const size_t plane = (size_t)C * L;
+#pragma unroll
+        for (int gi = 0; gi < 4; ++gi) {
+            float z[W];
+            tmem_ld(z, tm + gi * W);
+            if (valid) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int e = 4 * gi + i, m = j + GT * (e / RL) + NSL * (e % RL);
+                    out[m] = z[i];
+                    if constexpr (LAG) {
+                        out[plane + m] = z[8 + 6 * i];
+                        out[2 * plane + m] = z[8 + 6 * i + 1];
+                    }
+                }
+            }
+        }
+        __syncthreads();   // every thread has taken this unit's number and left the last transform's buffers
+    }
+    if (failed && tid == 0) {
+        atomicOr(q.err, 1u);
+        mbar_wait(bar, phase ^ 1);   // the copy still in flight, bounded
+    }
+    __syncthreads();
+    if (warp == 0) tmem_free(tm_base, COLS);
+}
+
+template <int LT, bool BF16, bool LAG, bool HALF>
+cudaError_t launch_corr_t(const CorrArgs& a, int sms, cudaStream_t st) {
+    auto kern = corr_kernel<LT, BF16, LAG, HALF>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
+    if (e != cudaSuccess) return e;
+    const int grid = a.units < CORR_CTAS_PER_SM * sms ? a.units : CORR_CTAS_PER_SM * sms;
+    kern<<<grid, CORR_THREADS, a.smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace cc

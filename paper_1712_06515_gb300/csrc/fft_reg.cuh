@@ -33,13 +33,18 @@ __device__ __forceinline__ void dft2(float2& a, float2& b) {
     b = csub(t, b);
 }
 
+// a - i b and a + i b, component by component: the swapped, negated operand costs nothing there
+// (a paired sum would need it assembled in registers first)
+__device__ __forceinline__ float2 cadd_negi(float2 a, float2 b) { return make_float2(a.x + b.y, a.y - b.x); }
+__device__ __forceinline__ float2 cadd_posi(float2 a, float2 b) { return make_float2(a.x - b.y, a.y + b.x); }
+
 // forward 4-point DFT in place, natural order
 __device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2& a3) {
-    const float2 s0 = cadd(a0, a2), d0 = csub(a0, a2), s1 = cadd(a1, a3), d1 = mul_negi(csub(a1, a3));
+    const float2 s0 = cadd(a0, a2), d0 = csub(a0, a2), s1 = cadd(a1, a3), t = csub(a1, a3);
     a0 = cadd(s0, s1);
     a2 = csub(s0, s1);
-    a1 = cadd(d0, d1);
-    a3 = csub(d0, d1);
+    a1 = cadd_negi(d0, t);
+    a3 = cadd_posi(d0, t);
 }
 
 // multiplication by exp(-2 pi i e / 16) for the constant exponents of the 4x4 split
@@ -55,10 +60,9 @@ __device__ __forceinline__ float2 w16(float2 a) {
 }
 
 // 16-point DFT: n = 4 n1 + n2, k = k1 + 4 k2; inner 4-point DFTs over n1, twiddles
-// W16^(n2 k1), outer 4-point DFTs over n2.  Result in natural order.
-__device__ __forceinline__ void dft16(float2 (&v)[16]) {
-#pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) dft4(v[n2], v[n2 + 4], v[n2 + 8], v[n2 + 12]);
+// W16^(n2 k1), outer 4-point DFTs over n2.  Result in natural order.  dft16_outer: the part
+// after the inner DFTs.
+__device__ __forceinline__ void dft16_outer(float2 (&v)[16]) {
     // v[n2 + 4 k1] = Y[n2][k1]
     v[5] = w16<1>(v[5]);
     v[9] = w16<2>(v[9]);
@@ -79,6 +83,26 @@ __device__ __forceinline__ void dft16(float2 (&v)[16]) {
         for (int k2 = 0; k2 < 4; ++k2) t[k1 + 4 * k2] = v[4 * k1 + k2];
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = t[i];
+}
+
+__device__ __forceinline__ void dft16(float2 (&v)[16]) {
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) dft4(v[n2], v[n2 + 4], v[n2 + 8], v[n2 + 12]);
+    dft16_outer(v);
+}
+
+// The 16-point DFT of an input whose upper half is zero: v[0..7] given, v[8..15] not read.
+// The inner DFTs over (v[n2], v[n2 + 4], 0, 0) take half the sums.
+__device__ __forceinline__ void dft16_in8(float2 (&v)[16]) {
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) {
+        const float2 a = v[n2], b = v[n2 + 4];
+        v[n2] = cadd(a, b);
+        v[n2 + 4] = cadd_negi(a, b);
+        v[n2 + 8] = csub(a, b);
+        v[n2 + 12] = cadd_posi(a, b);
+    }
+    dft16_outer(v);
 }
 
 // The 16-point DFT of dft16 restricted to its outputs X[0..7], left in v[0..7] (v[8..15]

@@ -101,7 +101,7 @@ bool fused_layout(const cc_plan* plan, int64_t n_t, FusedLayout* lay) {
 // detectors (it depends on the source time only); the barycentric part per detector.
 __global__ void __launch_bounds__(256)
 knots_kernel(DevParams p, const cc_template* __restrict__ tm, int64_t t_base, int64_t nkn,
-             KnotRec* __restrict__ out) {
+             KnotRec* __restrict__ out, int* __restrict__ zero_word) {
     __shared__ double dk[CC_MAX_DET][256 + 3];
     __shared__ Orbit orb_s;
     const int Q = p.Q;
@@ -109,6 +109,8 @@ knots_kernel(DevParams p, const cc_template* __restrict__ tm, int64_t t_base, in
     const int64_t k0 = (int64_t)blockIdx.x * 256;
     // the orbit's FP64 set-up (a reciprocal, and trigonometry for e != 0) once per block
     if (threadIdx.x == 0) orb_s = make_orbit(p, tm[t]);
+    // a later kernel's unit counter, cleared here instead of by a memset of its own
+    if (zero_word && threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.z == 0) *zero_word = 0;
     __syncthreads();
     const Orbit orb = orb_s;
     for (int i = threadIdx.x; i < 256 + 3; i += 256) {
@@ -128,13 +130,14 @@ knots_kernel(DevParams p, const cc_template* __restrict__ tm, int64_t t_base, in
 int64_t knot_rows(const cc_plan* plan) { return (plan->N_tau + KNOT - 1) / KNOT; }
 
 // Knot records of templates t_dev[0 .. n_t) into kn ([n_t][Q][knot_rows]).
-cc_status launch_knots(cc_plan* plan, const cc_template* t_dev, int64_t n_t, KnotRec* kn, cudaStream_t st) {
+cc_status launch_knots(cc_plan* plan, const cc_template* t_dev, int64_t n_t, KnotRec* kn, cudaStream_t st,
+                       int* zero_word) {
     const DevParams& p = plan->dp;
     const int64_t nkn = knot_rows(plan);
     for (int64_t t0 = 0; t0 < n_t; t0 += 65535) {
         const int64_t nt = std::min<int64_t>(65535, n_t - t0);
         dim3 gk((unsigned)((nkn + 255) / 256), 1u, (unsigned)nt);
-        knots_kernel<<<gk, 256, 0, st>>>(p, t_dev + t0, 0, nkn, kn + (size_t)t0 * p.Q * nkn);
+        knots_kernel<<<gk, 256, 0, st>>>(p, t_dev + t0, 0, nkn, kn + (size_t)t0 * p.Q * nkn, zero_word);
         count_launch();
     }
     cudaError_t e = cudaGetLastError();
@@ -183,7 +186,7 @@ cc_status launch_fused(cc_plan* plan, const cc_template* t_dev, int64_t n_t, flo
         const int64_t nt = std::min(step, n_t - tb);
         if (pre) {
             dim3 gk((unsigned)((nkn + 255) / 256), 1u, (unsigned)nt);
-            knots_kernel<<<gk, 256, 0, st>>>(p, t_dev, tb, nkn, kn_ws);
+            knots_kernel<<<gk, 256, 0, st>>>(p, t_dev, tb, nkn, kn_ws, nullptr);
             count_launch();
         }
         cudaLaunchConfig_t cfg = {};

@@ -1,12 +1,17 @@
-// Spectrum + pair-sum kernel of the two-pass search for coset length L = 4096 (the
-// 120-day single band: N_FFT = 32768 = 8 cosets of 4096, N_s = 3600 samples per
-// segment): a persistent kernel whose segment samples arrive by TMA bulk copies.
+// Spectra and pair sums at the output bins on 4096-point cosets: a persistent kernel whose
+// segment samples arrive by TMA bulk copies.  Two users:
+//   * the two-pass search of segments longer than 4096 samples stored in BF16 (the long-lag
+//     band): the folded rows are rounded to BF16 per output coset, so the products belong to
+//     these cosets' bins; every other two-pass search sums its products on the lag grid
+//     (corr_kernel.cuh), about a quarter of the transform work;
+//   * with SPECTRA set, the staged segment-FFT stage (whole segments, e.g. the 120-day single
+//     band: N_FFT = 32768 = 8 cosets of 4096, N_s = 3600 samples per segment).
 //
 // Per (template, weight, chunk of segments, coset) unit a CTA walks the chunk's
 // segments; per segment it transforms detector 0's and detector 1's samples (each the
 // zero-padded N_FFT-point DFT restricted to coset c, Sec. III B 4: an L-point transform
 // of the samples times exp(-2 pi i (b0 + c) s / N_FFT)) and folds the two spectra into
-// the pair sum of Eq. final-formatted-rho, as segpair_kernel does.  What differs:
+// the pair sum of Eq. final-formatted-rho:
 //
 //   * staging: the N_s samples of the next (detector, segment) transform are copied
 //     from HBM/L2 into shared memory by one cp.async.bulk (TMA, completion on an
@@ -44,6 +49,7 @@
 #include <algorithm>
 
 #include "segpair.cuh"
+#include "tma.cuh"
 
 namespace cc {
 
@@ -51,50 +57,8 @@ namespace {
 
 constexpr int TT_THREADS = 256;
 constexpr int TT_L = 4096;
-constexpr long long WAIT_LIMIT_CYCLES = 2000000000LL;   // ~1 s at 2 GHz
 constexpr int FOLD_MAX_F = 16;     // folds of a long segment onto the 4096 positions
 constexpr int FOLD_MAX_C = 1024;   // cosets of a folded plan
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait for the phase with the given parity; false when the limit ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity))
-        if (clock64() - t0 > WAIT_LIMIT_CYCLES) return false;
-    return true;
-}
-
-// 1-D bulk copy global -> shared (16-byte aligned addresses, size a multiple of 16),
-// completing `bytes` transactions on the mbarrier.
-__device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(bar))
-                 : "memory");
-}
 
 __device__ __forceinline__ unsigned sm_id() {
     unsigned id;
@@ -409,10 +373,9 @@ segpair_tma_kernel(DevParams p, TmaWork q, const void* __restrict__ ab, const fl
 // every q, instead of each coset re-reading and re-twiddling the whole segment.  The
 // persistent kernel applies W_N^((b0+c) p) as it does for whole segments.
 // grid: x = segment K, y = detector X * 2 + weight w, z = template of the batch.
-// ab: [n_t][Q][2][N_tau], z: [n_t][Q][2][M][C][L] (both in the plan's storage type).
-template <bool BF16>
+// ab: [n_t][Q][2][N_tau], z: [n_t][Q][2][M][C][L], bf16 pairs.
 __global__ void __launch_bounds__(TT_THREADS)
-fold_kernel(DevParams p, const void* __restrict__ ab, const float4* __restrict__ norm, void* __restrict__ z) {
+fold_cosets_kernel(DevParams p, const void* __restrict__ ab, const float4* __restrict__ norm, void* __restrict__ z) {
     __shared__ float2 wc[FOLD_MAX_C];   // W_C^n
     constexpr int L = TT_L;
     const int64_t K = blockIdx.x;
@@ -439,8 +402,7 @@ fold_kernel(DevParams p, const void* __restrict__ ab, const float4* __restrict__
             const int64_t sidx = pp + (int64_t)f * L;
             a[f] = make_float2(0.f, 0.f);
             if (f < F && sidx < N_s) {
-                if constexpr (BF16) a[f] = __bfloat1622float2(((const __nv_bfloat162*)ab)[row + sidx]);
-                else a[f] = __ldg((const float2*)ab + row + sidx);
+                a[f] = __bfloat1622float2(((const __nv_bfloat162*)ab)[row + sidx]);
             }
         }
         for (int qq = 0; qq < C; ++qq) {
@@ -449,18 +411,17 @@ fold_kernel(DevParams p, const void* __restrict__ ab, const float4* __restrict__
             for (int f = 1; f < FOLD_MAX_F; ++f)
                 if (f < F) acc = cadd(acc, cmul(a[f], wc[(qq * f) & (C - 1)]));
             const size_t o = zrow + (size_t)qq * L + pp;
-            if constexpr (BF16) ((__nv_bfloat162*)z)[o] = __float22bfloat162_rn(acc);
-            else ((float2*)z)[o] = acc;
+            ((__nv_bfloat162*)z)[o] = __float22bfloat162_rn(acc);
         }
     }
 }
 
-// fold_kernel for C = 64 cosets (the long-lag band: N_FFT = 2^18 = 64 x 4096) and at most
+// fold_cosets_kernel for C = 64 cosets (the long-lag band: N_FFT = 2^18 = 64 x 4096) and at most
 // 16 folds, by a radix-8 split of the 64-point DFT over the fold index: with q = u + 8 v
 // and f = f1 + 8 f2, W_64^(q f) = W_8^(v f1) W_64^(u f1) W_8^(u f2), so
 // Z_(u+8v) = DFT8_v[ W_64^(u f1) (a_(f1) + a_(f1+8) W_8^u) ]: per residue u a twiddle and
 // one register 8-point DFT instead of 64 x F products.
-template <bool BF16, int MAXF>
+template <int MAXF>
 __global__ void __launch_bounds__(TT_THREADS, 3)
 fold64_kernel(DevParams p, const void* __restrict__ ab, const float4* __restrict__ norm, void* __restrict__ z) {
     static_assert(MAXF > 8 && MAXF <= 16, "folds f = f1 + 8 f2 with f2 < 2");
@@ -486,8 +447,7 @@ fold64_kernel(DevParams p, const void* __restrict__ ab, const float4* __restrict
             const int64_t sidx = pp + (int64_t)f * L;
             a[f] = make_float2(0.f, 0.f);
             if (f < F && sidx < N_s) {
-                if constexpr (BF16) a[f] = __bfloat1622float2(((const __nv_bfloat162*)ab)[row + sidx]);
-                else a[f] = __ldg((const float2*)ab + row + sidx);
+                a[f] = __bfloat1622float2(((const __nv_bfloat162*)ab)[row + sidx]);
             }
         }
 #pragma unroll
@@ -503,8 +463,7 @@ fold64_kernel(DevParams p, const void* __restrict__ ab, const float4* __restrict
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const size_t o = zrow + (size_t)(u + 8 * j) * L + pp;
-                if constexpr (BF16) ((__nv_bfloat162*)z)[o] = __float22bfloat162_rn(v[j]);
-                else ((float2*)z)[o] = v[j];
+                ((__nv_bfloat162*)z)[o] = __float22bfloat162_rn(v[j]);
             }
         }
     }
@@ -548,18 +507,15 @@ int occupancy(size_t smem) {
 
 }  // namespace
 
-// Coset length 4096, segments of an even number of samples (a multiple of 4 with BF16
-// storage: rows then start on 16-byte boundaries for the bulk copies), Q <= 2, R <= 1, the
-// output bins in the lower half of each coset transform; segments longer than 4096
-// samples are folded first (at most FOLD_MAX_F folds and FOLD_MAX_C cosets).
+// Folded segments in BF16: more than 4096 samples, a multiple of 4 (rows then start on 16-byte
+// boundaries for the bulk copies), at most FOLD_MAX_F folds and FOLD_MAX_C cosets, Q <= 2,
+// R <= 1, the output bins in the lower half of each coset transform.
 bool segpair_tma_supported(const cc_plan* plan) {
     const DevParams& p = plan->dp;
-    const bool padded = p.L < TT_L && plan->tuning.transform_len == TT_L && p.C4 > 0;   // N_s <= L < 4096
-    if ((p.L != TT_L && !padded) || p.Q > 2 || p.R > 1 || p.pair_mode == CC_PAIRS_CROSS_ONLY || plan->N_f < 1)
+    if (p.store != CC_STORE_BF16 || p.N_s <= TT_L || p.L != TT_L || p.Q > 2 || p.R > 1 ||
+        p.pair_mode == CC_PAIRS_CROSS_ONLY || plan->N_f < 1)
         return false;
-    if (p.N_s > TT_L && (p.C4 > FOLD_MAX_C || (p.N_s + TT_L - 1) / TT_L > FOLD_MAX_F)) return false;
-    // rows start on 16-byte boundaries for the bulk copies
-    if (p.N_s % (p.store == CC_STORE_BF16 ? 4 : 2)) return false;
+    if (p.C4 > FOLD_MAX_C || (p.N_s + TT_L - 1) / TT_L > FOLD_MAX_F || p.N_s % 4) return false;
     TmaWork q;
     size_t bytes;
     if (!tma_layout(plan, &q, &bytes)) return false;
@@ -580,48 +536,39 @@ int segpair_tma_chunks(const cc_plan* plan, int64_t n_t) {
     return (int)std::max<int64_t>(1, std::min<int64_t>({want, maxch, 32767}));
 }
 
-bool segpair_tma_folded(const cc_plan* plan) { return plan->dp.N_s > TT_L; }
-
-// Bytes of the fold kernel's output per template (0 for whole segments).
+// Bytes of the fold kernel's output per template.
 size_t segpair_tma_fold_bytes(const cc_plan* plan) {
-    if (!segpair_tma_folded(plan)) return 0;
     const DevParams& p = plan->dp;
-    return (size_t)p.Q * 2 * p.M * p.C4 * TT_L * (p.store == CC_STORE_BF16 ? 4 : 8);
+    return (size_t)p.Q * 2 * p.M * p.C4 * TT_L * 4;
 }
 
-cc_status launch_fold(cc_plan* plan, int64_t n_t, const void* ab, const float4* norm, void* z, cudaStream_t st) {
+cc_status launch_fold_bf16(cc_plan* plan, int64_t n_t, const void* ab, const float4* norm, void* z, cudaStream_t st) {
     const DevParams& p = plan->dp;
     if (n_t > 65535 || p.M > 0x7fffffff) return fail(CC_ERR_UNSUPPORTED, "fold launch size");
     const dim3 grid((unsigned)p.M, (unsigned)(2 * p.Q), (unsigned)n_t);
-    const bool bf16 = p.store == CC_STORE_BF16;
     const int64_t F = (p.N_s + TT_L - 1) / TT_L;
-    if (p.C4 == 64 && F <= 9) {   // the long-lag band: nine folds
-        if (bf16) fold64_kernel<true, 9><<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
-        else fold64_kernel<false, 9><<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
-    } else if (p.C4 == 64) {
-        if (bf16) fold64_kernel<true, 16><<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
-        else fold64_kernel<false, 16><<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
-    } else {
-        if (bf16) fold_kernel<true><<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
-        else fold_kernel<false><<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
-    }
+    if (p.C4 == 64 && F <= 9)   // the long-lag band: nine folds
+        fold64_kernel<9><<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
+    else if (p.C4 == 64)
+        fold64_kernel<16><<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
+    else
+        fold_cosets_kernel<<<grid, TT_THREADS, 0, st>>>(p, ab, norm, z);
     count_launch();
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? CC_OK : cuda_fail(e, "fold launch");
 }
 
-cc_status launch_segpair_tma(cc_plan* plan, const SegPairLayout& lay, int64_t n_t, const void* ab,
+cc_status launch_segpair_tma(cc_plan* plan, int n_chunks, int64_t chunk_len, int64_t n_t, const void* ab,
                              const float4* norm, float* raw, int* counters, cudaStream_t st) {
     const DevParams& p = plan->dp;
     TmaWork q;
     size_t bytes;
     if (!tma_layout(plan, &q, &bytes)) return fail(CC_ERR_UNSUPPORTED, "segpair_tma layout");
-    q.n_chunks = lay.n_chunks;
-    q.chunk_len = lay.chunk_len;
-    q.units = n_t * 2 * lay.n_chunks;
+    q.n_chunks = n_chunks;
+    q.chunk_len = chunk_len;
+    q.units = n_t * 2 * n_chunks;
     if (q.units > 0x7fffffff) return fail(CC_ERR_UNSUPPORTED, "too many work units in one launch");
-    const bool bf16 = p.store == CC_STORE_BF16;
-    const int occ = bf16 ? occupancy<true, false>(bytes) : occupancy<false, false>(bytes);
+    const int occ = occupancy<true, false>(bytes);
     if (occ < 1) return fail(CC_ERR_UNSUPPORTED, "segpair_tma kernel does not fit an SM");
     int dev = 0, sms = 152;
     cudaError_t e = cudaGetDevice(&dev);
@@ -630,12 +577,7 @@ cc_status launch_segpair_tma(cc_plan* plan, const SegPairLayout& lay, int64_t n_
     const int64_t grid = std::min<int64_t>((int64_t)occ * sms, q.units * p.C4);
     if ((e = cudaMemsetAsync(counters, 0, sizeof(int) * p.C4, st)) != cudaSuccess)
         return cuda_fail(e, "unit counters");
-    if (bf16)
-        segpair_tma_kernel<true, false><<<(unsigned)grid, TT_THREADS, bytes, st>>>(p, q, ab, norm, raw, counters,
-                                                                                  nullptr);
-    else
-        segpair_tma_kernel<false, false><<<(unsigned)grid, TT_THREADS, bytes, st>>>(p, q, ab, norm, raw, counters,
-                                                                                   nullptr);
+    segpair_tma_kernel<true, false><<<(unsigned)grid, TT_THREADS, bytes, st>>>(p, q, ab, norm, raw, counters, nullptr);
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "segpair_tma launch");

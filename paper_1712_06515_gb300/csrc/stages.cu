@@ -62,14 +62,16 @@ __host__ __device__ inline int resample_window_len(const DevParams& p) {
 // of the pre-pass, [n_t][Q][nkn]) the FP64 knots are not recomputed, and a segment whose
 // detector times all fall in gaps is skipped: its norms are written as zero and its
 // a_r, b_r are written as zero (`write_inactive`, the staged stage: every weight there is
-// zero) or left unwritten (the two-pass search reads a segment only when its norms are
-// nonzero).  Without `kn` every sample is computed.  The parameter block comes last: with
+// zero) or left unwritten (the two-pass search reads a segment only when its flag is
+// nonzero); `act` (two-pass search, Q <= 2; [2][M][t_pad] bytes, detector 0 and the last one)
+// receives whether the segment was computed.  Without `kn` every sample is computed.  The parameter block comes last: with
 // it first, the offsets of the small parameters after it moved with its size, and at some
 // sizes the two-pass variant compiled to 52 registers instead of 32 and ran 15 % slower.
 template <int DT, bool PRE>
 __global__ void __launch_bounds__(RS_THREADS)
 resample_kernel(const cc_template* __restrict__ tm, int64_t t_base, void* ab, float4* __restrict__ norm,
-                const KnotRec* __restrict__ kn, int64_t nkn, int use_window, int write_inactive, DevParams p) {
+                const KnotRec* __restrict__ kn, int64_t nkn, int use_window, int write_inactive,
+                uint8_t* __restrict__ act, int t_pad, DevParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float red[32];
     __shared__ int active;
@@ -119,6 +121,7 @@ resample_kernel(const cc_template* __restrict__ tm, int64_t t_base, void* ab, fl
             }
         }
         __syncthreads();
+        if (act && tid == 0) act[((X == p.Q - 1 ? p.M : 0) + K) * t_pad + t] = active != 0;
         if (!active) {
             if (tid == 0) norm[(t * p.Q + X) * p.M + K] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (write_inactive) {
@@ -446,7 +449,8 @@ size_t resample_smem_bytes(const DevParams& p, bool window) {
 }
 
 cc_status launch_resample(cc_plan* plan, const cc_template* t_dev, int64_t n_t, void* ab,
-                          float* norm, cudaStream_t st, const KnotRec* kn, int64_t nkn, int write_inactive) {
+                          float* norm, cudaStream_t st, const KnotRec* kn, int64_t nkn, int write_inactive,
+                          uint8_t* act, int t_pad) {
     const DevParams& p = plan->dp;
     // with knot records, the segment's window of x is staged in shared memory when it
     // leaves room for several blocks per SM
@@ -464,14 +468,16 @@ cc_status launch_resample(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
     for (int64_t t0 = 0; t0 < n_t; t0 += MAX_GRID_YZ) {
         const int64_t nt = std::min<int64_t>(MAX_GRID_YZ, n_t - t0);
         dim3 grid((unsigned)p.M, (unsigned)p.Q, (unsigned)nt);
-        kern<<<grid, RS_THREADS, sm, st>>>(t_dev, t0, ab, (float4*)norm, kn, nkn, use_window, write_inactive, p);
+        kern<<<grid, RS_THREADS, sm, st>>>(t_dev, t0, ab, (float4*)norm, kn, nkn, use_window, write_inactive,
+                                           act, t_pad, p);
         count_launch();
     }
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? CC_OK : cuda_fail(e, "resample launch");
 }
 
-cc_status launch_knots(cc_plan* plan, const cc_template* t_dev, int64_t n_t, KnotRec* kn, cudaStream_t st);
+cc_status launch_knots(cc_plan* plan, const cc_template* t_dev, int64_t n_t, KnotRec* kn, cudaStream_t st,
+                       int* zero_word = nullptr);
 
 // Knot records of one template's detectors, bytes.
 size_t knot_bytes_per_template(const cc_plan* plan) {
@@ -491,7 +497,7 @@ cc_status resample_with_knots(cc_plan* plan, const cc_template* t_dev, int64_t n
         const int64_t nc = std::min(kbatch, n_t - c0);
         cc_status s = launch_knots(plan, t_dev + c0, nc, kn, st);
         if (s != CC_OK) return s;
-        s = launch_resample(plan, t_dev + c0, nc, (char*)ab + ab_t * c0, norm + nm_t * c0, st, kn, nkn, 1);
+        s = launch_resample(plan, t_dev + c0, nc, (char*)ab + ab_t * c0, norm + nm_t * c0, st, kn, nkn, 1, nullptr, 0);
         if (s != CC_OK) return s;
     }
     return CC_OK;
@@ -637,7 +643,7 @@ cc_status crosscorr_resample(cc_plan* plan, const void* const* x_dev, const cc_t
         kbatch = std::max<int64_t>(1, std::min<int64_t>(n_t, (int64_t)(KNOT_WS_BUDGET / krow)));
         if ((s = ensure_workspace(plan, krow * kbatch)) != CC_OK) return s;
     }
-    if (kbatch < 1) return launch_resample(plan, t_dev, n_t, ab_dev, norm_dev, (cudaStream_t)stream, nullptr, 0, 0);
+    if (kbatch < 1) return launch_resample(plan, t_dev, n_t, ab_dev, norm_dev, (cudaStream_t)stream, nullptr, 0, 0, nullptr, 0);
     return resample_with_knots(plan, t_dev, n_t, ab_dev, norm_dev, (cudaStream_t)stream, (KnotRec*)plan->ws, kbatch);
 }
 

@@ -1,0 +1,66 @@
+"""Parity of the two-pass search on the lag grid (corr_kernel and the transforms after it)
+against the FP64 oracle at the sizes where its shapes change: the shortest and longest segment
+of each transform length, odd lengths (no bulk copies), template counts that leave series of a
+group empty, two cosets, folded segments in FP32, both storage types.  Tolerances as in the
+other parity tests: 1e-4 max(1, max|rho|) (FP32), 1e-2 (BF16 storage)."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts too
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_1712_06515_gb300 as cc  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+# (N_s, segments, templates, keywords)
+SHAPES = [
+    (33, 24, 5, {}), (64, 24, 17, {}), (65, 24, 9, dict(pair_mode=2)), (128, 24, 1, dict(T_max=0.0)),
+    (129, 16, 3, {}), (255, 16, 5, dict(n_det=1, pair_mode=2)), (256, 16, 9, {}), (257, 12, 2, {}), (512, 12, 5, dict(T_max=0.0)),
+    (513, 8, 3, {}), (1024, 8, 3, dict(pair_mode=2)), (1025, 8, 2, {}), (2047, 6, 2, {}), (2048, 6, 3, dict(T_max=0.0)),
+    (2049, 5, 2, {}), (2050, 5, 2, dict(pair_mode=2)), (4095, 4, 1, {}), (4096, 4, 2, dict(n_det=1, pair_mode=2)),
+    (4097, 4, 1, {}), (8192, 4, 2, dict(T_max=0.0)), (8194, 3, 1, {}), (16385, 3, 1, {}),
+]
+
+
+def run(n_s, m, n_t, kw, store=cc.STORE_FP32, **tune):
+    kw = dict(dict(T_max=float(n_s)), **kw)
+    sft = next(float(d) for d in range(n_s // 2 + 1, n_s + 1) if n_s % d == 0) / 1.0
+    ds = synth.tiny(seed=61, n_samples=n_s * m + n_s // 3, T_sft=sft, T_short=float(n_s), f_band=0.1 if n_s > 200 else 0.4,
+                    n_templates=n_t, duty=0.7, mean_lock_s=1.5 * n_s, **kw)
+    ref = oracle.rho(ds)
+    with cc.CrossCorrPlan(ds.cfg, ds.dets, store=store) as plan:
+        assert plan.search_path == cc.PATH_TWO_PASS
+        plan.set_tuning(**tune)
+        x = torch.from_numpy(ds.x64).to(DEV)
+        tm = torch.from_numpy(ds.templates).to(DEV)
+        runs = [plan.search(x, tm).cpu().numpy() for _ in range(2)]
+        plan.check()
+    assert np.array_equal(runs[0], runs[1])     # units are computed in a fixed order
+    tol = 1e-4 if store == cc.STORE_FP32 else 1e-2
+    for t in range(n_t):
+        err = float(np.abs(runs[0][t].astype(np.float64) - ref[t]).max())
+        lim = tol * max(1.0, float(np.abs(ref[t]).max()))
+        assert err <= lim, f"template {t}: max |drho| = {err:.3e} > {lim:.3e}"
+
+
+@pytest.mark.parametrize("n_s,m,n_t,kw", SHAPES)
+def test_shapes(n_s, m, n_t, kw):
+    run(n_s, m, n_t, kw)
+
+
+@pytest.mark.parametrize("n_s,m,n_t", [(66, 24, 5), (100, 24, 9), (250, 12, 3), (1000, 8, 2), (3000, 4, 2), (8193, 3, 1)])
+def test_shapes_bf16(n_s, m, n_t):
+    """BF16 rows: whole 16-byte pieces and not, and an odd folded segment (FP32 folded rows)."""
+    run(n_s, m, n_t, {}, store=cc.STORE_BF16)
+
+
+@pytest.mark.parametrize("tune", [dict(batch_templates=2), dict(chunk_waves=1), dict(chunk_waves=400), dict(transform_len=4096)])
+def test_splits(tune):
+    run(600, 40, 5, {}, **tune)
