@@ -128,6 +128,142 @@ topk_pass2(const float* __restrict__ cv, const long long* __restrict__ ci, long 
     }
 }
 
+// ---------------------------------------------------------------------------
+// One pass over rho for the usual case (k well below the number of groups): every warp takes
+// groups of contiguous values and notes each group's maximum; the last block to finish takes
+// the k-th largest of those maxima as a threshold -- at least k values reach it --, rereads the
+// groups that reach it (about k of them), collects their values above it and sorts those.
+// Bound by the one read of rho.  Values are compared by an unsigned key that orders as `better`
+// does (NaN as -inf, -0 as +0); ties end in the sort by index.  When the collection overflows
+// (values bunched into few groups, or many equal ones) the count says so and the caller takes
+// the block-list passes above.
+// ---------------------------------------------------------------------------
+constexpr int SEL_THREADS = 1024;
+constexpr int SEL_GROUPS = 16384;      // maxima
+constexpr int SEL_CAP = 8192;          // collected candidates
+
+struct SelHead {                       // followed by the hits' indices [k] and values [k]
+    unsigned count, err, done, pad;
+};
+
+__device__ __forceinline__ unsigned sel_key(float v) {
+    v = isnan(v) ? -INFINITY : v + 0.0f;
+    const unsigned u = __float_as_uint(v);
+    return u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
+}
+
+// Largest key of values [b, e) over the warp (aligned: b and rho allow 16-byte loads).
+__device__ __forceinline__ unsigned group_max(const float* __restrict__ rho, long long b, long long e, bool aligned) {
+    const int lane = threadIdx.x & 31;
+    unsigned m = 0;
+    if (aligned) {
+        const float4* p = (const float4*)(rho + b);
+        const long long n4 = (e - b) >> 2;
+#pragma unroll 4
+        for (long long i = lane; i < n4; i += 32) {
+            const float4 v = __ldg(p + i);
+            m = max(max(m, max(sel_key(v.x), sel_key(v.y))), max(sel_key(v.z), sel_key(v.w)));
+        }
+        b += n4 << 2;
+    }
+    for (long long i = b + lane; i < e; i += 32) m = max(m, sel_key(__ldg(rho + i)));
+    return __reduce_max_sync(0xffffffffu, m);
+}
+
+__global__ void __launch_bounds__(SEL_THREADS)
+topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups, int k, int aligned,
+            unsigned* __restrict__ maxima, SelHead* head, long long* __restrict__ out_i, float* __restrict__ out_v,
+            const unsigned* __restrict__ err) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ bool last;
+    __shared__ unsigned hist[256], s_prefix;
+    __shared__ int s_need, ncand;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nw = gridDim.x * (SEL_THREADS / 32);
+    for (int g = blockIdx.x * (SEL_THREADS / 32) + warp; g < n_groups; g += nw) {
+        const long long b = (long long)g * gsize, e = b + gsize < n ? b + gsize : n;
+        const unsigned m = group_max(rho, b, e, aligned);
+        if (lane == 0) maxima[g] = m;
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(&head->done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // the k-th largest maximum, eight bits at a time
+    if (tid == 0) {
+        s_prefix = 0;
+        s_need = k;
+        ncand = 0;
+    }
+    for (int shift = 24; shift >= 0; shift -= 8) {
+        if (tid < 256) hist[tid] = 0;
+        __syncthreads();
+        const unsigned prefix = s_prefix, mask = shift == 24 ? 0u : 0xffffffffu << (shift + 8);
+        for (int g = tid; g < n_groups; g += SEL_THREADS) {
+            const unsigned m = __ldcg(maxima + g);
+            if ((m & mask) == prefix) atomicAdd(&hist[(m >> shift) & 255u], 1u);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            int need = s_need, d = 255;
+            while (d > 0 && (int)hist[d] < need) need -= (int)hist[d--];
+            s_need = need;
+            s_prefix = prefix | ((unsigned)d << shift);
+        }
+        __syncthreads();
+    }
+    const unsigned thr = s_prefix;
+    Cand* s = (Cand*)smem;
+    for (int g0 = warp * 32; g0 < n_groups; g0 += SEL_THREADS)
+        for (unsigned hit = __ballot_sync(0xffffffffu, g0 + lane < n_groups && __ldcg(maxima + g0 + lane) >= thr); hit; hit &= hit - 1) {
+        const int g = g0 + __ffs(hit) - 1;
+        const long long b = (long long)g * gsize, e = b + gsize < n ? b + gsize : n;
+        for (long long i = b + lane; i < e; i += 32) {
+            const float v = __ldg(rho + i);
+            if (sel_key(v) >= thr) {
+                const int pos = atomicAdd(&ncand, 1);
+                if (pos < SEL_CAP) {
+                    Cand c;
+                    c.v = isnan(v) ? -INFINITY : v;
+                    c.pad = 0;
+                    c.idx = i;
+                    s[pos] = c;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const int m = ncand;
+    if (m <= SEL_CAP) {
+        int size = 2;
+        while (size < m) size <<= 1;
+        for (int i = m + tid; i < size; i += SEL_THREADS) s[i] = worst_cand();
+        bitonic_sort(s, size);
+        for (int i = tid; i < k; i += SEL_THREADS) {
+            out_i[i] = s[i].idx;
+            out_v[i] = s[i].v;
+        }
+    }
+    if (tid == 0) {
+        head->count = (unsigned)m;
+        head->err = __ldcg(err);
+    }
+}
+
+static void fill_hits(const cc_plan* plan, int nk, const long long* idx, const float* val, cc_hit* out) {
+    for (int i = 0; i < nk; ++i) {
+        cc_hit h;
+        memset(&h, 0, sizeof(h));
+        h.tmpl = idx[i] / plan->N_f;
+        h.bin = (int32_t)(idx[i] % plan->N_f);
+        h.freq = plan->freq[h.bin];
+        h.rho = val[i];
+        out[i] = h;
+    }
+}
+
 }  // namespace cc
 
 extern "C" cc_status crosscorr_rho_topk(cc_plan* plan, const float* rho_dev, int64_t n_t, int k,
@@ -141,14 +277,8 @@ extern "C" cc_status crosscorr_rho_topk(cc_plan* plan, const float* rho_dev, int
     if (n == 0) return CC_OK;
     if (!rho_dev) return fail(CC_ERR_INVALID, "rho_dev is null");
     cudaStream_t st = (cudaStream_t)stream;
-    int KP = 1;
-    while (KP < k) KP <<= 1;
-    KP = std::max(KP, 2 * TOPK_THREADS);   // candidate buffer must exceed one tile
-    int nb = (int)std::min<long long>(TOPK_BLOCKS, (n + 65535) / 65536);
-    nb = std::max(nb, 1);
-    size_t cand = (size_t)nb * KP;
-    // Candidate lists live in a buffer of their own, sized once for the largest k and
-    // block count, so top-k never touches (or grows) the search workspace: a search
+    // Group maxima and candidate lists live in a buffer of their own, sized once for the
+    // largest k and block count, so top-k never touches (or grows) the search workspace: a search
     // queued on another stream for this plan keeps its workspace intact.
     if (!plan->topk_ws) {
         cudaError_t ea = cudaMalloc(&plan->topk_ws, topk_buffer_bytes());
@@ -157,6 +287,44 @@ extern "C" cc_status crosscorr_rho_topk(cc_plan* plan, const float* rho_dev, int
             return cuda_fail(ea, "top-k candidate buffer");
         }
     }
+    const int nk = (int)std::min<long long>(k, n);
+    // Groups of at least 256 values, at most SEL_GROUPS of them; the threshold needs k groups and
+    // is close to the k-th value while there are several times more.
+    const long long gsize = std::max<long long>(256, ((n + SEL_GROUPS - 1) / SEL_GROUPS + 127) / 128 * 128);
+    const long long n_groups = (n + gsize - 1) / gsize;
+    if (n_groups >= 2 * (long long)nk) {
+        SelHead* head = (SelHead*)plan->topk_ws;
+        long long* oi = (long long*)(head + 1);
+        float* ov = (float*)(oi + nk);
+        unsigned* maxima = (unsigned*)((char*)(head + 1) + (size_t)TOPK_MAX * 12);
+        const size_t sm = (size_t)SEL_CAP * sizeof(Cand);
+        cudaError_t e = cudaFuncSetAttribute(topk_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e == cudaSuccess) e = cudaMemsetAsync(head, 0, sizeof(SelHead), st);
+        if (e != cudaSuccess) return cuda_fail(e, "top-k selection set-up");
+        const int aligned = ((uintptr_t)rho_dev & 15) == 0;
+        const int blocks = (int)std::min<long long>(152, (n_groups + SEL_THREADS / 32 - 1) / (SEL_THREADS / 32));
+        topk_select<<<blocks, SEL_THREADS, sm, st>>>(rho_dev, n, (int)gsize, (int)n_groups, nk, aligned, maxima, head, oi, ov,
+                                                     plan->dp.err);
+        count_launch();
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "topk launch");
+        std::vector<char> back(sizeof(SelHead) + (size_t)nk * 12);
+        e = cudaMemcpyAsync(back.data(), head, back.size(), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail(e, "topk copy");
+        const SelHead* h = (const SelHead*)back.data();
+        if (h->err) return crosscorr_plan_check(plan, stream);   // a failed bounded wait of the searches before
+        if (h->count <= (unsigned)SEL_CAP) {
+            const long long* hi = (const long long*)(h + 1);
+            fill_hits(plan, nk, hi, (const float*)(hi + nk), hits_host);
+            return CC_OK;
+        }
+    }
+    int KP = 1;
+    while (KP < k) KP <<= 1;
+    KP = std::max(KP, 2 * TOPK_THREADS);   // candidate buffer must exceed one tile
+    int nb = (int)std::min<long long>(TOPK_BLOCKS, (n + 65535) / 65536);
+    nb = std::max(nb, 1);
+    size_t cand = (size_t)nb * KP;
     char* w = (char*)plan->topk_ws;
     long long* ci = (long long*)w;
     long long* fi = ci + cand;
@@ -184,15 +352,6 @@ extern "C" cc_status crosscorr_rho_topk(cc_plan* plan, const float* rho_dev, int
     e = cudaMemcpy(&err_word, plan->dp.err, sizeof(err_word), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "reading the device error word");
     if (err_word) return crosscorr_plan_check(plan, stream);
-    const int nk = (int)std::min<long long>(k, n);
-    for (int i = 0; i < nk; ++i) {
-        cc_hit h;
-        memset(&h, 0, sizeof(h));
-        h.tmpl = hi[i] / plan->N_f;
-        h.bin = (int32_t)(hi[i] % plan->N_f);
-        h.freq = plan->freq[h.bin];
-        h.rho = hv[i];
-        hits_host[i] = h;
-    }
+    fill_hits(plan, nk, hi.data(), hv.data(), hits_host);
     return CC_OK;
 }
