@@ -16,6 +16,7 @@ namespace cc {
 namespace {
 
 constexpr int SS_THREADS = 256;
+constexpr int SS_CHUNK = 32;               // T_sft blocks of a persistent-warp CTA, at most
 constexpr int SS_WARP_SMEM = 72 * 1024;   // shared-memory budget of a persistent-warp CTA
 
 // one CTA per T_sft block: the block's SFT (or zeros for a gap) -> N' output samples
@@ -81,9 +82,20 @@ constexpr float kC52 = -0.809016994374947424f;  // cos(4 pi / 5)
 constexpr float kS51 = 0.951056516295153572f;   // sin(2 pi / 5)
 constexpr float kS52 = 0.587785252292473129f;   // sin(4 pi / 5)
 
+constexpr float kR2 = 0.707106781186547524f;    // sqrt(1/2)
+constexpr float kC91 = 0.766044443118978035f;   // cos(2 pi / 9), sin
+constexpr float kS91 = 0.642787609686539327f;
+constexpr float kC92 = 0.173648177666930349f;   // cos(4 pi / 9), sin
+constexpr float kS92 = 0.984807753012208059f;
+constexpr float kC94 = -0.939692620785908384f;  // cos(8 pi / 9), sin
+constexpr float kS94 = 0.342020143325668733f;
+
 __device__ __forceinline__ float2 f2add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 f2sub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 f2scale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+__device__ __forceinline__ float2 f2mul(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
 __device__ __forceinline__ float2 f2negi(float2 a) { return make_float2(a.y, -a.x); }   // -i a
 
 // forward DFT of radix R in place on v[0 .. R-1] (exp(-2 pi i n k / R))
@@ -218,8 +230,46 @@ __device__ __forceinline__ void dft_r(float2 (&v)[R]) {
         v[2] = f2sub(s0, s1);
         v[1] = f2add(d0, d1);
         v[3] = f2sub(d0, d1);
+    } else if constexpr (R == 8) {   // 2 x 4: n = 4 n1 + n2, k = k1 + 2 k2
+        float2 e[4], o[4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            e[n] = f2add(v[n], v[n + 4]);
+            o[n] = f2sub(v[n], v[n + 4]);
+        }
+        o[1] = f2scale(make_float2(o[1].x + o[1].y, o[1].y - o[1].x), kR2);    // W8
+        o[2] = f2negi(o[2]);
+        o[3] = f2scale(make_float2(o[3].y - o[3].x, -o[3].x - o[3].y), kR2);   // W8^3
+        dft_r<4>(e);
+        dft_r<4>(o);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[2 * k] = e[k];
+            v[2 * k + 1] = o[k];
+        }
+    } else if constexpr (R == 9) {   // 3 x 3: n = 3 n1 + n2, k = k1 + 3 k2, twiddles W9^(n2 k1)
+        float2 a[3][3];
+#pragma unroll
+        for (int n2 = 0; n2 < 3; ++n2) {
+            a[n2][0] = v[n2];
+            a[n2][1] = v[n2 + 3];
+            a[n2][2] = v[n2 + 6];
+            dft_r<3>(a[n2]);
+        }
+        a[1][1] = f2mul(a[1][1], make_float2(kC91, -kS91));
+        a[1][2] = f2mul(a[1][2], make_float2(kC92, -kS92));
+        a[2][1] = f2mul(a[2][1], make_float2(kC92, -kS92));
+        a[2][2] = f2mul(a[2][2], make_float2(kC94, -kS94));
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) {
+            float2 b[3] = {a[0][k1], a[1][k1], a[2][k1]};
+            dft_r<3>(b);
+            v[k1] = b[0];
+            v[k1 + 3] = b[1];
+            v[k1 + 6] = b[2];
+        }
     } else {
-        static_assert(R == 5, "radix 2, 3, 4 or 5");
+        static_assert(R == 5, "radix 2, 3, 4, 5, 8 or 9");
         const float2 a14 = f2add(v[1], v[4]), d14 = f2sub(v[1], v[4]);
         const float2 a23 = f2add(v[2], v[3]), d23 = f2sub(v[2], v[3]);
         const float2 p1 = make_float2(v[0].x + kC51 * a14.x + kC52 * a23.x, v[0].y + kC51 * a14.y + kC52 * a23.y);
@@ -235,12 +285,13 @@ __device__ __forceinline__ void dft_r(float2 (&v)[R]) {
 }
 
 // One Stockham pass of radix R over N' points by one warp (lanes stride the butterflies);
-// CONJ conjugates the inputs (the first pass, reading the staged band).
-template <int R, bool CONJ>
+// CONJ conjugates the inputs (the first pass, reading the staged band).  LAST: the outputs
+// X_j, j + r ns, go straight to the series, as (-1)^j conj(X_j) times the block's factor.
+template <int R, bool CONJ, bool LAST>
 __device__ __forceinline__ void warp_pass_r(const float2* src, float2* dst, const float2* twf, int nb, int tstep,
-                                            int ns, uint32_t nsm, int nss, int lane) {
+                                            int ns, uint32_t nsm, int nss, int lane, float2 rot) {
     for (int j = lane; j < nb; j += 32) {
-        const int k = ns == 1 ? 0 : j - (int)(((uint64_t)(uint32_t)j * nsm) >> nss) * ns;   // j mod ns
+        const int k = LAST ? j : ns == 1 ? 0 : j - (int)(((uint64_t)(uint32_t)j * nsm) >> nss) * ns;   // j mod ns
         float2 v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -250,109 +301,119 @@ __device__ __forceinline__ void warp_pass_r(const float2* src, float2* dst, cons
         if (ns > 1) {
             const int tk = k * tstep;
 #pragma unroll
-            for (int r = 1; r < R; ++r) {
-                const float2 w = twf[tk * r];
-                v[r] = make_float2(v[r].x * w.x - v[r].y * w.y, v[r].x * w.y + v[r].y * w.x);
-            }
+            for (int r = 1; r < R; ++r) v[r] = f2mul(v[r], twf[tk * r]);
         }
         dft_r<R>(v);
-        float2* d = dst + (j - k) * R + k;
+        if constexpr (LAST) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) d[r * ns] = v[r];
+            for (int r = 0; r < R; ++r) {
+                const int o = j + r * ns;
+                const float2 f = (o & 1) ? make_float2(-rot.x, -rot.y) : rot;
+                dst[o] = make_float2(fmaf(v[r].x, f.x, v[r].y * f.y), fmaf(v[r].x, f.y, -v[r].y * f.x));
+            }
+        } else {
+            float2* d = dst + (j - k) * R + k;
+#pragma unroll
+            for (int r = 0; r < R; ++r) d[r * ns] = v[r];
+        }
     }
 }
 
-template <bool CONJ>
+template <bool CONJ, bool LAST>
 __device__ __forceinline__ void warp_pass(const float2* src, float2* dst, const float2* twf, const Radices& rad,
-                                          int p, int lane) {
+                                          int p, int lane, float2 rot) {
     const int nb = rad.nb[p], tstep = rad.tstep[p], ns = rad.ns[p], nss = rad.nss[p];
     const uint32_t nsm = rad.nsm[p];
     switch (rad.r[p]) {   // the same for the whole warp
-        case 2: warp_pass_r<2, CONJ>(src, dst, twf, nb, tstep, ns, nsm, nss, lane); break;
-        case 3: warp_pass_r<3, CONJ>(src, dst, twf, nb, tstep, ns, nsm, nss, lane); break;
-        case 4: warp_pass_r<4, CONJ>(src, dst, twf, nb, tstep, ns, nsm, nss, lane); break;
-        default: warp_pass_r<5, CONJ>(src, dst, twf, nb, tstep, ns, nsm, nss, lane); break;
+        case 2: warp_pass_r<2, CONJ, LAST>(src, dst, twf, nb, tstep, ns, nsm, nss, lane, rot); break;
+        case 3: warp_pass_r<3, CONJ, LAST>(src, dst, twf, nb, tstep, ns, nsm, nss, lane, rot); break;
+        case 4: warp_pass_r<4, CONJ, LAST>(src, dst, twf, nb, tstep, ns, nsm, nss, lane, rot); break;
+        case 8: warp_pass_r<8, CONJ, LAST>(src, dst, twf, nb, tstep, ns, nsm, nss, lane, rot); break;
+        case 9: warp_pass_r<9, CONJ, LAST>(src, dst, twf, nb, tstep, ns, nsm, nss, lane, rot); break;
+        default: warp_pass_r<5, CONJ, LAST>(src, dst, twf, nb, tstep, ns, nsm, nss, lane, rot); break;
     }
 }
 
-// N' up to 1536: persistent warps, each taking its next T_sft block from a global counter
-// (locked SFTs and gaps fall unevenly on a fixed stride; the counter balances them).  Per
-// warp three N'-point shared buffers: the next locked SFT's bins are staged by cp.async
-// while the current one runs its passes, so its HBM latency overlaps the transform; the
-// forward twiddles exp(-2 pi i e / N') are formed once per CTA (FP64).  Only warp-level
-// synchronisation after the one CTA barrier of the twiddle table.
+// N' up to 1536: a CTA takes `chunk` consecutive T_sft blocks, its warps one block after the
+// other from a shared counter (locked SFTs and gaps come in runs of hours: the CTAs' sizes
+// differ, and more CTAs than fit at once even that out).  Per warp three N'-point shared
+// buffers: the next locked SFT's bins are staged by cp.async while the current one runs its
+// passes; radices up to 9 keep those few (three for N' = 360) and the last one writes the
+// series.  The forward twiddles exp(-2 pi i e / N') and the blocks' phase factors are formed
+// once per CTA.  Only warp-level synchronisation after that.
+// What bounds it: HBM (read the locked bands, write the series) and the shared-memory passes.
 __global__ void __launch_bounds__(SS_THREADS)
 sft_fft_warp_kernel(const float2* __restrict__ band, const int64_t* __restrict__ block_sft, int64_t n_blocks,
-                    int n_prime, double T_sft, double f_h, Radices rad, unsigned int* __restrict__ next_block,
-                    float2* __restrict__ x) {
+                    int n_prime, double T_sft, double f_h, Radices rad, int chunk, float2* __restrict__ x) {
     extern __shared__ __align__(16) float2 sw[];
+    __shared__ int64_t s_sft[SS_CHUNK];
+    __shared__ float2 s_rot[SS_CHUNK];
+    __shared__ int s_next;
     float2* twf = sw;                                  // [N' rounded up to even]
     const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float2* stage = sw + ((n_prime + 1) & ~1) + (size_t)g * 3 * n_prime;
     float2* bufA = stage + n_prime;
     float2* bufB = bufA + n_prime;
-    for (int e = threadIdx.x; e < n_prime; e += blockDim.x) {
-        double sn, cs;
-        sincospi(-2.0 * (double)e / (double)n_prime, &sn, &cs);
-        twf[e] = make_float2((float)cs, (float)sn);
+    const int64_t b0 = (int64_t)blockIdx.x * chunk;
+    const int nb = (int)imin64(chunk, n_blocks - b0);
+    if (threadIdx.x == 0) s_next = 0;
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+        s_sft[i] = __ldg(block_sft + b0 + i);
+        // SFT-start phase in FP64, reduced to cycles, and 1 / T_sft
+        const double cyc = f_h * ((double)(b0 + i) * T_sft);
+        const float c = (float)(cyc - floor(cyc)), scale = (float)(1.0 / T_sft);
+        float sn, cs;
+        sincospif(2.0f * c, &sn, &cs);
+        s_rot[i] = make_float2(cs * scale, -sn * scale);
     }
+    for (int e = threadIdx.x; e < n_prime; e += blockDim.x) twf[e] = unit_root(e, n_prime);
     __syncthreads();
-    auto grab = [&]() -> int64_t {
-        unsigned int v = 0;
-        if (lane == 0) v = atomicAdd(next_block, 1u);
-        return (int64_t)__shfl_sync(0xffffffffu, v, 0);
+    auto grab = [&]() -> int {
+        int v = 0;
+        if (lane == 0) v = atomicAdd(&s_next, 1);
+        return __shfl_sync(0xffffffffu, v, 0);
     };
-    int64_t b = grab();
-    int64_t s = b < n_blocks ? __ldg(block_sft + b) : -1;
-    if (s >= 0) {
-        const float2* zs = band + s * (int64_t)n_prime;
-        for (int m = lane; m < n_prime; m += 32) cp_async8(stage + m, zs + m);
-    }
-    cp_async_commit();
-    const float scale = (float)(1.0 / T_sft);
-    while (b < n_blocks) {
-        const int64_t bn = grab();
-        const int64_t sn = bn < n_blocks ? __ldg(block_sft + bn) : -1;
-        float2* xo = x + b * (int64_t)n_prime;
-        if (s >= 0) {
+    auto fetch = [&](int i) {
+        if (i < nb && s_sft[i] >= 0) {
+            const float2* zs = band + s_sft[i] * (int64_t)n_prime;
+            for (int m = lane; m < n_prime; m += 32) cp_async8(stage + m, zs + m);
+        }
+        cp_async_commit();
+    };
+    int i = grab();
+    fetch(i);
+    while (i < nb) {
+        const int in = grab();
+        float2* xo = x + (b0 + i) * (int64_t)n_prime;
+        const float2 rot = s_rot[i];
+        if (s_sft[i] >= 0) {
             cp_async_wait_all();
             __syncwarp();
-            warp_pass<true>(stage, bufA, twf, rad, 0, lane);
-            __syncwarp();                              // the stage is free: every lane has read it
-        }
-        if (sn >= 0) {
-            const float2* zs = band + sn * (int64_t)n_prime;
-            for (int m = lane; m < n_prime; m += 32) cp_async8(stage + m, zs + m);
-            cp_async_commit();
-        }
-        if (s >= 0) {
-            float2* src = bufA;
-            float2* dst = bufB;
-            for (int p = 1; p < rad.n; ++p) {
+            if (rad.n == 1) {
+                warp_pass<true, true>(stage, xo, twf, rad, 0, lane, rot);
                 __syncwarp();
-                warp_pass<false>(src, dst, twf, rad, p, lane);
-                float2* t = src;
-                src = dst;
-                dst = t;
+                fetch(in);
+            } else {
+                warp_pass<true, false>(stage, bufA, twf, rad, 0, lane, rot);
+                __syncwarp();                          // the stage is free: every lane has read it
+                fetch(in);
+                float2* src = bufA;
+                float2* dst = bufB;
+                for (int p = 1; p < rad.n - 1; ++p) {
+                    warp_pass<false, false>(src, dst, twf, rad, p, lane, rot);
+                    __syncwarp();
+                    float2* t = src;
+                    src = dst;
+                    dst = t;
+                }
+                warp_pass<false, true>(src, xo, twf, rad, rad.n - 1, lane, rot);
+                __syncwarp();                          // the buffers' reads are done before the next pass 0
             }
-            __syncwarp();
-            // SFT-start phase in FP64, reduced to cycles; output (-1)^j conj(X_j) / T_sft times it
-            const double cyc = f_h * ((double)b * T_sft);
-            const float c = (float)(cyc - floor(cyc));
-            float sn2, cs;
-            sincospif(2.0f * c, &sn2, &cs);
-            const float2 rot = make_float2(cs, -sn2);
-            for (int j = lane; j < n_prime; j += 32) {
-                const float sg = (j & 1) ? -scale : scale;
-                const float2 a = make_float2(src[j].x * sg, -src[j].y * sg);
-                xo[j] = make_float2(fmaf(a.x, rot.x, -a.y * rot.y), fmaf(a.x, rot.y, a.y * rot.x));
-            }
-            __syncwarp();                              // bufA / bufB reads done before the next pass 0
         } else {
             for (int j = lane; j < n_prime; j += 32) xo[j] = make_float2(0.f, 0.f);
+            fetch(in);
         }
-        s = sn;
-        b = bn;
+        i = in;
     }
     cp_async_wait_all();
 }
@@ -388,6 +449,28 @@ bool factor_radices(int64_t n, Radices* rad) {
     return true;
 }
 
+// The radices of the warp kernel: eights and nines first (fewer passes), two fours instead of
+// an eight and a two.
+void widen_radices(int64_t N, Radices* rad) {
+    int two = 0, three = 0, five = 0, r[SS_MAX_PASSES], k = 0;
+    for (int64_t m = N; m % 2 == 0; m /= 2) ++two;
+    for (int64_t m = N; m % 3 == 0; m /= 3) ++three;
+    for (int64_t m = N; m % 5 == 0; m /= 5) ++five;
+    while (two >= 3 && two != 4) {
+        r[k++] = 8;
+        two -= 3;
+    }
+    while (two >= 2) {
+        r[k++] = 4;
+        two -= 2;
+    }
+    if (two) r[k++] = 2;
+    for (; three >= 2; three -= 2) r[k++] = 9;
+    if (three) r[k++] = 3;
+    for (; five > 0; --five) r[k++] = 5;
+    set_passes(N, r, k, rad);
+}
+
 // Shared-memory wavefronts of one warp access to 8-byte elements at `idx` (32 banks of
 // 4 bytes, 128-byte rows): the largest number of distinct rows any bank is asked for.
 int warp_wavefronts(const int* idx, int nl) {
@@ -418,11 +501,13 @@ int64_t order_wavefronts(int64_t N, const int* r, int n) {
             for (int q = 0; q < R; ++q) {
                 for (int l = 0; l < nl; ++l) idx[l] = j0 + l + q * nb;
                 total += warp_wavefronts(idx, nl);
-                for (int l = 0; l < nl; ++l) {
-                    const int j = j0 + l, k = j % ns;
-                    idx[l] = (j - k) * R + k + q * ns;
+                if (p + 1 < n) {   // the last pass writes the series
+                    for (int l = 0; l < nl; ++l) {
+                        const int j = j0 + l, k = j % ns;
+                        idx[l] = (j - k) * R + k + q * ns;
+                    }
+                    total += warp_wavefronts(idx, nl);
                 }
-                total += warp_wavefronts(idx, nl);
                 if (ns > 1 && q > 0) {
                     for (int l = 0; l < nl; ++l) idx[l] = ((j0 + l) % ns) * q * tstep;
                     total += warp_wavefronts(idx, nl);
@@ -473,8 +558,8 @@ extern "C" cc_status crosscorr_sfts_to_series(const void* band_dev, const int64_
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
     if (fft && n_prime <= 1536) {
-        // persistent warps: three N'-point buffers per warp plus the CTA's twiddle table,
-        // as many warps per CTA (at most 8) as fit in 72 KB; one wave of CTAs
+        // three N'-point buffers per warp plus the CTA's twiddle table, as many warps per CTA
+        // (at most 8) as fit in 72 KB
         const size_t per = 3 * sizeof(float2) * n_prime, tw_b = sizeof(float2) * ((n_prime + 1) & ~1);
         const int groups = (int)std::max<int64_t>(1, std::min<int64_t>(SS_THREADS / 32, (SS_WARP_SMEM - tw_b) / per));
         const size_t smem = tw_b + per * groups;
@@ -496,6 +581,7 @@ extern "C" cc_status crosscorr_sfts_to_series(const void* band_dev, const int64_
                 sms = it->second.sms;
                 rad = it->second.rad;
             } else {
+                widen_radices(n_prime, &rad);
                 order_for_banks(n_prime, &rad);
                 // the attribute is the kernel's, shared by every N': set to the largest shape
                 // (72 KB, or one group of three 1536-point buffers and the table: 49 KB)
@@ -509,22 +595,17 @@ extern "C" cc_status crosscorr_sfts_to_series(const void* band_dev, const int64_
                 shapes[{dev, n_prime}] = Shape{occ, sms, rad};
             }
         }
-        const int64_t ctas = std::max<int64_t>(1, std::min<int64_t>((n_blocks + groups - 1) / groups,
-                                                                    (int64_t)std::max(1, occ) * sms));
-        // the block counter: stream-ordered, zeroed before and freed after the kernel
-        unsigned int* ctr = nullptr;
-        if ((e = cudaMallocAsync((void**)&ctr, sizeof(unsigned int), st)) != cudaSuccess)
-            return cuda_fail(e, "sfts_to_series block counter");
-        if ((e = cudaMemsetAsync(ctr, 0, sizeof(unsigned int), st)) != cudaSuccess) {
-            cudaFreeAsync(ctr, st);
-            return cuda_fail(e, "sfts_to_series block counter");
-        }
-        sft_fft_warp_kernel<<<(unsigned)ctas, 32 * groups, smem, st>>>((const float2*)band_dev, block_sft_dev,
-                                                                       n_blocks, (int)n_prime, T_sft, f_h, rad,
-                                                                       ctr, (float2*)x_dev);
+        // blocks per CTA: two per warp while that leaves at least four CTAs per resident slot, more
+        // while there are plenty (the tables are formed per CTA)
+        const int64_t slots = (int64_t)std::max(1, occ) * sms;
+        int64_t chunk = std::min<int64_t>(SS_CHUNK, std::max<int64_t>(groups, n_blocks / (4 * slots)));
+        if (n_blocks < slots * groups) chunk = std::max<int64_t>(1, std::min<int64_t>(groups, (n_blocks + slots - 1) / slots));
+        const int64_t ctas = (n_blocks + chunk - 1) / chunk;
+        sft_fft_warp_kernel<<<(unsigned)ctas, 32 * groups, smem, st>>>((const float2*)band_dev, block_sft_dev, n_blocks,
+                                                                       (int)n_prime, T_sft, f_h, rad, (int)chunk,
+                                                                       (float2*)x_dev);
         count_launch();
         e = cudaGetLastError();
-        cudaFreeAsync(ctr, st);
         return e == cudaSuccess ? CC_OK : cuda_fail(e, "sft_fft_warp_kernel launch");
     }
     // twiddles: exp(+2 pi i j / N') for the direct DFT, exp(-2 pi i j / N') for the FFT
