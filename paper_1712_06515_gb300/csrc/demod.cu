@@ -433,100 +433,162 @@ __global__ void __launch_bounds__(128) demod_sep_kernel(DevParams p, int m_lo, i
     if (act) rho[(size_t)t * p.N_f + k] = den > 0.f ? 1.41421356237309505f * raw * rsqrtf(den) : 0.f;
 }
 
-// The method's pair loop: one thread per (template, output bin) over the locked SFTs in
-// time order (the separable kernel's records and pipelined loads).  A ring of R_s + 1
-// blocks holds, per slot (block mod (R_s + 1), detector), the thread's y and Xi^2
-// (thread-private columns of shared memory) and the SFT's prescaled filter weights
-// (shared).  A slot that is not a partner of the current SFT -- a block outside the
-// window, a gap, a later detector of the current block -- has zero weights, so the
-// partner loop is one fixed-length sum without branches.  The filter weights
-// Gamma_KL = a^'_K a^'_L + b^'_K b^'_L of the next SFT against every slot are formed once
-// per CTA (slot j by thread j mod blockDim) while the ring is updated, so the loop reads
-// one shared value per slot.  Before the first SFT of a block the slots of that block
-// (and of any skipped block) are cleared.
-__global__ void __launch_bounds__(256) demod_pair_kernel(DevParams p, int m_lo, int nbins, int n_blk, int Rs,
-                                                         const float2* __restrict__ z,
-                                                         const DemodTiming* __restrict__ recs, int n_list,
-                                                         const double* __restrict__ dfreq,
-                                                         const int64_t* __restrict__ kbar, int64_t t_base,
-                                                         float* __restrict__ rho) {
+// The method's pair loop: one thread per (template, output bin) over the locked SFTs in time
+// order (the separable kernel's records), PT consecutive SFTs at a time.  The partners of SFT i
+// are the entries of the list from the first one of block l_i - R_s up to i - 1, so those of a
+// tile of PT SFTs are a contiguous range before the tile plus pairs inside it.  A ring of the
+// last NR = (R_s + 1) Q entries holds, per entry, the thread's y and Xi^2 (thread-private columns
+// of shared memory) and the SFT's prescaled filter weights (shared); per tile the CTA forms
+// Gamma_KL = a^'_K a^'_L + b^'_K b^'_L of every ring entry against the PT SFTs (zero where it is
+// not a partner), and every thread reads each entry once for PT pairs: four shared-memory
+// wavefronts per PT pairs and warp, where one SFT at a time took four per pair and bound the
+// kernel.  Records reach shared memory by cp.async three tiles ahead, the SFT bins registers
+// one tile ahead.
+constexpr int PT = 4;
+
+__global__ void __launch_bounds__(256, 3) demod_pair_kernel(DevParams p, int m_lo, int nbins, int n_blk, int Rs,
+                                                            const float2* __restrict__ z,
+                                                            const DemodTiming* __restrict__ recs, int n_list,
+                                                            const int* __restrict__ boff, const double* __restrict__ dfreq,
+                                                            const int64_t* __restrict__ kbar, int64_t t_base,
+                                                            float* __restrict__ rho) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int nthr = blockDim.x, tid = threadIdx.x;
-    const int Q = p.Q, W = (Rs + 1) * Q;
-    float2* ry = (float2*)sm;                          // [W][nthr] y
-    float* rx = (float*)(ry + (size_t)W * nthr);       // [W][nthr] Xi^2
-    float2* rab = (float2*)(rx + (size_t)W * nthr);    // [W] (a^', b^'), zero: not a partner
-    float* sg = (float*)(rab + W);                     // [W] Gamma of the current SFT per slot
+    const int NR = (Rs + 1) * p.Q;
+    float4* sg = (float4*)sm;                          // [NR] Gamma of the tile's SFTs against each ring entry
+    float4* sq = sg + NR;                              // [NR] their squares
+    float4* rec4 = sq + NR;                            // [4 tiles][PT][2] records
+    float* sin_ = (float*)(rec4 + 4 * PT * 2);         // [PT (PT - 1) / 2] Gamma of the pairs inside the tile, padded to 8
+    float2* rab = (float2*)(sin_ + 8);                 // [NR] (a^', b^')
+    float2* ry = rab + NR + (NR & 1);                  // [NR][nthr] y
+    float* rx = (float*)(ry + (size_t)NR * nthr);      // [NR][nthr] Xi^2
+    __shared__ int s_lo;
     const int64_t t = t_base + blockIdx.y;
     const int k = blockIdx.x * nthr + tid;
     const bool act = k < (int)p.N_f;
-    const DemodTiming* rt = recs + (size_t)(t - t_base) * (n_list + 2);
-    for (int j = 0; j < W; ++j) {
-        ry[(size_t)j * nthr + tid] = make_float2(0.f, 0.f);
-        rx[(size_t)j * nthr + tid] = 0.f;
-    }
-    for (int j = tid; j < W; j += nthr) {
-        rab[j] = make_float2(0.f, 0.f);
-        sg[j] = 0.f;                                   // the first SFT has no partner
-    }
+    const float4* rt = (const float4*)(recs + (size_t)(t - t_base) * (n_list + 2));
     if (n_list == 0) {
         if (act) rho[(size_t)t * p.N_f + k] = 0.f;
         return;
     }
+    // records of tile n (padding past the list: no bins, no weight) into slot n mod 4
+    auto stage = [&](int n) {
+        if (tid < 2 * PT) {
+            const int i = min(n * PT + (tid >> 1), n_list);
+            const uint32_t d = (uint32_t)__cvta_generic_to_shared(rec4 + (n & 3) * PT * 2 + tid);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(rt + 2 * i + (tid & 1)) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto rec = [&](int i) { return SepRec{rec4[((i / PT) & 3) * PT * 2 + (i % PT) * 2], rec4[((i / PT) & 3) * PT * 2 + (i % PT) * 2 + 1]}; };
+    stage(0);
+    stage(1);
+    stage(2);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
     const float df = (float)__ldg(dfreq + (act ? k : 0));
     const int64_t kb = __ldg(kbar + (act ? k : 0));
     const float kh = (float)(kb >> 7), kl = (float)(kb & 127);
     float raw = 0.f, rawc = 0.f, den = 0.f, denc = 0.f;
-    auto step = [&](SepRec& Rc, SftIn& Fc, const SepRec& Rn, SftIn& Fn, int i) {
-        rec_fetch(Fn, Rn, df, kh, kl, m_lo, nbins, n_blk, z);
-        const float a = Rc.t1.y, b = Rc.t1.z;
-        const int key = __float_as_int(Rc.t1.w);
-        const int l = key >> 2, X = key & 3;
-        const int ln = __float_as_int(Rn.t1.w) >> 2;    // block of SFT i + 1 (padding: the last block)
-        Rc = load_rec(rt + i + 2);
-        float xi2;
-        const float2 y = sft_y(Fc, xi2);
-        float pr = 0.f, pq = 0.f;
-        for (int j = 0; j < W; ++j) {
-            const float g = sg[j];
-            const float2 yl = ry[(size_t)j * nthr + tid];
-            pr = fmaf(g, fmaf(y.x, yl.x, y.y * yl.y), pr);
-            pq = fmaf(g * g, rx[(size_t)j * nthr + tid], pq);
-        }
-        kahan_add(raw, rawc, pr);
-        kahan_add(den, denc, xi2 * pq);
-        __syncthreads();                               // every thread is done with the ring
-        const int bl = l % (Rs + 1), slot = bl * Q + X;
-        ry[(size_t)slot * nthr + tid] = y;
-        rx[(size_t)slot * nthr + tid] = xi2;
-        // the ring's weights after SFT i (its own slot set; SFT i + 1 opening block ln
-        // clears the slots of blocks l + 1 .. ln, all of them after R_s + 1 blocks) and
-        // Gamma of SFT i + 1 against each slot
-        const float an = Rn.t1.y, bn = Rn.t1.z;
-        const int jump = ln - l;
-        for (int j = tid; j < W; j += nthr) {
-            float2 ab = j == slot ? make_float2(a, b) : rab[j];
-            if (jump > 0) {
-                const int d = j / Q - bl;                 // block-slot distance after l, 0 .. R_s
-                const int dd = d <= 0 ? d + Rs + 1 : d;   // 1 .. R_s + 1
-                if (dd <= jump) ab = make_float2(0.f, 0.f);
+    SftIn F[PT];
+#pragma unroll
+    for (int q = 0; q < PT; ++q) rec_fetch(F[q], rec(q), df, kh, kl, m_lo, nbins, n_blk, z);
+    int slot0 = 0;                                     // ring slot of the tile's first SFT
+    for (int n = 0; n * PT < n_list; ++n) {
+        const int i0 = n * PT;
+        const int have = min(i0, NR);                  // ring entries before the tile
+        // the tile's first entries of the windows, and Gamma against the ring
+        for (int j = tid; j < have + 8; j += nthr) {
+            if (j < have) {
+                const int e = i0 - 1 - j;              // j-th entry before the tile
+                int s = slot0 - 1 - j;
+                s += s < 0 ? NR : 0;
+                const float2 ab = rab[s];
+                float g[PT];
+#pragma unroll
+                for (int q = 0; q < PT; ++q) {
+                    const float4 r1 = rec4[(n & 3) * PT * 2 + 2 * q + 1];
+                    const int l = __float_as_int(r1.w) >> 2;
+                    g[q] = e >= __ldg(boff + max(0, l - Rs)) ? fmaf(r1.y, ab.x, r1.z * ab.y) : 0.f;
+                }
+                sg[s] = make_float4(g[0], g[1], g[2], g[3]);
+                sq[s] = make_float4(g[0] * g[0], g[1] * g[1], g[2] * g[2], g[3] * g[3]);
+            } else if (j < have + 6) {                 // pairs (q, r), r < q, of the tile: index q (q - 1) / 2 + r
+                const int c = j - have, q = c < 1 ? 1 : c < 3 ? 2 : 3, r = c - q * (q - 1) / 2;
+                const float4 a = rec4[(n & 3) * PT * 2 + 2 * q + 1], b = rec4[(n & 3) * PT * 2 + 2 * r + 1];
+                const int la = __float_as_int(a.w) >> 2;
+                sin_[c] = i0 + r >= __ldg(boff + max(0, la - Rs)) ? fmaf(a.y, b.y, a.z * b.z) : 0.f;
+            } else if (j == have + 6) {
+                s_lo = __ldg(boff + max(0, (__float_as_int(rec4[(n & 3) * PT * 2 + 1].w) >> 2) - Rs));
             }
-            rab[j] = ab;
-            sg[j] = fmaf(an, ab.x, bn * ab.y);
         }
+        stage(n + 3);
+        asm volatile("cp.async.wait_group 2;" ::: "memory");   // tile n + 1's records
         __syncthreads();
-    };
-    SepRec ra = load_rec(rt);
-    SepRec rb = load_rec(rt + 1);
-    SftIn fa, fb;
-    rec_fetch(fa, ra, df, kh, kl, m_lo, nbins, n_blk, z);
-    int i = 0;
-    for (; i + 1 < n_list; i += 2) {
-        step(ra, fa, rb, fb, i);
-        step(rb, fb, ra, fa, i + 1);
+        float2 y[PT];
+        float xi[PT], pr[PT], pq[PT];
+#pragma unroll
+        for (int q = 0; q < PT; ++q) {
+            y[q] = sft_y(F[q], xi[q]);
+            pr[q] = pq[q] = 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < PT; ++q) rec_fetch(F[q], rec(i0 + PT + q), df, kh, kl, m_lo, nbins, n_blk, z);
+        const int cnt = i0 - max(s_lo, i0 - have);
+        int s = slot0 - cnt;
+        s += s < 0 ? NR : 0;
+        const float2* cy = ry + (size_t)s * nthr + tid;
+        const float* cx = rx + (size_t)s * nthr + tid;
+#pragma unroll 2
+        for (int j = 0; j < cnt; ++j) {
+            const float4 g = sg[s], h = sq[s];
+            const float2 yl = *cy;
+            const float xl = *cx;
+            pr[0] = fmaf(g.x, fmaf(y[0].x, yl.x, y[0].y * yl.y), pr[0]);
+            pr[1] = fmaf(g.y, fmaf(y[1].x, yl.x, y[1].y * yl.y), pr[1]);
+            pr[2] = fmaf(g.z, fmaf(y[2].x, yl.x, y[2].y * yl.y), pr[2]);
+            pr[3] = fmaf(g.w, fmaf(y[3].x, yl.x, y[3].y * yl.y), pr[3]);
+            pq[0] = fmaf(h.x, xl, pq[0]);
+            pq[1] = fmaf(h.y, xl, pq[1]);
+            pq[2] = fmaf(h.z, xl, pq[2]);
+            pq[3] = fmaf(h.w, xl, pq[3]);
+            ++s;
+            cy += nthr;
+            cx += nthr;
+            if (s == NR) {
+                s = 0;
+                cy = ry + tid;
+                cx = rx + tid;
+            }
+        }
+        // pairs inside the tile, then the ring takes its SFTs
+#pragma unroll
+        for (int q = 1; q < PT; ++q)
+#pragma unroll
+            for (int r = 0; r < q; ++r) {
+                const float g = sin_[q * (q - 1) / 2 + r];
+                pr[q] = fmaf(g, fmaf(y[q].x, y[r].x, y[q].y * y[r].y), pr[q]);
+                pq[q] = fmaf(g * g, xi[r], pq[q]);
+            }
+        int w = slot0;
+#pragma unroll
+        for (int q = 0; q < PT; ++q) {
+            kahan_add(raw, rawc, pr[q]);
+            kahan_add(den, denc, xi[q] * pq[q]);
+            if (NR >= PT || q >= PT - NR) {            // (a ring shorter than the tile keeps its last SFTs)
+                ry[(size_t)w * nthr + tid] = y[q];
+                rx[(size_t)w * nthr + tid] = xi[q];
+                if (tid == q) {
+                    const float4 r1 = rec4[(n & 3) * PT * 2 + 2 * q + 1];
+                    rab[w] = make_float2(r1.y, r1.z);
+                }
+            }
+            w = w + 1 == NR ? 0 : w + 1;
+        }
+        slot0 = w;
+        __syncthreads();
     }
-    if (i < n_list) step(ra, fa, rb, fb, i);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     // rho = (2 raw) / sqrt(2 den)
     if (act) rho[(size_t)t * p.N_f + k] = den > 0.f ? 1.41421356237309505f * raw * rsqrtf(den) : 0.f;
 }
@@ -670,7 +732,7 @@ extern "C" cc_status crosscorr_demod_search(cc_plan* plan, const cc_template* t_
     int nthr = sep ? 128 : 256;
     auto ring_bytes = [&](int nt) {
         return sep ? (sep_ring ? (size_t)(Rs + 1) * 7 * nt * sizeof(float) : 0)
-                   : (size_t)W * nt * 12 + (size_t)W * 12;
+                   : (size_t)W * nt * 12 + (size_t)W * 40 + 8 + 4 * PT * 32 + 32;
     };
     while (nthr > 32 && ring_bytes(nthr) > DM_RING_BUDGET) nthr /= 2;
     if (ring_bytes(nthr) > DM_RING_BUDGET) return fail(CC_ERR_UNSUPPORTED, "T_max / T_sft too large for the pair ring");
@@ -680,15 +742,19 @@ extern "C" cc_status crosscorr_demod_search(cc_plan* plan, const cc_template* t_
     // timing records for a batch of templates: the list of locked SFTs plus two padding
     const size_t per_t = sizeof(DemodTiming) * ((size_t)n_list + 2);
     const int64_t batch = std::max<int64_t>(1, std::min<int64_t>({n_t, (int64_t)((size_t)2 << 30) / (int64_t)per_t, 65535}));
-    if (sep) {
-        // CTA size of the separable kernel (every thread does the same work, issue-bound):
-        // the fewest resident-thread slots over whole waves of the first batch,
-        // ceil(CTAs / (resident CTAs x SMs)) x resident threads per SM
+    {
+        // CTA size (every thread does the same work): the fewest resident-thread slots over whole
+        // waves of the first batch, ceil(CTAs / (resident CTAs x SMs)) x resident threads per SM
         int dev = 0, sms = 152;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const void* kern = sep_ring ? (const void*)demod_sep_kernel<true> : (const void*)demod_sep_kernel<false>;
+        const void* kern = !sep ? (const void*)demod_pair_kernel
+                                : sep_ring ? (const void*)demod_sep_kernel<true> : (const void*)demod_sep_kernel<false>;
         int64_t best = -1;
-        for (int nt : {128, 96, 64}) {
+        for (int nt : {256, 192, 128, 96, 64}) {
+            if (nt > (sep ? 128 : 256) || ring_bytes(nt) > DM_RING_BUDGET) continue;
+            if (ring_bytes(nt) > 48 * 1024 &&
+                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes(nt)) != cudaSuccess)
+                continue;
             int occ = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, nt, ring_bytes(nt)) != cudaSuccess || occ < 1)
                 continue;
@@ -730,7 +796,7 @@ extern "C" cc_status crosscorr_demod_search(cc_plan* plan, const cc_template* t_
         else
             demod_pair_kernel<<<grid, nthr, smem, st>>>(
                 p, plan->demod_m_lo, plan->demod_nbins, n_blk, Rs, (const float2*)plan->demod_z,
-                (const DemodTiming*)plan->ws, n_list, (const double*)plan->demod_df,
+                (const DemodTiming*)plan->ws, n_list, (const int*)plan->demod_boff, (const double*)plan->demod_df,
                 (const int64_t*)plan->demod_kbar, t0, rho_dev);
         count_launch();
         if (ev1) cudaEventRecord(ev1, st);
