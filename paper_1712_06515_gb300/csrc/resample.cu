@@ -28,7 +28,7 @@ namespace cc {
 
 namespace {
 
-constexpr int RG_MAX_WARPS = 16;
+constexpr int RG_MAX_WARPS = 12;      // 56 registers a thread at three blocks per SM (40 spill)
 constexpr int RG_TILE = 3616;         // samples of a staged tile: three blocks of 73 KB per SM
 
 template <int DT>
@@ -42,7 +42,10 @@ __device__ __forceinline__ float2 sinc_pairs(const SincTab<DT>& tb, const float2
     float2 E = make_float2(0.f, 0.f), O = make_float2(0.f, 0.f);
 #pragma unroll
     for (int k = 1; k <= DT; ++k) {
-        const float g = __fdividef(1.0f, fmaf(d2, tb.ca[k - 1], tb.cb[k - 1])), h = g * (float)k;
+        // one MUFU; the argument is between 0.75 and 13 k^2 in size, far from denormals
+        float g;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(g) : "f"(fmaf(d2, tb.ca[k - 1], tb.cb[k - 1])));
+        const float h = g * (float)k;
         const float2 xm = xc[-k], xp = xc[k];
         const float2 e = cadd(xp, xm), o = csub(xp, xm);
         E.x = fmaf(g, e.x, E.x);
@@ -106,7 +109,7 @@ resample_group_kernel(float2* __restrict__ ab, float4* __restrict__ norm, const 
     }
     if (lane == 0 && sub == 0) {
         s_on[tl] = on;
-        if (t < n_t && act) act[((X == p.Q - 1 ? p.M : 0) + (size_t)K) * t_pad + t] = on;
+        if (t < n_t && act) act[((X == p.Q - 1 ? p.M : 0) + K) * t_pad + t] = on;
     }
     __syncthreads();
     int lo = 0x7fffffff, hi = -0x7fffffff;
@@ -259,8 +262,11 @@ cc_status launch_resample_group(cc_plan* plan, int64_t n_t, void* ab, float* nor
     // warps per block by the segment's knot intervals; templates per block: up to eight (the
     // window is staged once for them), fewer while there are less than two blocks per SM
     const int warps = p.N_s <= 512 ? 4 : p.N_s <= 1536 ? 8 : RG_MAX_WARPS;
-    int tg = std::min(warps, 8);
-    while (tg > 1 && (tg >= 2 * n_t || p.M * p.Q * ((n_t + tg - 1) / tg) < 304)) tg /= 2;
+    static const int groups[] = {12, 6, 3, 2, 1, 0}, groups8[] = {8, 4, 2, 1, 0};
+    const int* gp = warps == 12 ? groups : warps == 8 ? groups8 : groups8 + 1;
+    if (warps == 12) ++gp;
+    while (gp[1] && (gp[0] >= 2 * n_t || p.M * p.Q * ((n_t + gp[0] - 1) / gp[0]) < 304)) ++gp;
+    const int tg = gp[0];
     const int64_t tiles = (p.N_s + RG_TILE - 1) / RG_TILE;
     const int tile = (int)(((p.N_s + tiles - 1) / tiles + 31) & ~(int64_t)31);
     // the window of a tile: its samples, the drift of the delay over the segment

@@ -448,10 +448,15 @@ size_t resample_smem_bytes(const DevParams& p, bool window) {
     return (size_t)nk * (sizeof(KnotRec) + sizeof(double));
 }
 
+cc_status launch_resample_group(cc_plan* plan, int64_t n_t, void* ab, float* norm, cudaStream_t st, const KnotRec* kn,
+                                int64_t nkn, int write_inactive, uint8_t* act, int t_pad);
+
 cc_status launch_resample(cc_plan* plan, const cc_template* t_dev, int64_t n_t, void* ab,
                           float* norm, cudaStream_t st, const KnotRec* kn, int64_t nkn, int write_inactive,
                           uint8_t* act, int t_pad) {
     const DevParams& p = plan->dp;
+    if (kn && p.store == CC_STORE_FP32)
+        return launch_resample_group(plan, n_t, ab, norm, st, kn, nkn, write_inactive, act, t_pad);
     // with knot records, the segment's window of x is staged in shared memory when it
     // leaves room for several blocks per SM
     const int use_window = kn && resample_smem_bytes(p, true) <= 96 * 1024;

@@ -1,0 +1,78 @@
+"""Parity of the grouped resampling kernel (several templates per block, FP32 storage) with the
+FP64 oracle, per sample: segment lengths around its warp and tile splits, template counts that
+leave a group partly empty, templates so far apart that samples miss the staged window, generic
+and compile-time stencils, the learned interpolator.  Bounds as in the other stage tests: a_r,
+b_r within 2e-5 of max, norms within 2e-5 relative; samples within 1e-5 of a stencil or block
+tie are left out."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU hosts too
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_1712_06515_gb300 as cc  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+
+def check(n_s, m, n_t, learned=False, templates=None, tol=2e-5, **kw):
+    ds = synth.tiny(seed=71, n_samples=n_s * m + 5, T_sft=float(kw.pop("T_sft", n_s)), T_max=float(n_s), T_short=float(n_s),
+                    f_band=0.5 if learned else 0.1, n_templates=n_t, duty=0.7, mean_lock_s=1.5 * n_s, templates=templates, **kw)
+    p = oracle.make_plan(ds.cfg)
+    interp = None
+    with cc.CrossCorrPlan(ds.cfg, ds.dets, interp=cc.INTERP_LEARNED if learned else cc.INTERP_EXACT) as plan:
+        if learned:
+            from oracle import learned as ol
+            from paper_1712_06515_gb300 import learned_interp
+            model = ol.load(learned_interp.WEIGHTS)
+            interp = lambda x, j, d: ol.interpolate(x, j, d, model, plan.nu_c)   # noqa: E731
+        ab, norm = plan.resample(torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV))
+        ab, norm = ab.cpu().numpy(), norm.cpu().numpy()
+    r = np.arange(p.M * p.N_s)
+    rot = np.exp(-2j * np.pi * ((p.f_r * r * p.dt) % 1.0))
+    nsft = int(round(ds.cfg.T_sft / ds.cfg.dt))
+    for t in sorted({0, n_t // 2, n_t - 1}):
+        for q, det in enumerate(ds.dets):
+            xr, js, de = oracle.resample(ds.x[q], det, ds.cfg, p, ds.templates[t], interp)
+            al, be, s2 = oracle.weights(det, ds.cfg, js, de)
+            ok = (np.abs(np.abs(de) - 0.5) > 1e-5) & ((np.abs(de) > 1e-5) | (js % nsft != 0))
+            if learned:
+                ok &= np.abs(de) > 1e-5
+            for w, ref in ((0, al * xr * rot), (1, be * xr * rot)):
+                err = np.abs(ab[t, q, w] - ref)[ok].max()
+                assert err <= tol * max(1e-30, np.abs(ref).max()), (t, q, w, err)
+            for i, ref in enumerate(oracle.segment_norms(al, be, s2, p)):
+                lim = 2e-5 * np.abs(oracle.segment_norms(al, be, s2, p)).max()
+                assert np.abs(norm[t, q, :, i] - ref).max() <= lim
+
+
+@pytest.mark.parametrize("n_s,m,n_t", [(64, 20, 5), (127, 12, 4), (129, 12, 1), (512, 6, 9), (513, 6, 7), (1536, 4, 9),
+                                       (1537, 4, 13), (3616, 3, 5), (3617, 3, 2), (7300, 2, 1)])
+def test_segment_lengths(n_s, m, n_t):
+    check(n_s, m, n_t)
+
+
+@pytest.mark.parametrize("D", [1, 7, 16, 32])
+def test_stencils(D):
+    check(600, 6, 3, D=D, T_sft=200)
+
+
+def test_learned():
+    check(600, 6, 3, learned=True, T_sft=200, f_h=150.0)
+
+
+def test_templates_far_apart():
+    """Projected axes from 0.1 to 45 s in one group: delays differ by up to 90 samples, beyond the
+    staged window's slack.  The heterodyne phase f_h pp is an FP32 product of up to f_h a_p Omega
+    KNOT cycles per knot interval, three roundings of it: 2 pi 3 2^-24 of that more than the bound
+    of the other tests."""
+    tm = np.array([[0.1, synth.T_ASC_O1, synth.SCO_X1_P], [45.0, synth.T_ASC_O1, synth.SCO_X1_P],
+                   [45.0, synth.T_ASC_O1 + 0.5 * synth.SCO_X1_P, synth.SCO_X1_P], [1.44, synth.T_ASC_O1, synth.SCO_X1_P]])
+    tol = 2e-5 + 2 * np.pi * 3 * 2.0 ** -24 * 120.0 * 45.0 * (2 * np.pi / synth.SCO_X1_P) * 128
+    check(600, 8, 4, templates=tm, T_sft=200, tol=tol)
