@@ -143,7 +143,7 @@ struct cc_plan {
     // two-pass search, lag grid: coset and pass twiddles [C][272] of the plan's grid and of one
     // coset, roots of its transform length and of 4096 (plan-owned)
     const float2 *corr_twk = nullptr, *corr_twk1 = nullptr, *corr_twL = nullptr, *corr_tw4096 = nullptr;
-    const float4 *corr_tw8 = nullptr, *corr_tw8_1 = nullptr;   // [C][256][2] last-pass powers (corr.cuh)
+    const float2 *corr_twp = nullptr, *corr_twp4096 = nullptr;   // last-pass powers (corr_powers)
     int* segfft_ctr = nullptr;                // [C4] unit counters of the staged segment FFT (plan-owned)
     bool ws_external = false;                 // ws is caller memory (crosscorr_plan_set_workspace)
     // diagnostic event pairs around fused-kernel launches (crosscorr_plan_set_kernel_timing)

@@ -41,8 +41,15 @@ CC_CORR_INST(extern, 1024)
 CC_CORR_INST(extern, 2048)
 CC_CORR_INST(extern, 4096)
 CC_CORR_INST_FULL(extern)
+CC_CORR_INST_MULTI(extern, 256)
+CC_CORR_INST_MULTI(extern, 512)
+CC_CORR_INST_MULTI(extern, 1024)
+CC_CORR_INST_MULTI(extern, 2048)
+CC_CORR_INST_MULTI(extern, 4096)
+CC_CORR_INST_MULTI_FULL(extern)
 
 constexpr size_t TWO_PASS_WS_BUDGET = (size_t)24 << 30;   // a_r, b_r (and folded rows) of one template batch
+constexpr size_t MULTI_WS_BUDGET = (size_t)4 << 30;       // the same for three and four detectors (the fused path's plans)
 constexpr int LAG_THREADS = 256;
 constexpr int ROW_BLOCK = 32;        // partial rows summed by one block of corr_rows_kernel
 
@@ -202,12 +209,29 @@ static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 static size_t al128(size_t b) { return (b + 127) & ~(size_t)127; }
 
 struct CorrLayout {
-    int L, C, T, half, folded, bf16_rows, planes, n_rows, n_blocks, n_lags;
+    int L, C, T, half, padded, folded, bf16_rows, planes, n_rows, n_blocks, n_lags;
     int64_t G, t_pad;
     CorrArgs a;
     // workspace pieces of a batch, bytes
     size_t ab, z, norm, act, D, raw, rows2, U, h, kn, total;
 };
+
+std::vector<float2> corr_powers(int64_t L, int64_t C) {
+    const int64_t GT = L / 16, RL = L >= 512 ? L / 256 : L / 16, nb = 16 / RL, G = C * L;
+    int np = 0;
+    while ((1 << np) < RL) ++np;
+    std::vector<float2> v((size_t)(C * nb * np * GT));
+    for (int64_t c = 0; c < C; ++c)
+        for (int64_t i = 0; i < nb; ++i)
+            for (int n = 0; n < np; ++n)
+                for (int64_t j = 0; j < GT; ++j) {
+                    // the thread's butterfly: column k, row i0 + RL i of the second pass's outputs
+                    const int64_t b = L >= 512 ? 16 * ((j & 15) % RL + RL * i) + (j >> 4) + RL * ((j & 15) / RL) : j + GT * i;
+                    const double a = -2.0 * M_PI * (double)(((c + C * b) << n) % G) / (double)G;
+                    v[(size_t)(((c * nb + i) * np + n) * GT + j)] = make_float2((float)cos(a), (float)sin(a));
+                }
+    return v;
+}
 
 // Whether the plan takes the two-pass kernels by name (CC_PATH_TWO_PASS): Q <= 2, R <= 1, no
 // cross-only pair set, coset length 64..4096, every bin in the lower half of its coset.
@@ -216,6 +240,15 @@ bool two_pass_supported(const cc_plan* plan) {
     if (p.Q > 2 || p.R > 1 || p.pair_mode == CC_PAIRS_CROSS_ONLY) return false;
     if (p.L < 64 || p.L > 4096 || plan->N_f < 1) return false;
     return 2 * ((plan->kbar.back() - plan->k0) / p.C) < p.L;
+}
+
+// Whether the lag grid serves the plan: the conditions of two_pass_supported but any output bins
+// (the last transform reaches all of them); with three or four detectors FP32 storage and at
+// least 256-point transforms (one activity bit per detector and template of a series group).
+bool lag_grid_supported(const cc_plan* plan) {
+    const DevParams& p = plan->dp;
+    if (p.R > 1 || p.pair_mode == CC_PAIRS_CROSS_ONLY || p.L < 64 || p.L > 4096 || plan->N_f < 1) return false;
+    return p.Q <= 2 || (p.store == CC_STORE_FP32 && p.L >= 128);
 }
 
 static int sm_count() {
@@ -228,6 +261,7 @@ static int sm_count() {
 static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     const DevParams& p = plan->dp;
     const bool padded = plan->tuning.transform_len == CORR_POINTS && p.L < CORR_POINTS;
+    y->padded = padded;
     y->folded = p.N_s > CORR_POINTS;
     y->half = 2 * p.N_s <= CORR_POINTS;
     y->L = y->half && !padded ? 2 * p.L : CORR_POINTS;
@@ -245,12 +279,11 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     a.row_bytes = (uint32_t)(a.n_in * esz);
     a.row_stride = (uint32_t)((y->half ? y->L / 2 : y->L) * esz);   // whole inputs, zero beyond the samples
     a.tma = a.row_bytes % 16 == 0;   // bulk copies: rows of whole 16-byte pieces start on 16-byte boundaries
-    const size_t buf = (size_t)y->T * padded_len(y->L) * sizeof(float2);
     size_t o = al128((size_t)y->T * a.row_stride);
     a.off_y = (uint32_t)o;
-    o = al128(o + buf);
-    a.off_z = (uint32_t)o;
-    o = al128(o + buf);
+    o = al128(o + (size_t)2 * CORR_POINTS * sizeof(float2));
+    a.off_tw = (uint32_t)o;
+    o += (272 + 1024) * sizeof(float2);
     a.off_act = (uint32_t)o;
     o += (CORR_MAX_CHUNK + 1) * sizeof(uint32_t);
     a.off_bar = (uint32_t)o;
@@ -286,7 +319,7 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     y->ab = al256(b * plan->Q * 2 * plan->N_tau * (plan->cfg.store == CC_STORE_BF16 ? 4 : 8));
     y->z = y->folded ? al256(b * plan->Q * 2 * plan->M * y->G * esz) : 0;
     y->norm = al256(b * plan->Q * plan->M * sizeof(float4));
-    y->act = al256((size_t)2 * plan->M * y->t_pad);
+    y->act = al256((size_t)plan->Q * plan->M * y->t_pad);
     y->D = al256(b * sizeof(double));
     y->raw = al256(b * y->n_rows * y->planes * y->G * sizeof(float));
     y->rows2 = al256(b * y->n_blocks * y->planes * y->G * sizeof(float));
@@ -302,7 +335,7 @@ static int64_t two_pass_batch(const cc_plan* plan, int64_t n_t) {
                        (plan->N_s > CORR_POINTS ? (size_t)plan->Q * 2 * plan->M * 2 * fold_count(plan) * CORR_POINTS * 8
                                                 : 0);
     const int64_t b = plan->tuning.batch_templates > 0 ? plan->tuning.batch_templates
-                                                       : (int64_t)std::max<size_t>(1, TWO_PASS_WS_BUDGET / per);
+                                                       : (int64_t)std::max<size_t>(1, (plan->Q > 2 ? MULTI_WS_BUDGET : TWO_PASS_WS_BUDGET) / per);
     return std::max<int64_t>(1, std::min<int64_t>({b, n_t, 65535}));
 }
 
@@ -388,20 +421,34 @@ size_t two_pass_workspace_bytes(const cc_plan* plan, int64_t n_t) {
 
 template <bool BF16, bool LAG>
 static cudaError_t launch_corr_l(const CorrLayout& y, int sms, cudaStream_t st) {
-    if (!y.half) return launch_corr_t<4096, BF16, LAG, false>(y.a, sms, st);
+    if (!y.half) return launch_corr_t<4096, BF16, LAG, false, false>(y.a, sms, st);
     switch (y.L) {
-        case 128: return launch_corr_t<128, BF16, LAG, true>(y.a, sms, st);
-        case 256: return launch_corr_t<256, BF16, LAG, true>(y.a, sms, st);
-        case 512: return launch_corr_t<512, BF16, LAG, true>(y.a, sms, st);
-        case 1024: return launch_corr_t<1024, BF16, LAG, true>(y.a, sms, st);
-        case 2048: return launch_corr_t<2048, BF16, LAG, true>(y.a, sms, st);
-        case 4096: return launch_corr_t<4096, BF16, LAG, true>(y.a, sms, st);
+        case 128: return launch_corr_t<128, BF16, LAG, true, false>(y.a, sms, st);
+        case 256: return launch_corr_t<256, BF16, LAG, true, false>(y.a, sms, st);
+        case 512: return launch_corr_t<512, BF16, LAG, true, false>(y.a, sms, st);
+        case 1024: return launch_corr_t<1024, BF16, LAG, true, false>(y.a, sms, st);
+        case 2048: return launch_corr_t<2048, BF16, LAG, true, false>(y.a, sms, st);
+        case 4096: return launch_corr_t<4096, BF16, LAG, true, false>(y.a, sms, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <bool LAG>
+static cudaError_t launch_corr_multi(const CorrLayout& y, int sms, cudaStream_t st) {
+    if (!y.half) return launch_corr_t<4096, false, LAG, false, true>(y.a, sms, st);
+    switch (y.L) {
+        case 256: return launch_corr_t<256, false, LAG, true, true>(y.a, sms, st);
+        case 512: return launch_corr_t<512, false, LAG, true, true>(y.a, sms, st);
+        case 1024: return launch_corr_t<1024, false, LAG, true, true>(y.a, sms, st);
+        case 2048: return launch_corr_t<2048, false, LAG, true, true>(y.a, sms, st);
+        case 4096: return launch_corr_t<4096, false, LAG, true, true>(y.a, sms, st);
     }
     return cudaErrorInvalidValue;
 }
 
 static cudaError_t launch_corr(const CorrLayout& y, cudaStream_t st) {
     const int sms = sm_count();
+    if (y.a.Q > 2) return y.planes > 1 ? launch_corr_multi<true>(y, sms, st) : launch_corr_multi<false>(y, sms, st);
     if (y.bf16_rows) return y.planes > 1 ? launch_corr_l<true, true>(y, sms, st) : launch_corr_l<true, false>(y, sms, st);
     return y.planes > 1 ? launch_corr_l<false, true>(y, sms, st) : launch_corr_l<false, false>(y, sms, st);
 }
@@ -453,8 +500,7 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         a.ctr = ctr;
         a.err = p.err;
         a.twk = y.C == 1 ? plan->corr_twk1 : plan->corr_twk;
-        a.tw8 = y.C == 1 ? plan->corr_tw8_1 : plan->corr_tw8;
-        a.twL = y.L == CORR_POINTS ? plan->corr_tw4096 : plan->corr_twL;
+        a.twp = y.padded ? plan->corr_twp4096 : plan->corr_twp;
         a.N_s = p.N_s;
         a.M = (int)p.M;
         a.N_tau = p.N_tau;
@@ -483,7 +529,7 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         }
         q.U = U;
         q.h = y.C > 2 ? h : nullptr;
-        q.twL = a.twL;
+        q.twL = y.L == CORR_POINTS ? plan->corr_tw4096 : plan->corr_twL;
         q.norm = (const float4*)norm;
         q.D = D;
         q.M = p.M;

@@ -14,33 +14,36 @@ constexpr int CORR_POINTS = 4096;   // points of one CTA's transforms: 4096 / L 
 // Everything corr_kernel needs.
 struct CorrArgs {
     const void* src;        // a_r, b_r [n_t][Q][2][N_tau], or folded rows Z [n_t][Q][2][M][C][4096]
-    const uint8_t* act;     // [2][M][t_pad]: detector 0 / the last detector has weight in (segment, template)
+    const uint8_t* act;     // [Q][M][t_pad]: the detector has weight in (segment, template)
     float* raw;             // [n_t][2 n_chunks][planes][C][L] partial sums (planes: A, and Re B, Im B with a lag)
     int* ctr;               // unit counter, zero at launch
     unsigned* err;          // the plan's device error word
     const float2* twk;      // [C][272] coset and second-pass twiddles on the grid of G = C L points
-    const float4* tw8;      // [C][256][2] powers 1, 2, 4, 8 of W_G^(c + C j), G = 4096 C (last pass of L = 4096)
-    const float2* twL;      // exp(-2 pi i j / L)
+    const float2* twp;      // [C][butterflies][powers][L / 16] last-pass twiddle powers per thread (corr_powers)
     int64_t N_s, N_tau;
     int M, chunk_len, n_t, t_pad, Q, C, n_chunks, units;
     int n_in;               // samples of a staged row: N_s, or 4096 positions of a folded row
     int folded, tma, all_ordered, wait_test;
-    uint32_t row_bytes, row_stride, off_y, off_z, off_act, off_bar, smem;
+    uint32_t row_bytes, row_stride, off_y, off_tw, off_act, off_bar, smem;
 };
 
-template <int LT, bool BF16, bool LAG, bool HALF>
+template <int LT, bool BF16, bool LAG, bool HALF, bool MULTI>
 cudaError_t launch_corr_t(const CorrArgs& a, int sms, cudaStream_t st);
 
-#define CC_CORR_INST(KW, L)                                                                    \
-    KW template cudaError_t launch_corr_t<L, false, false, true>(const CorrArgs&, int, cudaStream_t);  \
-    KW template cudaError_t launch_corr_t<L, false, true, true>(const CorrArgs&, int, cudaStream_t);   \
-    KW template cudaError_t launch_corr_t<L, true, false, true>(const CorrArgs&, int, cudaStream_t);   \
-    KW template cudaError_t launch_corr_t<L, true, true, true>(const CorrArgs&, int, cudaStream_t);
-#define CC_CORR_INST_FULL(KW)                                                                  \
-    KW template cudaError_t launch_corr_t<4096, false, false, false>(const CorrArgs&, int, cudaStream_t); \
-    KW template cudaError_t launch_corr_t<4096, false, true, false>(const CorrArgs&, int, cudaStream_t);  \
-    KW template cudaError_t launch_corr_t<4096, true, false, false>(const CorrArgs&, int, cudaStream_t);  \
-    KW template cudaError_t launch_corr_t<4096, true, true, false>(const CorrArgs&, int, cudaStream_t);
+#define CC_CORR_ONE(KW, L, B, G, H, MU) KW template cudaError_t launch_corr_t<L, B, G, H, MU>(const CorrArgs&, int, cudaStream_t);
+#define CC_CORR_INST(KW, L) \
+    CC_CORR_ONE(KW, L, false, false, true, false) CC_CORR_ONE(KW, L, false, true, true, false) \
+    CC_CORR_ONE(KW, L, true, false, true, false) CC_CORR_ONE(KW, L, true, true, true, false)
+#define CC_CORR_INST_FULL(KW) \
+    CC_CORR_ONE(KW, 4096, false, false, false, false) CC_CORR_ONE(KW, 4096, false, true, false, false) \
+    CC_CORR_ONE(KW, 4096, true, false, false, false) CC_CORR_ONE(KW, 4096, true, true, false, false)
+// three or four detectors (FP32 rows)
+#define CC_CORR_INST_MULTI(KW, L) CC_CORR_ONE(KW, L, false, false, true, true) CC_CORR_ONE(KW, L, false, true, true, true)
+#define CC_CORR_INST_MULTI_FULL(KW) CC_CORR_ONE(KW, 4096, false, false, false, true) CC_CORR_ONE(KW, 4096, false, true, false, true)
+
+// Threads' last-pass twiddle powers for C cosets of L points (host, at plan creation): thread j
+// of a transform, butterfly i, power 2^n of W_G^(c + C b), G = C L, at ((c nb + i) np + n) L/16 + j.
+std::vector<float2> corr_powers(int64_t L, int64_t C);
 
 // Work units per resident CTA slot (2 per SM), shared by the layout and the launch.
 constexpr int CORR_CTAS_PER_SM = 2;

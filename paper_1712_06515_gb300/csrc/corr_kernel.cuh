@@ -11,7 +11,7 @@
 //
 // With T_K(j) the transform of segment K from its own first sample on, S_K the sum over
 // detectors, the kernel accumulates over segments, per template and weight,
-//   A(j) = sum_K Re(conj(T1_K) T0_K)   (|S_K|^2 with every ordered pair), real,
+//   A(j) = sum_K sum_(X<Y) Re(conj(T_YK) T_XK)   (|S_K|^2 with every ordered pair), real,
 //   B(j) = sum_K conj(S_K) S_(K-1)     (R = 1), complex,
 // each in compensated FP32.
 //
@@ -31,10 +31,14 @@
 //   * the running sums, their compensations and S_(K-1) -- 128 words per thread -- live in
 //     tensor memory, 32 columns per group of four bins, read and written by
 //     tcgen05.ld/st once per segment: registers hold only the transform (16 points), and
-//     detector 0's spectrum, so two CTAs of 128 registers fit an SM without spills;
+//     detector 0's spectrum (MULTI, three or four detectors: the
+//     sum of the earlier ones), so two CTAs of 128 registers fit an SM without spills;
 //   * twiddles as in the staged kernel: the coset factor of sample s = t + 256 r is split
 //     between a factor per r (first pass) and the table of the second and the powers of the
-//     last pass.
+//     last pass.  The coset's tables (10 KB) are kept in shared memory: read through L1, whose
+//     share beside 2 x 110 KB is 8 KB, they cost 8 % of the kernel;
+//   * one CTA barrier per transform: the second pass's outputs that a last-pass butterfly needs
+//     come from one column of threads, which share a half-warp and exchange them in place.
 //
 // What bounds it (L = 4096): the FP32 pipe and the shared-memory exchanges of the two inner
 // passes, each about 1500 cycles per 4096-point transform and SM.
@@ -92,14 +96,42 @@ struct CorrShape {
     static constexpr int L = LT;
     static constexpr int T = CORR_POINTS / L;            // transforms per CTA
     static constexpr int GT = L / 16;                    // threads per transform
-    static constexpr int PL = padded_len(L);
     static constexpr bool PASS2 = L >= 512;              // a radix-16 pass with NS = 16
     static constexpr int RL = PASS2 ? L / 256 : L / 16;  // radix of the last pass
     static constexpr int NSL = L / RL;                   // its butterflies
     static constexpr int BPT = 16 / RL;                  // of them per thread
+    static constexpr int NP = RL == 16 ? 4 : RL == 8 ? 3 : RL == 4 ? 2 : 1;   // twiddle powers of one: 1, 2, 4, 8
     static constexpr int TA = T > 1 ? T / 2 : 1;         // templates of a series group
     static_assert(T * GT == CORR_THREADS && NSL == GT * BPT, "16 points per thread in every pass");
 };
+
+// x[r] *= w^r, r < R, from the powers 1, 2, 4, 8 of w (as many as R needs).
+template <int R>
+__device__ __forceinline__ void twiddle_powers(float2 (&x)[16], const float2 (&w)[4]) {
+    x[1] = cmul(x[1], w[0]);
+    if constexpr (R >= 4) {
+        const float2 w3 = cmul(w[1], w[0]);
+        x[2] = cmul(x[2], w[1]);
+        x[3] = cmul(x[3], w3);
+        if constexpr (R >= 8) {
+            x[4] = cmul(x[4], w[2]);
+            x[5] = cmul(x[5], cmul(w[2], w[0]));
+            x[6] = cmul(x[6], cmul(w[2], w[1]));
+            x[7] = cmul(x[7], cmul(w[2], w3));
+            if constexpr (R == 16) {
+                const float2 w12 = cmul(w[3], w[2]);
+                x[8] = cmul(x[8], w[3]);
+                x[9] = cmul(x[9], cmul(w[3], w[0]));
+                x[10] = cmul(x[10], cmul(w[3], w[1]));
+                x[11] = cmul(x[11], cmul(w[3], w3));
+                x[12] = cmul(x[12], w12);
+                x[13] = cmul(x[13], cmul(w12, w[0]));
+                x[14] = cmul(x[14], cmul(w12, w[1]));
+                x[15] = cmul(x[15], cmul(w12, w3));
+            }
+        }
+    }
+}
 
 // Compensated sums of two FP32 values in paired operations (the same rounding as kahan_add
 // on each): y = v - c, t = s + y, c = (t - s) - y.
@@ -119,15 +151,17 @@ __device__ __forceinline__ uint32_t act_bits(const uint8_t* p, int valid) {
     return b;
 }
 
-template <int LT, bool BF16, bool LAG, bool HALF>
+template <int LT, bool BF16, bool LAG, bool HALF, bool MULTI>
 __global__ void __launch_bounds__(CORR_THREADS, CORR_CTAS_PER_SM)
 corr_kernel(const CorrArgs q) {
     using S = CorrShape<LT>;
-    constexpr int L = S::L, T = S::T, GT = S::GT, PL = S::PL, RL = S::RL, NSL = S::NSL, BPT = S::BPT, TA = S::TA;
+    constexpr int L = S::L, T = S::T, GT = S::GT, RL = S::RL, NSL = S::NSL, BPT = S::BPT, TA = S::TA, NP = S::NP;
     constexpr int W = LAG ? 32 : 8;                  // tensor-memory words per group of four bins
     constexpr uint32_t COLS = LAG ? 256 : 64;        // two warps of a lane quarter, four groups each
     constexpr uint32_t ESZ = BF16 ? 4 : 8;
     constexpr int PLANES = LAG ? 3 : 1;
+    constexpr int SH = MULTI ? 8 : 16;               // activity bits of a detector in a segment's word
+    static_assert(TA <= SH, "one activity bit per template of the group");
     extern __shared__ __align__(128) unsigned char sm[];
     unsigned char* stage = sm;
     uint64_t* bar = (uint64_t*)(sm + q.off_bar);
@@ -136,9 +170,20 @@ corr_kernel(const CorrArgs q) {
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = tid / GT, j = tid % GT;
-    float2* Y = (float2*)(sm + q.off_y) + g * PL;
-    float2* Z = (float2*)(sm + q.off_z) + g * PL;
+    // Exchange buffers: element p of a transform lies at 16 (p >> 4) + ((p ^ (p >> 4)) & 15), so
+    // that 16 lanes reach 16 different banks down a column as well as along a row (8-point last
+    // passes of neighbouring groups also take different halves).  ey: this thread's group.
+    float2* const ex = (float2*)(sm + q.off_y);
+    const int gsw = GT == 8 ? 8 * (g & 1) : 0;
+    // second and last pass: thread j takes column k, rows i + RL r (see below)
+    const int hw = j >> 4, i0 = S::PASS2 ? (j & 15) % RL : 0, k = S::PASS2 ? hw + RL * ((j & 15) / RL) : 0;
+    const int wr1 = g * L + 16 * j + ((j & 15) ^ gsw);                     // ^ r: pass 1's output r
+    const int rd2 = g * L + 16 * i0 + (k ^ i0);                            // pass 2's row i0, column k
+    const int rd3 = g * L + 16 * RL * i0 + 16 * i0 + (k ^ i0 ^ ((RL * i0) & 15));
     uint32_t* aw = (uint32_t*)(sm + q.off_act);      // per segment of the chunk: activity bits
+    float2* const twk = (float2*)(sm + q.off_tw);    // the coset's first- and second-pass twiddles,
+    float2* const twp = twk + 272;                   // and the last pass's powers
+    int c_held = -1;
     const int C = q.C, M = q.M;
     const size_t act_x = (size_t)M * q.t_pad;        // bytes of one detector's activity
 
@@ -176,31 +221,37 @@ corr_kernel(const CorrArgs q) {
         // this thread's series: template t, weight w
         const int ser = sg * T + g;
         const int t = ser >> 1, w = ser & 1;
-        const bool valid = t < q.n_t;
-        // activity of the chunk's segments: bit i, template i of the group has weight of
-        // detector 0; bit 16 + i, of the last detector
+        // the coset's tables, when it changes
+        if (c != c_held) {
+            for (int i = tid; i < 272; i += CORR_THREADS) twk[i] = __ldg(q.twk + (size_t)c * 272 + i);
+            for (int i = tid; i < BPT * NP * GT; i += CORR_THREADS) twp[i] = __ldg(q.twp + (size_t)c * BPT * NP * GT + i);
+            c_held = c;
+        }
+        // activity of the chunk's segments: bit X SH + i, template i of the group has weight of
+        // detector X
         {
             const int t0 = (sg * T) >> 1, nvalid = min(TA, q.n_t - t0);
             for (int K = Kl + tid; K < Kb; K += CORR_THREADS) {
                 const uint8_t* p = q.act + (size_t)K * q.t_pad + t0;
-                uint32_t b = act_bits<TA>(p + act_x, nvalid) << 16;
-                if (q.Q > 1) b |= act_bits<TA>(p, nvalid);
+                uint32_t b = act_bits<TA>(p, nvalid);
+                for (int X = 1; X < q.Q; ++X) b |= act_bits<TA>(p + X * act_x, nvalid) << (X * SH);
                 aw[K - Kl] = b;
             }
         }
         __syncthreads();
         // the transform after (K, X) in unit order; X = -1 starts at segment K
         auto next_after = [&](int K, int X, int& nK, int& nX) -> bool {
-            if (X == 0 && q.Q > 1 && (aw[K - Kl] >> 16)) {
+            uint32_t b = X + 1 < q.Q ? aw[K - Kl] >> ((X + 1) * SH) : 0u;
+            if (b) {
                 nK = K;
-                nX = q.Q - 1;
+                nX = X + 1 + (__ffs(b) - 1) / SH;
                 return true;
             }
-            for (int k = X < 0 ? K : K + 1; k < Kb; ++k) {
-                const uint32_t b = aw[k - Kl];
+            for (int k = K + 1; k < Kb; ++k) {
+                b = aw[k - Kl];
                 if (b) {
                     nK = k;
-                    nX = (b & 0xffffu) ? 0 : q.Q - 1;
+                    nX = (__ffs(b) - 1) / SH;
                     return true;
                 }
             }
@@ -225,7 +276,7 @@ corr_kernel(const CorrArgs q) {
                     }
                 } else if (warp == 0 && next_after(K, X, nK, nX)) {
                     const int s2 = sg * T + lane, tt = s2 >> 1;
-                    const uint32_t b = aw[nK - Kl] >> (nX == q.Q - 1 ? 16 : 0);
+                    const uint32_t b = aw[nK - Kl] >> (nX * SH);
                     const bool on = lane < T && ((b >> (lane >> 1)) & 1u);
                     const int n = __popc(__ballot_sync(0xffffffffu, on));
                     if (lane == 0) {
@@ -236,7 +287,7 @@ corr_kernel(const CorrArgs q) {
                     if (on) tma_load_1d(stage + lane * q.row_stride, row(nK, nX, tt, s2 & 1), q.row_bytes, bar);
                 }
             } else {
-                if (next_after(K, X, nK, nX) && ((aw[nK - Kl] >> (nX == q.Q - 1 ? 16 : 0)) & own_bit)) {
+                if (next_after(K, X, nK, nX) && ((aw[nK - Kl] >> (nX * SH)) & own_bit)) {
                     const char* src = row(nK, nX, t, w);
                     unsigned char* dst = stage + g * q.row_stride;
                     for (int s = j; s < q.n_in; s += GT) cp_async<ESZ>(dst + s * ESZ, src + s * ESZ);
@@ -252,9 +303,6 @@ corr_kernel(const CorrArgs q) {
 #pragma unroll
             for (int gi = 0; gi < 4; ++gi) tmem_st(tm + gi * W, z);
         }
-        // last pass of L = 4096: e, 2 e, 4 e and 8 e-th powers of W_G^(c + C tid)
-        const float4* __restrict__ tw8 = q.tw8 + ((size_t)c * CORR_THREADS + j) * 2;
-        const float2* __restrict__ twk = q.twk + (size_t)c * 272;
 
         if (!(q.wait_test && first_unit)) issue_after(Kl, -1);
         first_unit = false;
@@ -267,13 +315,20 @@ corr_kernel(const CorrArgs q) {
                 prev_zero = true;
                 continue;
             }
-            const bool a0 = (bits & 0xffffu) != 0, al = (bits >> 16) != 0;
+            const bool acc_on = !LAG || K >= Ka;
             float2 v[16], f0[16];
 #pragma unroll
             for (int e = 0; e < 16; ++e) v[e] = make_float2(0.f, 0.f);
+            if constexpr (MULTI) {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) f0[e] = make_float2(0.f, 0.f);
+            }
+            bool have = false;   // MULTI: f0 holds a sum of detectors
 #pragma unroll 1
-            for (int pass = a0 ? 0 : 1; pass < (al ? 2 : 1); ++pass) {
-                if (pass == 1) {
+            for (int X = 0; X < q.Q; ++X) {
+                const uint32_t xbits = (bits >> (X * SH)) & ((1u << SH) - 1u);
+                if (!xbits) continue;
+                if (!MULTI && X == 1) {
 #pragma unroll
                     for (int e = 0; e < 16; ++e) f0[e] = v[e];   // detector 0's spectrum (zero without weight)
                 }
@@ -292,91 +347,100 @@ corr_kernel(const CorrArgs q) {
                     if constexpr (BF16) v[r] = __bfloat1622float2(((const __nv_bfloat162*)st)[j + r * GT]);
                     else v[r] = ((const float2*)st)[j + r * GT];
                 }
-                if (T > 1 && !((pass == 0 ? bits : bits >> 16) & own_bit)) {   // no weight: the row was not copied
+                if (T > 1 && !(xbits & own_bit)) {   // no weight: the row was not copied
 #pragma unroll
                     for (int r = 0; r < 8; ++r) v[r] = make_float2(0.f, 0.f);
                 }
-                // buffers alternate between transforms when there is no second pass
-                float2* buf = S::PASS2 || parity == 0 ? Y : Z;
+                // buffers alternate between transforms: one CTA barrier each
+                float2* buf = ex + (parity ? CORR_POINTS : 0);
                 parity ^= 1;
                 if constexpr (HALF) {
                     dft16_in8(v);
                 } else {
                     if (c > 0) {
 #pragma unroll
-                        for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(twk + r));
+                        for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], twk[r]);
                     }
                     dft16(v);
                 }
-                {
-                    float2* d = buf + 17 * j;   // padi(16 j + r)
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) d[r] = v[r];
-                }
+                for (int r = 0; r < 16; ++r) buf[wr1 ^ r] = v[r];
                 // every thread has read the stage and written its outputs; all agree on a failed wait
                 if (__syncthreads_or(!ok)) {
                     failed = true;
                     break;
                 }
-                issue_after(K, pass == 0 && q.Q > 1 ? 0 : q.Q - 1);
-                const float2* src = buf;
+                issue_after(K, X);
+                // last pass: butterfly (i) of this thread leaves outputs m = b + NSL r in v[i RL + r]
                 if constexpr (S::PASS2) {
-                    const int k = j & 15;
-                    const float2* s = Y + padi(j);
+                    // second pass on column k = j' mod 16 of the rows j' >> 4 + RL r (j' the Stockham
+                    // index): the last pass needs the outputs of the RL threads of that column only,
+                    // which sit in one half-warp and exchange them in place, without a CTA barrier
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) v[r] = s[r * pstride<S::PASS2 ? GT : 16>()];
+                    for (int r = 0; r < 16; ++r) v[r] = buf[(rd2 ^ ((RL * r) & 15)) + 16 * RL * r];
 #pragma unroll
-                    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(twk + 16 + r * 16 + k));
+                    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], twk[16 + r * 16 + k]);
                     dft16(v);
-                    float2* d = Z + padi((j - k) * 16 + k);
+                    __syncwarp();
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) d[r * pstride<16>()] = v[r];
-                    __syncthreads();
-                    src = Z;
-                }
-                // last pass into registers: butterfly b = j + GT i leaves outputs m = b + NSL r
-                // in v[i RL + r]
-                if constexpr (L == 4096) {
-                    const float2* s = src + padi(j);
-                    const float4 p0 = __ldg(tw8), p1 = __ldg(tw8 + 1);
+                    for (int r = 0; r < 16; ++r) {
+                        const int cx = r & (RL - 1);
+                        buf[(rd2 ^ (16 * cx + (cx ^ ((RL * r) & 15)))) + 16 * RL * r] = v[r];
+                    }
+                    __syncwarp();
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) v[r] = s[r * pstride<256>()];
-                    const float2 b1 = make_float2(p0.x, p0.y), b2 = make_float2(p0.z, p0.w);
-                    const float2 b4 = make_float2(p1.x, p1.y), b8 = make_float2(p1.z, p1.w);
-                    const float2 b3 = cmul(b2, b1), b12 = cmul(b8, b4);
-                    v[1] = cmul(v[1], b1);
-                    v[2] = cmul(v[2], b2);
-                    v[3] = cmul(v[3], b3);
-                    v[4] = cmul(v[4], b4);
-                    v[5] = cmul(v[5], cmul(b4, b1));
-                    v[6] = cmul(v[6], cmul(b4, b2));
-                    v[7] = cmul(v[7], cmul(b4, b3));
-                    v[8] = cmul(v[8], b8);
-                    v[9] = cmul(v[9], cmul(b8, b1));
-                    v[10] = cmul(v[10], cmul(b8, b2));
-                    v[11] = cmul(v[11], cmul(b8, b3));
-                    v[12] = cmul(v[12], b12);
-                    v[13] = cmul(v[13], cmul(b12, b1));
-                    v[14] = cmul(v[14], cmul(b12, b2));
-                    v[15] = cmul(v[15], cmul(b12, b3));
-                    dft16(v);
+                    for (int i = 0; i < BPT; ++i)
+#pragma unroll
+                        for (int r = 0; r < RL; ++r)
+                            v[i * RL + r] = buf[(rd3 ^ (17 * r) ^ ((RL * RL * i) & 15)) + 16 * RL * RL * i];
                 } else {
 #pragma unroll
-                    for (int i = 0; i < BPT; ++i) {
-                        const int b = j + GT * i;
-                        const float2* s = src + padi(b);
-                        float2 x[16];
+                    for (int i = 0; i < BPT; ++i)
 #pragma unroll
-                        for (int r = 0; r < RL; ++r) x[r] = s[r * pstride<NSL>()];
-                        apply_twiddles<RL>(x, q.twL, b, L - 1);
-                        dft_r<RL>(x);
+                        for (int r = 0; r < RL; ++r)
+                            v[i * RL + r] = buf[g * L + 16 * r + (((j + GT * i) ^ r ^ gsw) & 15)];
+                }
 #pragma unroll
-                        for (int r = 0; r < RL; ++r) v[i * RL + r] = x[r];
+                for (int i = 0; i < BPT; ++i) {
+                    float2 x[16];
+#pragma unroll
+                    for (int r = 0; r < RL; ++r) x[r] = v[i * RL + r];
+                    float2 pw[4];
+#pragma unroll
+                    for (int n = 0; n < NP; ++n) pw[n] = twp[(i * NP + n) * GT + j];
+                    twiddle_powers<RL>(x, pw);
+                    dft_r<RL>(x);
+#pragma unroll
+                    for (int r = 0; r < RL; ++r) v[i * RL + r] = x[r];
+                }
+                if constexpr (MULTI) {
+                    // pairs of this detector with the earlier ones: A += Re(conj(F) sum), sum += F
+                    if (have && acc_on && !q.all_ordered) {
+                        tmem_wait_st();
+#pragma unroll
+                        for (int gi = 0; gi < 4; ++gi) {
+                            float z[8];
+                            tmem_ld(z, tm + gi * W);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const int e = 4 * gi + 2 * h;
+                                float2 s = make_float2(z[2 * h], z[2 * h + 1]), cp = make_float2(z[4 + 2 * h], z[5 + 2 * h]);
+                                kahan2(s, cp, make_float2(redot(v[e], f0[e]), redot(v[e + 1], f0[e + 1])));
+                                z[2 * h] = s.x;
+                                z[2 * h + 1] = s.y;
+                                z[4 + 2 * h] = cp.x;
+                                z[5 + 2 * h] = cp.y;
+                            }
+                            tmem_st(tm + gi * W, z);
+                        }
                     }
+                    have = true;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) f0[e] = cadd(f0[e], v[e]);
                 }
             }
             if (failed) break;
-            if (!al) {   // the last detector has no weight
+            if (!MULTI && !(bits >> SH)) {   // the second detector has no weight, or there is none
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
                     f0[e] = v[e];
@@ -384,7 +448,6 @@ corr_kernel(const CorrArgs q) {
                 }
             }
             // pair terms of segment K
-            const bool acc_on = !LAG || K >= Ka;
             tmem_wait_st();
 #pragma unroll
             for (int gi = 0; gi < 4; ++gi) {
@@ -393,8 +456,8 @@ corr_kernel(const CorrArgs q) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int e = 4 * gi + 2 * h;
-                    const float2 S0 = cadd(f0[e], v[e]), S1 = cadd(f0[e + 1], v[e + 1]);
-                    if (acc_on) {
+                    const float2 S0 = MULTI ? f0[e] : cadd(f0[e], v[e]), S1 = MULTI ? f0[e + 1] : cadd(f0[e + 1], v[e + 1]);
+                    if (acc_on && (!MULTI || q.all_ordered)) {
                         const float2 d = q.all_ordered ? make_float2(redot(S0, S0), redot(S1, S1))
                                                        : make_float2(redot(v[e], f0[e]), redot(v[e + 1], f0[e + 1]));
                         float2 s = make_float2(z[2 * h], z[2 * h + 1]), cp = make_float2(z[4 + 2 * h], z[5 + 2 * h]);
@@ -428,27 +491,37 @@ corr_kernel(const CorrArgs q) {
             prev_zero = false;
         }
         if (failed) break;
-        // the unit's sums to its row
+        // the unit's sums to its row, through the exchange buffers (padded) for whole lines
         tmem_wait_st();
-        float* out = q.raw + (((size_t)t * 2 * q.n_chunks + (size_t)w * q.n_chunks + chunk) * PLANES * C + c) * L;
-        const size_t plane = (size_t)C * L;
+        __syncthreads();   // every thread has left the last transform's buffers
+        float* fl = (float*)ex;
+        constexpr int FP = CORR_POINTS + CORR_POINTS / 16;
 #pragma unroll
         for (int gi = 0; gi < 4; ++gi) {
             float z[W];
             tmem_ld(z, tm + gi * W);
-            if (valid) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int e = 4 * gi + i, m = j + GT * (e / RL) + NSL * (e % RL);
-                    out[m] = z[i];
-                    if constexpr (LAG) {
-                        out[plane + m] = z[8 + 6 * i];
-                        out[2 * plane + m] = z[8 + 6 * i + 1];
-                    }
+            for (int i = 0; i < 4; ++i) {
+                const int e = 4 * gi + i, b = e / RL;
+                const int m = g * L + (S::PASS2 ? 16 * (i0 + RL * b) + k : j + GT * b) + NSL * (e % RL);
+                const int o = m + (m >> 4);
+                fl[o] = z[i];
+                if constexpr (LAG) {
+                    fl[FP + o] = z[8 + 6 * i];
+                    fl[2 * FP + o] = z[8 + 6 * i + 1];
                 }
             }
         }
-        __syncthreads();   // every thread has taken this unit's number and left the last transform's buffers
+        __syncthreads();
+#pragma unroll
+        for (int pl = 0; pl < PLANES; ++pl)
+            for (int o = tid; o < CORR_POINTS; o += CORR_THREADS) {
+                const int so = sg * T + o / L, to = so >> 1;
+                if (to < q.n_t)
+                    q.raw[((((size_t)to * 2 * q.n_chunks + (size_t)(so & 1) * q.n_chunks + chunk) * PLANES + pl) * C + c) * L + o % L] =
+                        fl[pl * FP + o + (o >> 4)];
+            }
+        __syncthreads();   // the next unit's first pass rewrites the buffers
     }
     if (failed && tid == 0) {
         atomicOr(q.err, 1u);
@@ -458,9 +531,9 @@ corr_kernel(const CorrArgs q) {
     if (warp == 0) tmem_free(tm_base, COLS);
 }
 
-template <int LT, bool BF16, bool LAG, bool HALF>
+template <int LT, bool BF16, bool LAG, bool HALF, bool MULTI>
 cudaError_t launch_corr_t(const CorrArgs& a, int sms, cudaStream_t st) {
-    auto kern = corr_kernel<LT, BF16, LAG, HALF>;
+    auto kern = corr_kernel<LT, BF16, LAG, HALF, MULTI>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.smem);
     if (e != cudaSuccess) return e;
     const int grid = a.units < CORR_CTAS_PER_SM * sms ? a.units : CORR_CTAS_PER_SM * sms;

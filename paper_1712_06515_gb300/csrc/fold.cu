@@ -77,7 +77,7 @@ fold_kernel(const void* __restrict__ ab, const uint8_t* __restrict__ act, int t_
     const int64_t K = blockIdx.x, M = gridDim.x;
     const int X = blockIdx.y >> 1, w = blockIdx.y & 1;
     const int64_t t = blockIdx.z;
-    if (!__ldg(act + ((X == Q - 1 ? M : 0) + K) * t_pad + t)) return;
+    if (!__ldg(act + ((size_t)X * M + K) * t_pad + t)) return;
     const size_t row = (((size_t)t * Q + X) * 2 + w) * N_tau + (size_t)(K * N_s);
     const size_t zrow = ((((size_t)t * Q + X) * 2 + w) * M + K) * C * FOLD_L;
     for (int pp = threadIdx.x; pp < FOLD_L; pp += CORR_THREADS) {
@@ -108,7 +108,7 @@ fold_any_kernel(const void* __restrict__ ab, const uint8_t* __restrict__ act, in
     const int64_t K = blockIdx.x, M = gridDim.x;
     const int X = blockIdx.y >> 1, w = blockIdx.y & 1;
     const int64_t t = blockIdx.z;
-    if (!__ldg(act + ((X == Q - 1 ? M : 0) + K) * t_pad + t)) return;
+    if (!__ldg(act + ((size_t)X * M + K) * t_pad + t)) return;
     const size_t row = (((size_t)t * Q + X) * 2 + w) * N_tau + (size_t)(K * N_s);
     const size_t zrow = ((((size_t)t * Q + X) * 2 + w) * M + K) * C * FOLD_L;
     for (int c = 0; c < C; ++c)

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "corr.cuh"
 
 namespace {
 thread_local std::string g_last_error;
@@ -450,23 +451,7 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
             }
         return v;
     };
-    auto last_powers = [](int64_t Cn) {
-        std::vector<float4> v((size_t)Cn * 512);
-        const uint64_t G = (uint64_t)Cn * 4096;
-        for (uint64_t c2 = 0; c2 < (uint64_t)Cn; ++c2)
-            for (uint64_t j = 0; j < 256; ++j) {
-                float w[8];
-                for (int i = 0; i < 4; ++i) {
-                    const double ang = -2.0 * M_PI * (double)(((c2 + (uint64_t)Cn * j) << i) % G) / (double)G;
-                    w[2 * i] = (float)cos(ang);
-                    w[2 * i + 1] = (float)sin(ang);
-                }
-                v[(c2 * 256 + j) * 2] = make_float4(w[0], w[1], w[2], w[3]);
-                v[(c2 * 256 + j) * 2 + 1] = make_float4(w[4], w[5], w[6], w[7]);
-            }
-        return v;
-    };
-    const std::vector<float4> g8 = last_powers(Cg), g81 = last_powers(1);
+    const std::vector<float2> gp = cc::corr_powers(Lg, Cg), gp4 = cc::corr_powers(4096, 1);
     const std::vector<float2> gk = grid_twiddles(Cg), gk1 = grid_twiddles(1), gl = roots(Lg), g4 = roots(4096);
     // coset maps of the 4096-point decomposition (the same as the plan's when L = 4096)
     std::vector<int> off4, ck4, cm4;
@@ -493,8 +478,8 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
         (st = upload(p, gk.data(), gk.size(), &p->corr_twk)) != CC_OK ||
         (st = upload(p, gk1.data(), gk1.size(), &p->corr_twk1)) != CC_OK ||
         (st = upload(p, gl.data(), gl.size(), &p->corr_twL)) != CC_OK ||
-        (st = upload(p, g8.data(), g8.size(), &p->corr_tw8)) != CC_OK ||
-        (st = upload(p, g81.data(), g81.size(), &p->corr_tw8_1)) != CC_OK ||
+        (st = upload(p, gp.data(), gp.size(), &p->corr_twp)) != CC_OK ||
+        (st = upload(p, gp4.data(), gp4.size(), &p->corr_twp4096)) != CC_OK ||
         (st = upload(p, g4.data(), g4.size(), &p->corr_tw4096)) != CC_OK ||
         (!off4.empty() && ((st = upload(p, off4.data(), off4.size(), &dp.coset4_off)) != CC_OK ||
                            (st = upload(p, ck4.data(), ck4.size(), &dp.coset4_k)) != CC_OK ||

@@ -109,7 +109,7 @@ resample_group_kernel(float2* __restrict__ ab, float4* __restrict__ norm, const 
     }
     if (lane == 0 && sub == 0) {
         s_on[tl] = on;
-        if (t < n_t && act) act[((X == p.Q - 1 ? p.M : 0) + K) * t_pad + t] = on;
+        if (t < n_t && act) act[((size_t)X * p.M + K) * t_pad + t] = on;
     }
     __syncthreads();
     int lo = 0x7fffffff, hi = -0x7fffffff;

@@ -63,8 +63,7 @@ __host__ __device__ inline int resample_window_len(const DevParams& p) {
 // detector times all fall in gaps is skipped: its norms are written as zero and its
 // a_r, b_r are written as zero (`write_inactive`, the staged stage: every weight there is
 // zero) or left unwritten (the two-pass search reads a segment only when its flag is
-// nonzero); `act` (two-pass search, Q <= 2; [2][M][t_pad] bytes, detector 0 and the last one)
-// receives whether the segment was computed.  Without `kn` every sample is computed.  The parameter block comes last: with
+// nonzero); `act` (two-pass search; [Q][M][t_pad] bytes) receives whether the segment was computed.  Without `kn` every sample is computed.  The parameter block comes last: with
 // it first, the offsets of the small parameters after it moved with its size, and at some
 // sizes the two-pass variant compiled to 52 registers instead of 32 and ran 15 % slower.
 template <int DT, bool PRE>
@@ -121,7 +120,7 @@ resample_kernel(const cc_template* __restrict__ tm, int64_t t_base, void* ab, fl
             }
         }
         __syncthreads();
-        if (act && tid == 0) act[((X == p.Q - 1 ? p.M : 0) + K) * t_pad + t] = active != 0;
+        if (act && tid == 0) act[((size_t)X * p.M + K) * t_pad + t] = active != 0;
         if (!active) {
             if (tid == 0) norm[(t * p.Q + X) * p.M + K] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (write_inactive) {
