@@ -13,6 +13,7 @@ cc_status launch_norm_pairs(cc_plan* plan, const void* F, const float* norm, int
                             float* rawws, float* rho, cudaStream_t st);
 size_t pair_workspace_bytes(const cc_plan* plan, int64_t n_t);
 bool two_pass_supported(const cc_plan* plan);
+bool lag_grid_supported(const cc_plan* plan);
 size_t two_pass_workspace_bytes(const cc_plan* plan, int64_t n_t);
 cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, float* rho, cudaStream_t st);
 
@@ -56,12 +57,20 @@ static bool fused_supported(const cc_plan* plan) {
     return plan->cfg.store == CC_STORE_FP32 && fused_layout(plan, 1, &lay);
 }
 
+// The two-pass kernels also serve plans whose output bins reach the upper half of their cosets
+// (f_band near 1/dt), which CC_PATH_TWO_PASS by name leaves to the others: 64 templates of a
+// one-day 1 Hz band take 0.2 ms on the lag grid, 7.8 ms on the cluster kernel.
 static int resolve_path(const cc_plan* plan) {
     if (plan->search_path != CC_PATH_AUTO) return plan->search_path;
-    if (two_pass_supported(plan)) return CC_PATH_TWO_PASS;
+    if (plan->Q <= 2 && lag_grid_supported(plan)) return CC_PATH_TWO_PASS;
     if (fused_supported(plan)) return CC_PATH_FUSED;
     return CC_PATH_STAGED;
 }
+
+// Three and four detectors on the fused path: the lag grid in batches of a few GB, where the
+// cluster kernel transforms every segment at all output frequencies in a 8-CTA cluster per
+// template (48 templates of ten days and three detectors: 43.6 ms there, 1.8 ms here).
+static bool fused_on_lag_grid(const cc_plan* plan) { return plan->Q > 2 && lag_grid_supported(plan); }
 
 }  // namespace cc
 
@@ -86,7 +95,7 @@ extern "C" cc_status crosscorr_plan_workspace_size(const cc_plan* plan, int64_t 
     const int path = resolve_path(plan);
     FusedLayout lay;
     int64_t kbatch, batch;
-    if (path == CC_PATH_TWO_PASS) *bytes = two_pass_workspace_bytes(plan, n_t);
+    if (path == CC_PATH_TWO_PASS || (path == CC_PATH_FUSED && fused_on_lag_grid(plan))) *bytes = two_pass_workspace_bytes(plan, n_t);
     else if (path == CC_PATH_FUSED && fused_plan(plan, n_t, &lay, &kbatch, bytes)) {
     } else staged_batch(plan, n_t, &batch, bytes);
     return CC_OK;
@@ -112,6 +121,13 @@ extern "C" cc_status crosscorr_search(cc_plan* plan, const void* const* x_dev, c
     cudaStream_t st = (cudaStream_t)stream;
     const int path = resolve_path(plan);
     if (path == CC_PATH_TWO_PASS) return search_two_pass(plan, t_dev, n_t, rho_dev, st);
+    if (path == CC_PATH_FUSED && fused_on_lag_grid(plan)) {
+        // a workspace that cannot hold a batch (the caller's, or no memory for the plan's own)
+        // leaves the search to the cluster kernel
+        const size_t need = two_pass_workspace_bytes(plan, n_t);
+        if (plan->ws_external ? plan->ws_bytes >= need : ensure_workspace(plan, need) == CC_OK)
+            return search_two_pass(plan, t_dev, n_t, rho_dev, st);
+    }
     FusedLayout lay;
     int64_t kbatch;
     size_t fbytes;

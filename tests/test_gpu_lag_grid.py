@@ -61,6 +61,42 @@ def test_shapes_bf16(n_s, m, n_t):
     run(n_s, m, n_t, {}, store=cc.STORE_BF16)
 
 
+@pytest.mark.parametrize("n_det,n_s,m,n_t,kw", [
+    (3, 65, 24, 9, {}), (4, 128, 24, 17, dict(pair_mode=2)), (3, 256, 16, 3, dict(T_max=0.0)), (4, 257, 12, 2, {}),
+    (3, 600, 12, 3, dict(pair_mode=2)), (3, 1025, 8, 2, {}), (4, 2049, 5, 2, {}), (3, 4097, 4, 1, {})])
+def test_three_and_four_detectors(n_det, n_s, m, n_t, kw):
+    """The fused path's plans on the lag grid."""
+    kw = dict(dict(T_max=float(n_s)), **kw)
+    ds = synth.tiny(seed=67, n_samples=n_s * m, T_sft=float(n_s), T_short=float(n_s), f_band=0.1 if n_s > 200 else 0.4,
+                    n_templates=n_t, n_det=n_det, duty=0.7, mean_lock_s=1.5 * n_s, **kw)
+    ref = oracle.rho(ds)
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        x = torch.from_numpy(ds.x64).to(DEV)
+        tm = torch.from_numpy(ds.templates).to(DEV)
+        got = plan.search(x, tm).cpu().numpy()
+        plan.check()
+    for t in range(n_t):
+        err = float(np.abs(got[t].astype(np.float64) - ref[t]).max())
+        assert err <= 1e-4 * max(1.0, float(np.abs(ref[t]).max())), (t, err)
+
+
+@pytest.mark.parametrize("f_band,store", [(1.0, 0), (0.9, 0), (1.0, 1)])
+def test_wide_band(f_band, store):
+    """Output bins over the whole sampled band: the lag grid reaches them all; the path by name
+    still refuses such a plan."""
+    ds = synth.tiny(seed=73, n_samples=240 * 40, T_sft=240.0, T_max=0.0, T_short=240.0, f_band=f_band, n_templates=5, duty=0.8,
+                    mean_lock_s=2400.0)
+    ref = oracle.rho(ds)
+    with cc.CrossCorrPlan(ds.cfg, ds.dets, store=store) as plan:
+        assert plan.search_path == cc.PATH_TWO_PASS
+        with pytest.raises(cc.CrossCorrError):
+            plan.set_path(cc.PATH_TWO_PASS)
+        got = plan.search(torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV)).cpu().numpy()
+    tol = 1e-4 if store == 0 else 1e-2
+    for t in range(5):
+        assert np.abs(got[t] - ref[t]).max() <= tol * max(1.0, np.abs(ref[t]).max())
+
+
 @pytest.mark.parametrize("tune", [dict(batch_templates=2), dict(chunk_waves=1), dict(chunk_waves=400), dict(transform_len=4096)])
 def test_splits(tune):
     run(600, 40, 5, {}, **tune)
