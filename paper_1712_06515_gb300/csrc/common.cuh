@@ -151,13 +151,15 @@ struct cc_plan {
     std::vector<cudaEvent_t> timing_events;   // [2 * n] start, stop
     size_t timing_used = 0;                   // pairs recorded since the last read
     // detector-frame (demodulation) search: SFT bins and weights, twiddles, bin tables
-    void* demod_z = nullptr;                  // [Q][n_blk][nbins] float2
+    void* demod_z = nullptr;                  // [Q][n_blk][nbins + 2] float2
     void* demod_w = nullptr;                  // [Q][n_blk] float4 (a^, b^, locked, 0)
     void* demod_tw = nullptr;                 // [nsft] float2
     void* demod_df = nullptr;                 // [N_f] double: f - f_h of the output bins
     void* demod_kbar = nullptr;               // [N_f] int64
     void* demod_list = nullptr;               // [n_list] int: locked SFTs in time order, 4 l + X
     void* demod_boff = nullptr;               // [n_blk + 1] int: first list entry of each block
+    void* demod_start = nullptr;              // [n_list + pad] int: first partner of each list entry
+    void* demod_ctl = nullptr;                // [n_list + pad] int: control words of the separable kernel (demod.cu)
     int demod_nlist = 0;
     bool demod_ready = false;
     int demod_form = CC_DEMOD_PAIRS;          // crosscorr_plan_set_demod_form

@@ -35,11 +35,17 @@ constexpr size_t DM_RING_BUDGET = 160 * 1024;
 constexpr size_t DM_SEP_RING = 40 * 1024;   // separable form: block-sum ring per CTA (R_s <= 10)
 
 struct DemodTiming {   // per (template, locked SFT): 32 bytes
-    float A0, A1;       // signal bin position x = A0 + df A1 (df = f - f_h of the output bin)
+    float A0, A1;       // signal bin position x - 1/2 = A0 + df A1 (df = f - f_h of the output bin)
     float C0, C1;       // heterodyned phase (cycles) = C0 + kbar C1 with kbar = 128 kh + kl:
     float C128, pad0;   //   C0 + kh C128 + kl C1 (mod 1); pad0, pad1: the SFT's a^, b^
-    float pad1, pad2;   //   divided by sqrt(10); pad2: its list key 4 l + X (int bits)
+    float pad1, pad2;   //   divided by sqrt(10); pad2: its row of SFT bins, X n_blk + l (int bits)
 };
+
+// What the separable kernel does when the list reaches a new block, from the list alone
+// (crosscorr_demod_prepare): bits 0-1 DM_*, bit 2: the partial sums join the compensated totals,
+// bits 3-16 and 17-30: the ring slots of the finished and of the new block.
+enum { DM_SAME = 0, DM_STEP = 1, DM_REFRESH = 2, DM_EMPTY = 3 };
+constexpr int DM_LIST_PAD = 8;   // padding entries of the per-entry tables
 
 // DFT bins m_lo .. m_lo + nbins - 1 of one T_sft block of detector X, normalised to unit
 // variance, each times (-1)^m: the two-bin interpolation's alternating sign
@@ -50,7 +56,8 @@ sft_kernel(DevParams p, int nsft, int m_lo, int nbins, int n_blk, const float2* 
            float2* __restrict__ z, float4* __restrict__ wts) {
     extern __shared__ __align__(16) float2 xs[];
     const int l = blockIdx.x, X = blockIdx.y;
-    float2* zo = z + ((size_t)X * n_blk + l) * nbins;
+    float2* zo = z + ((size_t)X * n_blk + l) * (nbins + 2);   // two zero columns end a row
+    if (threadIdx.x < 2) zo[nbins + threadIdx.x] = make_float2(0.f, 0.f);
     const float2 sw = (l < (int)p.n_sig[X]) ? __ldg(p.sigw[X] + l) : make_float2(0.f, 0.f);
     const bool locked = sw.x > 0.f;
     if (threadIdx.x == 0) {
@@ -138,7 +145,7 @@ __device__ DemodTiming demod_timing(const DevParams& p, const cc_template& T, in
     const double Tsft = nsft * p.dt;
     DemodTiming r;
     // x = (f (dtau - 1) + df) T_sft with f = f_h + df
-    r.A0 = (float)(p.f_h * (dtau - 1.0) * Tsft);
+    r.A0 = (float)(p.f_h * (dtau - 1.0) * Tsft - 0.5);
     r.A1 = (float)(dtau * Tsft);
     // phase f tau - f_h t = f_h d + df (t + d), df = df0 + kbar dK
     const double tau = tmid + d;
@@ -152,7 +159,7 @@ __device__ DemodTiming demod_timing(const DevParams& p, const cc_template& T, in
 }
 
 // The search kernels' records: one per locked SFT of the time-ordered list, the timing of
-// demod_timing with the SFT's filter weights (divided by sqrt(10)) and list key (4 l + X) in
+// demod_timing with the SFT's filter weights (divided by sqrt(10)) and its row of bins in
 // the spare words; two padding records (no bins) follow the list.
 __global__ void demod_timing_list_kernel(DevParams p, const cc_template* __restrict__ tm, int nsft, int n_blk,
                                          double df0, double dK, const int* __restrict__ list, int n_list,
@@ -164,7 +171,7 @@ __global__ void demod_timing_list_kernel(DevParams p, const cc_template* __restr
     if (i >= n_list) {                                 // padding: no bins (x far below the band)
         r.A0 = -1.0e9f;
         r.A1 = r.C0 = r.C1 = r.C128 = r.pad0 = r.pad1 = 0.f;
-        r.pad2 = __int_as_float(__ldg(list + n_list - 1));
+        r.pad2 = __int_as_float(0);
     } else {
         const int key = __ldg(list + i);
         const int l = key >> 2, X = key & 3;
@@ -172,7 +179,7 @@ __global__ void demod_timing_list_kernel(DevParams p, const cc_template* __restr
         const float4 wk = __ldg(wts + (size_t)X * n_blk + l);
         r.pad0 = wk.x * 0.316227766016837933f;         // a^ / sqrt(10)
         r.pad1 = wk.y * 0.316227766016837933f;
-        r.pad2 = __int_as_float(key);
+        r.pad2 = __int_as_float(X * n_blk + l);
     }
     out[(size_t)t * (n_list + 2) + i] = r;
 }
@@ -189,254 +196,327 @@ __global__ void demod_timing_list_kernel(DevParams p, const cc_template* __restr
 // so that rounding cannot drift.  s_(l - R_s) comes from a per-thread ring of block sums in
 // shared memory when R_s is small (RING), otherwise it is recomputed from the SFT bins.
 // Results equal the per-pair loop's up to FP32 rounding.
-struct SepSums {
-    float ayx, ayy, byx, byy, uaa, uab, ubb;
+struct SepSums {     // (paired operations: the kernel is bound by instruction issue)
+    float2 ay, by;   // sum a^ y, sum b^ y
+    float2 u;        // sum Xi^2 a^^2, sum Xi^2 a^ b^
+    float ubb;       // sum Xi^2 b^^2
 };
 
-__device__ __forceinline__ void sep_zero(SepSums& a) { a = SepSums{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}; }
-
-__device__ __forceinline__ void sep_axpy(SepSums& a, const SepSums& b, float sg) {
-    a.ayx = fmaf(sg, b.ayx, a.ayx);
-    a.ayy = fmaf(sg, b.ayy, a.ayy);
-    a.byx = fmaf(sg, b.byx, a.byx);
-    a.byy = fmaf(sg, b.byy, a.byy);
-    a.uaa = fmaf(sg, b.uaa, a.uaa);
-    a.uab = fmaf(sg, b.uab, a.uab);
-    a.ubb = fmaf(sg, b.ubb, a.ubb);
+__device__ __forceinline__ void sep_zero(SepSums& a) {
+    a.ay = a.by = a.u = make_float2(0.f, 0.f);
+    a.ubb = 0.f;
 }
 
-// SFT (X, l)'s contribution (a^ y, b^ y, Xi^2 a^^2, Xi^2 a^ b^, Xi^2 b^^2) to the sums
-__device__ __forceinline__ void sep_add_sft(SepSums& a, float2 y, float xi2, float4 wk) {
-    const float xa = xi2 * wk.x, xb = xi2 * wk.y;
-    a.ayx = fmaf(wk.x, y.x, a.ayx);
-    a.ayy = fmaf(wk.x, y.y, a.ayy);
-    a.byx = fmaf(wk.y, y.x, a.byx);
-    a.byy = fmaf(wk.y, y.y, a.byy);
-    a.uaa = fmaf(xa, wk.x, a.uaa);
-    a.uab = fmaf(xa, wk.y, a.uab);
-    a.ubb = fmaf(xb, wk.y, a.ubb);
+__device__ __forceinline__ void sep_add(SepSums& a, const SepSums& b) {
+    a.ay = cadd(a.ay, b.ay);
+    a.by = cadd(a.by, b.by);
+    a.u = cadd(a.u, b.u);
+    a.ubb += b.ubb;
 }
 
-// One SFT's inputs for the separable kernel, fetched ahead of its arithmetic: kappa =
-// floor(x) - x of the signal bin position, the heterodyne phase in cycles reduced to
-// [-1/2, 1/2], and the two stored bins floor(x), floor(x) + 1 (zero when out of the band).
+__device__ __forceinline__ void sep_sub(SepSums& a, const SepSums& b) {
+    a.ay = csub(a.ay, b.ay);
+    a.by = csub(a.by, b.by);
+    a.u = csub(a.u, b.u);
+    a.ubb -= b.ubb;
+}
+
+// An SFT's factors, the same for every bin (a^, b^ over sqrt(10)): (a^, a^), (b^, b^),
+// (a^^2, a^ b^), b^^2.
+struct SftW {
+    float2 a, b, u;
+    float bb;
+};
+
+__device__ __forceinline__ SftW sft_w(float a, float b) {
+    return SftW{make_float2(a, a), make_float2(b, b), make_float2(a * a, a * b), b * b};
+}
+
+// One SFT's contribution (a^ y, b^ y, Xi^2 a^^2, Xi^2 a^ b^, Xi^2 b^^2) to the sums
+__device__ __forceinline__ void sep_add_sft(SepSums& s, float2 y, float xi2, const SftW& w) {
+    s.ay = __ffma2_rn(w.a, y, s.ay);
+    s.by = __ffma2_rn(w.b, y, s.by);
+    s.u = make_float2(fmaf(xi2, w.u.x, s.u.x), fmaf(xi2, w.u.y, s.u.y));
+    s.ubb = fmaf(xi2, w.bb, s.ubb);
+}
+
+// One SFT's inputs, fetched ahead of its arithmetic: h = x - m - 1/2 in [-1/2, 1/2] of the
+// signal bin position x between bins m and m + 1, the heterodyne phase in cycles reduced to
+// [-1/2, 1/2], and the two stored bins (zero when out of the band).
 struct SftIn {
-    float k0, cyc;
+    float h, cyc;
     float2 z0, z1;
 };
 
-// The demodulated bin y (the two-bin sinc interpolation of the pair kernel, rotated by the
-// heterodyne phase) and the interpolation weight Xi^2.  The two sinc weights
-// s0 = sin(pi kappa) / (pi kappa), s1 = -sin(pi kappa) / (pi (kappa + 1)) take the series
-// at whichever of kappa, kappa + 1 lies within 1/2 of zero and one quotient for the other
-// (its denominator at least 1/2 in size).  The rotation takes the phase in [-1/2, 1/2)
-// cycles to the fast sine/cosine, whose absolute error there (2^-21.4) is far below the
-// statistic's FP32 rounding.
+// The two sinc weights of kappa = -f and 1 - f, f = h + 1/2: with
+// g(h) = sin(pi f) / (pi f (1 - f)) = cos(pi h) / (pi (1/4 - h^2)), an entire even function,
+// sinc(f) = g (1 - f) and sinc(1 - f) = g f.  g as a polynomial in h^2 by Chebyshev fit on
+// |h| <= 1/2 (largest error 4e-12).
+__device__ __forceinline__ float2 sinc_weights(float h) {
+    const float u = h * h;
+    float g = -0.000581711926f;
+    g = fmaf(g, u, 0.00805632297f);
+    g = fmaf(g, u, -0.0728914161f);
+    g = fmaf(g, u, 0.406804216f);
+    g = fmaf(g, u, -1.19022713f);
+    g = fmaf(g, u, 1.27323954f);
+    return make_float2(g * (0.5f - h), g * (0.5f + h));
+}
+
+// The demodulated bin y (the two-bin sinc interpolation, rotated by the heterodyne phase) and
+// the interpolation weight Xi^2.  The rotation takes the phase in [-1/2, 1/2] cycles to the fast
+// sine/cosine, whose absolute error there (2^-21.4) is far below the statistic's FP32 rounding.
 __device__ __forceinline__ float2 sft_y(const SftIn& q, float& xi2) {
-    const bool near0 = q.k0 >= -0.5f;                // kappa in [-1/2, 0]: series at kappa
-    const float r = near0 ? q.k0 : q.k0 + 1.f;
-    const float far = near0 ? q.k0 + 1.f : q.k0;
-    const float sv = sinc_pi(r);
-    const float other = -__fdividef(r * sv, far);
-    const float s0 = near0 ? sv : other, s1 = near0 ? other : sv;
-    xi2 = s0 * s0 + s1 * s1;
-    const float2 u = make_float2(fmaf(s0, q.z0.x, s1 * q.z1.x), fmaf(s0, q.z0.y, s1 * q.z1.y));
+    const float2 s = sinc_weights(q.h);
+    xi2 = fmaf(s.x, s.x, s.y * s.y);
+    const float2 u = make_float2(fmaf(s.x, q.z0.x, s.y * q.z1.x), fmaf(s.x, q.z0.y, s.y * q.z1.y));
     float sn, cs;
     __sincosf(6.28318530717958648f * q.cyc, &sn, &cs);
     return make_float2(fmaf(u.x, cs, u.y * sn), fmaf(u.y, cs, -u.x * sn));
 }
 
-// One record of the separable kernel's list: timing, weights and key of SFT i.
+// One record of the list: timing, weights and row of SFT i.
 struct SepRec {
     float4 t0;   // A0, A1, C0, C1
-    float4 t1;   // C128, a^, b^, key (int bits: 4 l + X)
+    float4 t1;   // C128, a^, b^, row (int bits)
 };
 
-__device__ __forceinline__ SepRec load_rec(const DemodTiming* __restrict__ r) {
-    const float4* q = reinterpret_cast<const float4*>(r);
-    return SepRec{__ldg(q), __ldg(q + 1)};
-}
-
+// x - 1/2 rounded to the nearest integer m by adding 1.5 x 2^23 (|x| < 2^22 for any real SFT; a
+// tie gives f = 0 or 1 with the same weights on the same bins), m also read from the sum's bits.
 __device__ __forceinline__ void rec_fetch(SftIn& q, const SepRec& r, float df, float kh, float kl, int m_lo,
-                                          int nbins, int n_blk, const float2* __restrict__ z) {
-    const int key = __float_as_int(r.t1.w);
-    const float x = fmaf(df, r.t0.y, r.t0.x);
-    const float fm = floorf(x);
-    q.k0 = fm - x;
-    const int idx = (int)fm - m_lo;
+                                          int nbins, const float2* __restrict__ z) {
+    constexpr float MAGIC = 12582912.f;
+    const float xs = fmaf(df, r.t0.y, r.t0.x), t = xs + MAGIC;
+    q.h = xs - (t - MAGIC);
+    const int i = __float_as_int(t) - (0x4b400000 + m_lo);
+    const int c = (unsigned)i < (unsigned)(nbins - 1) ? i : nbins;   // the zero columns
     const float cyc = fmaf(kl, r.t0.w, fmaf(kh, r.t1.x, r.t0.z));
     q.cyc = cyc - rintf(cyc);
-    q.z0 = q.z1 = make_float2(0.f, 0.f);
-    if (idx >= 0 && idx + 1 < nbins) {
-        const float2* zr = z + ((size_t)(key & 3) * n_blk + (key >> 2)) * nbins + idx;
-        q.z0 = __ldg(zr);
-        q.z1 = __ldg(zr + 1);
-    }
+    const float2* zr = z + (size_t)(unsigned)__float_as_int(r.t1.w) * (unsigned)(nbins + 2) + c;
+    q.z0 = __ldg(zr);
+    q.z1 = __ldg(zr + 1);
 }
 
-// One thread per (template, output bin) walks the list of locked SFTs in time order (gaps
-// never enter the loop).  The SFT records of one template are shared by its CTAs; their
-// filter weights come scaled by 1/sqrt(10), so Gamma_KL = a^'_K a^'_L + b^'_K b^'_L and the
+// A thread takes SB output bins of one template (a CTA's threads apart) and walks the list of
+// locked SFTs in time order (gaps never enter the loop): what is the same for every bin -- the
+// records, the weights' products, the list's control words -- is read and formed once for them.
+// The filter weights come scaled by 1/sqrt(10), so Gamma_KL = a^'_K a^'_L + b^'_K b^'_L and the
 // factors 1/10 and 1/100 drop out (the pair sum is then half the statistic's raw sum).
 // V holds the sums over SFT K's partners so far (window W plus the current block); block
 // sums go to the window when the block index changes: one step adds s_l and subtracts
 // s_(l - R_s); a jump over empty blocks, and every 4 (R_s + 1) steps, sums the window
-// exactly.  The record list carries two padding records (no bins) past its end so that
-// the pipeline's loads need no guards.
+// exactly.  Records and control words reach shared memory by cp.async, SG at a time, one group
+// ahead; SFT i + 1's bins load while SFT i is summed.  What bounds it: instruction issue (66 %
+// active with the twelve warps whose rings fit an SM, 115 instructions per SFT and 32 bins).
+constexpr int SB = 2, SG = 16;
+
 template <bool RING>
-__global__ void __launch_bounds__(128) demod_sep_kernel(DevParams p, int m_lo, int nbins, int n_blk, int Rs, int refresh,
+__global__ void __launch_bounds__(128) demod_sep_kernel(DevParams p, int m_lo, int nbins, int n_blk, int Rs,
                                  const float2* __restrict__ z, const DemodTiming* __restrict__ recs, int n_list,
-                                 const int* __restrict__ boff, const double* __restrict__ dfreq,
-                                 const int64_t* __restrict__ kbar, int64_t t_base, float* __restrict__ rho) {
-    extern __shared__ __align__(16) float sring[];     // RING: [R_s + 1][7][nthr] block sums, thread-private
-    const int nthr = blockDim.x, tid = threadIdx.x;
+                                 const int* __restrict__ boff, const int* __restrict__ list, const int* __restrict__ ctl,
+                                 const double* __restrict__ dfreq, const int64_t* __restrict__ kbar, int64_t t_base,
+                                 float* __restrict__ rho) {
+    extern __shared__ __align__(16) float sring[];     // RING: [R_s + 1][7 words][SB][nthr] block sums, thread-private
+    __shared__ __align__(16) float4 s_rec[3][SG][2];
+    __shared__ __align__(16) int s_ctl[3][SG];
+    const int nthr = blockDim.x, tid = threadIdx.x, rst = SB * nthr;
     const int64_t t = t_base + blockIdx.y;
-    const int k = blockIdx.x * nthr + tid;
-    const bool act = k < (int)p.N_f;
+    const int k0 = blockIdx.x * rst + tid;
     const DemodTiming* rt = recs + (size_t)(t - t_base) * (n_list + 2);
     if (n_list == 0) {                                 // no locked SFT
-        if (act) rho[(size_t)t * p.N_f + k] = 0.f;
+        for (int q = 0; q < SB; ++q)
+            if (k0 + q * nthr < (int)p.N_f) rho[(size_t)t * p.N_f + k0 + q * nthr] = 0.f;
         return;
     }
     if (RING)
-        for (int j = 0; j < (Rs + 1) * 7; ++j) sring[(size_t)j * nthr + tid] = 0.f;
+        for (int j = 0; j < (Rs + 1) * 7 * SB; ++j) sring[(size_t)j * nthr + tid] = 0.f;
     // threads past the last bin compute bin 0's statistic and store nothing
-    const float df = (float)__ldg(dfreq + (act ? k : 0));
-    const int64_t kb = __ldg(kbar + (act ? k : 0));
-    const float kh = (float)(kb >> 7), kl = (float)(kb & 127);
-    auto ring_get = [&](int slot) {
-        const float* r = sring + (size_t)slot * 7 * nthr + tid;
-        return SepSums{r[0], r[nthr], r[2 * nthr], r[3 * nthr], r[4 * nthr], r[5 * nthr], r[6 * nthr]};
+    float df[SB], kh[SB], kl[SB];
+#pragma unroll
+    for (int q = 0; q < SB; ++q) {
+        const int k = k0 + q * nthr < (int)p.N_f ? k0 + q * nthr : 0;
+        df[q] = (float)__ldg(dfreq + k);
+        const int64_t kb = __ldg(kbar + k);
+        kh[q] = (float)(kb >> 7);
+        kl[q] = (float)(kb & 127);
+    }
+    auto ring_get = [&](int slot, int q) {
+        const float* r = sring + slot * 7 * rst;
+        const float2* r2 = (const float2*)r + q * nthr + tid;
+        return SepSums{r2[0], r2[rst], r2[2 * rst], r[6 * rst + q * nthr + tid]};
     };
-    auto ring_put = [&](int slot, const SepSums& v) {
-        float* r = sring + (size_t)slot * 7 * nthr + tid;
-        r[0] = v.ayx;
-        r[nthr] = v.ayy;
-        r[2 * nthr] = v.byx;
-        r[3 * nthr] = v.byy;
-        r[4 * nthr] = v.uaa;
-        r[5 * nthr] = v.uab;
-        r[6 * nthr] = v.ubb;
+    auto ring_put = [&](int slot, int q, const SepSums& v) {
+        float* r = sring + slot * 7 * rst;
+        float2* r2 = (float2*)r + q * nthr + tid;
+        r2[0] = v.ay;
+        r2[rst] = v.by;
+        r2[2 * rst] = v.u;
+        r[6 * rst + q * nthr + tid] = v.ubb;
     };
     // block j's sums from its SFT bins (no ring)
-    auto block_sums = [&](int j, SepSums& sj) {
+    auto block_sums = [&](int j, int q, SepSums& sj) {
         sep_zero(sj);
         const int e = __ldg(boff + j + 1);
         for (int i = __ldg(boff + j); i < e; ++i) {
-            const SepRec r = load_rec(rt + i);
-            SftIn q;
-            rec_fetch(q, r, df, kh, kl, m_lo, nbins, n_blk, z);
+            const float4* r4 = (const float4*)(rt + i);
+            const SepRec r{__ldg(r4), __ldg(r4 + 1)};
+            SftIn in;
+            rec_fetch(in, r, df[q], kh[q], kl[q], m_lo, nbins, z);
             float xi2;
-            const float2 y = sft_y(q, xi2);
-            sep_add_sft(sj, y, xi2, make_float4(r.t1.y, r.t1.z, 1.f, 0.f));
+            const float2 y = sft_y(in, xi2);
+            sep_add_sft(sj, y, xi2, sft_w(r.t1.y, r.t1.z));
         }
     };
-    float raw = 0.f, rawc = 0.f, den = 0.f, denc = 0.f;
-    SepSums W, V;
-    sep_zero(W);
-    sep_zero(V);
-    int steps = 0;
-    int lcur = 0, scur = 0;                            // block lcur and its ring slot lcur mod (R_s + 1)
+    // group n (entries n SG ..) into buffer n mod 3; past the list: the padding record, no control
+    auto stage = [&](int n) {
+        if (tid < 2 * SG + SG / 4) {
+            if (tid < 2 * SG) {
+                const int i = min(n * SG + (tid >> 1), n_list);
+                const uint32_t d = (uint32_t)__cvta_generic_to_shared(&s_rec[n % 3][tid >> 1][tid & 1]);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"((const float4*)(rt + i) + (tid & 1)) : "memory");
+            } else if (n * SG < n_list) {
+                const uint32_t d = (uint32_t)__cvta_generic_to_shared(&s_ctl[n % 3][4 * (tid - 2 * SG)]);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(ctl + n * SG + 4 * (tid - 2 * SG)) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float raw[SB], rawc[SB], den[SB], denc[SB];
     // the pair and normalisation terms go to plain FP32 partial sums that join the
     // compensated totals at most every 64 SFTs (at a block change)
-    float raw_p = 0.f, den_p = 0.f;
-    int nacc = 0;
-    // SFT i: Rc its record, Fc its fetched inputs; Rn the record of SFT i + 1, Fn receives
-    // SFT i + 1's inputs.  The bins of SFT i + 1 and the record of SFT i + 2 (into Rc once
-    // read) load while SFT i is summed; two calls per iteration with the roles swapped keep
-    // the pipeline in place without register copies.
-    auto step = [&](SepRec& Rc, SftIn& Fc, const SepRec& Rn, SftIn& Fn, int i) {
-        rec_fetch(Fn, Rn, df, kh, kl, m_lo, nbins, n_blk, z);
-        const float4 wk = make_float4(Rc.t1.y, Rc.t1.z, 1.f, 0.f);
-        const int l = __float_as_int(Rc.t1.w) >> 2;
-        Rc = load_rec(rt + i + 2);
-        if (l != lcur) {                               // block lcur is complete: the window of block l
-            if (Rs > 0) {
-                if (RING) {
-                    const bool step1 = l == lcur + 1 && ++steps < refresh;
-                    SepSums Pb = V;                    // block lcur's sums
-                    sep_axpy(Pb, W, -1.f);
-                    ring_put(scur, Pb);
-                    if (step1) {
-                        scur = scur == Rs ? 0 : scur + 1;       // slot of l: s_(l - R_s - 1) = s_(lcur - R_s)
-                        const SepSums old = ring_get(scur);
-                        W = V;
-                        sep_axpy(W, old, -1.f);
-                    } else {
-                        const SepSums zero{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                        const int nz = min(l - lcur - 1, Rs + 1);   // empty blocks lcur + 1 .. l - 1
-                        for (int j = 1; j <= nz; ++j) {
-                            scur = scur == Rs ? 0 : scur + 1;
-                            ring_put(scur, zero);
+    float raw_p[SB], den_p[SB];
+    SepSums W[SB], V[SB];
+    SftIn F[SB];
+    stage(0);
+    stage(1);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < SB; ++q) {
+        raw[q] = rawc[q] = den[q] = denc[q] = raw_p[q] = den_p[q] = 0.f;
+        sep_zero(W[q]);
+        sep_zero(V[q]);
+        rec_fetch(F[q], SepRec{s_rec[0][0][0], s_rec[0][0][1]}, df[q], kh[q], kl[q], m_lo, nbins, z);
+    }
+    const int groups = (n_list + SG - 1) / SG;
+    for (int n = 0, buf = 0; n < groups; ++n) {
+        const int next = buf == 2 ? 0 : buf + 1;
+        // group n + 1's records are needed by this group's last fetch
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                               // and every thread has left group n - 1's buffer
+        stage(n + 2);
+        const int cnt = min(SG, n_list - n * SG);
+#pragma unroll 2
+        for (int e = 0; e < cnt; ++e) {
+            const float4 w4 = s_rec[buf][e][1];
+            const SftW w = sft_w(w4.y, w4.z);
+            const int cw = s_ctl[buf][e];
+            const float4* nr = e + 1 < SG ? s_rec[buf][e + 1] : s_rec[next][0];
+            float2 y[SB];
+            float xi2[SB];
+#pragma unroll
+            for (int q = 0; q < SB; ++q) {
+                y[q] = sft_y(F[q], xi2[q]);
+                rec_fetch(F[q], SepRec{nr[0], nr[1]}, df[q], kh[q], kl[q], m_lo, nbins, z);
+            }
+            const int op = cw & 3;
+            if (op != DM_SAME) {                       // the block before is complete: the new block's window
+                const int from = (cw >> 3) & 0x3fff, to = (cw >> 17) & 0x3fff;
+                const int i = n * SG + e;
+                if (Rs == 0) {
+                } else if (RING) {
+#pragma unroll
+                    for (int q = 0; q < SB; ++q) {
+                        SepSums Pb = V[q];             // the finished block's sums
+                        sep_sub(Pb, W[q]);
+                        ring_put(from, q, Pb);
+                    }
+                    if (op == DM_STEP) {               // slot `to` holds s_(l - R_s - 1)
+#pragma unroll
+                        for (int q = 0; q < SB; ++q) {
+                            W[q] = V[q];
+                            sep_sub(W[q], ring_get(to, q));
                         }
-                        scur = l % (Rs + 1);
-                        sep_zero(W);
-                        for (int j = 0; j <= Rs; ++j)
-                            if (j != scur) sep_axpy(W, ring_get(j), 1.f);
-                        steps = 0;
+                    } else {
+                        const int l = __ldg(list + i) >> 2, lcur = __ldg(list + i - 1) >> 2;
+                        SepSums zero;
+                        sep_zero(zero);
+                        const int nz = min(l - lcur - 1, Rs + 1);   // empty blocks lcur + 1 .. l - 1
+#pragma unroll
+                        for (int q = 0; q < SB; ++q) {
+                            int s = from;
+                            for (int j = 1; j <= nz; ++j) {
+                                s = s == Rs ? 0 : s + 1;
+                                ring_put(s, q, zero);
+                            }
+                            sep_zero(W[q]);
+                            for (int j = 0; j <= Rs; ++j)
+                                if (j != to) sep_add(W[q], ring_get(j, q));
+                        }
                     }
-                } else if (l - lcur > Rs) {            // every block of the new window is empty
-                    sep_zero(W);
-                    steps = 0;
-                } else if (++steps < refresh) {        // blocks lcur - R_s .. l - R_s - 1 leave
-                    W = V;
-                    for (int j = max(0, lcur - Rs); j < l - Rs; ++j) {
-                        SepSums old;
-                        block_sums(j, old);
-                        sep_axpy(W, old, -1.f);
-                    }
+                } else if (op == DM_EMPTY) {           // every block of the new window is empty
+#pragma unroll
+                    for (int q = 0; q < SB; ++q) sep_zero(W[q]);
                 } else {
-                    SepSums Wn = V;                    // blocks l - R_s .. lcur (those after are empty)
-                    sep_axpy(Wn, W, -1.f);
-                    for (int j = max(0, l - Rs); j < lcur; ++j) {
+                    const int l = __ldg(list + i) >> 2, lcur = __ldg(list + i - 1) >> 2;
+#pragma unroll
+                    for (int q = 0; q < SB; ++q) {
                         SepSums sj;
-                        block_sums(j, sj);
-                        sep_axpy(Wn, sj, 1.f);
+                        if (op == DM_STEP) {           // blocks lcur - R_s .. l - R_s - 1 leave
+                            W[q] = V[q];
+                            for (int j = max(0, lcur - Rs); j < l - Rs; ++j) {
+                                block_sums(j, q, sj);
+                                sep_sub(W[q], sj);
+                            }
+                        } else {                       // blocks l - R_s .. lcur (those after are empty)
+                            SepSums Wn = V[q];
+                            sep_sub(Wn, W[q]);
+                            for (int j = max(0, l - Rs); j < lcur; ++j) {
+                                block_sums(j, q, sj);
+                                sep_add(Wn, sj);
+                            }
+                            W[q] = Wn;
+                        }
                     }
-                    W = Wn;
-                    steps = 0;
+                }
+#pragma unroll
+                for (int q = 0; q < SB; ++q) {
+                    V[q] = W[q];
+                    if (cw & 4) {
+                        kahan_add(raw[q], rawc[q], raw_p[q]);
+                        kahan_add(den[q], denc[q], den_p[q]);
+                        raw_p[q] = den_p[q] = 0.f;
+                    }
                 }
             }
-            V = W;
-            lcur = l;
-            if (steps == 0 || nacc >= 64) {
-                kahan_add(raw, rawc, raw_p);
-                kahan_add(den, denc, den_p);
-                raw_p = den_p = 0.f;
-                nacc = 0;
+            const float ab2 = 2.f * w.u.y;
+#pragma unroll
+            for (int q = 0; q < SB; ++q) {
+                const float2 g = __ffma2_rn(w.a, V[q].ay, __fmul2_rn(w.b, V[q].by));
+                raw_p[q] = fmaf(y[q].x, g.x, fmaf(y[q].y, g.y, raw_p[q]));   // Re(conj(y) g)
+                const float nq = fmaf(w.u.x, V[q].u.x, fmaf(ab2, V[q].u.y, w.bb * V[q].ubb));
+                den_p[q] = fmaf(xi2[q], nq, den_p[q]);
+                sep_add_sft(V[q], y[q], xi2[q], w);
             }
         }
-        float xi2;
-        const float2 y = sft_y(Fc, xi2);
-        const float gx = fmaf(wk.x, V.ayx, wk.y * V.byx), gy = fmaf(wk.x, V.ayy, wk.y * V.byy);
-        raw_p = fmaf(y.x, gx, fmaf(y.y, gy, raw_p));                 // Re(conj(y) g)
-        const float nq = fmaf(wk.x * wk.x, V.uaa, fmaf(2.f * wk.x * wk.y, V.uab, wk.y * wk.y * V.ubb));
-        den_p = fmaf(xi2, nq, den_p);
-        ++nacc;
-        sep_add_sft(V, y, xi2, wk);
-    };
-    SepRec ra = load_rec(rt);
-    SepRec rb = load_rec(rt + 1);
-    SftIn fa, fb;
-    rec_fetch(fa, ra, df, kh, kl, m_lo, nbins, n_blk, z);
-    lcur = __float_as_int(ra.t1.w) >> 2;
-    scur = lcur % (Rs + 1);
-    int i = 0;
-    for (; i + 1 < n_list; i += 2) {
-        step(ra, fa, rb, fb, i);
-        step(rb, fb, ra, fa, i + 1);
+        buf = next;
     }
-    if (i < n_list) step(ra, fa, rb, fb, i);
-    kahan_add(raw, rawc, raw_p);
-    kahan_add(den, denc, den_p);
-    // rho = (2 raw) / sqrt(2 den)
-    if (act) rho[(size_t)t * p.N_f + k] = den > 0.f ? 1.41421356237309505f * raw * rsqrtf(den) : 0.f;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+    for (int q = 0; q < SB; ++q) {
+        kahan_add(raw[q], rawc[q], raw_p[q]);
+        kahan_add(den[q], denc[q], den_p[q]);
+        // rho = (2 raw) / sqrt(2 den)
+        if (k0 + q * nthr < (int)p.N_f)
+            rho[(size_t)t * p.N_f + k0 + q * nthr] = den[q] > 0.f ? 1.41421356237309505f * raw[q] * rsqrtf(den[q]) : 0.f;
+    }
 }
 
 // The method's pair loop: one thread per (template, output bin) over the locked SFTs in time
 // order (the separable kernel's records), PT consecutive SFTs at a time.  The partners of SFT i
 // are the entries of the list from the first one of block l_i - R_s up to i - 1, so those of a
-// tile of PT SFTs are a contiguous range before the tile plus pairs inside it.  A ring of the
+// tile of PT SFTs are a contiguous range before the tile plus pairs inside it (start: the first
+// partner of each entry).  A ring of the
 // last NR = (R_s + 1) Q entries holds, per entry, the thread's y and Xi^2 (thread-private columns
 // of shared memory) and the SFT's prescaled filter weights (shared); per tile the CTA forms
 // Gamma_KL = a^'_K a^'_L + b^'_K b^'_L of every ring entry against the PT SFTs (zero where it is
@@ -446,14 +526,16 @@ __global__ void __launch_bounds__(128) demod_sep_kernel(DevParams p, int m_lo, i
 // one tile ahead.
 constexpr int PT = 4;
 
-__global__ void __launch_bounds__(256, 3) demod_pair_kernel(DevParams p, int m_lo, int nbins, int n_blk, int Rs,
+template <int NT>
+__global__ void __launch_bounds__(NT, 768 / NT) demod_pair_kernel(DevParams p, int m_lo, int nbins, int n_blk, int Rs,
                                                             const float2* __restrict__ z,
                                                             const DemodTiming* __restrict__ recs, int n_list,
-                                                            const int* __restrict__ boff, const double* __restrict__ dfreq,
+                                                            const int* __restrict__ start, const double* __restrict__ dfreq,
                                                             const int64_t* __restrict__ kbar, int64_t t_base,
                                                             float* __restrict__ rho) {
     extern __shared__ __align__(16) unsigned char sm[];
-    const int nthr = blockDim.x, tid = threadIdx.x;
+    constexpr int nthr = NT;
+    const int tid = threadIdx.x;
     const int NR = (Rs + 1) * p.Q;
     float4* sg = (float4*)sm;                          // [NR] Gamma of the tile's SFTs against each ring entry
     float4* sq = sg + NR;                              // [NR] their squares
@@ -492,7 +574,7 @@ __global__ void __launch_bounds__(256, 3) demod_pair_kernel(DevParams p, int m_l
     float raw = 0.f, rawc = 0.f, den = 0.f, denc = 0.f;
     SftIn F[PT];
 #pragma unroll
-    for (int q = 0; q < PT; ++q) rec_fetch(F[q], rec(q), df, kh, kl, m_lo, nbins, n_blk, z);
+    for (int q = 0; q < PT; ++q) rec_fetch(F[q], rec(q), df, kh, kl, m_lo, nbins, z);
     int slot0 = 0;                                     // ring slot of the tile's first SFT
     for (int n = 0; n * PT < n_list; ++n) {
         const int i0 = n * PT;
@@ -508,18 +590,16 @@ __global__ void __launch_bounds__(256, 3) demod_pair_kernel(DevParams p, int m_l
 #pragma unroll
                 for (int q = 0; q < PT; ++q) {
                     const float4 r1 = rec4[(n & 3) * PT * 2 + 2 * q + 1];
-                    const int l = __float_as_int(r1.w) >> 2;
-                    g[q] = e >= __ldg(boff + max(0, l - Rs)) ? fmaf(r1.y, ab.x, r1.z * ab.y) : 0.f;
+                    g[q] = e >= __ldg(start + i0 + q) ? fmaf(r1.y, ab.x, r1.z * ab.y) : 0.f;
                 }
                 sg[s] = make_float4(g[0], g[1], g[2], g[3]);
                 sq[s] = make_float4(g[0] * g[0], g[1] * g[1], g[2] * g[2], g[3] * g[3]);
             } else if (j < have + 6) {                 // pairs (q, r), r < q, of the tile: index q (q - 1) / 2 + r
                 const int c = j - have, q = c < 1 ? 1 : c < 3 ? 2 : 3, r = c - q * (q - 1) / 2;
                 const float4 a = rec4[(n & 3) * PT * 2 + 2 * q + 1], b = rec4[(n & 3) * PT * 2 + 2 * r + 1];
-                const int la = __float_as_int(a.w) >> 2;
-                sin_[c] = i0 + r >= __ldg(boff + max(0, la - Rs)) ? fmaf(a.y, b.y, a.z * b.z) : 0.f;
+                sin_[c] = i0 + r >= __ldg(start + i0 + q) ? fmaf(a.y, b.y, a.z * b.z) : 0.f;
             } else if (j == have + 6) {
-                s_lo = __ldg(boff + max(0, (__float_as_int(rec4[(n & 3) * PT * 2 + 1].w) >> 2) - Rs));
+                s_lo = __ldg(start + i0);
             }
         }
         stage(n + 3);
@@ -533,33 +613,33 @@ __global__ void __launch_bounds__(256, 3) demod_pair_kernel(DevParams p, int m_l
             pr[q] = pq[q] = 0.f;
         }
 #pragma unroll
-        for (int q = 0; q < PT; ++q) rec_fetch(F[q], rec(i0 + PT + q), df, kh, kl, m_lo, nbins, n_blk, z);
+        for (int q = 0; q < PT; ++q) rec_fetch(F[q], rec(i0 + PT + q), df, kh, kl, m_lo, nbins, z);
         const int cnt = i0 - max(s_lo, i0 - have);
-        int s = slot0 - cnt;
-        s += s < 0 ? NR : 0;
-        const float2* cy = ry + (size_t)s * nthr + tid;
-        const float* cx = rx + (size_t)s * nthr + tid;
-#pragma unroll 2
-        for (int j = 0; j < cnt; ++j) {
-            const float4 g = sg[s], h = sq[s];
-            const float2 yl = *cy;
-            const float xl = *cx;
-            pr[0] = fmaf(g.x, fmaf(y[0].x, yl.x, y[0].y * yl.y), pr[0]);
-            pr[1] = fmaf(g.y, fmaf(y[1].x, yl.x, y[1].y * yl.y), pr[1]);
-            pr[2] = fmaf(g.z, fmaf(y[2].x, yl.x, y[2].y * yl.y), pr[2]);
-            pr[3] = fmaf(g.w, fmaf(y[3].x, yl.x, y[3].y * yl.y), pr[3]);
-            pq[0] = fmaf(h.x, xl, pq[0]);
-            pq[1] = fmaf(h.y, xl, pq[1]);
-            pq[2] = fmaf(h.z, xl, pq[2]);
-            pq[3] = fmaf(h.w, xl, pq[3]);
-            ++s;
-            cy += nthr;
-            cx += nthr;
-            if (s == NR) {
-                s = 0;
-                cy = ry + tid;
-                cx = rx + tid;
+        // the range in the ring, in up to two runs of consecutive slots
+        auto run = [&](int s0, int m) {
+            const float2* cy = ry + s0 * nthr + tid;
+            const float* cx = rx + s0 * nthr + tid;
+#pragma unroll 4
+            for (int j = 0; j < m; ++j) {
+                const float4 g = sg[s0 + j], h = sq[s0 + j];
+                const float2 yl = cy[j * nthr];
+                const float xl = cx[j * nthr];
+                pr[0] = fmaf(g.x, fmaf(y[0].x, yl.x, y[0].y * yl.y), pr[0]);
+                pr[1] = fmaf(g.y, fmaf(y[1].x, yl.x, y[1].y * yl.y), pr[1]);
+                pr[2] = fmaf(g.z, fmaf(y[2].x, yl.x, y[2].y * yl.y), pr[2]);
+                pr[3] = fmaf(g.w, fmaf(y[3].x, yl.x, y[3].y * yl.y), pr[3]);
+                pq[0] = fmaf(h.x, xl, pq[0]);
+                pq[1] = fmaf(h.y, xl, pq[1]);
+                pq[2] = fmaf(h.z, xl, pq[2]);
+                pq[3] = fmaf(h.w, xl, pq[3]);
             }
+        };
+        const int s = slot0 - cnt;
+        if (s < 0) {
+            run(s + NR, -s);
+            run(0, slot0);
+        } else {
+            run(s, cnt);
         }
         // pairs inside the tile, then the ring takes its SFTs
 #pragma unroll
@@ -592,6 +672,14 @@ __global__ void __launch_bounds__(256, 3) demod_pair_kernel(DevParams p, int m_l
     // rho = (2 raw) / sqrt(2 den)
     if (act) rho[(size_t)t * p.N_f + k] = den > 0.f ? 1.41421356237309505f * raw * rsqrtf(den) : 0.f;
 }
+
+// R_s = floor(T_max / T_sft): blocks back that hold partners; whether the separable form keeps
+// their sums in its shared-memory ring.
+int demod_blocks_back(const cc_plan* plan) {
+    const double Tsft = (double)llround(plan->cfg.T_sft / plan->cfg.dt) * plan->cfg.dt;
+    return (int)std::floor(plan->cfg.T_max / Tsft + 1e-9);
+}
+bool demod_sep_ring(int Rs) { return (size_t)(Rs + 1) * 7 * 128 * sizeof(float) <= DM_SEP_RING; }
 
 }  // namespace
 }  // namespace cc
@@ -640,7 +728,7 @@ extern "C" cc_status crosscorr_demod_prepare(cc_plan* plan, const void* const* x
         tw[j] = make_float2((float)cos(a), (float)sin(a));
     }
     if ((e = cudaMalloc(&plan->demod_tw, sizeof(float2) * nsft)) != cudaSuccess ||
-        (e = cudaMalloc(&plan->demod_z, sizeof(float2) * (size_t)p.Q * n_blk * nbins)) != cudaSuccess ||
+        (e = cudaMalloc(&plan->demod_z, sizeof(float2) * (size_t)p.Q * n_blk * (nbins + 2))) != cudaSuccess ||
         (e = cudaMalloc(&plan->demod_w, sizeof(float4) * (size_t)p.Q * n_blk)) != cudaSuccess)
         return cuda_fail(e, "demodulation SFT allocation");
     cudaStream_t st = (cudaStream_t)stream;
@@ -685,11 +773,42 @@ extern "C" cc_status crosscorr_demod_prepare(cc_plan* plan, const void* const* x
                 if (w[(size_t)X * n_blk + l].z != 0.f) list.push_back((int)(4 * l + X));
         }
         boff[n_blk] = (int)list.size();
-        for (void* ptr : {plan->demod_list, plan->demod_boff})
+        // per entry: its first partner, and the separable kernel's control word (a refresh after
+        // 4 (R_s + 1) single-block steps: the FP32 rounding of the running sums cannot drift
+        // further; totals at most every 64 SFTs)
+        const int Rs = demod_blocks_back(plan), refresh = 4 * (Rs + 1);
+        const bool ring = demod_sep_ring(Rs);
+        std::vector<int> start(list.size() + DM_LIST_PAD, (int)list.size()), ctl(list.size() + 2 * SG, 0);
+        int steps = 0, nacc = 0;
+        for (size_t i = 0; i < list.size(); ++i, ++nacc) {
+            const int l = list[i] >> 2;
+            start[i] = boff[std::max(0, l - Rs)];
+            const int lcur = i ? list[i - 1] >> 2 : l;
+            if (l == lcur) continue;
+            int op = DM_SAME;
+            if (Rs == 0) {
+                op = DM_STEP;
+            } else if (ring) {
+                op = l == lcur + 1 && ++steps < refresh ? DM_STEP : DM_REFRESH;
+            } else {
+                op = l - lcur > Rs ? DM_EMPTY : ++steps < refresh ? DM_STEP : DM_REFRESH;
+            }
+            if (op != DM_STEP) steps = 0;
+            const bool flush = steps == 0 || nacc >= 64;
+            if (flush) nacc = 0;
+            ctl[i] = op | (flush ? 4 : 0);
+            if (ring) ctl[i] |= lcur % (Rs + 1) << 3 | l % (Rs + 1) << 17;
+        }
+        for (void* ptr : {plan->demod_list, plan->demod_boff, plan->demod_start, plan->demod_ctl})
             if (ptr) cudaFree(ptr);
-        plan->demod_list = plan->demod_boff = nullptr;
+        plan->demod_list = plan->demod_boff = plan->demod_start = plan->demod_ctl = nullptr;
         if ((e = cudaMalloc(&plan->demod_list, sizeof(int) * std::max<size_t>(1, list.size()))) != cudaSuccess ||
             (e = cudaMalloc(&plan->demod_boff, sizeof(int) * boff.size())) != cudaSuccess ||
+            (e = cudaMalloc(&plan->demod_start, sizeof(int) * start.size())) != cudaSuccess ||
+            (e = cudaMalloc(&plan->demod_ctl, sizeof(int) * ctl.size())) != cudaSuccess ||
+            (e = cudaMemcpy(plan->demod_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice)) !=
+                cudaSuccess ||
+            (e = cudaMemcpy(plan->demod_ctl, ctl.data(), sizeof(int) * ctl.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
             (!list.empty() && (e = cudaMemcpy(plan->demod_list, list.data(), sizeof(int) * list.size(),
                                               cudaMemcpyHostToDevice)) != cudaSuccess) ||
             (e = cudaMemcpy(plan->demod_boff, boff.data(), sizeof(int) * boff.size(), cudaMemcpyHostToDevice)) !=
@@ -722,44 +841,53 @@ extern "C" cc_status crosscorr_demod_search(cc_plan* plan, const cc_template* t_
     if (!t_dev || !rho_dev) return fail(CC_ERR_INVALID, "null device pointer");
     const DevParams& p = plan->dp;
     const int n_blk = plan->demod_nblk, nsft = plan->demod_nsft;
-    const double Tsft = nsft * plan->cfg.dt;
-    const int Rs = (int)std::floor(plan->cfg.T_max / Tsft + 1e-9);
+    const int Rs = demod_blocks_back(plan);
     const int W = (Rs + 1) * p.Q;
     const bool sep = plan->demod_form == CC_DEMOD_SEPARABLE;
     const int n_list = plan->demod_nlist;
-    // separable form: 128 threads, the ring of block sums while it stays within DM_SEP_RING
-    const bool sep_ring = sep && (size_t)(Rs + 1) * 7 * 128 * sizeof(float) <= DM_SEP_RING;
+    // separable form: the ring of block sums while 128 bins of it stay within DM_SEP_RING
+    const bool sep_ring = sep && demod_sep_ring(Rs);
     int nthr = sep ? 128 : 256;
     auto ring_bytes = [&](int nt) {
-        return sep ? (sep_ring ? (size_t)(Rs + 1) * 7 * nt * sizeof(float) : 0)
+        return sep ? (sep_ring ? (size_t)(Rs + 1) * 7 * SB * nt * sizeof(float) : 0)
                    : (size_t)W * nt * 12 + (size_t)W * 40 + 8 + 4 * PT * 32 + 32;
     };
+    const int bins = sep ? SB : 1;   // output bins of a thread
     while (nthr > 32 && ring_bytes(nthr) > DM_RING_BUDGET) nthr /= 2;
     if (ring_bytes(nthr) > DM_RING_BUDGET) return fail(CC_ERR_UNSUPPORTED, "T_max / T_sft too large for the pair ring");
-    // exact window sum (over the ring, or recomputed from the bins) after 4 (R_s + 1)
-    // single-block steps: the FP32 rounding of the running sums cannot drift further
-    const int refresh = 4 * (Rs + 1);
     // timing records for a batch of templates: the list of locked SFTs plus two padding
     const size_t per_t = sizeof(DemodTiming) * ((size_t)n_list + 2);
     const int64_t batch = std::max<int64_t>(1, std::min<int64_t>({n_t, (int64_t)((size_t)2 << 30) / (int64_t)per_t, 65535}));
+    auto kernel = [&](int nt) -> const void* {
+        if (sep) return sep_ring ? (const void*)demod_sep_kernel<true> : (const void*)demod_sep_kernel<false>;
+        switch (nt) {
+            case 256: return (const void*)demod_pair_kernel<256>;
+            case 192: return (const void*)demod_pair_kernel<192>;
+            case 128: return (const void*)demod_pair_kernel<128>;
+            case 96: return (const void*)demod_pair_kernel<96>;
+            case 64: return (const void*)demod_pair_kernel<64>;
+            default: return (const void*)demod_pair_kernel<32>;
+        }
+    };
     {
-        // CTA size (every thread does the same work): the fewest resident-thread slots over whole
-        // waves of the first batch, ceil(CTAs / (resident CTAs x SMs)) x resident threads per SM
+        // CTA size (every thread does the same work, in whole waves of the first batch): the least
+        // waves x warps resident on an SM, a wave of few warps counted as one of eleven (its time
+        // is the latency of a thread's steps; the separable form's two bins a thread fill the
+        // issue slots from there on)
         int dev = 0, sms = 152;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const void* kern = !sep ? (const void*)demod_pair_kernel
-                                : sep_ring ? (const void*)demod_sep_kernel<true> : (const void*)demod_sep_kernel<false>;
         int64_t best = -1;
-        for (int nt : {256, 192, 128, 96, 64}) {
-            if (nt > (sep ? 128 : 256) || ring_bytes(nt) > DM_RING_BUDGET) continue;
+        for (int nt : {256, 192, 128, 112, 96, 80, 64, 48}) {
+            if (sep ? nt > 128 : nt == 112 || nt == 80 || nt == 48) continue;
+            if (ring_bytes(nt) > DM_RING_BUDGET) continue;
             if (ring_bytes(nt) > 48 * 1024 &&
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes(nt)) != cudaSuccess)
+                cudaFuncSetAttribute(kernel(nt), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes(nt)) != cudaSuccess)
                 continue;
             int occ = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, nt, ring_bytes(nt)) != cudaSuccess || occ < 1)
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel(nt), nt, ring_bytes(nt)) != cudaSuccess || occ < 1)
                 continue;
-            const int64_t ctas = (plan->N_f + nt - 1) / nt * std::min(batch, n_t);
-            const int64_t est = (ctas + (int64_t)occ * sms - 1) / ((int64_t)occ * sms) * occ * nt;
+            const int64_t ctas = (plan->N_f + (int64_t)bins * nt - 1) / ((int64_t)bins * nt) * std::min(batch, n_t);
+            const int64_t est = (ctas + (int64_t)occ * sms - 1) / ((int64_t)occ * sms) * std::max(11, occ * ((nt + 31) / 32));
             if (best < 0 || est < best) {
                 best = est;
                 nthr = nt;
@@ -772,8 +900,7 @@ extern "C" cc_status crosscorr_demod_search(cc_plan* plan, const cc_template* t_
     cudaError_t e;
     const size_t smem = ring_bytes(nthr);
     if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(sep ? (const void*)demod_sep_kernel<true> : (const void*)demod_pair_kernel,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        (e = cudaFuncSetAttribute(kernel(nthr), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return cuda_fail(e, "demodulation smem attribute");
     const double df0 = plan->f_r - 0.5 / plan->cfg.dt, dK = 1.0 / plan->T_FFT;
     for (int64_t t0 = 0; t0 < n_t; t0 += batch) {
@@ -787,17 +914,20 @@ extern "C" cc_status crosscorr_demod_search(cc_plan* plan, const cc_template* t_
         cudaEvent_t ev0, ev1;   // diagnostic timing of the pair loop (crosscorr_plan_set_kernel_timing)
         timing_pair(plan, &ev0, &ev1);
         if (ev0) cudaEventRecord(ev0, st);
-        const dim3 grid((unsigned)((plan->N_f + nthr - 1) / nthr), (unsigned)nb);
-        if (sep)
-            (sep_ring ? demod_sep_kernel<true> : demod_sep_kernel<false>)<<<grid, nthr, smem, st>>>(
-                p, plan->demod_m_lo, plan->demod_nbins, n_blk, Rs, refresh, (const float2*)plan->demod_z,
-                (const DemodTiming*)plan->ws, n_list, (const int*)plan->demod_boff, (const double*)plan->demod_df,
-                (const int64_t*)plan->demod_kbar, t0, rho_dev);
-        else
-            demod_pair_kernel<<<grid, nthr, smem, st>>>(
-                p, plan->demod_m_lo, plan->demod_nbins, n_blk, Rs, (const float2*)plan->demod_z,
-                (const DemodTiming*)plan->ws, n_list, (const int*)plan->demod_boff, (const double*)plan->demod_df,
-                (const int64_t*)plan->demod_kbar, t0, rho_dev);
+        const dim3 grid((unsigned)((plan->N_f + (int64_t)bins * nthr - 1) / ((int64_t)bins * nthr)), (unsigned)nb);
+        const float2* zp = (const float2*)plan->demod_z;
+        const DemodTiming* rp = (const DemodTiming*)plan->ws;
+        const int *bo = (const int*)plan->demod_boff, *li = (const int*)plan->demod_list, *ct = (const int*)plan->demod_ctl,
+                  *sp = (const int*)plan->demod_start;
+        const double* dfp = (const double*)plan->demod_df;
+        const int64_t* kp = (const int64_t*)plan->demod_kbar;
+        void* as[] = {(void*)&p, (void*)&plan->demod_m_lo, (void*)&plan->demod_nbins, (void*)&n_blk, (void*)&Rs, (void*)&zp,
+                      (void*)&rp, (void*)&n_list, (void*)&bo, (void*)&li, (void*)&ct, (void*)&dfp, (void*)&kp, (void*)&t0,
+                      (void*)&rho_dev};
+        void* ap[] = {(void*)&p, (void*)&plan->demod_m_lo, (void*)&plan->demod_nbins, (void*)&n_blk, (void*)&Rs, (void*)&zp,
+                      (void*)&rp, (void*)&n_list, (void*)&sp, (void*)&dfp, (void*)&kp, (void*)&t0, (void*)&rho_dev};
+        if ((e = cudaLaunchKernel(kernel(nthr), grid, dim3((unsigned)nthr), sep ? as : ap, smem, st)) != cudaSuccess)
+            return cuda_fail(e, "demodulation launch");
         count_launch();
         if (ev1) cudaEventRecord(ev1, st);
     }
