@@ -20,9 +20,8 @@ namespace cc {
 constexpr int KNOT = 128;
 constexpr int MAX_D = 32;
 constexpr int MAX_TAPS = 2 * MAX_D + 1;
-constexpr int N_BIN_ITER = 4;   // fixed-point steps of the binary delay b = a_p sin(Omega (tau + b - T_asc))
-constexpr int N_SSB_ITER = 4;   // fixed-point steps of t = u - Delta(t)
-constexpr int N_KEPLER_ITER = 8; // joint fixed-point / Newton steps of the elliptical binary delay
+constexpr int N_BIN_ITER = 4;   // fixed-point steps of the binary delay b = a_p sin(Omega (tau + b - T_asc)), at most
+constexpr int N_KEPLER_ITER = 8; // Newton steps of the elliptical binary delay, at most
 constexpr int MAX_L = 4096;     // largest coset FFT: 256 threads, one radix-16 butterfly each per pass
 
 // Learned interpolator: 8 taps from a 2 -> 64 -> 64 -> 8 tanh network, tabulated at
@@ -311,16 +310,29 @@ __device__ __forceinline__ Orbit make_orbit(const DevParams& p, const cc_templat
 // FP64 sincospi at theta0, then fixed-point steps through the angle-addition formula
 // with sin/cos of the small angle Omega b (|Omega b| <= 1.4e-4 rad) from their series
 // (remainders below 1e-26); the contraction a_p Omega ~ 1.3e-4 per step leaves
-// < 1e-15 s after N_BIN_ITER steps.  Elliptical orbit: b = R(tau + b)/c with E from
-// Kepler's equation, one Newton step per fixed-point step from the previous E (the mean
-// anomaly moves by Omega db ~ 1e-4 rad per step), N_KEPLER_ITER steps (Newton from
-// E = M + e sin M converges quadratically to FP64 precision well within them for e < 0.95).
-// SSB part: t = u - Delta(t), u = tau + b, iterated on Delta from Delta(u) (contraction
-// |Delta'| <= 1e-4).  Both work on the small quantities b and Delta so d = Delta - b
+// a_p (a_p Omega)^(n + 1) after n steps: as many steps as take that below the rounding of b
+// (three for Sco X-1), at most N_BIN_ITER.  Elliptical orbit: b = R(tau + b)/c with E from
+// Kepler's equation at the mean anomaly M0 + Omega b(E), by Newton's method on both at once
+// from E = M0 + e sin M0 + e^2/2 sin 2 M0; quadratic convergence ends it after three or four
+// steps for moderate e (at most N_KEPLER_ITER), when a step is below the rounding of E.
+// SSB part: t = u - Delta(t), u = tau + b: Delta is linear between table nodes, so one Newton
+// step from t1 = u - Delta(u) (0.05 s off at most) is exact unless a node lies between, and a
+// second one from there is.  Both work on the small quantities b and Delta so d = Delta - b
 // keeps FP64 precision.  The binary part depends on the source time only, so a caller
 // with several detectors computes it once (knot_binary) and the SSB part per detector
 // (knot_ssb); knot_delay is the two together.
-__device__ __forceinline__ double knot_binary(const Orbit& o, double tau) {
+__device__ __forceinline__ int binary_steps(const Orbit& o) {
+    const float q = (float)fabs(o.a_p * 6.283185307179586 * o.invP);
+    float r = q * q;   // relative error after one step
+    int n = 1;
+    while (n < N_BIN_ITER && r > 4.4e-16f) {
+        r *= q;
+        ++n;
+    }
+    return n;
+}
+
+__device__ __forceinline__ double knot_binary(const Orbit& o, double tau, int steps) {
     double b;
     if (o.e == 0.0) {
         const double x0 = (tau - o.tasc_rel) * o.invP;        // orbital phase in cycles
@@ -328,8 +340,8 @@ __device__ __forceinline__ double knot_binary(const Orbit& o, double tau) {
         sincospi(2.0 * x0, &s0, &c0);
         const double om = 6.283185307179586 * o.invP;         // Omega
         b = o.a_p * s0;
-#pragma unroll
-        for (int it = 0; it < N_BIN_ITER; ++it) {
+#pragma unroll 1
+        for (int it = 0; it < steps; ++it) {
             const double dl = om * b, d2 = dl * dl;
             const double sd = dl * (1.0 - d2 * (1.0 / 6.0) * (1.0 - d2 * (1.0 / 20.0)));
             const double cd = 1.0 - d2 * 0.5 * (1.0 - d2 * (1.0 / 12.0));
@@ -340,33 +352,60 @@ __device__ __forceinline__ double knot_binary(const Orbit& o, double tau) {
         xm -= floor(xm);
         const double M0 = 6.283185307179586 * xm;             // mean anomaly at tau, [0, 2 pi)
         const double om = 6.283185307179586 * o.invP;
-        double E = M0 + o.e * sinpi(2.0 * xm), sE, cE;
-        sincos_rad(E, &sE, &cE);
-        b = 0.0;
+        double sM, cM, sE, cE;
+        sincospi(2.0 * xm, &sM, &cM);
+        double E = M0 + o.e * sM * (1.0 + o.e * cM);
+        const double as = o.a_p * o.sinw, ac = o.a_p * o.cosw * o.sq;
 #pragma unroll 1
-        for (int it = 0; it < N_KEPLER_ITER; ++it) {
-            const double M = M0 + om * b;                      // mean anomaly at u = tau + b
-            E -= (E - o.e * sE - M) / (1.0 - o.e * cE);
+        for (int it = 0;; ++it) {
             sincos_rad(E, &sE, &cE);
-            b = o.a_p * (o.sinw * (cE - o.e) + o.cosw * o.sq * sE);
+            b = as * (cE - o.e) + ac * sE;
+            if (it == N_KEPLER_ITER) break;
+            // f(E) = E - e sin E - M0 - Omega b(E)
+            const double db = ac * cE - as * sE;               // db / dE
+            const double dE = (E - o.e * sE - M0 - om * b) / (1.0 - o.e * cE - om * db);
+            E -= dE;
+            if (fabs(dE) < 1.0e-9) {   // what is left is O(dE^2): b there to first order
+                b -= dE * db;
+                break;
+            }
         }
     }
     return b;
 }
 
+// Table value and slope (per second) of the interval holding t (end intervals extrapolate).
+__device__ __forceinline__ double table_at(const double* tab, double t0, double inv_dt, int n, double t, double* slope) {
+    const double u = (t - t0) * inv_dt;
+    double fi = floor(u);
+    int i = (int)fi;
+    if (i < 0 || i > n - 2) {
+        i = u < 0.0 ? 0 : n - 2;
+        fi = (double)i;
+    }
+    const double v0 = __ldg(tab + i), dv = __ldg(tab + i + 1) - v0;
+    *slope = dv * inv_dt;
+    return fma(u - fi, dv, v0);
+}
+
 __device__ __forceinline__ double knot_ssb(const DevParams& p, int X, double tau, double b) {
     const double* tab = p.ssb[X];
     const double t0 = p.eph_t0[X], inv = p.inv_eph_dt[X];
-    const int64_t n = p.n_eph[X];
+    const int n = (int)p.n_eph[X];
     const double u = tau + b;
-    double dl = table_lerp(tab, t0, inv, n, u);
+    double m;
+    double dl = table_at(tab, t0, inv, n, u, &m);
 #pragma unroll
-    for (int it = 0; it < N_SSB_ITER; ++it) dl = table_lerp(tab, t0, inv, n, u - dl);
+    for (int it = 0; it < 2; ++it) {
+        // residual r = Delta(u - dl) - dl; dl + r / (1 + m) solves the interval's linear equation
+        const double r = table_at(tab, t0, inv, n, u - dl, &m) - dl;
+        dl = fma(r, 1.0 - m * (1.0 - m), dl);
+    }
     return dl - b;
 }
 
 __device__ __forceinline__ double knot_delay(const DevParams& p, int X, const Orbit& o, double tau) {
-    return knot_ssb(p, X, tau, knot_binary(o, tau));
+    return knot_ssb(p, X, tau, knot_binary(o, tau, binary_steps(o)));
 }
 
 // Knot record from the delays at knots k-1, k, k+1, k+2 (seconds) of a knot at

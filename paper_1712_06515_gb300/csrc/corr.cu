@@ -60,7 +60,7 @@ struct LagArgs {
     float2* h;              // [n_t][n_lags] (C > 2)
     const float2* twL;      // exp(-2 pi i j / L)
     const float4* norm;     // [n_t][Q][M]
-    double* D;              // [n_t]
+    double* D;              // [n_t] sqrt(2 / normalisation), 0 without weight
     int64_t M;
     int L, log2L, C, planes, n_rows, n_lags, N_s, Q, R, pair_mode;
 };
@@ -82,7 +82,7 @@ __device__ __forceinline__ double norm_pair(float4 a, float4 b) {
     return (double)a.x * b.x + (double)a.y * b.y + 2.0 * (double)a.z * b.z;
 }
 
-// grid: x = coset c (x = C, y = 0: the normalisation D of template z), y = A or B, z = template.
+// grid: x = coset c (x = C, y = 0: the normalisation factor of template z), y = A or B, z = template.
 __global__ void __launch_bounds__(LAG_THREADS)
 corr_lags_kernel(const LagArgs q) {
     extern __shared__ __align__(16) float2 buf[];
@@ -110,7 +110,7 @@ corr_lags_kernel(const LagArgs q) {
         if (threadIdx.x == 0) {
             double s = 0.0;
             for (int w = 0; w < LAG_THREADS / 32; ++w) s += red[w];
-            q.D[t] = s;
+            q.D[t] = s > 0.0 ? 1.4142135623730951 / sqrt(s) : 0.0;
         }
         return;
     }
@@ -195,11 +195,10 @@ corr_rho_kernel(const LagArgs q, int L, int log2L, const float2* __restrict__ tw
     }
     __syncthreads();
     const float2* res = fft_stockham(buf, buf + L, L, log2L, twL);
-    const double D = q.D[t];
-    const double sc = D > 0.0 ? 1.4142135623730951 / sqrt(D) : 0.0;
+    const double sc = q.D[t];
     const int e = __ldg(off + c + 1);
     for (int i = __ldg(off + c) + threadIdx.x; i < e; i += LAG_THREADS)
-        rho[t * N_f + __ldg(ck + i)] = D > 0.0 ? (float)((double)res[__ldg(cm + i)].x * sc) : 0.f;
+        rho[t * N_f + __ldg(ck + i)] = sc > 0.0 ? (float)((double)res[__ldg(cm + i)].x * sc) : 0.f;
 }
 
 // ---------------------------------------------------------------------------
@@ -290,15 +289,15 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     a.smem = (uint32_t)(o + 16);
     // Chunks of segments: units are equal, handed out one by one to two CTAs per SM, each
     // rereads its first segment's predecessor (R = 1) and writes one row (about the traffic of
-    // another segment): the count with the least ceil(units / slots) (length + overhead), at
-    // most M / (4 R + 1) chunks; with cc_tuning.chunk_waves, that many units per slot.
+    // another segment): the count with the least ceil(units / slots) (length + overhead); with
+    // cc_tuning.chunk_waves, that many units per slot, at most M / (4 R + 1) chunks.
     const int64_t slots = (int64_t)CORR_CTAS_PER_SM * sm_count();
     const int64_t per_chunk = (2 * n_t + y->T - 1) / y->T * y->C;
     const int64_t minch = (p.M + CORR_MAX_CHUNK - 1) / CORR_MAX_CHUNK;
-    const int64_t maxch = std::max<int64_t>(minch, p.M / (4 * p.R + 1));
+    const int64_t maxch = std::max<int64_t>(minch, p.M);
     int64_t nch = minch;
     if (plan->tuning.chunk_waves > 0) {
-        nch = std::max(minch, std::min<int64_t>(maxch, (plan->tuning.chunk_waves * slots + per_chunk - 1) / per_chunk));
+        nch = std::max(minch, std::min<int64_t>(std::max<int64_t>(1, p.M / (4 * p.R + 1)), (plan->tuning.chunk_waves * slots + per_chunk - 1) / per_chunk));
     } else {
         const int64_t most = std::max(minch, std::min<int64_t>(maxch, (32 * slots + per_chunk - 1) / per_chunk));
         int64_t best = -1;

@@ -96,31 +96,38 @@ bool fused_layout(const cc_plan* plan, int64_t n_t, FusedLayout* lay) {
 }
 
 // Knot records (FP64 delays at every KNOT-th source sample, four per record) for a batch
-// of templates: one thread per record of every detector, the block's 256 records plus
-// three halo knots.  The binary-orbit part of each delay is computed once for all
-// detectors (it depends on the source time only); the barycentric part per detector.
-__global__ void __launch_bounds__(256)
+// of templates: a block computes KN_BLOCK consecutive delays of every detector, one a thread,
+// and writes the records whose four knots it holds.  The binary-orbit part of each delay is
+// computed once for all detectors (it depends on the source time only); the barycentric part
+// per detector.  Bound by the FP64 rate.
+constexpr int KN_BLOCK = 128, KN_OUT = KN_BLOCK - 3;
+
+__global__ void __launch_bounds__(KN_BLOCK)
 knots_kernel(DevParams p, const cc_template* __restrict__ tm, int64_t t_base, int64_t nkn,
              KnotRec* __restrict__ out, int* __restrict__ zero_word) {
-    __shared__ double dk[CC_MAX_DET][256 + 3];
+    __shared__ double dk[CC_MAX_DET][KN_BLOCK];
     __shared__ Orbit orb_s;
+    __shared__ int steps_s;
     const int Q = p.Q;
     const int64_t tl = blockIdx.z, t = t_base + tl;
-    const int64_t k0 = (int64_t)blockIdx.x * 256;
+    const int64_t k0 = (int64_t)blockIdx.x * KN_OUT;
     // the orbit's FP64 set-up (a reciprocal, and trigonometry for e != 0) once per block
-    if (threadIdx.x == 0) orb_s = make_orbit(p, tm[t]);
+    if (threadIdx.x == 0) {
+        orb_s = make_orbit(p, tm[t]);
+        steps_s = binary_steps(orb_s);
+    }
     // a later kernel's unit counter, cleared here instead of by a memset of its own
     if (zero_word && threadIdx.x == 32 && blockIdx.x == 0 && blockIdx.z == 0) *zero_word = 0;
     __syncthreads();
     const Orbit orb = orb_s;
-    for (int i = threadIdx.x; i < 256 + 3; i += 256) {
-        const double tau = (double)((k0 - 1 + i) * KNOT) * p.dt;
-        const double b = knot_binary(orb, tau);
-        for (int X = 0; X < Q; ++X) dk[X][i] = knot_ssb(p, X, tau, b);
+    {
+        const double tau = (double)((k0 - 1 + threadIdx.x) * KNOT) * p.dt;
+        const double b = knot_binary(orb, tau, steps_s);
+        for (int X = 0; X < Q; ++X) dk[X][threadIdx.x] = knot_ssb(p, X, tau, b);
     }
     __syncthreads();
     const int64_t k = k0 + threadIdx.x;
-    if (k < nkn)
+    if (threadIdx.x < KN_OUT && k < nkn)
         for (int X = 0; X < Q; ++X)
             out[((size_t)tl * Q + X) * nkn + k] =
                 make_knot(p, dk[X][threadIdx.x], dk[X][threadIdx.x + 1], dk[X][threadIdx.x + 2],
@@ -136,8 +143,8 @@ cc_status launch_knots(cc_plan* plan, const cc_template* t_dev, int64_t n_t, Kno
     const int64_t nkn = knot_rows(plan);
     for (int64_t t0 = 0; t0 < n_t; t0 += 65535) {
         const int64_t nt = std::min<int64_t>(65535, n_t - t0);
-        dim3 gk((unsigned)((nkn + 255) / 256), 1u, (unsigned)nt);
-        knots_kernel<<<gk, 256, 0, st>>>(p, t_dev + t0, 0, nkn, kn + (size_t)t0 * p.Q * nkn, zero_word);
+        dim3 gk((unsigned)((nkn + KN_OUT - 1) / KN_OUT), 1u, (unsigned)nt);
+        knots_kernel<<<gk, KN_BLOCK, 0, st>>>(p, t_dev + t0, 0, nkn, kn + (size_t)t0 * p.Q * nkn, zero_word);
         count_launch();
     }
     cudaError_t e = cudaGetLastError();
@@ -185,8 +192,8 @@ cc_status launch_fused(cc_plan* plan, const cc_template* t_dev, int64_t n_t, flo
     for (int64_t tb = 0; tb < n_t; tb += step) {
         const int64_t nt = std::min(step, n_t - tb);
         if (pre) {
-            dim3 gk((unsigned)((nkn + 255) / 256), 1u, (unsigned)nt);
-            knots_kernel<<<gk, 256, 0, st>>>(p, t_dev, tb, nkn, kn_ws, nullptr);
+            dim3 gk((unsigned)((nkn + KN_OUT - 1) / KN_OUT), 1u, (unsigned)nt);
+            knots_kernel<<<gk, KN_BLOCK, 0, st>>>(p, t_dev, tb, nkn, kn_ws, nullptr);
             count_launch();
         }
         cudaLaunchConfig_t cfg = {};
