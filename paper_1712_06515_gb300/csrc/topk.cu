@@ -176,8 +176,7 @@ topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups,
             const unsigned* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ bool last;
-    __shared__ unsigned hist[256], s_prefix;
-    __shared__ int s_need, ncand;
+    __shared__ int cnt[33], ncand;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nw = gridDim.x * (SEL_THREADS / 32);
     for (int g = blockIdx.x * (SEL_THREADS / 32) + warp; g < n_groups; g += nw) {
@@ -191,37 +190,34 @@ topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups,
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // the k-th largest maximum, eight bits at a time
-    if (tid == 0) {
-        s_prefix = 0;
-        s_need = k;
-        ncand = 0;
+    // the k-th largest maximum, bit by bit: the largest value that k maxima reach (a histogram of
+    // them would serialise: they share their leading bits)
+    unsigned mine[SEL_GROUPS / SEL_THREADS];
+#pragma unroll
+    for (int i = 0; i < SEL_GROUPS / SEL_THREADS; ++i) {
+        const int g = i * SEL_THREADS + tid;
+        mine[i] = g < n_groups ? __ldcg(maxima + g) : 0u;
     }
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        if (tid < 256) hist[tid] = 0;
+    if (tid < 33) cnt[tid] = 0;
+    if (tid == 0) ncand = 0;
+    __syncthreads();
+    unsigned thr = 0;
+    for (int bit = 31; bit >= 0; --bit) {
+        const unsigned c = thr | (1u << bit);
+        int n_ge = 0;
+#pragma unroll
+        for (int i = 0; i < SEL_GROUPS / SEL_THREADS; ++i) n_ge += mine[i] >= c;
+        n_ge = __reduce_add_sync(0xffffffffu, n_ge);
+        if (lane == 0 && n_ge) atomicAdd(&cnt[bit], n_ge);
         __syncthreads();
-        const unsigned prefix = s_prefix, mask = shift == 24 ? 0u : 0xffffffffu << (shift + 8);
-        for (int g = tid; g < n_groups; g += SEL_THREADS) {
-            const unsigned m = __ldcg(maxima + g);
-            if ((m & mask) == prefix) atomicAdd(&hist[(m >> shift) & 255u], 1u);
-        }
-        __syncthreads();
-        if (tid == 0) {
-            int need = s_need, d = 255;
-            while (d > 0 && (int)hist[d] < need) need -= (int)hist[d--];
-            s_need = need;
-            s_prefix = prefix | ((unsigned)d << shift);
-        }
-        __syncthreads();
+        if (cnt[bit] >= k) thr = c;
     }
-    const unsigned thr = s_prefix;
     Cand* s = (Cand*)smem;
     for (int g0 = warp * 32; g0 < n_groups; g0 += SEL_THREADS)
         for (unsigned hit = __ballot_sync(0xffffffffu, g0 + lane < n_groups && __ldcg(maxima + g0 + lane) >= thr); hit; hit &= hit - 1) {
         const int g = g0 + __ffs(hit) - 1;
         const long long b = (long long)g * gsize, e = b + gsize < n ? b + gsize : n;
-        for (long long i = b + lane; i < e; i += 32) {
-            const float v = __ldg(rho + i);
+        auto take = [&](float v, long long i) {
             if (sel_key(v) >= thr) {
                 const int pos = atomicAdd(&ncand, 1);
                 if (pos < SEL_CAP) {
@@ -232,7 +228,22 @@ topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups,
                     s[pos] = c;
                 }
             }
+        };
+        long long i0 = b;
+        if (aligned) {
+            const float4* p = (const float4*)(rho + b);
+            const long long n4 = (e - b) >> 2;
+#pragma unroll 4
+            for (long long i = lane; i < n4; i += 32) {
+                const float4 v = __ldg(p + i);
+                take(v.x, b + 4 * i);
+                take(v.y, b + 4 * i + 1);
+                take(v.z, b + 4 * i + 2);
+                take(v.w, b + 4 * i + 3);
+            }
+            i0 += n4 << 2;
         }
+        for (long long i = i0 + lane; i < e; i += 32) take(__ldg(rho + i), i);
     }
     __syncthreads();
     const int m = ncand;
