@@ -115,6 +115,10 @@ typedef struct {
     double omega;  /* argument of periapsis w [rad] */
 } cc_template;
 
+/* Circular templates t3_dev, device double [n_t][3] rows (a_p, T_asc, P), as cc_template rows
+ * t_dev (device [n_t]) with e = omega = 0; asynchronous on `stream`. */
+cc_status crosscorr_templates_circular(const double* t3_dev, int64_t n_t, cc_template* t_dev, void* stream);
+
 /* One top-k record. */
 typedef struct {
     int64_t tmpl;  /* template index within the rho array */

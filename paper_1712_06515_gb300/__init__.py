@@ -25,6 +25,11 @@ STORE_FP32, STORE_BF16 = 0, 1
 INTERP_EXACT, INTERP_LEARNED = 0, 1
 PATH_AUTO, PATH_FUSED, PATH_TWO_PASS, PATH_STAGED = 0, 1, 2, 3
 
+# the records of crosscorr_rho_topk as the C ABI lays them out
+_HIT = np.dtype({"names": ["tmpl", "bin", "freq", "rho"], "formats": [np.int64, np.int32, np.float64, np.float32],
+                 "offsets": [getattr(CcHit, f).offset for f in ("tmpl", "bin", "freq", "rho")],
+                 "itemsize": ctypes.sizeof(CcHit)})
+
 build = _lib.build
 load = _lib.load
 
@@ -58,8 +63,20 @@ def templates5(templates):
     import torch
     if templates.shape[-1] == 5:
         return templates
+    if templates.is_cuda and templates.dim() == 2 and templates.dtype == torch.float64 and templates.is_contiguous():
+        return _circular(templates, None)
     z = torch.zeros((templates.shape[0], 2), dtype=templates.dtype, device=templates.device)
     return torch.cat([templates, z], dim=1).contiguous()
+
+
+def _circular(t3, stream):
+    """[n, 3] contiguous CUDA rows widened to [n, 5] by the library, on `stream`."""
+    import torch
+    lib = _lib.load()
+    out = torch.empty((t3.shape[0], 5), dtype=torch.float64, device=t3.device)
+    check("crosscorr_templates_circular", lib.crosscorr_templates_circular(_dptr(t3), t3.shape[0], _dptr(out),
+                                                                          _stream_handle(stream)))
+    return out
 
 
 def metric(T_obs: float, T_sft: float, T_max: float, Q: int, f: float, a_p: float, T_asc: float, P: float,
@@ -208,6 +225,10 @@ class CrossCorrPlan:
     # -- helpers ---------------------------------------------------------------
     def _xptrs(self, x):
         import torch
+        if (isinstance(x, torch.Tensor) and x.dim() == 2 and x.is_contiguous() and x.is_cuda and x.dtype == torch.complex64
+                and tuple(x.shape) == (self.Q, self.cfg.n_samples)):
+            base, row = _dptr(x), 8 * x.shape[1]   # one tensor of every detector's series: no views needed
+            return (c_void_p * self.Q)(*[base + i * row for i in range(self.Q)]), [x]
         if isinstance(x, torch.Tensor):
             xs = [x[i] for i in range(x.shape[0])]
         else:
@@ -368,10 +389,11 @@ class CrossCorrPlan:
         hits = (CcHit * max(n, 1))()
         check("crosscorr_rho_topk", self._lib.crosscorr_rho_topk(
             self._h, _dptr(rho), n_t, k, hits, _stream_handle(stream)))
+        rec = np.frombuffer(hits, dtype=_HIT, count=n)
         out = np.zeros(n, dtype=[("tmpl", np.int64), ("bin", np.int32), ("freq", np.float64),
                                  ("rho", np.float32)])
-        for i in range(n):
-            out[i] = (hits[i].tmpl, hits[i].bin, hits[i].freq, hits[i].rho)
+        for name in out.dtype.names:
+            out[name] = rec[name]
         return out
 
     def close(self):

@@ -138,6 +138,7 @@ SIGNATURES = {
                                  POINTER(c_double)]),
     "crosscorr_lattice": (c_int, [POINTER(c_double), c_double, POINTER(c_double), POINTER(c_double), c_void_p,
                                   c_int64, POINTER(c_int64)]),
+    "crosscorr_templates_circular": (c_int, [c_void_p, c_int64, c_void_p, c_void_p]),
     "crosscorr_sfts_to_series": (c_int, [c_void_p, c_void_p, c_int64, c_int64, c_double, c_double, c_void_p,
                                          c_void_p]),
     "crosscorr_demod_search": (c_int, [c_void_p, c_void_p, c_int64, c_void_p, c_void_p]),

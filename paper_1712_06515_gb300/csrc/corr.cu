@@ -544,8 +544,8 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         q.pair_mode = p.pair_mode;
         const size_t sm1 = (size_t)2 * y.L * sizeof(float2), sm2 = (size_t)2 * p.L * sizeof(float2);
         const int big = (int)(2 * CORR_POINTS * sizeof(float2));
-        if ((e = cudaFuncSetAttribute(corr_lags_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(corr_rho_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess)
+        if ((sm1 > 48 * 1024 && (e = cudaFuncSetAttribute(corr_lags_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess) ||
+            (sm2 > 48 * 1024 && (e = cudaFuncSetAttribute(corr_rho_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess))
             return cuda_fail(e, "lag kernels smem attribute");
         corr_lags_kernel<<<dim3((unsigned)(y.C + 1), y.planes > 1 ? 2u : 1u, (unsigned)nb), LAG_THREADS, sm1, st>>>(q);
         count_launch();

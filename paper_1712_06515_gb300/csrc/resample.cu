@@ -243,9 +243,11 @@ cudaError_t launch_group(dim3 grid, int threads, size_t smem, cudaStream_t st, f
         tb.ca[k - 1] = (float)ca;
         tb.cb[k - 1] = (float)(-(double)(k * k) * ca);
     }
-    cudaError_t e = cudaFuncSetAttribute(resample_group_kernel<DT, LEARNED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(resample_group_kernel<DT, LEARNED>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     resample_group_kernel<DT, LEARNED><<<grid, threads, smem, st>>>(ab, norm, kn, nkn, n_t, tg, wpt, tile, cap,
                                                                     write_inactive, act, t_pad, tb, p);
     return cudaGetLastError();

@@ -74,6 +74,25 @@ static bool fused_on_lag_grid(const cc_plan* plan) { return plan->Q > 2 && lag_g
 
 }  // namespace cc
 
+static __global__ void templates_circular_kernel(const double* __restrict__ t3, int64_t n, double* __restrict__ t5) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 5 * n) return;
+    const int64_t r = i / 5, c = i - 5 * r;
+    t5[i] = c < 3 ? t3[3 * r + c] : 0.0;
+}
+
+extern "C" cc_status crosscorr_templates_circular(const double* t3_dev, int64_t n_t, cc_template* t_dev, void* stream) {
+    using namespace cc;
+    static_assert(sizeof(cc_template) == 5 * sizeof(double), "rows of five doubles");
+    if (n_t < 0 || n_t > (int64_t)1 << 36) return fail(CC_ERR_INVALID, "n_t must be in [0, 2^36]");
+    if (n_t == 0) return CC_OK;
+    if (!t3_dev || !t_dev) return fail(CC_ERR_INVALID, "null device pointer");
+    templates_circular_kernel<<<(unsigned)((5 * n_t + 255) / 256), 256, 0, (cudaStream_t)stream>>>(t3_dev, n_t, (double*)t_dev);
+    count_launch();
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? CC_OK : cuda_fail(e, "templates launch");
+}
+
 extern "C" cc_status crosscorr_plan_set_path(cc_plan* plan, int path) {
     using namespace cc;
     if (!plan) return fail(CC_ERR_INVALID, "plan is null");
