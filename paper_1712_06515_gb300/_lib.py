@@ -22,7 +22,7 @@ LIBPATH = os.path.join(LIBDIR, "libcrosscorr.so")
 
 SOURCES = ["plan.cu", "stages.cu", "search.cu", "topk.cu", "fused.cu", "fused_l64_256.cu", "fused_l512_1024.cu",
            "fused_l2048.cu", "fused_l4096.cu", "noalloc.cu", "learned.cu", "corr.cu", "corr_l128_512.cu",
-           "corr_l1024_2048.cu", "corr_l4096.cu", "corr_multi.cu", "fold.cu", "resample.cu", "segpair_tma.cu", "peak.cu", "demod.cu", "sftseries.cu", "lattice.cu"]
+           "corr_l1024_2048.cu", "corr_l4096.cu", "corr_multi.cu", "fold.cu", "resample.cu", "segpair_tma.cu", "segfft_rows.cu", "peak.cu", "demod.cu", "sftseries.cu", "lattice.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I" + INCLUDE]
 

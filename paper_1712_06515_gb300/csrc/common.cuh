@@ -143,7 +143,11 @@ struct cc_plan {
     // coset, roots of its transform length and of 4096 (plan-owned)
     const float2 *corr_twk = nullptr, *corr_twk1 = nullptr, *corr_twL = nullptr, *corr_tw4096 = nullptr;
     const float2 *corr_twp = nullptr, *corr_twp4096 = nullptr;   // last-pass powers (corr_powers)
-    int* segfft_ctr = nullptr;                // [C4] unit counters of the staged segment FFT (plan-owned)
+    // staged segment FFT by rows (segfft_rows.cu; segments of up to 4096 samples, plan-owned):
+    // last-pass powers [C4][4][256], output bin of each coset position [C4][2048], row counter
+    const float2* rows_twp = nullptr;
+    const int* rows_kmap = nullptr;
+    int* segfft_ctr = nullptr;
     bool ws_external = false;                 // ws is caller memory (crosscorr_plan_set_workspace)
     // diagnostic event pairs around fused-kernel launches (crosscorr_plan_set_kernel_timing)
     bool kernel_timing = false;

@@ -426,6 +426,33 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
             }
         }
     }
+    // Staged segment FFT by rows: powers 1, 2, 4, 8 of W_N^(bc + C4 b) for thread j's last-pass
+    // butterfly b = 16 (j mod 16) + j / 16 (the column order of the half-warp exchange), and the
+    // output bin of coset position m (-1: none).  Beyond 64 cosets the kernel computes the powers.
+    // Two bins of one position (nu_R a rounding below one) leave the stage to the general kernel.
+    std::vector<float2> rtw;
+    std::vector<int> rkm;
+    if (C4 > 0 && p->N_s <= 4096 && p->N_s % 2 == 0 && p->Q <= 2 && (p->kbar.back() - p->k0) / C4 < 2048) {
+        const int64_t tabled = C4 <= 64 ? C4 : 0;
+        rtw.resize((size_t)tabled * 1024);
+        rkm.assign((size_t)C4 * 2048, -1);
+        for (int64_t c2 = 0; c2 < tabled; ++c2)
+            for (int n = 0; n < 4; ++n)
+                for (int64_t j = 0; j < 256; ++j) {
+                    const uint64_t ct = (uint64_t)((b0 + c2) % N) + (uint64_t)C4 * (16 * (j & 15) + (j >> 4));
+                    const double ang = -2.0 * M_PI * (double)((ct << n) % (uint64_t)N) / (double)N;
+                    rtw[(size_t)(c2 * 4 + n) * 256 + j] = make_float2((float)cos(ang), (float)sin(ang));
+                }
+        for (int64_t k = 0; k < p->N_f; ++k) {
+            const int64_t kp = p->kbar[k] - p->k0;
+            int& bin = rkm[(size_t)(kp % C4) * 2048 + kp / C4];
+            if (bin >= 0) {
+                rkm.clear();
+                break;
+            }
+            bin = (int)k;
+        }
+    }
     // The lag grid of the two-pass search (corr.cu): G = Cg x Lg points, the same split of the
     // coset twiddles W_G^(c s) and the second pass's twiddles; [1] for one coset (c = 0).
     const int64_t Lg = 2 * p->N_s <= 4096 ? 2 * L : 4096;
@@ -476,6 +503,8 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
         (st = upload(p, cm.data(), cm.size(), &dp.coset_m)) != CC_OK ||
         (st = upload(p, tw.data(), tw.size(), &dp.twL)) != CC_OK ||
         (st = upload(p, twk.data(), twk.size(), &dp.twk)) != CC_OK ||
+        (!rtw.empty() && (st = upload(p, rtw.data(), rtw.size(), &p->rows_twp)) != CC_OK) ||
+        (!rkm.empty() && (st = upload(p, rkm.data(), rkm.size(), &p->rows_kmap)) != CC_OK) ||
         (st = upload(p, gk.data(), gk.size(), &p->corr_twk)) != CC_OK ||
         (st = upload(p, gk1.data(), gk1.size(), &p->corr_twk1)) != CC_OK ||
         (st = upload(p, gl.data(), gl.size(), &p->corr_twL)) != CC_OK ||
