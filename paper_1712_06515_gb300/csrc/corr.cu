@@ -212,7 +212,7 @@ struct CorrLayout {
     int64_t G, t_pad;
     CorrArgs a;
     // workspace pieces of a batch, bytes
-    size_t ab, z, norm, act, D, raw, rows2, U, h, kn, total;
+    size_t ab, z, norm, act, D, raw, scratch, rows2, U, h, kn, total;
 };
 
 std::vector<float2> corr_powers(int64_t L, int64_t C) {
@@ -303,7 +303,8 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
         int64_t best = -1;
         for (int64_t n = minch; n <= most; n += 1 + n / 16) {
             const int64_t len = (p.M + n - 1) / n, waves = (per_chunk * ((p.M + len - 1) / len) + slots - 1) / slots;
-            const int64_t cost = waves * (len + p.R + 1);
+            // more rows than a block of corr_rows_kernel takes cost that launch, about three segments' time
+            const int64_t cost = waves * (len + p.R + 1) + (2 * n > ROW_BLOCK ? 3 : 0);
             if (best < 0 || cost < best) {
                 best = cost;
                 nch = n;
@@ -321,11 +322,14 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     y->act = al256((size_t)plan->Q * plan->M * y->t_pad);
     y->D = al256(b * sizeof(double));
     y->raw = al256(b * y->n_rows * y->planes * y->G * sizeof(float));
+    // compensated sums: only units of more than one plain run touch them
+    const int64_t ctas = std::min<int64_t>(slots, per_chunk * a.n_chunks);
+    y->scratch = a.chunk_len > CORR_FLUSH ? al256((size_t)ctas * (y->planes > 1 ? 96 : 32) * CORR_THREADS * sizeof(float)) : 0;
     y->rows2 = al256(b * y->n_blocks * y->planes * y->G * sizeof(float));
     y->U = al256(b * (y->planes > 1 ? 2 : 1) * y->G * sizeof(float2));
     y->h = y->C > 2 ? al256(b * y->n_lags * sizeof(float2)) : 0;
     y->kn = al256(b * plan->Q * knot_rows(plan) * sizeof(KnotRec));
-    y->total = y->ab + y->z + y->norm + y->act + y->D + y->raw + y->rows2 + y->U + y->h + y->kn + 256;
+    y->total = y->ab + y->z + y->norm + y->act + y->D + y->raw + y->scratch + y->rows2 + y->U + y->h + y->kn + 256;
 }
 
 // Templates per batch: as many as the budget of a_r, b_r and folded rows holds.
@@ -477,6 +481,7 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         uint8_t* act = (uint8_t*)take(y.act);
         double* D = (double*)take(y.D);
         float* raw = (float*)take(y.raw);
+        float* scratch = (float*)take(y.scratch);
         float* rows2 = (float*)take(y.rows2);
         float2* U = (float2*)take(y.U);
         float2* h = (float2*)take(y.h);
@@ -496,6 +501,7 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         a.src = y.folded ? z : ab;
         a.act = act;
         a.raw = raw;
+        a.scratch = scratch;
         a.ctr = ctr;
         a.err = p.err;
         a.twk = y.C == 1 ? plan->corr_twk1 : plan->corr_twk;

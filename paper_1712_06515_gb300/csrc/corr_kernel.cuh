@@ -13,7 +13,8 @@
 // detectors, the kernel accumulates over segments, per template and weight,
 //   A(j) = sum_K sum_(X<Y) Re(conj(T_YK) T_XK)   (|S_K|^2 with every ordered pair), real,
 //   B(j) = sum_K conj(S_K) S_(K-1)     (R = 1), complex,
-// each in compensated FP32.
+// each in FP32: at most CORR_FLUSH segments plainly, those sums compensated (a run of that
+// length rounds to a twentieth of what the transforms' own rounding leaves in its terms).
 //
 // A CTA of 256 threads holds 4096 points, 16 per thread: T = 4096 / L transforms of L
 // points, each one (template, weight) series (L = 4096: one).  G = L for N_s <= 2048
@@ -28,11 +29,13 @@
 //   * the rows of the next (detector, segment) arrive by cp.async.bulk (TMA) on an mbarrier
 //     under the current transform's later passes (16-byte rows; otherwise by 8- or 4-byte
 //     cp.async);
-//   * the running sums, their compensations and S_(K-1) -- 128 words per thread -- live in
-//     tensor memory, 32 columns per group of four bins, read and written by
-//     tcgen05.ld/st once per segment: registers hold only the transform (16 points), and
-//     detector 0's spectrum (MULTI, three or four detectors: the
-//     sum of the earlier ones), so two CTAs of 128 registers fit an SM without spills;
+//   * the running sums, S_(K-1) and detector 0's spectrum -- 112 words per thread -- live in
+//     tensor memory, 32 columns per group of four bins, read and written by tcgen05.ld/st once
+//     per segment: registers hold only the transform (16 points), so two CTAs of 128 registers
+//     fit an SM.  MULTI (three or four detectors) keeps the sum of the earlier detectors in
+//     registers; without a lag so are the sums (16 words) and detector 0's spectrum;
+//   * the compensated sums of a unit sit in global memory (L2), a slot per CTA, touched every
+//     CORR_FLUSH segments;
 //   * twiddles as in the staged kernel: the coset factor of sample s = t + 256 r is split
 //     between a factor per r (first pass) and the table of the second and the powers of the
 //     last pass.  The coset's tables (10 KB) are kept in shared memory: read through L1, whose
@@ -133,14 +136,6 @@ __device__ __forceinline__ void twiddle_powers(float2 (&x)[16], const float2 (&w
     }
 }
 
-// Compensated sums of two FP32 values in paired operations (the same rounding as kahan_add
-// on each): y = v - c, t = s + y, c = (t - s) - y.
-__device__ __forceinline__ void kahan2(float2& s, float2& c, float2 v) {
-    const float2 y = csub(v, c), t = cadd(s, y);
-    c = csub(csub(t, s), y);
-    s = t;
-}
-
 // The TA activity bytes (0 or 1) at p, aligned to TA, of which the first `valid` count, as bits.
 template <int TA>
 __device__ __forceinline__ uint32_t act_bits(const uint8_t* p, int valid) {
@@ -156,8 +151,11 @@ __global__ void __launch_bounds__(CORR_THREADS, CORR_CTAS_PER_SM)
 corr_kernel(const CorrArgs q) {
     using S = CorrShape<LT>;
     constexpr int L = S::L, T = S::T, GT = S::GT, RL = S::RL, NSL = S::NSL, BPT = S::BPT, TA = S::TA, NP = S::NP;
-    constexpr int W = LAG ? 32 : 8;                  // tensor-memory words per group of four bins
-    constexpr uint32_t COLS = LAG ? 256 : 64;        // two warps of a lane quarter, four groups each
+    // tensor-memory words per group of four bins: A [4], B [4] re im, S of the segment before
+    // [4], detector 0's spectrum [4] (F0T)
+    constexpr bool F0T = LAG && !MULTI;
+    constexpr int W = 32, OF = 20;
+    constexpr uint32_t COLS = 8 * W;                 // two warps of a lane quarter, four groups each
     constexpr uint32_t ESZ = BF16 ? 4 : 8;
     constexpr int PLANES = LAG ? 3 : 1;
     constexpr int SH = MULTI ? 8 : 16;               // activity bits of a detector in a segment's word
@@ -187,7 +185,7 @@ corr_kernel(const CorrArgs q) {
     const int C = q.C, M = q.M;
     const size_t act_x = (size_t)M * q.t_pad;        // bytes of one detector's activity
 
-    if (warp == 0) tmem_alloc(&s_tmem, COLS);
+    if (LAG && warp == 0) tmem_alloc(&s_tmem, COLS);
     if (tid == 0) {
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -201,7 +199,7 @@ corr_kernel(const CorrArgs q) {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tm_base = s_tmem;
+    const uint32_t tm_base = LAG ? s_tmem : 0u;
     const uint32_t tm = tm_base + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * (COLS / 2);
     const uint32_t own_bit = T > 1 ? 1u << (g >> 1) : 1u;
     uint32_t phase = 0;
@@ -296,14 +294,63 @@ corr_kernel(const CorrArgs q) {
             }
         };
 
-        {   // zero sums
+        float sA[16];           // !LAG: the sums
+        if constexpr (LAG) {    // zero sums
             float z[W];
 #pragma unroll
             for (int i = 0; i < W; ++i) z[i] = 0.f;
 #pragma unroll
             for (int gi = 0; gi < 4; ++gi) tmem_st(tm + gi * W, z);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) sA[e] = 0.f;
         }
-
+        bool flushed = false;   // the unit's compensated sums hold something
+        int run = 0;            // segments in the plain sums
+        // the plain sums into the compensated ones; the last time the totals go to the row buffer
+        float* const acc = q.scratch + (size_t)blockIdx.x * (LAG ? 96 : 32) * CORR_THREADS + tid;
+        float* const fl = (float*)ex;
+        constexpr int FP = CORR_POINTS + CORR_POINTS / 16;
+        auto put = [&](bool final, int e, int n, int pl, float val) {   // sum n of the thread: element e, plane pl
+            float* const p = acc + (size_t)2 * n * CORR_THREADS;
+            float sum = val, comp = 0.f;
+            if (flushed) {
+                sum = p[0];
+                comp = p[CORR_THREADS];
+                kahan_add(sum, comp, val);
+            }
+            if (final) {
+                const int b = e / RL, m = g * L + (S::PASS2 ? 16 * (i0 + RL * b) + k : j + GT * b) + NSL * (e % RL);
+                fl[pl * FP + m + (m >> 4)] = sum;
+            } else {
+                p[0] = sum;
+                p[CORR_THREADS] = comp;
+            }
+        };
+        auto flush = [&](bool final) {
+            if constexpr (LAG) {
+                tmem_wait_st();
+#pragma unroll 1
+                for (int gi = 0; gi < 4; ++gi) {
+                    float z[W];
+                    tmem_ld(z, tm + gi * W);
+#pragma unroll
+                    for (int n = 0; n < 12; ++n) {
+                        put(final, 4 * gi + (n < 4 ? n : (n - 4) >> 1), gi * 12 + n, n < 4 ? 0 : 1 + ((n - 4) & 1), z[n]);
+                        z[n] = 0.f;
+                    }
+                    if (!final) tmem_st(tm + gi * W, z);
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    put(final, e, e, 0, sA[e]);
+                    sA[e] = 0.f;
+                }
+            }
+            flushed = true;
+            run = 0;
+        };
         if (!(q.wait_test && first_unit)) issue_after(Kl, -1);
         first_unit = false;
         bool prev_zero = true;
@@ -316,22 +363,20 @@ corr_kernel(const CorrArgs q) {
                 continue;
             }
             const bool acc_on = !LAG || K >= Ka;
-            float2 v[16], f0[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) v[e] = make_float2(0.f, 0.f);
-            if constexpr (MULTI) {
+            if (acc_on && ++run > CORR_FLUSH) {
+                flush(false);
+                run = 1;
+            }
+            float2 v[16], f0[16];   // f0 (unless F0T): detector 0's spectrum, MULTI: the earlier ones' sum
+            bool have = false;      // an earlier detector's spectrum is kept
+            if constexpr (!F0T) {
 #pragma unroll
                 for (int e = 0; e < 16; ++e) f0[e] = make_float2(0.f, 0.f);
             }
-            bool have = false;   // MULTI: f0 holds a sum of detectors
 #pragma unroll 1
             for (int X = 0; X < q.Q; ++X) {
                 const uint32_t xbits = (bits >> (X * SH)) & ((1u << SH) - 1u);
                 if (!xbits) continue;
-                if (!MULTI && X == 1) {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) f0[e] = v[e];   // detector 0's spectrum (zero without weight)
-                }
                 bool ok = true;
                 if (q.tma) {
                     ok = mbar_wait(bar, phase);
@@ -414,104 +459,91 @@ corr_kernel(const CorrArgs q) {
                     for (int r = 0; r < RL; ++r) v[i * RL + r] = x[r];
                 }
                 if constexpr (MULTI) {
-                    // pairs of this detector with the earlier ones: A += Re(conj(F) sum), sum += F
+                    // this detector's pairs with the earlier ones, then their sum
                     if (have && acc_on && !q.all_ordered) {
-                        tmem_wait_st();
+                        if constexpr (LAG) {
+                            tmem_wait_st();
 #pragma unroll
-                        for (int gi = 0; gi < 4; ++gi) {
-                            float z[8];
-                            tmem_ld(z, tm + gi * W);
+                            for (int gi = 0; gi < 4; ++gi) {
+                                float z[8];
+                                tmem_ld(z, tm + gi * W);
 #pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const int e = 4 * gi + 2 * h;
-                                float2 s = make_float2(z[2 * h], z[2 * h + 1]), cp = make_float2(z[4 + 2 * h], z[5 + 2 * h]);
-                                kahan2(s, cp, make_float2(redot(v[e], f0[e]), redot(v[e + 1], f0[e + 1])));
-                                z[2 * h] = s.x;
-                                z[2 * h + 1] = s.y;
-                                z[4 + 2 * h] = cp.x;
-                                z[5 + 2 * h] = cp.y;
+                                for (int i = 0; i < 4; ++i)
+                                    z[i] = fmaf(v[4 * gi + i].x, f0[4 * gi + i].x, fmaf(v[4 * gi + i].y, f0[4 * gi + i].y, z[i]));
+                                tmem_st(tm + gi * W, z);
                             }
-                            tmem_st(tm + gi * W, z);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) sA[e] = fmaf(v[e].x, f0[e].x, fmaf(v[e].y, f0[e].y, sA[e]));
                         }
                     }
                     have = true;
 #pragma unroll
                     for (int e = 0; e < 16; ++e) f0[e] = cadd(f0[e], v[e]);
+                } else if (X + 1 < q.Q && (bits >> SH) != 0) {   // the second detector pairs with this one
+                    if constexpr (F0T) {
+#pragma unroll
+                        for (int gi = 0; gi < 4; ++gi) {
+                            float z[8];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                z[2 * i] = v[4 * gi + i].x;
+                                z[2 * i + 1] = v[4 * gi + i].y;
+                            }
+                            tmem_st(tm + gi * W + OF, z);
+                        }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) f0[e] = v[e];
+                    }
+                    have = true;
                 }
             }
             if (failed) break;
-            if (!MULTI && !(bits >> SH)) {   // the second detector has no weight, or there is none
+            // pair terms of segment K
+            if constexpr (LAG) {
+                tmem_wait_st();
+#pragma unroll
+                for (int gi = 0; gi < 4; ++gi) {
+                    float z[W];
+                    tmem_ld(z, tm + gi * W);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int e = 4 * gi + i;
+                        float2 Sk = MULTI ? f0[e] : v[e];
+                        if (!MULTI && have) {
+                            const float2 f = F0T ? make_float2(z[OF + 2 * i], z[OF + 2 * i + 1]) : f0[e];
+                            Sk = cadd(f, v[e]);
+                            if (acc_on && !q.all_ordered) z[i] = fmaf(v[e].x, f.x, fmaf(v[e].y, f.y, z[i]));
+                        }
+                        if (acc_on && q.all_ordered) z[i] = fmaf(Sk.x, Sk.x, fmaf(Sk.y, Sk.y, z[i]));
+                        float* const B = z + 4 + 2 * i;
+                        float* const P = z + 12 + 2 * i;
+                        if (acc_on && !prev_zero) {
+                            B[0] = fmaf(Sk.x, P[0], fmaf(Sk.y, P[1], B[0]));
+                            B[1] = fmaf(Sk.x, P[1], fmaf(-Sk.y, P[0], B[1]));
+                        }
+                        P[0] = Sk.x;
+                        P[1] = Sk.y;
+                    }
+                    tmem_st(tm + gi * W, z);
+                }
+            } else if (q.all_ordered) {
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
-                    f0[e] = v[e];
-                    v[e] = make_float2(0.f, 0.f);
+                    const float2 Sk = MULTI ? f0[e] : cadd(f0[e], v[e]);
+                    sA[e] = fmaf(Sk.x, Sk.x, fmaf(Sk.y, Sk.y, sA[e]));
                 }
-            }
-            // pair terms of segment K
-            tmem_wait_st();
+            } else if (!MULTI && have) {
 #pragma unroll
-            for (int gi = 0; gi < 4; ++gi) {
-                float z[W];
-                tmem_ld(z, tm + gi * W);   // A[4], its compensation[4]; B[4] re im, compensation, S of segment K - 1
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int e = 4 * gi + 2 * h;
-                    const float2 S0 = MULTI ? f0[e] : cadd(f0[e], v[e]), S1 = MULTI ? f0[e + 1] : cadd(f0[e + 1], v[e + 1]);
-                    if (acc_on && (!MULTI || q.all_ordered)) {
-                        const float2 d = q.all_ordered ? make_float2(redot(S0, S0), redot(S1, S1))
-                                                       : make_float2(redot(v[e], f0[e]), redot(v[e + 1], f0[e + 1]));
-                        float2 s = make_float2(z[2 * h], z[2 * h + 1]), cp = make_float2(z[4 + 2 * h], z[5 + 2 * h]);
-                        kahan2(s, cp, d);
-                        z[2 * h] = s.x;
-                        z[2 * h + 1] = s.y;
-                        z[4 + 2 * h] = cp.x;
-                        z[5 + 2 * h] = cp.y;
-                    }
-                    if constexpr (LAG) {
-#pragma unroll
-                        for (int i = 0; i < 2; ++i) {
-                            float* zb = z + 8 + 6 * (2 * h + i);
-                            const float2 Sk = i == 0 ? S0 : S1;
-                            if (acc_on && !prev_zero) {
-                                const float2 d = make_float2(fmaf(Sk.x, zb[4], Sk.y * zb[5]), fmaf(Sk.x, zb[5], -Sk.y * zb[4]));
-                                float2 s = make_float2(zb[0], zb[1]), cp = make_float2(zb[2], zb[3]);
-                                kahan2(s, cp, d);
-                                zb[0] = s.x;
-                                zb[1] = s.y;
-                                zb[2] = cp.x;
-                                zb[3] = cp.y;
-                            }
-                            zb[4] = Sk.x;
-                            zb[5] = Sk.y;
-                        }
-                    }
-                }
-                tmem_st(tm + gi * W, z);
+                for (int e = 0; e < 16; ++e) sA[e] = fmaf(v[e].x, f0[e].x, fmaf(v[e].y, f0[e].y, sA[e]));
             }
             prev_zero = false;
         }
         if (failed) break;
         // the unit's sums to its row, through the exchange buffers (padded) for whole lines
-        tmem_wait_st();
         __syncthreads();   // every thread has left the last transform's buffers
-        float* fl = (float*)ex;
-        constexpr int FP = CORR_POINTS + CORR_POINTS / 16;
-#pragma unroll
-        for (int gi = 0; gi < 4; ++gi) {
-            float z[W];
-            tmem_ld(z, tm + gi * W);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int e = 4 * gi + i, b = e / RL;
-                const int m = g * L + (S::PASS2 ? 16 * (i0 + RL * b) + k : j + GT * b) + NSL * (e % RL);
-                const int o = m + (m >> 4);
-                fl[o] = z[i];
-                if constexpr (LAG) {
-                    fl[FP + o] = z[8 + 6 * i];
-                    fl[2 * FP + o] = z[8 + 6 * i + 1];
-                }
-            }
-        }
+        flush(true);
         __syncthreads();
 #pragma unroll
         for (int pl = 0; pl < PLANES; ++pl)
@@ -528,7 +560,7 @@ corr_kernel(const CorrArgs q) {
         mbar_wait(bar, phase ^ 1);   // the copy still in flight, bounded
     }
     __syncthreads();
-    if (warp == 0) tmem_free(tm_base, COLS);
+    if (LAG && warp == 0) tmem_free(tm_base, COLS);
 }
 
 template <int LT, bool BF16, bool LAG, bool HALF, bool MULTI>
