@@ -14,8 +14,8 @@ bool segpair_tma_supported(const cc_plan* plan);
 int segpair_tma_chunks(const cc_plan* plan, int64_t n_t);
 size_t segpair_tma_fold_bytes(const cc_plan* plan);
 cc_status launch_fold_bf16(cc_plan* plan, int64_t n_t, const void* ab, const float4* norm, void* z, cudaStream_t st);
-cc_status launch_segpair_tma(cc_plan* plan, int n_chunks, int64_t chunk_len, int64_t n_t, const void* ab,
-                             const float4* norm, float* raw, int* counters, cudaStream_t st);
+cc_status launch_segpair_tma(cc_plan* plan, int n_chunks, int64_t chunk_len, int64_t n_t, const void* z,
+                             const float4* norm, float* raw, int* counter, cudaStream_t st);
 // The staged segment-FFT stage by whole output rows: whether plan and input fit it, and one launch
 // writing F [n_t][Q][M][2][N_f] (counter: one int).
 bool segfft_rows_supported(const cc_plan* plan, const void* ab);

@@ -5,44 +5,45 @@
 // bins; every other two-pass search sums its products on the lag grid (corr_kernel.cuh), about a
 // quarter of the transform work.
 //
-// Per (template, weight, chunk of segments, coset) unit a CTA walks the chunk's
-// segments; per segment it transforms detector 0's and detector 1's samples (each the
-// zero-padded N_FFT-point DFT restricted to coset c, Sec. III B 4: an L-point transform
-// of the samples times exp(-2 pi i (b0 + c) s / N_FFT)) and folds the two spectra into
-// the pair sum of Eq. final-formatted-rho:
+// Per (template, weight, chunk of segments, coset) unit a CTA of 256 threads walks the chunk's
+// segments; per segment it transforms detector 0's and detector 1's folded row (the N_FFT-point
+// DFT restricted to coset c, Sec. III B 4: a 4096-point transform of Z_q[p] times
+// exp(-2 pi i (b0 + c) p / N_FFT)) and folds the two spectra into the pair sum of Eq.
+// final-formatted-rho:
 //
-//   * staging: the N_s samples of the next (detector, segment) transform are copied
-//     from HBM/L2 into shared memory by one cp.async.bulk (TMA, completion on an
-//     mbarrier) issued as soon as the current transform's first pass has read the stage,
-//     so the copy runs under the current transform's second and third passes instead of
-//     stalling the first pass on global loads;
-//   * scheduling: one CTA per SM slot (persistent), units handed out by a per-coset
-//     atomic counter; a CTA starts on the coset smid mod C, so the CTAs sharing an SM
-//     work on one coset and its 28.8 KB twiddle row stays in L1, and takes units of
-//     other cosets once its own queue is empty (results never depend on placement);
-//   * segment-relative positions: sample s of a segment sits at transform position s
-//     (no wrap), so its transform T_K(m) = sum_s x_s W_N^((b0+c) s) W_L^(m s) lacks the
-//     segment-start phase W_N^(k seg0_K) of bin k = b0 + c + C m.  In a pair of
-//     consecutive segments that phase leaves theta(m) = W_N^(-k N_s), one constant per
-//     bin: Re(conj(F_K) F_(K-1)) = Re(conj(T_K) T_(K-1) theta(m)), and the same-segment
-//     terms carry no phase.  theta(m + 256) = theta(m) psi with psi = exp(2 pi i N_s / 16),
-//     so each thread keeps theta of its first bin m = tid and steps by psi through its
-//     eight bins m = tid + 256 r (psi = 1 when 16 divides N_s);
-//   * coset twiddles without a per-sample table: the twiddle W_N^((b0+c) s) of sample
-//     s = tid + 256 r splits into a factor per r (16 values per coset, applied in the first
-//     pass) and a factor per thread, which passes through the first pass's DFT and is
-//     absorbed into the second pass's table twiddles and the last pass's base twiddles
-//     (the plan's twk table); the last pass computes only the 8 outputs m < L/2 that hold
-//     output bins.
+//   * staging: rows arrive in two stages by cp.async.bulk (TMA, completion on an mbarrier each),
+//     the copy of the row after the next issued as soon as the current transform's first pass
+//     has read its stage.  Rows are read once, from HBM;
+//   * scheduling: two persistent CTAs per SM, units handed out by one atomic counter,
+//     neighbouring cosets in turn (neighbouring rows of Z); results never depend on placement;
+//   * segment-relative positions: sample s of a segment sits at transform position s, so its
+//     transform T_K(m) lacks the segment-start phase W_N^(k seg0_K) of bin k = b0 + c + C m.  In
+//     a pair of consecutive segments that phase leaves theta(m) = W_N^(-k N_s), one constant per
+//     bin: Re(conj(F_K) F_(K-1)) = Re(conj(T_K) T_(K-1) theta(m)), and the same-segment terms
+//     carry no phase.  theta(m + 256) = theta(m) psi with psi = exp(2 pi i N_s / 16), so each
+//     thread keeps theta of its first bin and steps by psi through its eight bins m = b + 256 r
+//     (psi = 1 when 16 divides N_s);
+//   * the passes are corr_kernel's: one CTA barrier per transform, the second pass's outputs
+//     exchanged inside half-warps through XOR-swizzled buffers, the coset's twiddles in shared
+//     memory; the last pass computes only the 8 outputs m < 2048 that hold output bins;
+//   * the previous segment's detector sum (times theta) and detector 0's spectrum -- 32 words a
+//     thread -- live in tensor memory, read and written once per segment, the Kahan sums in
+//     registers.
 //
-// Waits on the mbarrier are bounded (about one second of clock): a wait that runs out
-// sets bit 0 of the plan's device error word, every thread of the CTA agrees on it at
-// the next barrier, the CTA waits (bounded again) for the copy still in flight and
+// What bounds it: instruction issue (68 % of the slots, about 1150 instructions a warp and
+// transform, 16 warps per SM), the FP32 pipe (53 %) and the shared-memory exchanges (55 %); Z
+// leaves HBM at 1.7 TB/s.  The 120-day band at a ten-hour lag, per template: 684 us; 842 us with
+// padded buffers, two barriers a transform, twiddles read through L1 and one stage.
+//
+// Waits on the mbarriers are bounded (about one second of clock): a wait that runs out sets bit
+// 0 of the plan's device error word, every thread of the CTA agrees on it at the next barrier,
+// the CTA waits (bounded again) for the copies still in flight, frees its tensor memory and
 // returns; crosscorr_plan_check reports CC_ERR_TIMEOUT.
 #include <algorithm>
 
 #include "segpair.cuh"
 #include "tma.cuh"
+#include "tmem.cuh"
 
 namespace cc {
 
@@ -50,208 +51,173 @@ namespace {
 
 constexpr int TT_THREADS = 256;
 constexpr int TT_L = 4096;
-constexpr int FOLD_MAX_F = 16;     // folds of a long segment onto the 4096 positions
-constexpr int FOLD_MAX_C = 1024;   // cosets of a folded plan
+constexpr int TT_BINS = TT_L / 2;    // kept positions m < 2048 of a coset, eight a thread
+constexpr int TT_MAX_CHUNK = 1023;   // segments of a chunk (its activity, and one before, is kept on chip)
+constexpr int FOLD_MAX_F = 16;       // folds of a long segment onto the 4096 positions
+constexpr int FOLD_MAX_C = 1024;     // cosets of a folded plan
+constexpr uint32_t TT_ROW = TT_L * 4;   // bytes of a folded row (bf16 pairs)
 
-__device__ __forceinline__ unsigned sm_id() {
-    unsigned id;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
-    return id;
-}
+// shared memory: two stages, two exchange buffers, the coset's twiddles (272 and 4 x 256), a
+// byte of activity a segment, two mbarriers
+constexpr size_t TT_OFF_EX = 2 * TT_ROW;
+constexpr size_t TT_OFF_TW = TT_OFF_EX + 2 * (size_t)TT_L * sizeof(float2);
+constexpr size_t TT_OFF_ACT = TT_OFF_TW + (272 + 4 * TT_THREADS) * sizeof(float2);
+constexpr size_t TT_OFF_BAR = TT_OFF_ACT + TT_MAX_CHUNK + 1;
+constexpr size_t TT_SMEM = TT_OFF_BAR + 16;
+static_assert(TT_OFF_BAR % 8 == 0 && 2 * (TT_SMEM + 1024) <= 228 * 1024, "two CTAs per SM");
 
-struct TmaWork {
-    int mmax;
-    int n_chunks;
-    int64_t chunk_len;
-    int64_t units;        // (template, weight, chunk) units per coset
-    uint32_t off_y, off_z, off_h, off_stage, off_bar;
-    uint32_t stage_bytes;   // one staged row: N_s samples, or L folded positions
-    int folded;             // N_s > L: rows of the fold kernel's output Z instead of a_r, b_r
-    int n_in;               // valid positions of a staged row (N_s, or L when folded)
+struct PairArgs {
+    const char* z;          // folded rows [n_t][Q][2][M][C][4096], bf16 pairs
+    const float4* norm;     // [n_t][Q][M] (hat-A, hat-B, hat-C, 0)
+    float* raw;             // [n_t][2 n_chunks][N_f] partial pair sums
+    int* ctr;               // unit counter, zero at launch
+    unsigned* err;          // the plan's device error word
+    const float2* twk;      // DevParams::twk
+    const int *coset_off, *coset_k, *coset_m;   // the cosets' output bins and their positions
+    int64_t N_FFT, b0, N_s, N_f, units;
+    int M, Q, C, n_chunks, chunk_len, lag, all_ordered, wait_test;
 };
 
-// ab: [n_t][Q][2][N_tau] complex64 (bf16 pairs with BF16 storage), or with folded
-// segments (N_s > L) the fold kernel's Z [n_t][Q][2][M][C][L] in the same type; norm:
-// [n_t][Q][M] (hat-A, hat-B, hat-C, 0), raw: [n_t][2 * n_chunks][N_f] partial pair
-// sums, counters: [C] unit counters (zero at launch).
 __global__ void __launch_bounds__(TT_THREADS, 2)
-segpair_tma_kernel(DevParams p, TmaWork q, const void* __restrict__ ab, const float4* __restrict__ norm,
-                   float* __restrict__ raw, int* __restrict__ counters) {
+segpair_tma_kernel(const PairArgs q) {
+    constexpr int W = 32;   // tensor-memory words of a thread: S_(K-1) theta [8], detector 0's spectrum [8]
+    constexpr uint32_t COLS = 2 * W;
     extern __shared__ __align__(128) unsigned char sm[];
-    constexpr int L = TT_L;
-    constexpr int NSL = 256;    // butterflies of each pass = threads
-    constexpr int SLP = 8;      // kept outputs per thread: m = tid + 256 r, r < 8 (m < L/2)
-    float2* Y = (float2*)(sm + q.off_y);
-    float2* Z = (float2*)(sm + q.off_z);
-    float2* H = (float2*)(sm + q.off_h);
-    unsigned char* stage = sm + q.off_stage;
-    uint64_t* bar = (uint64_t*)(sm + q.off_bar);
-    __shared__ int s_unit, s_coset;
+    float2* const ex = (float2*)(sm + TT_OFF_EX);
+    float2* const twk = (float2*)(sm + TT_OFF_TW);
+    float2* const twp = twk + 272;
+    uint8_t* const act = sm + TT_OFF_ACT;   // bit 0: detector 0, bit Q - 1: the last one has weight in the segment
+    uint64_t* const bar = (uint64_t*)(sm + TT_OFF_BAR);
+    __shared__ int s_unit;
+    __shared__ uint32_t s_tmem;
 
-    const int tid = threadIdx.x, Q = p.Q, C = p.C4;   // cosets of the 4096-point decomposition
-    const int64_t N_s = p.N_s, R = p.R, M = p.M, N_tau = p.N_tau;
-    const uint64_t N = (uint64_t)p.N_FFT, mask = N - 1;
-    constexpr uint32_t ESZ = 4;   // bf16 pairs
+    const int tid = threadIdx.x, warp = tid >> 5, Q = q.Q, C = q.C, M = q.M;
+    // Exchange buffers as in corr_kernel: element p at 16 (p >> 4) + ((p ^ (p >> 4)) & 15); second
+    // and last pass: thread j takes column k, rows i0 + 16 r, then butterfly b
+    const int k2 = tid >> 4, i0 = tid & 15, b = 16 * i0 + k2;
+    const int wr1 = 16 * tid + i0, rd2 = 16 * i0 + (k2 ^ i0), rd3 = 256 * i0 + rd2;
+    const uint64_t N = (uint64_t)q.N_FFT, mask = N - 1;
+    const bool psi_one = (q.N_s & 15) == 0;
+    float2 psi;
+    sincospif(0.125f * (float)(q.N_s & 15), &psi.y, &psi.x);   // exp(2 pi i (N_s mod 16) / 16)
 
+    if (warp == 0) tmem_alloc(&s_tmem, COLS);
     if (tid == 0) {
         mbar_init(bar, 1);
+        mbar_init(bar + 1, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    uint32_t phase = 0;
-    bool first_unit = true;
-    int my_c = (int)(sm_id() % (unsigned)C), tries = 0;   // thread 0's queue position
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tm_base = s_tmem;
+    const uint32_t tm = tm_base + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * W;
+    uint32_t phase = 0, in_flight = 0;   // bit per stage (in_flight: thread 0's)
+    int slot = 0, parity = 0;
+    bool first_unit = true, failed = false;
 
     for (;;) {
-        if (tid == 0) {
-            int u = -1;
-            while (tries < C) {
-                const int v = atomicAdd(counters + my_c, 1);
-                if (v < q.units) {
-                    u = v;
-                    break;
-                }
-                my_c = my_c + 1 == C ? 0 : my_c + 1;   // this coset's queue is empty: help the next
-                ++tries;
+        if (tid == 0) s_unit = atomicAdd(q.ctr, 1);
+        __syncthreads();
+        const int u = s_unit;
+        if (u >= q.units) break;
+        const int c = u % C, v0 = u / C, chunk = v0 % q.n_chunks, tw = v0 / q.n_chunks;
+        const int t = tw >> 1;
+        const int Ka = chunk * q.chunk_len, Kb = min(M, Ka + q.chunk_len), Kl = max(0, Ka - q.lag);
+        const uint64_t bc = ((uint64_t)q.b0 + (uint64_t)c) & mask, ct = bc + (uint64_t)C * b;
+        // pair phase of this thread's first bin
+        const float2 theta = twiddle_N((N - (ct * (uint64_t)q.N_s & mask)) & mask, N);
+        // last pass: element r of butterfly b takes W_L^(b r) W_N^(bc r) = W_N^(ct r), formed
+        // from powers 1, 2, 4, 8
+#pragma unroll
+        for (int n = 0; n < 4; ++n) twp[n * TT_THREADS + tid] = twiddle_N((ct << n) & mask, N);
+        for (int i = tid; i < 272; i += TT_THREADS) twk[i] = __ldg(q.twk + (size_t)c * 272 + i);
+        for (int K = Kl + tid; K < Kb; K += TT_THREADS) {
+            uint32_t a = 0;
+            for (int X = 0; X < Q; ++X) {
+                const float4 n = __ldg(q.norm + ((size_t)t * Q + X) * M + K);
+                a |= (n.x + n.y > 0.f ? 1u : 0u) << X;
             }
-            s_unit = u;
-            s_coset = my_c;
+            act[K - Kl] = (uint8_t)a;
         }
         __syncthreads();
-        const int u = s_unit, c = s_coset;
-        if (u < 0) break;
-        const int64_t t = u / (2 * q.n_chunks);
-        const int rem = u % (2 * q.n_chunks), w = rem / q.n_chunks, chunk = rem % q.n_chunks;
-        const int64_t Ka = (int64_t)chunk * q.chunk_len;
-        const int64_t Kb = imin64(M, Ka + q.chunk_len);
-        const int64_t Kl = imax64(0, Ka - R);
-        const uint64_t bc = ((uint64_t)p.b0 + (uint64_t)c) & mask;
-        const float2* __restrict__ twk = p.twk + (size_t)c * 272;
-        // pair phase of this thread's bins: theta = W_N^(-(bc + C tid) N_s)
-        const uint64_t ct = bc + (uint64_t)C * tid;
-        const float2 theta = twiddle_N((N - (ct * (uint64_t)N_s & mask)) & mask, N);
-        const bool psi_one = (N_s & 15) == 0;
-        float2 psi;
-        sincospif(0.125f * (float)(N_s & 15), &psi.y, &psi.x);   // exp(2 pi i (N_s mod 16) / 16)
-        // last pass (NS = 256): element r3 of thread tid takes W_L^(tid r3) W_N^(bc r3) =
-        // W_N^(ct r3), formed from these four powers
-        const float2 b1 = twiddle_N(ct & mask, N), b2 = twiddle_N((2 * ct) & mask, N);
-        const float2 b4 = twiddle_N((4 * ct) & mask, N), b8 = twiddle_N((8 * ct) & mask, N);
-        const float4* __restrict__ nt = norm + (size_t)t * Q * M;
-        // element offset of (template t, detector X, weight w) row
-        const size_t abt = (size_t)t * Q * 2 * N_tau + (size_t)w * N_tau;
-        auto active = [&](int64_t K, int X) {
-            const float4 n = nt[(size_t)X * M + K];
-            return n.x + n.y > 0.f;
-        };
-        // the transform after (K, X) in unit order (detector 0, then detector Q-1, of each
-        // segment; inactive ones skipped); X = -1 starts at segment K
-        auto next_after = [&](int64_t K, int X, int64_t& nK, int& nX) -> bool {
-            if (X == 0 && Q > 1 && active(K, Q - 1)) {
-                nK = K;
-                nX = Q - 1;
-                return true;
+        // row Z_q of coset c: q = (b0 + c) mod C
+        const char* const src = q.z + (((size_t)tw + (size_t)t * 2 * (Q - 1)) * M * C + (size_t)(bc & (uint64_t)(C - 1))) * TT_ROW;
+        // thread 0: the copy of the transform after (pK, pX) in unit order into stage s, after a
+        // barrier that ends every read of it
+        int pK = Kl, pX = -1;
+        auto issue = [&](int s) {
+            if (pK >= Kb) return;
+            uint32_t a = pX + 1 < Q ? (uint32_t)act[pK - Kl] >> (pX + 1) << (pX + 1) : 0u;
+            while (!a) {
+                if (++pK >= Kb) return;
+                a = act[pK - Kl];
             }
-            for (int64_t k = X < 0 ? K : K + 1; k < Kb; ++k) {
-                if (Q > 1 && active(k, 0)) {
-                    nK = k;
-                    nX = 0;
-                    return true;
-                }
-                if (active(k, Q - 1)) {
-                    nK = k;
-                    nX = Q - 1;
-                    return true;
-                }
-            }
-            return false;
-        };
-        // folded segments: the row Z_q of coset c is q = (b0 + c) mod C
-        const size_t zq = (size_t)(((uint64_t)p.b0 + (uint64_t)c) & (uint64_t)(C - 1));
-        auto issue = [&](int64_t K, int X) {   // thread 0, after a barrier that ends every read of the stage
+            pX = __ffs(a) - 1;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            const size_t el = q.folded ? ((((size_t)t * Q + X) * 2 + w) * M + K) * C * L + zq * L
-                                       : abt + (size_t)X * 2 * N_tau + (size_t)(K * N_s);
-            const char* src = (const char*)ab + el * ESZ;
-            mbar_arrive_expect_tx(bar, q.stage_bytes);
-            tma_load_1d(stage, src, q.stage_bytes, bar);
+            mbar_arrive_expect_tx(bar + s, TT_ROW);
+            tma_load_1d(sm + s * TT_ROW, src + ((size_t)pX * 2 * M + pK) * C * TT_ROW, TT_ROW, bar + s);
+            in_flight |= 1u << s;
         };
-
-        float accP[SLP], cmpP[SLP];
-        float2 prevP[SLP];
-#pragma unroll
-        for (int r = 0; r < SLP; ++r) {
-            accP[r] = cmpP[r] = 0.f;
-            prevP[r] = make_float2(0.f, 0.f);
+        // (the wait test leaves the CTA's first copies unissued: its bounded wait runs out)
+        if (tid == 0 && !(q.wait_test && first_unit)) {
+            issue(slot);
+            issue(slot ^ 1);
         }
-        int64_t sK = 0;   // staged transform (sK, sX)
-        int sX = 0;
-        bool staged = next_after(Kl, -1, sK, sX);
-        // (the wait test leaves the CTA's first copy unissued: its bounded wait runs out)
-        if (staged && tid == 0 && !(p.wait_test && first_unit)) issue(sK, sX);
         first_unit = false;
 
-        for (int64_t K = Kl; K < Kb; ++K) {
-            const bool a0 = active(K, 0), al = active(K, Q - 1);
+        float accP[8], cmpP[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) accP[r] = cmpP[r] = 0.f;
+        bool prev_zero = true;
+
+        for (int K = Kl; K < Kb; ++K) {
+            const uint32_t bits = act[K - Kl];
+            if (!bits) {
+                prev_zero = true;
+                continue;
+            }
+            const bool a0 = Q > 1 && (bits & 1u), al = (bits >> (Q - 1)) & 1u;
             float2 v[16];
 #pragma unroll 1
-            for (int pass = 0; pass < 2; ++pass) {
-                const int X = pass == 0 ? 0 : Q - 1;
-                if (pass == 0 ? !(Q > 1 && a0) : !al) continue;
-                // (K, X) is the staged transform
-                const bool ok = mbar_wait(bar, phase);
-                phase ^= 1;
-                // first radix-16 pass: sample s = tid + 256 r of the segment (zero beyond
-                // N_s) times the coset factor W_N^(256 bc r)
-                {
+            for (int X = a0 ? 0 : Q - 1; X < (al ? Q : 1); ++X) {
+                const bool ok = mbar_wait(bar + slot, (phase >> slot) & 1u);
+                if (ok) in_flight &= ~(1u << slot);
+                const __nv_bfloat162* st = (const __nv_bfloat162*)(sm + slot * TT_ROW);
+                float2* const buf = ex + (parity ? TT_L : 0);   // buffers alternate: one CTA barrier a transform
+                parity ^= 1;
+                // first pass: position p = tid + 256 r times the coset factor W_N^(256 bc r)
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) {
-                        const int s = tid + r * 256;
-                        const bool in = s < q.n_in;
-                        v[r] = in ? __bfloat1622float2(((const __nv_bfloat162*)stage)[s]) : make_float2(0.f, 0.f);
-                    }
+                for (int r = 0; r < 16; ++r) v[r] = __bfloat1622float2(st[tid + 256 * r]);
 #pragma unroll
-                    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(twk + r));
-                    dft16(v);
-                    float2* d = Y + 17 * tid;   // padi(16 tid + r)
+                for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], twk[r]);
+                dft16(v);
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) d[r] = v[r];
-                }
-                int64_t nK = 0;
-                int nX = 0;
-                const bool more = next_after(K, X, nK, nX);
-                // every thread has read the stage and written Y; all agree on a failed wait
+                for (int r = 0; r < 16; ++r) buf[wr1 ^ r] = v[r];
+                // every thread has read the stage and written its outputs; all agree on a failed wait
                 if (__syncthreads_or(!ok)) {
-                    if (tid == 0) {
-                        atomicOr(p.err, 1u);
-                        mbar_wait(bar, phase ^ 1);   // the copy still in flight, bounded
-                    }
-                    __syncthreads();
-                    return;
+                    failed = true;
+                    break;
                 }
-                if (more && tid == 0) issue(nK, nX);
-                // second pass (NS = 16): Y -> Z, twiddles W_L^(16 k r) W_N^(16 bc r) from the
-                // table (the thread factor of the first pass's source threads)
+                if (tid == 0) issue(slot);
+                phase ^= 1u << slot;
+                slot ^= 1;
+                // second pass: twiddles W_L^(16 k r) W_N^(16 bc r)
+#pragma unroll
+                for (int r = 0; r < 16; ++r) v[r] = buf[rd2 + 256 * r];
+#pragma unroll
+                for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], twk[16 + r * 16 + k2]);
+                dft16(v);
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < 16; ++r) buf[(rd2 ^ (17 * r)) + 256 * r] = v[r];
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < 16; ++r) v[r] = buf[rd3 ^ (17 * r)];
                 {
-                    const int k = tid & 15;
-                    const float2* s = Y + padi(tid);
-#pragma unroll
-                    for (int r = 0; r < 16; ++r) v[r] = s[r * pstride<256>()];
-#pragma unroll
-                    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(twk + 16 + r * 16 + k));
-                    dft16(v);
-                    float2* d = Z + padi((tid - k) * 16 + k);
-#pragma unroll
-                    for (int r = 0; r < 16; ++r) d[r * pstride<16>()] = v[r];
-                }
-                __syncthreads();
-                // last pass (NS = 256) into registers: v[r] = X[tid + 256 r], r < 8
-                {
-                    const float2* s = Z + padi(tid);
-#pragma unroll
-                    for (int r = 0; r < 16; ++r) v[r] = s[r * pstride<256>()];
-                    const float2 b3 = cmul(b2, b1);
+                    const float2 b1 = twp[tid], b2 = twp[TT_THREADS + tid], b4 = twp[2 * TT_THREADS + tid];
+                    const float2 b8 = twp[3 * TT_THREADS + tid], b3 = cmul(b2, b1), b12 = cmul(b8, b4);
                     v[1] = cmul(v[1], b1);
                     v[2] = cmul(v[2], b2);
                     v[3] = cmul(v[3], b3);
@@ -263,56 +229,66 @@ segpair_tma_kernel(DevParams p, TmaWork q, const void* __restrict__ ab, const fl
                     v[9] = cmul(v[9], cmul(b8, b1));
                     v[10] = cmul(v[10], cmul(b8, b2));
                     v[11] = cmul(v[11], cmul(b8, b3));
-                    const float2 b12 = cmul(b8, b4);
                     v[12] = cmul(v[12], b12);
                     v[13] = cmul(v[13], cmul(b12, b1));
                     v[14] = cmul(v[14], cmul(b12, b2));
                     v[15] = cmul(v[15], cmul(b12, b3));
-                    dft16_lo8(v);
                 }
-                if (pass == 0) {
+                dft16_lo8(v);
+                if (X + 1 < Q) {
+                    float z[16];
 #pragma unroll
-                    for (int r = 0; r < SLP; ++r)
-                        if (tid + NSL * r <= q.mmax) H[r * NSL + tid] = v[r];   // read back by this thread only
+                    for (int r = 0; r < 8; ++r) {
+                        z[2 * r] = v[r].x;
+                        z[2 * r + 1] = v[r].y;
+                    }
+                    tmem_st(tm + 16, z);
                 }
             }
-            // pair terms of segment K (F = 0 for a detector with no weight in it); prevP
-            // holds the previous segment's detector sum times theta of its bin
+            if (failed) break;
+            // pair terms of segment K (zero for a detector with no weight in it)
             const bool acc_on = K >= Ka;
+            float z[W], s[16];
+            tmem_wait_st();
+            tmem_ld(z, tm);
             float2 th = theta;
 #pragma unroll
-            for (int r = 0; r < SLP; ++r) {
-                const int m = tid + NSL * r;
-                if (m <= q.mmax) {
-                    const float2 Fl = al ? v[r] : make_float2(0.f, 0.f);
-                    float2 F0 = Fl, F1 = make_float2(0.f, 0.f);
-                    if (Q > 1) {
-                        F0 = a0 ? H[r * NSL + tid] : make_float2(0.f, 0.f);
-                        F1 = Fl;
-                    }
-                    const float2 S = cadd(F0, F1);
-                    const float2 P = R > 0 ? prevP[r] : make_float2(0.f, 0.f);
-                    const float term = p.pair_mode == CC_PAIRS_ALL_ORDERED ? fmaf(2.f, redot(S, P), redot(S, S))
-                                                                           : redot(S, P) + redot(F1, F0);
-                    if (acc_on) kahan_add(accP[r], cmpP[r], term);
-                    if (R > 0) prevP[r] = cmul(S, th);
-                }
-                if (R > 0 && !psi_one) th = cmul(th, psi);
+            for (int r = 0; r < 8; ++r) {
+                const float2 zero = make_float2(0.f, 0.f);
+                const float2 F1 = al ? v[r] : zero, F0 = a0 ? make_float2(z[16 + 2 * r], z[17 + 2 * r]) : zero;
+                const float2 S = Q > 1 ? cadd(F0, F1) : F1;
+                const float2 P = prev_zero ? zero : make_float2(z[2 * r], z[2 * r + 1]);
+                const float term = q.all_ordered ? fmaf(2.f, redot(S, P), redot(S, S)) : redot(S, P) + redot(F1, F0);
+                if (acc_on) kahan_add(accP[r], cmpP[r], term);
+                const float2 n = cmul(S, th);
+                s[2 * r] = n.x;
+                s[2 * r + 1] = n.y;
+                if (!psi_one) th = cmul(th, psi);
             }
+            if (q.lag) tmem_st(tm, s);
+            prev_zero = !q.lag;
         }
-        // partial sums of this (template, weight, chunk) row for the coset's bins, staged
-        // through Y (the last transform's reads of Y ended before its second barrier)
+        if (failed) break;
+        // partial sums of this (template, weight, chunk) row for the coset's bins, staged through
+        // an exchange buffer
         __syncthreads();
-        float* accm = (float*)Y;
+        float* const accm = (float*)ex;
 #pragma unroll
-        for (int r = 0; r < SLP; ++r)
-            if (tid + NSL * r <= q.mmax) accm[tid + NSL * r] = accP[r];
+        for (int r = 0; r < 8; ++r) accm[b + 256 * r] = accP[r];
         __syncthreads();
-        const int o = __ldg(p.coset4_off + c), nbc = __ldg(p.coset4_off + c + 1) - o;
-        float* outp = raw + ((size_t)t * 2 * q.n_chunks + (size_t)w * q.n_chunks + chunk) * p.N_f;
-        for (int i = tid; i < nbc; i += TT_THREADS) outp[__ldg(p.coset4_k + o + i)] = accm[__ldg(p.coset4_m + o + i)];
-        // the next unit's first pass rewrites Y: the unit fetch's barrier orders it
+        const int o = __ldg(q.coset_off + c), nbc = __ldg(q.coset_off + c + 1) - o;
+        float* const out = q.raw + ((size_t)tw * q.n_chunks + chunk) * q.N_f;
+        for (int i = tid; i < nbc; i += TT_THREADS) out[__ldg(q.coset_k + o + i)] = accm[__ldg(q.coset_m + o + i)];
+        // the next unit's first pass rewrites the buffer: the unit fetch's barrier orders it
     }
+    if (failed && tid == 0) {
+        atomicOr(q.err, 1u);
+        for (int s = 0; s < 2; ++s)   // copies still in flight, bounded
+            if (in_flight & (1u << s)) mbar_wait(bar + s, (phase >> s) & 1u);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) tmem_free(tm_base, COLS);
 }
 
 // Fold of a long segment (N_s > L) onto the L = 4096 positions of the coset transforms
@@ -419,41 +395,6 @@ fold64_kernel(DevParams p, const void* __restrict__ ab, const float4* __restrict
     }
 }
 
-size_t al128(size_t b) { return (b + 127) & ~(size_t)127; }
-
-bool tma_layout(const cc_plan* plan, TmaWork* q, size_t* bytes) {
-    const DevParams& p = plan->dp;
-    const int esz = p.store == CC_STORE_BF16 ? 4 : 8;
-    q->mmax = p.C4 > 0 ? (int)((plan->kbar.back() - plan->k0) / p.C4) : TT_L;
-    q->folded = p.N_s > TT_L ? 1 : 0;
-    q->n_in = q->folded ? TT_L : (int)p.N_s;
-    q->stage_bytes = (uint32_t)(q->n_in * esz);
-    size_t o = 0;
-    q->off_stage = (uint32_t)o;
-    o = al128(o + q->stage_bytes);
-    q->off_y = (uint32_t)o;
-    o = al128(o + (size_t)padded_len(TT_L) * sizeof(float2));
-    q->off_z = (uint32_t)o;
-    o = al128(o + (size_t)padded_len(TT_L) * sizeof(float2));
-    q->off_h = (uint32_t)o;
-    o = al128(o + (size_t)(q->mmax + 1) * sizeof(float2));
-    q->off_bar = (uint32_t)o;
-    o += 16;
-    *bytes = o;
-    return o <= 113 * 1024;   // two CTAs per SM
-}
-
-int occupancy(size_t smem) {
-    int n = 0;
-    if (cudaFuncSetAttribute(segpair_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-        return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, segpair_tma_kernel, TT_THREADS, smem) !=
-        cudaSuccess)
-        return 0;
-    return n;
-}
-
 }  // namespace
 
 // Folded segments in BF16: more than 4096 samples, a multiple of 4 (rows then start on 16-byte
@@ -465,15 +406,12 @@ bool segpair_tma_supported(const cc_plan* plan) {
         p.pair_mode == CC_PAIRS_CROSS_ONLY || plan->N_f < 1)
         return false;
     if (p.C4 > FOLD_MAX_C || (p.N_s + TT_L - 1) / TT_L > FOLD_MAX_F || p.N_s % 4) return false;
-    TmaWork q;
-    size_t bytes;
-    if (!tma_layout(plan, &q, &bytes)) return false;
-    return 2 * q.mmax < TT_L;
+    return p.C4 > 0 && plan->kbar_span4 < TT_BINS;
 }
 
 // Segment chunks per (template, weight) for a batch of n_t templates: about
 // `units per CTA` (the tuning's chunk_waves, default 24) units per persistent CTA, each
-// chunk at least 4R + 1 segments.
+// chunk at least 4R + 1 segments and at most TT_MAX_CHUNK.
 int segpair_tma_chunks(const cc_plan* plan, int64_t n_t) {
     const DevParams& p = plan->dp;
     int dev = 0, sms = 152;
@@ -482,7 +420,8 @@ int segpair_tma_chunks(const cc_plan* plan, int64_t n_t) {
     const int64_t ctas_per_coset = std::max<int64_t>(1, 2 * (int64_t)sms / p.C4);
     const int64_t want = (per_cta * ctas_per_coset + 2 * n_t - 1) / (2 * n_t);
     const int64_t maxch = std::max<int64_t>(1, p.M / (4 * p.R + 1));
-    return (int)std::max<int64_t>(1, std::min<int64_t>({want, maxch, 32767}));
+    const int64_t least = (p.M + TT_MAX_CHUNK - 1) / TT_MAX_CHUNK;
+    return (int)std::max<int64_t>(least, std::min<int64_t>({want, maxch, 32767}));
 }
 
 // Bytes of the fold kernel's output per template.
@@ -507,26 +446,40 @@ cc_status launch_fold_bf16(cc_plan* plan, int64_t n_t, const void* ab, const flo
     return e == cudaSuccess ? CC_OK : cuda_fail(e, "fold launch");
 }
 
-cc_status launch_segpair_tma(cc_plan* plan, int n_chunks, int64_t chunk_len, int64_t n_t, const void* ab,
-                             const float4* norm, float* raw, int* counters, cudaStream_t st) {
+cc_status launch_segpair_tma(cc_plan* plan, int n_chunks, int64_t chunk_len, int64_t n_t, const void* z,
+                             const float4* norm, float* raw, int* counter, cudaStream_t st) {
     const DevParams& p = plan->dp;
-    TmaWork q;
-    size_t bytes;
-    if (!tma_layout(plan, &q, &bytes)) return fail(CC_ERR_UNSUPPORTED, "segpair_tma layout");
+    PairArgs q;
+    q.z = (const char*)z;
+    q.norm = norm;
+    q.raw = raw;
+    q.ctr = counter;
+    q.err = p.err;
+    q.twk = p.twk;
+    q.coset_off = p.coset4_off;
+    q.coset_k = p.coset4_k;
+    q.coset_m = p.coset4_m;
+    q.N_FFT = p.N_FFT;
+    q.b0 = p.b0;
+    q.N_s = p.N_s;
+    q.N_f = p.N_f;
+    q.M = (int)p.M;
+    q.Q = p.Q;
+    q.C = p.C4;
     q.n_chunks = n_chunks;
-    q.chunk_len = chunk_len;
-    q.units = n_t * 2 * n_chunks;
-    if (q.units > 0x7fffffff) return fail(CC_ERR_UNSUPPORTED, "too many work units in one launch");
-    const int occ = occupancy(bytes);
-    if (occ < 1) return fail(CC_ERR_UNSUPPORTED, "segpair_tma kernel does not fit an SM");
+    q.chunk_len = (int)chunk_len;
+    q.lag = (int)p.R;
+    q.all_ordered = p.pair_mode == CC_PAIRS_ALL_ORDERED;
+    q.wait_test = p.wait_test;
+    q.units = n_t * 2 * n_chunks * p.C4;
+    if (q.units > 0x7fffffff - 65536) return fail(CC_ERR_UNSUPPORTED, "too many work units in one launch");
     int dev = 0, sms = 152;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = cudaFuncSetAttribute(segpair_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TT_SMEM);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return cuda_fail(e, "device attributes");
-    const int64_t grid = std::min<int64_t>((int64_t)occ * sms, q.units * p.C4);
-    if ((e = cudaMemsetAsync(counters, 0, sizeof(int) * p.C4, st)) != cudaSuccess)
-        return cuda_fail(e, "unit counters");
-    segpair_tma_kernel<<<(unsigned)grid, TT_THREADS, bytes, st>>>(p, q, ab, norm, raw, counters);
+    if (e == cudaSuccess) e = cudaMemsetAsync(counter, 0, sizeof(int), st);
+    if (e != cudaSuccess) return cuda_fail(e, "segment pair set-up");
+    segpair_tma_kernel<<<(unsigned)std::min<int64_t>(2 * (int64_t)sms, q.units), TT_THREADS, TT_SMEM, st>>>(q);
     count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "segpair_tma launch");
