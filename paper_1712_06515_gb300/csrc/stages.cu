@@ -454,12 +454,12 @@ cc_status launch_resample(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
                           float* norm, cudaStream_t st, const KnotRec* kn, int64_t nkn, int write_inactive,
                           uint8_t* act, int t_pad) {
     const DevParams& p = plan->dp;
-    if (kn && p.store == CC_STORE_FP32)
-        return launch_resample_group(plan, n_t, ab, norm, st, kn, nkn, write_inactive, act, t_pad);
-    // with knot records, the segment's window of x is staged in shared memory when it
-    // leaves room for several blocks per SM
+    // with knot records, the segment's window of x is staged in shared memory when it leaves room
+    // for several blocks per SM; longer segments go tile by tile
     const int use_window = kn && resample_smem_bytes(p, true) <= 96 * 1024;
-    const size_t sm = kn ? (use_window ? resample_smem_bytes(p, true) : 0) : resample_smem_bytes(p, false);
+    if (kn && (p.store == CC_STORE_FP32 || !use_window))
+        return launch_resample_group(plan, n_t, ab, norm, st, kn, nkn, write_inactive, act, t_pad);
+    const size_t sm = resample_smem_bytes(p, kn != nullptr);
     // compile-time half width for the common stencils of the exact interpolator
     const int DT = p.interp == CC_INTERP_EXACT && (p.D == 8 || p.D == 16) ? p.D : 0;
     auto kern = kn ? (DT == 8 ? resample_kernel<8, true> : DT == 16 ? resample_kernel<16, true> : resample_kernel<0, true>)

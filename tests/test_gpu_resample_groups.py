@@ -76,3 +76,28 @@ def test_templates_far_apart():
                    [45.0, synth.T_ASC_O1 + 0.5 * synth.SCO_X1_P, synth.SCO_X1_P], [1.44, synth.T_ASC_O1, synth.SCO_X1_P]])
     tol = 2e-5 + 2 * np.pi * 3 * 2.0 ** -24 * 120.0 * 45.0 * (2 * np.pi / synth.SCO_X1_P) * 128
     check(600, 8, 4, templates=tm, T_sft=200, tol=tol)
+
+
+@pytest.mark.parametrize("n_s,m,n_t,D,learned", [(12400, 2, 1, 8, False), (18049, 2, 5, 16, False), (36000, 2, 7, 8, False),
+                                                 (20000, 2, 3, 5, False), (15000, 2, 4, 8, True)])
+def test_long_bf16_segments(n_s, m, n_t, D, learned):
+    """BF16 storage beyond one staged window against FP32 storage, whose samples the tests above
+    compare with the oracle, rounded to BF16 here: the two kernels' FP32 values differ by some
+    1e-6 of max, less than a hundredth of the BF16 step of most samples, so at most 1 % of them
+    may round the other way, and those by one step (2^-7 of the value; 2e-5 of max on either
+    side near zero).  A sample within FP32 rounding of a block's edge may take either block's
+    noise: at most one in 10^4.  The norms to their 2e-5."""
+    ds = synth.tiny(seed=73, n_samples=n_s * m + 5, T_sft=200.0, T_max=float(n_s), T_short=float(n_s), D=D,
+                    f_band=0.5 if learned else 0.1, n_templates=n_t, duty=0.7, mean_lock_s=3000.0)
+    interp = cc.INTERP_LEARNED if learned else cc.INTERP_EXACT
+    got = []
+    for store in (cc.STORE_FP32, cc.STORE_BF16):
+        with cc.CrossCorrPlan(ds.cfg, ds.dets, interp=interp, store=store) as plan:
+            ab, norm = plan.resample(torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV))
+            got.append(((torch.view_as_real(ab) if store == cc.STORE_FP32 else ab).float().cpu().numpy(), norm.cpu().numpy()))
+    (a32, n32), (a16, n16) = got
+    r32 = torch.from_numpy(a32).to(torch.bfloat16).float().numpy()
+    far = np.abs(a16 - r32) > 2.0 ** -7 * np.abs(r32) + 4e-5 * np.abs(r32).max()
+    assert float(far.mean()) <= 1e-4
+    assert float((a16 != r32).mean()) <= 1e-2
+    assert float(np.abs(n16 - n32).max()) <= 4e-5 * float(np.abs(n32).max())
