@@ -130,17 +130,22 @@ topk_pass2(const float* __restrict__ cv, const long long* __restrict__ ci, long 
 
 // ---------------------------------------------------------------------------
 // One pass over rho for the usual case (k well below the number of groups): every warp takes
-// groups of contiguous values and notes each group's maximum; the last block to finish takes
-// the k-th largest of those maxima as a threshold -- at least k values reach it --, rereads the
-// groups that reach it (about k of them), collects their values above it and sorts those.
-// Bound by the one read of rho.  Values are compared by an unsigned key that orders as `better`
-// does (NaN as -inf, -0 as +0); ties end in the sort by index.  When the collection overflows
-// (values bunched into few groups, or many equal ones) the count says so and the caller takes
-// the block-list passes above.
+// groups of contiguous values and notes each group's maximum; the last block to finish takes a
+// threshold that k of those maxima reach, and few more -- so at least k values reach it --,
+// rereads the groups that reach it, collects their values above it and sorts those.  Values
+// are compared by an unsigned key that orders as `better` does (NaN as -inf, -0 as +0); ties end
+// in the sort by index.  When the collection overflows (values bunched into few groups, or many
+// equal ones) the count says so and the caller takes the block-list passes above.
+//
+// What bounds it: the read of rho, then the one block's chain of latencies (24.7 M values,
+// k = 100: about 8 us to reread 119 groups, 3 us for the threshold, 2 us for the ranks).  The
+// whole call, with its copy and synchronisation, 73 us; 2140 us by the block lists alone.
 // ---------------------------------------------------------------------------
 constexpr int SEL_THREADS = 1024;
+constexpr int SEL_BLOCKS = 152;        // one per SM
 constexpr int SEL_GROUPS = 16384;      // maxima
 constexpr int SEL_CAP = 8192;          // collected candidates
+constexpr int SEL_BATCH = 8;           // 16-byte loads a lane has in flight while it rereads
 
 struct SelHead {                       // followed by the hits' indices [k] and values [k]
     unsigned count, err, done, pad;
@@ -152,22 +157,23 @@ __device__ __forceinline__ unsigned sel_key(float v) {
     return u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
 }
 
-// Largest key of values [b, e) over the warp (aligned: b and rho allow 16-byte loads).
+// Largest key of values [b, e) over the warp (aligned: b and rho allow 16-byte loads).  fmaxf
+// passes over NaN, as the key's order does.
 __device__ __forceinline__ unsigned group_max(const float* __restrict__ rho, long long b, long long e, bool aligned) {
     const int lane = threadIdx.x & 31;
-    unsigned m = 0;
+    float m = -INFINITY;
     if (aligned) {
         const float4* p = (const float4*)(rho + b);
         const long long n4 = (e - b) >> 2;
-#pragma unroll 4
+#pragma unroll 8
         for (long long i = lane; i < n4; i += 32) {
             const float4 v = __ldg(p + i);
-            m = max(max(m, max(sel_key(v.x), sel_key(v.y))), max(sel_key(v.z), sel_key(v.w)));
+            m = fmaxf(fmaxf(m, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
         }
         b += n4 << 2;
     }
-    for (long long i = b + lane; i < e; i += 32) m = max(m, sel_key(__ldg(rho + i)));
-    return __reduce_max_sync(0xffffffffu, m);
+    for (long long i = b + lane; i < e; i += 32) m = fmaxf(m, __ldg(rho + i));
+    return __reduce_max_sync(0xffffffffu, sel_key(m));
 }
 
 __global__ void __launch_bounds__(SEL_THREADS)
@@ -176,7 +182,8 @@ topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups,
             const unsigned* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ bool last;
-    __shared__ int cnt[33], ncand;
+    __shared__ int cnt[32], ncand, n_list;
+    __shared__ unsigned range[2];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nw = gridDim.x * (SEL_THREADS / 32);
     for (int g = blockIdx.x * (SEL_THREADS / 32) + warp; g < n_groups; g += nw) {
@@ -190,35 +197,65 @@ topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups,
     __syncthreads();
     if (!last) return;
     __threadfence();
-    // the k-th largest maximum, bit by bit: the largest value that k maxima reach (a histogram of
-    // them would serialise: they share their leading bits)
-    unsigned mine[SEL_GROUPS / SEL_THREADS];
+    // the threshold, bit by bit from above: the largest value so far that k maxima reach, until
+    // not many more than k do (a histogram of them would serialise: they share their leading
+    // bits).  A trial value outside the maxima's range needs no count.
+    unsigned mine[SEL_GROUPS / SEL_THREADS], lo = 0xffffffffu, hi = 0;
 #pragma unroll
     for (int i = 0; i < SEL_GROUPS / SEL_THREADS; ++i) {
         const int g = i * SEL_THREADS + tid;
         mine[i] = g < n_groups ? __ldcg(maxima + g) : 0u;
+        hi = max(hi, mine[i]);
+        if (g < n_groups) lo = min(lo, mine[i]);
     }
-    if (tid < 33) cnt[tid] = 0;
-    if (tid == 0) ncand = 0;
+    if (tid < 32) cnt[tid] = 0;
+    if (tid == 0) {
+        ncand = n_list = 0;
+        range[0] = 0xffffffffu;
+        range[1] = 0;
+    }
     __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+        atomicMin(&range[0], lo);
+        atomicMax(&range[1], hi);
+    }
+    __syncthreads();
+    lo = range[0];
+    hi = range[1];
     unsigned thr = 0;
     for (int bit = 31; bit >= 0; --bit) {
         const unsigned c = thr | (1u << bit);
+        if (c <= lo) thr = c;   // all of them, at least 2 k
+        if (c <= lo || c > hi) continue;
         int n_ge = 0;
 #pragma unroll
         for (int i = 0; i < SEL_GROUPS / SEL_THREADS; ++i) n_ge += mine[i] >= c;
         n_ge = __reduce_add_sync(0xffffffffu, n_ge);
         if (lane == 0 && n_ge) atomicAdd(&cnt[bit], n_ge);
         __syncthreads();
-        if (cnt[bit] >= k) thr = c;
+        const int reach = cnt[bit];
+        if (reach >= k) thr = c;
+        if (reach >= k && reach <= k + k / 8 + 32) break;
     }
     Cand* s = (Cand*)smem;
-    for (int g0 = warp * 32; g0 < n_groups; g0 += SEL_THREADS)
-        for (unsigned hit = __ballot_sync(0xffffffffu, g0 + lane < n_groups && __ldcg(maxima + g0 + lane) >= thr); hit; hit &= hit - 1) {
-        const int g = g0 + __ffs(hit) - 1;
+    unsigned short* list = (unsigned short*)(s + SEL_CAP);   // the groups that reach it
+#pragma unroll
+    for (int i = 0; i < SEL_GROUPS / SEL_THREADS; ++i) {
+        const int g = i * SEL_THREADS + tid;
+        if (g < n_groups && mine[i] >= thr) list[atomicAdd(&n_list, 1)] = (unsigned short)g;
+    }
+    __syncthreads();
+    // the threshold as a value: v >= floor_v where key(v) >= thr, but for one that every key
+    // reaches (-inf, and NaN with it)
+    const bool all = thr <= sel_key(-INFINITY);
+    const float floor_v = __uint_as_float(thr & 0x80000000u ? thr ^ 0x80000000u : ~thr);
+    for (int li = warp; li < n_list; li += SEL_THREADS / 32) {
+        const int g = list[li];
         const long long b = (long long)g * gsize, e = b + gsize < n ? b + gsize : n;
         auto take = [&](float v, long long i) {
-            if (sel_key(v) >= thr) {
+            if (all || v >= floor_v) {
                 const int pos = atomicAdd(&ncand, 1);
                 if (pos < SEL_CAP) {
                     Cand c;
@@ -232,22 +269,40 @@ topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups,
         long long i0 = b;
         if (aligned) {
             const float4* p = (const float4*)(rho + b);
-            const long long n4 = (e - b) >> 2;
-#pragma unroll 4
-            for (long long i = lane; i < n4; i += 32) {
-                const float4 v = __ldg(p + i);
-                take(v.x, b + 4 * i);
-                take(v.y, b + 4 * i + 1);
-                take(v.z, b + 4 * i + 2);
-                take(v.w, b + 4 * i + 3);
+            const int n4 = (int)((e - b) >> 2);
+            for (int i = lane; i < n4; i += 32 * SEL_BATCH) {   // the loads of a batch before its tests
+                float4 v[SEL_BATCH];
+#pragma unroll
+                for (int j = 0; j < SEL_BATCH; ++j)
+                    v[j] = i + 32 * j < n4 ? __ldg(p + i + 32 * j) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+#pragma unroll
+                for (int j = 0; j < SEL_BATCH; ++j) {
+                    if (!(all ? i + 32 * j < n4 : fmaxf(fmaxf(v[j].x, v[j].y), fmaxf(v[j].z, v[j].w)) >= floor_v)) continue;
+                    const long long at = b + 4 * (i + 32 * j);
+                    take(v[j].x, at);
+                    take(v[j].y, at + 1);
+                    take(v[j].z, at + 2);
+                    take(v[j].w, at + 3);
+                }
             }
-            i0 += n4 << 2;
+            i0 += (long long)n4 << 2;
         }
         for (long long i = i0 + lane; i < e; i += 32) take(__ldg(rho + i), i);
     }
     __syncthreads();
     const int m = ncand;
-    if (m <= SEL_CAP) {
+    if (m <= SEL_THREADS / 2) {   // few: each one's rank, counted by `per` neighbouring threads
+        const int per = m <= SEL_THREADS / 8 ? 8 : m <= SEL_THREADS / 4 ? 4 : 2;
+        const int ci = tid / per, part = tid & (per - 1);
+        Cand c = ci < m ? s[ci] : worst_cand();
+        int rank = 0;
+        for (int i = part; i < m; i += per) rank += better(s[i], c);
+        for (int o = 1; o < per; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        if (ci < m && part == 0 && rank < k) {
+            out_i[rank] = c.idx;
+            out_v[rank] = c.v;
+        }
+    } else if (m <= SEL_CAP) {
         int size = 2;
         while (size < m) size <<= 1;
         for (int i = m + tid; i < size; i += SEL_THREADS) s[i] = worst_cand();
@@ -299,21 +354,23 @@ extern "C" cc_status crosscorr_rho_topk(cc_plan* plan, const float* rho_dev, int
         }
     }
     const int nk = (int)std::min<long long>(k, n);
-    // Groups of at least 256 values, at most SEL_GROUPS of them; the threshold needs k groups and
-    // is close to the k-th value while there are several times more.
-    const long long gsize = std::max<long long>(256, ((n + SEL_GROUPS - 1) / SEL_GROUPS + 127) / 128 * 128);
+    // Groups of at least 256 values, at most three for each of the grid's warps (full rounds); the
+    // threshold needs k groups and is close to the k-th value while there are several times more.
+    const long long most = 3 * SEL_BLOCKS * (SEL_THREADS / 32);
+    static_assert(3 * SEL_BLOCKS * (SEL_THREADS / 32) <= SEL_GROUPS, "one maximum per group");
+    const long long gsize = std::max<long long>(256, ((n + most - 1) / most + 127) / 128 * 128);
     const long long n_groups = (n + gsize - 1) / gsize;
     if (n_groups >= 2 * (long long)nk) {
         SelHead* head = (SelHead*)plan->topk_ws;
         long long* oi = (long long*)(head + 1);
         float* ov = (float*)(oi + nk);
         unsigned* maxima = (unsigned*)((char*)(head + 1) + (size_t)TOPK_MAX * 12);
-        const size_t sm = (size_t)SEL_CAP * sizeof(Cand);
+        const size_t sm = (size_t)SEL_CAP * sizeof(Cand) + SEL_GROUPS * sizeof(unsigned short);
         cudaError_t e = cudaFuncSetAttribute(topk_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e == cudaSuccess) e = cudaMemsetAsync(head, 0, sizeof(SelHead), st);
         if (e != cudaSuccess) return cuda_fail(e, "top-k selection set-up");
         const int aligned = ((uintptr_t)rho_dev & 15) == 0;
-        const int blocks = (int)std::min<long long>(152, (n_groups + SEL_THREADS / 32 - 1) / (SEL_THREADS / 32));
+        const int blocks = (int)std::min<long long>(SEL_BLOCKS, (n_groups + SEL_THREADS / 32 - 1) / (SEL_THREADS / 32));
         topk_select<<<blocks, SEL_THREADS, sm, st>>>(rho_dev, n, (int)gsize, (int)n_groups, nk, aligned, maxima, head, oi, ov,
                                                      plan->dp.err);
         count_launch();
