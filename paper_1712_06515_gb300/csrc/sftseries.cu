@@ -207,6 +207,10 @@ __device__ __forceinline__ void cp_async8(float2* dst, const float2* src) {
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
 }
+__device__ __forceinline__ void cp_async16(float2* dst, const float2* src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
@@ -344,7 +348,7 @@ __device__ __forceinline__ void warp_pass(const float2* src, float2* dst, const 
 // What bounds it: HBM (read the locked bands, write the series) and the shared-memory passes.
 __global__ void __launch_bounds__(SS_THREADS)
 sft_fft_warp_kernel(const float2* __restrict__ band, const int64_t* __restrict__ block_sft, int64_t n_blocks,
-                    int n_prime, double T_sft, double f_h, Radices rad, int chunk, float2* __restrict__ x) {
+                    int n_prime, double T_sft, double f_h, Radices rad, int chunk, int wide, float2* __restrict__ x) {
     extern __shared__ __align__(16) float2 sw[];
     __shared__ int64_t s_sft[SS_CHUNK];
     __shared__ float2 s_rot[SS_CHUNK];
@@ -366,7 +370,11 @@ sft_fft_warp_kernel(const float2* __restrict__ band, const int64_t* __restrict__
         sincospif(2.0f * c, &sn, &cs);
         s_rot[i] = make_float2(cs * scale, -sn * scale);
     }
-    for (int e = threadIdx.x; e < n_prime; e += blockDim.x) twf[e] = unit_root(e, n_prime);
+    for (int e = threadIdx.x; e < n_prime; e += blockDim.x) {   // exp(-2 pi i e / N'), the angle within half a turn
+        float sn, cs;
+        sincospif(-2.0f * (float)(2 * e > n_prime ? e - n_prime : e) / (float)n_prime, &sn, &cs);
+        twf[e] = make_float2(cs, sn);
+    }
     __syncthreads();
     auto grab = [&]() -> int {
         int v = 0;
@@ -376,7 +384,10 @@ sft_fft_warp_kernel(const float2* __restrict__ band, const int64_t* __restrict__
     auto fetch = [&](int i) {
         if (i < nb && s_sft[i] >= 0) {
             const float2* zs = band + s_sft[i] * (int64_t)n_prime;
-            for (int m = lane; m < n_prime; m += 32) cp_async8(stage + m, zs + m);
+            if (wide)
+                for (int m = 2 * lane; m < n_prime; m += 64) cp_async16(stage + m, zs + m);
+            else
+                for (int m = lane; m < n_prime; m += 32) cp_async8(stage + m, zs + m);
         }
         cp_async_commit();
     };
@@ -410,7 +421,10 @@ sft_fft_warp_kernel(const float2* __restrict__ band, const int64_t* __restrict__
                 __syncwarp();                          // the buffers' reads are done before the next pass 0
             }
         } else {
-            for (int j = lane; j < n_prime; j += 32) xo[j] = make_float2(0.f, 0.f);
+            if (wide)
+                for (int j = 2 * lane; j < n_prime; j += 64) *(float4*)(xo + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+            else
+                for (int j = lane; j < n_prime; j += 32) xo[j] = make_float2(0.f, 0.f);
             fetch(in);
         }
         i = in;
@@ -601,8 +615,10 @@ extern "C" cc_status crosscorr_sfts_to_series(const void* band_dev, const int64_
         int64_t chunk = std::min<int64_t>(SS_CHUNK, std::max<int64_t>(groups, n_blocks / (4 * slots)));
         if (n_blocks < slots * groups) chunk = std::max<int64_t>(1, std::min<int64_t>(groups, (n_blocks + slots - 1) / slots));
         const int64_t ctas = (n_blocks + chunk - 1) / chunk;
+        // 16-byte copies where every row starts on such a boundary
+        const int wide = n_prime % 2 == 0 && (((uintptr_t)band_dev | (uintptr_t)x_dev) & 15) == 0;
         sft_fft_warp_kernel<<<(unsigned)ctas, 32 * groups, smem, st>>>((const float2*)band_dev, block_sft_dev, n_blocks,
-                                                                       (int)n_prime, T_sft, f_h, rad, (int)chunk,
+                                                                       (int)n_prime, T_sft, f_h, rad, (int)chunk, wide,
                                                                        (float2*)x_dev);
         count_launch();
         e = cudaGetLastError();
