@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(128) demod_sep_kernel(DevParams p, int m_lo, i
 // wavefronts per PT pairs and warp, where one SFT at a time took four per pair and bound the
 // kernel.  Records reach shared memory by cp.async three tiles ahead, the SFT bins registers
 // one tile ahead.
-constexpr int PT = 4;
+constexpr int PT = 4;   // (the ring's loop is written for four)
 
 template <int NT>
 __global__ void __launch_bounds__(NT, 768 / NT) demod_pair_kernel(DevParams p, int m_lo, int nbins, int n_blk, int Rs,
@@ -606,12 +606,13 @@ __global__ void __launch_bounds__(NT, 768 / NT) demod_pair_kernel(DevParams p, i
         asm volatile("cp.async.wait_group 2;" ::: "memory");   // tile n + 1's records
         __syncthreads();
         float2 y[PT];
-        float xi[PT], pr[PT], pq[PT];
+        float xi[PT];
 #pragma unroll
-        for (int q = 0; q < PT; ++q) {
-            y[q] = sft_y(F[q], xi[q]);
-            pr[q] = pq[q] = 0.f;
-        }
+        for (int q = 0; q < PT; ++q) y[q] = sft_y(F[q], xi[q]);
+        // the tile's sums, two SFTs to a paired operation
+        float2 r01 = make_float2(0.f, 0.f), r23 = r01, n01 = r01, n23 = r01;
+        const float2 x01 = make_float2(y[0].x, y[1].x), x23 = make_float2(y[2].x, y[3].x);
+        const float2 y01 = make_float2(y[0].y, y[1].y), y23 = make_float2(y[2].y, y[3].y);
 #pragma unroll
         for (int q = 0; q < PT; ++q) rec_fetch(F[q], rec(i0 + PT + q), df, kh, kl, m_lo, nbins, z);
         const int cnt = i0 - max(s_lo, i0 - have);
@@ -624,14 +625,11 @@ __global__ void __launch_bounds__(NT, 768 / NT) demod_pair_kernel(DevParams p, i
                 const float4 g = sg[s0 + j], h = sq[s0 + j];
                 const float2 yl = cy[j * nthr];
                 const float xl = cx[j * nthr];
-                pr[0] = fmaf(g.x, fmaf(y[0].x, yl.x, y[0].y * yl.y), pr[0]);
-                pr[1] = fmaf(g.y, fmaf(y[1].x, yl.x, y[1].y * yl.y), pr[1]);
-                pr[2] = fmaf(g.z, fmaf(y[2].x, yl.x, y[2].y * yl.y), pr[2]);
-                pr[3] = fmaf(g.w, fmaf(y[3].x, yl.x, y[3].y * yl.y), pr[3]);
-                pq[0] = fmaf(h.x, xl, pq[0]);
-                pq[1] = fmaf(h.y, xl, pq[1]);
-                pq[2] = fmaf(h.z, xl, pq[2]);
-                pq[3] = fmaf(h.w, xl, pq[3]);
+                const float2 lx = make_float2(yl.x, yl.x), ly = make_float2(yl.y, yl.y), l2 = make_float2(xl, xl);
+                r01 = __ffma2_rn(make_float2(g.x, g.y), __ffma2_rn(x01, lx, __fmul2_rn(y01, ly)), r01);
+                r23 = __ffma2_rn(make_float2(g.z, g.w), __ffma2_rn(x23, lx, __fmul2_rn(y23, ly)), r23);
+                n01 = __ffma2_rn(make_float2(h.x, h.y), l2, n01);
+                n23 = __ffma2_rn(make_float2(h.z, h.w), l2, n23);
             }
         };
         const int s = slot0 - cnt;
@@ -642,6 +640,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) demod_pair_kernel(DevParams p, i
             run(s, cnt);
         }
         // pairs inside the tile, then the ring takes its SFTs
+        float pr[PT] = {r01.x, r01.y, r23.x, r23.y}, pq[PT] = {n01.x, n01.y, n23.x, n23.y};
 #pragma unroll
         for (int q = 1; q < PT; ++q)
 #pragma unroll
