@@ -9,7 +9,7 @@
 // L2 transactions of the row's bytes, which took most of the stage's time.  Here two groups of
 // 256 threads take a coset each, C / 2 rounds, the samples staged once per row by a TMA bulk
 // copy; the outputs gather in a row buffer in shared memory, which leaves in whole lines.  The
-// exchanges are corr_kernel's (XOR-swizzled, the last one inside half-warps).  A row of zeros (a
+// exchanges are the pair kernels' (padded buffers, the last one inside half-warps).  A row of zeros (a
 // gapped segment, as the resampling stage writes it) is written without transforms.
 //
 // What bounds it: the FP32 pipe and shared memory of the transforms (about 16 warps per SM, as
@@ -28,6 +28,7 @@ namespace {
 
 constexpr int SR_THREADS = 512;
 constexpr int SR_L = 4096;
+constexpr int SR_EX = 17 * 256 + 16;   // elements of an exchange buffer
 
 struct RowsArgs {
     const void* ab;          // [n_t][Q][2][N_tau]
@@ -59,12 +60,12 @@ segfft_rows_kernel(RowsArgs q) {
     __shared__ int64_t s_next;
     __shared__ int s_nz[2];   // a nonzero sample in the row (two rows in turn)
     const int tid = threadIdx.x, grp = tid >> 8, j = tid & 255;
-    float2* ex = (float2*)(sm + q.off_ex) + grp * SR_L;
+    float2* ex = (float2*)(sm + q.off_ex) + grp * SR_EX;
     const int C = q.C;
     const uint64_t N = (uint64_t)q.N_FFT, mask = N - 1;
     // second and last pass: thread j takes column k, rows i + 16 r (see corr_kernel.cuh)
     const int k2 = j >> 4, i0 = j & 15;
-    const int wr1 = 16 * j + (j & 15), rd2 = 16 * i0 + (k2 ^ i0), rd3 = 256 * i0 + rd2;
+    const int wr1 = 17 * j + k2, rd2 = 17 * i0 + k2, rd3 = 273 * i0 + k2;   // rows at 17 R + (R >> 4), see segpair_tma.cu
     const int b = 16 * i0 + k2;                  // last-pass butterfly: outputs m = b + 256 r
 
     if (tid == 0) {
@@ -124,7 +125,7 @@ segfft_rows_kernel(RowsArgs q) {
                 for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(tw + r));
                 dft16(v);
 #pragma unroll
-                for (int r = 0; r < 16; ++r) ex[wr1 ^ r] = v[r];
+                for (int r = 0; r < 16; ++r) ex[wr1 + r] = v[r];
             }
             if (c0 == 0) {
                 if (__syncthreads_or(!ok)) {
@@ -147,16 +148,16 @@ segfft_rows_kernel(RowsArgs q) {
             if (on) {
                 const float2* __restrict__ tw = q.twk + (size_t)c * 272 + 16;
 #pragma unroll
-                for (int r = 0; r < 16; ++r) v[r] = ex[rd2 + 256 * r];
+                for (int r = 0; r < 16; ++r) v[r] = ex[rd2 + 273 * r];
 #pragma unroll
                 for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(tw + r * 16 + k2));
                 dft16(v);
                 __syncwarp();
 #pragma unroll
-                for (int r = 0; r < 16; ++r) ex[(rd2 ^ (17 * r)) + 256 * r] = v[r];
+                for (int r = 0; r < 16; ++r) ex[rd2 + 273 * r] = v[r];
                 __syncwarp();
 #pragma unroll
-                for (int r = 0; r < 16; ++r) v[r] = ex[rd3 ^ (17 * r)];
+                for (int r = 0; r < 16; ++r) v[r] = ex[rd3 + 17 * r];
                 const uint64_t ct = ((uint64_t)q.b0 + (uint64_t)c + (uint64_t)C * b) & mask;
                 float2 b1, b2, b4, b8;
                 if (q.twp) {
@@ -214,7 +215,7 @@ size_t rows_layout(const cc_plan* plan, RowsArgs* q, bool direct) {
     q->row_bytes = (uint32_t)(p.N_s * esz);
     size_t o = (size_t)SR_L * esz;
     q->off_ex = (uint32_t)o;
-    o += (size_t)2 * SR_L * sizeof(float2);
+    o += (size_t)2 * SR_EX * sizeof(float2);
     q->off_row = (uint32_t)o;
     if (!direct) o = al(o + (size_t)p.N_f * sizeof(float2));
     q->off_bar = (uint32_t)o;

@@ -24,7 +24,7 @@
 //     thread keeps theta of its first bin and steps by psi through its eight bins m = b + 256 r
 //     (psi = 1 when 16 divides N_s);
 //   * the passes are corr_kernel's: one CTA barrier per transform, the second pass's outputs
-//     exchanged inside half-warps through XOR-swizzled buffers, the coset's twiddles in shared
+//     exchanged inside half-warps through padded buffers, the coset's twiddles in shared
 //     memory; the last pass computes only the 8 outputs m < 2048 that hold output bins;
 //   * the previous segment's detector sum (times theta) and detector 0's spectrum -- 32 words a
 //     thread -- live in tensor memory, read and written once per segment, the Kahan sums in
@@ -51,6 +51,7 @@ namespace {
 
 constexpr int TT_THREADS = 256;
 constexpr int TT_L = 4096;
+constexpr int TT_EX = 17 * 256 + 16;  // elements of an exchange buffer
 constexpr int TT_BINS = TT_L / 2;    // kept positions m < 2048 of a coset, eight a thread
 constexpr int TT_MAX_CHUNK = 1023;   // segments of a chunk (its activity, and one before, is kept on chip)
 constexpr int FOLD_MAX_F = 16;       // folds of a long segment onto the 4096 positions
@@ -60,7 +61,7 @@ constexpr uint32_t TT_ROW = TT_L * 4;   // bytes of a folded row (bf16 pairs)
 // shared memory: two stages, two exchange buffers, the coset's twiddles (272 and 4 x 256), a
 // byte of activity a segment, two mbarriers
 constexpr size_t TT_OFF_EX = 2 * TT_ROW;
-constexpr size_t TT_OFF_TW = TT_OFF_EX + 2 * (size_t)TT_L * sizeof(float2);
+constexpr size_t TT_OFF_TW = TT_OFF_EX + 2 * (size_t)TT_EX * sizeof(float2);
 constexpr size_t TT_OFF_ACT = TT_OFF_TW + (272 + 4 * TT_THREADS) * sizeof(float2);
 constexpr size_t TT_OFF_BAR = TT_OFF_ACT + TT_MAX_CHUNK + 1;
 constexpr size_t TT_SMEM = TT_OFF_BAR + 16;
@@ -92,10 +93,11 @@ segpair_tma_kernel(const PairArgs q) {
     __shared__ uint32_t s_tmem;
 
     const int tid = threadIdx.x, warp = tid >> 5, Q = q.Q, C = q.C, M = q.M;
-    // Exchange buffers as in corr_kernel: element p at 16 (p >> 4) + ((p ^ (p >> 4)) & 15); second
-    // and last pass: thread j takes column k, rows i0 + 16 r, then butterfly b
+    // Exchange buffers: row R of 16 elements starts at 17 R + (R >> 4), so that 16 lanes reach 16
+    // different banks down a column, along a row and from block to block, at constant offsets in
+    // r.  Second and last pass: thread j takes column k2, rows i0 + 16 r, then butterfly b
     const int k2 = tid >> 4, i0 = tid & 15, b = 16 * i0 + k2;
-    const int wr1 = 16 * tid + i0, rd2 = 16 * i0 + (k2 ^ i0), rd3 = 256 * i0 + rd2;
+    const int wr1 = 17 * tid + k2, rd2 = 17 * i0 + k2, rd3 = 273 * i0 + k2;
     const uint64_t N = (uint64_t)q.N_FFT, mask = N - 1;
     const bool psi_one = (q.N_s & 15) == 0;
     float2 psi;
@@ -185,7 +187,7 @@ segpair_tma_kernel(const PairArgs q) {
                 const bool ok = mbar_wait(bar + slot, (phase >> slot) & 1u);
                 if (ok) in_flight &= ~(1u << slot);
                 const __nv_bfloat162* st = (const __nv_bfloat162*)(sm + slot * TT_ROW);
-                float2* const buf = ex + (parity ? TT_L : 0);   // buffers alternate: one CTA barrier a transform
+                float2* const buf = ex + (parity ? TT_EX : 0);   // buffers alternate: one CTA barrier a transform
                 parity ^= 1;
                 // first pass: position p = tid + 256 r times the coset factor W_N^(256 bc r)
 #pragma unroll
@@ -194,7 +196,7 @@ segpair_tma_kernel(const PairArgs q) {
                 for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], twk[r]);
                 dft16(v);
 #pragma unroll
-                for (int r = 0; r < 16; ++r) buf[wr1 ^ r] = v[r];
+                for (int r = 0; r < 16; ++r) buf[wr1 + r] = v[r];
                 // every thread has read the stage and written its outputs; all agree on a failed wait
                 if (__syncthreads_or(!ok)) {
                     failed = true;
@@ -205,16 +207,16 @@ segpair_tma_kernel(const PairArgs q) {
                 slot ^= 1;
                 // second pass: twiddles W_L^(16 k r) W_N^(16 bc r)
 #pragma unroll
-                for (int r = 0; r < 16; ++r) v[r] = buf[rd2 + 256 * r];
+                for (int r = 0; r < 16; ++r) v[r] = buf[rd2 + 273 * r];
 #pragma unroll
                 for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], twk[16 + r * 16 + k2]);
                 dft16(v);
                 __syncwarp();
 #pragma unroll
-                for (int r = 0; r < 16; ++r) buf[(rd2 ^ (17 * r)) + 256 * r] = v[r];
+                for (int r = 0; r < 16; ++r) buf[rd2 + 273 * r] = v[r];
                 __syncwarp();
 #pragma unroll
-                for (int r = 0; r < 16; ++r) v[r] = buf[rd3 ^ (17 * r)];
+                for (int r = 0; r < 16; ++r) v[r] = buf[rd3 + 17 * r];
                 {
                     const float2 b1 = twp[tid], b2 = twp[TT_THREADS + tid], b4 = twp[2 * TT_THREADS + tid];
                     const float2 b8 = twp[3 * TT_THREADS + tid], b3 = cmul(b2, b1), b12 = cmul(b8, b4);
