@@ -280,11 +280,11 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     a.tma = a.row_bytes % 16 == 0;   // bulk copies: rows of whole 16-byte pieces start on 16-byte boundaries
     size_t o = al128((size_t)y->T * a.row_stride);
     a.off_y = (uint32_t)o;
-    o = al128(o + (size_t)2 * CORR_POINTS * sizeof(float2));
+    o = al128(o + (size_t)2 * corr_buffer(y->T) * sizeof(float2));
     a.off_tw = (uint32_t)o;
     o += (272 + 1024) * sizeof(float2);
     a.off_act = (uint32_t)o;
-    o += (CORR_MAX_CHUNK + 1) * sizeof(uint32_t);
+    o += (CORR_MAX_CHUNK + 1) * corr_act_bytes(y->T);
     a.off_bar = (uint32_t)o;
     a.smem = (uint32_t)(o + 16);
     // Chunks of segments: units are equal, handed out one by one to two CTAs per SM, each

@@ -12,6 +12,12 @@ constexpr int CORR_MAX_CHUNK = 1023;    // segments of a chunk (its activity wor
 constexpr int CORR_FLUSH = 16;          // segments of a plain FP32 run of the sums
 constexpr int CORR_POINTS = 4096;   // points of one CTA's transforms: 4096 / L of L points each
 
+// T transforms a CTA: elements of an exchange buffer (T = 1: padded), activity bits of a detector
+// in a segment's word (a byte for T = 1) and the word's bytes.
+__host__ __device__ constexpr int corr_buffer(int T) { return T == 1 ? 17 * 256 + 16 : CORR_POINTS; }
+__host__ __device__ constexpr int corr_act_bits(int T, bool multi) { return T == 1 ? 1 : multi ? 8 : 16; }
+__host__ __device__ constexpr int corr_act_bytes(int T) { return T == 1 ? 1 : 4; }
+
 // Everything corr_kernel needs.
 struct CorrArgs {
     const void* src;        // a_r, b_r [n_t][Q][2][N_tau], or folded rows Z [n_t][Q][2][M][C][4096]

@@ -51,6 +51,8 @@
 // tensor memory and returns.
 #pragma once
 
+#include <type_traits>
+
 #include "corr.cuh"
 #include "tma.cuh"
 #include "tmem.cuh"
@@ -122,7 +124,9 @@ corr_kernel(const CorrArgs q) {
     constexpr uint32_t COLS = 8 * W;                 // two warps of a lane quarter, four groups each
     constexpr uint32_t ESZ = BF16 ? 4 : 8;
     constexpr int PLANES = LAG ? 3 : 1;
-    constexpr int SH = MULTI ? 8 : 16;               // activity bits of a detector in a segment's word
+    constexpr int SH = corr_act_bits(T, MULTI);      // activity bits of a detector in a segment's word
+    using AW = std::conditional_t<T == 1, uint8_t, uint32_t>;
+    constexpr bool PAD = T == 1;                     // exchange buffers padded instead of swizzled
     static_assert(TA <= SH, "one activity bit per template of the group");
     extern __shared__ __align__(128) unsigned char sm[];
     unsigned char* stage = sm;
@@ -134,15 +138,16 @@ corr_kernel(const CorrArgs q) {
     const int g = tid / GT, j = tid % GT;
     // Exchange buffers: element p of a transform lies at 16 (p >> 4) + ((p ^ (p >> 4)) & 15), so
     // that 16 lanes reach 16 different banks down a column as well as along a row (8-point last
-    // passes of neighbouring groups also take different halves).  ey: this thread's group.
+    // passes of neighbouring groups also take different halves).  PAD: row R of 16 elements at
+    // 17 R + (R >> 4), conflict-free alike and at constant offsets in r (4 % fewer instructions).
     float2* const ex = (float2*)(sm + q.off_y);
     const int gsw = GT == 8 ? 8 * (g & 1) : 0;
     // second and last pass: thread j takes column k, rows i + RL r (see below)
     const int hw = j >> 4, i0 = S::PASS2 ? (j & 15) % RL : 0, k = S::PASS2 ? hw + RL * ((j & 15) / RL) : 0;
-    const int wr1 = g * L + 16 * j + ((j & 15) ^ gsw);                     // ^ r: pass 1's output r
-    const int rd2 = g * L + 16 * i0 + (k ^ i0);                            // pass 2's row i0, column k
-    const int rd3 = g * L + 16 * RL * i0 + 16 * i0 + (k ^ i0 ^ ((RL * i0) & 15));
-    uint32_t* aw = (uint32_t*)(sm + q.off_act);      // per segment of the chunk: activity bits
+    const int wr1 = PAD ? 17 * j + hw : g * L + 16 * j + ((j & 15) ^ gsw);   // ^ r (PAD: + r): pass 1's output r
+    const int rd2 = PAD ? 17 * i0 + k : g * L + 16 * i0 + (k ^ i0);          // pass 2's row i0, column k
+    const int rd3 = PAD ? 273 * i0 + k : g * L + 16 * RL * i0 + 16 * i0 + (k ^ i0 ^ ((RL * i0) & 15));
+    AW* aw = (AW*)(sm + q.off_act);      // per segment of the chunk: activity bits
     float2* const twk = (float2*)(sm + q.off_tw);    // the coset's first- and second-pass twiddles,
     float2* const twp = twk + 272;                   // and the last pass's powers
     int c_held = -1;
@@ -197,7 +202,7 @@ corr_kernel(const CorrArgs q) {
                 const uint8_t* p = q.act + (size_t)K * q.t_pad + t0;
                 uint32_t b = act_bits<TA>(p, nvalid);
                 for (int X = 1; X < q.Q; ++X) b |= act_bits<TA>(p + X * act_x, nvalid) << (X * SH);
-                aw[K - Kl] = b;
+                aw[K - Kl] = (AW)b;
             }
         }
         __syncthreads();
@@ -361,7 +366,7 @@ corr_kernel(const CorrArgs q) {
                     for (int r = 0; r < 8; ++r) v[r] = make_float2(0.f, 0.f);
                 }
                 // buffers alternate between transforms: one CTA barrier each
-                float2* buf = ex + (parity ? CORR_POINTS : 0);
+                float2* buf = ex + (parity ? corr_buffer(T) : 0);
                 parity ^= 1;
                 if constexpr (HALF) {
                     dft16_in8(v);
@@ -373,7 +378,7 @@ corr_kernel(const CorrArgs q) {
                     dft16(v);
                 }
 #pragma unroll
-                for (int r = 0; r < 16; ++r) buf[wr1 ^ r] = v[r];
+                for (int r = 0; r < 16; ++r) buf[PAD ? wr1 + r : wr1 ^ r] = v[r];
                 // every thread has read the stage and written its outputs; all agree on a failed wait
                 if (__syncthreads_or(!ok)) {
                     failed = true;
@@ -386,7 +391,7 @@ corr_kernel(const CorrArgs q) {
                     // index): the last pass needs the outputs of the RL threads of that column only,
                     // which sit in one half-warp and exchange them in place, without a CTA barrier
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) v[r] = buf[(rd2 ^ ((RL * r) & 15)) + 16 * RL * r];
+                    for (int r = 0; r < 16; ++r) v[r] = buf[PAD ? rd2 + 273 * r : (rd2 ^ ((RL * r) & 15)) + 16 * RL * r];
 #pragma unroll
                     for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], twk[16 + r * 16 + k]);
                     dft16(v);
@@ -394,14 +399,14 @@ corr_kernel(const CorrArgs q) {
 #pragma unroll
                     for (int r = 0; r < 16; ++r) {
                         const int cx = r & (RL - 1);
-                        buf[(rd2 ^ (16 * cx + (cx ^ ((RL * r) & 15)))) + 16 * RL * r] = v[r];
+                        buf[PAD ? rd2 + 273 * r : (rd2 ^ (16 * cx + (cx ^ ((RL * r) & 15)))) + 16 * RL * r] = v[r];
                     }
                     __syncwarp();
 #pragma unroll
                     for (int i = 0; i < BPT; ++i)
 #pragma unroll
                         for (int r = 0; r < RL; ++r)
-                            v[i * RL + r] = buf[(rd3 ^ (17 * r) ^ ((RL * RL * i) & 15)) + 16 * RL * RL * i];
+                            v[i * RL + r] = buf[PAD ? rd3 + 17 * r : (rd3 ^ (17 * r) ^ ((RL * RL * i) & 15)) + 16 * RL * RL * i];
                 } else {
 #pragma unroll
                     for (int i = 0; i < BPT; ++i)
