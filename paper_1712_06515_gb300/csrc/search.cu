@@ -69,7 +69,7 @@ static int resolve_path(const cc_plan* plan) {
 
 // Three and four detectors on the fused path: the lag grid in batches of a few GB, where the
 // cluster kernel transforms every segment at all output frequencies in a 8-CTA cluster per
-// template (48 templates of ten days and three detectors: 43.6 ms there, 1.8 ms here).
+// template (48 templates of ten days and three detectors: 43.6 ms there, 1.9 ms here).
 static bool fused_on_lag_grid(const cc_plan* plan) { return plan->Q > 2 && lag_grid_supported(plan); }
 
 }  // namespace cc
@@ -138,14 +138,17 @@ extern "C" cc_status crosscorr_search(cc_plan* plan, const void* const* x_dev, c
     cc_status s = set_inputs(plan, x_dev);
     if (s != CC_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    const int path = resolve_path(plan);
-    if (path == CC_PATH_TWO_PASS) return search_two_pass(plan, t_dev, n_t, rho_dev, st);
-    if (path == CC_PATH_FUSED && fused_on_lag_grid(plan)) {
+    int path = resolve_path(plan);
+    // bands that only the automatic choice takes to the two-pass kernels
+    const bool wide = path == CC_PATH_TWO_PASS && plan->search_path == CC_PATH_AUTO && !two_pass_supported(plan);
+    if (path == CC_PATH_TWO_PASS && !wide) return search_two_pass(plan, t_dev, n_t, rho_dev, st);
+    if (wide || (path == CC_PATH_FUSED && fused_on_lag_grid(plan))) {
         // a workspace that cannot hold a batch (the caller's, or no memory for the plan's own)
-        // leaves the search to the cluster kernel
+        // leaves the search to the cluster or the stage kernels
         const size_t need = two_pass_workspace_bytes(plan, n_t);
         if (plan->ws_external ? plan->ws_bytes >= need : ensure_workspace(plan, need) == CC_OK)
             return search_two_pass(plan, t_dev, n_t, rho_dev, st);
+        if (wide) path = fused_supported(plan) ? CC_PATH_FUSED : CC_PATH_STAGED;
     }
     FusedLayout lay;
     int64_t kbatch;

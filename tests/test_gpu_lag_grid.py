@@ -97,6 +97,27 @@ def test_wide_band(f_band, store):
         assert np.abs(got[t] - ref[t]).max() <= tol * max(1.0, np.abs(ref[t]).max())
 
 
+@pytest.mark.parametrize("n_det", [2, 3])
+def test_small_workspace(n_det):
+    """A band that only the automatic choice takes to the lag grid, and three detectors, still run
+    in a caller's workspace of the cluster kernel's size, too small for the lag grid's batch."""
+    kw = dict(n_samples=240 * 40, T_sft=240.0, T_max=0.0, T_short=240.0, f_band=1.0, duty=0.8, mean_lock_s=2400.0)
+    ds = synth.tiny(seed=79, n_templates=6, n_det=n_det, **kw)
+    ref = oracle.rho(ds)
+    x, tm = torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV)
+    two = synth.tiny(seed=79, n_templates=6, n_det=2, **kw)   # the cluster kernel's bytes hardly depend on detectors
+    with cc.CrossCorrPlan(two.cfg, two.dets) as plan:
+        plan.set_path(cc.PATH_FUSED)
+        small = 2 * plan.workspace_size(6)
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        assert small < plan.workspace_size(6)
+        plan.set_workspace(torch.empty(small, dtype=torch.uint8, device=DEV))
+        got = plan.search(x, tm).cpu().numpy()
+        plan.check()
+    for t in range(6):
+        assert np.abs(got[t] - ref[t]).max() <= 1e-4 * max(1.0, np.abs(ref[t]).max())
+
+
 @pytest.mark.parametrize("tune", [dict(batch_templates=2), dict(chunk_waves=1), dict(chunk_waves=400), dict(transform_len=4096)])
 def test_splits(tune):
     run(600, 40, 5, {}, **tune)
