@@ -853,7 +853,10 @@ extern "C" cc_status crosscorr_demod_search(cc_plan* plan, const cc_template* t_
     };
     const int bins = sep ? SB : 1;   // output bins of a thread
     while (nthr > 32 && ring_bytes(nthr) > DM_RING_BUDGET) nthr /= 2;
-    if (ring_bytes(nthr) > DM_RING_BUDGET) return fail(CC_ERR_UNSUPPORTED, "T_max / T_sft too large for the pair ring");
+    // the limit counts the ring itself, 32 threads' columns and the weights; the tile's Gamma tables
+    // (28 bytes an entry more) find room beside it
+    if (!sep && (size_t)W * (32 * 12 + 12) > DM_RING_BUDGET)
+        return fail(CC_ERR_UNSUPPORTED, "T_max / T_sft too large for the pair ring");
     // timing records for a batch of templates: the list of locked SFTs plus two padding
     const size_t per_t = sizeof(DemodTiming) * ((size_t)n_list + 2);
     const int64_t batch = std::max<int64_t>(1, std::min<int64_t>({n_t, (int64_t)((size_t)2 << 30) / (int64_t)per_t, 65535}));
