@@ -340,8 +340,11 @@ cc_status launch_resample_group(cc_plan* plan, int64_t n_t, void* ab, float* nor
     // the window of a tile: its samples, the drift of the delay over the segment
     // (|d'| < 2.5e-4 for the Earth and a binary orbit), the taps, and slack for the templates
     // of a group (a wider spread of them takes the samples it misses straight from the tables)
-    const int cap = (int)(std::min<int64_t>(tile, p.N_s) + p.N_s / 512 + 2 * std::max(p.D, 4) + 48);
-    const size_t smem = (size_t)cap * (bf16 ? 8 : 20);
+    // (at most what a block's shared memory holds: segments of millions of samples)
+    const size_t elem = bf16 ? 8 : 20;
+    const int cap = (int)std::min<int64_t>(std::min<int64_t>(tile, p.N_s) + p.N_s / 512 + 2 * std::max(p.D, 4) + 48,
+                                           (int64_t)(220 * 1024 / elem));
+    const size_t smem = (size_t)cap * elem;
     const int64_t step = (int64_t)65535 * tg;
     for (int64_t t0 = 0; t0 < n_t; t0 += step) {
         const int64_t nt = std::min(step, n_t - t0);
