@@ -8,12 +8,15 @@
 // coset wrote 8 bytes into every sector of the row in turn, eight CTAs the row, four times the
 // L2 transactions of the row's bytes, which took most of the stage's time.  Here two groups of
 // 256 threads take a coset each, C / 2 rounds, the samples staged once per row by a TMA bulk
-// copy; the outputs gather in a row buffer in shared memory, which leaves in whole lines.  The
+// copy; the outputs gather in a row buffer in shared memory, which leaves by one bulk copy under
+// the next row's first pass (an odd number of bins: by plain stores).  The
 // exchanges are the pair kernels' (padded buffers, the last one inside half-warps).  A row of zeros (a
 // gapped segment, as the resampling stage writes it) is written without transforms.
 //
-// What bounds it: the FP32 pipe and shared memory of the transforms (about 16 warps per SM, as
-// registers and the 195 KB of buffers allow); 16 x the samples' bytes leave per row.
+// What bounds it: shared memory (65 % of its wavefronts) and issue, with the 16 warps per SM that
+// registers and 200 KB of buffers allow, and the barriers between a row's rounds.  20 days, three
+// templates (N_FFT = 32768, N_f = 12356): 433 us, 470 with plain stores of the row, 660 with a CTA
+// per coset; 510 MB leave.
 //
 // Waits on the mbarrier are bounded (about one second): a wait that runs out sets bit 0 of the
 // plan's error word, the CTA waits (bounded again) for the copy in flight and returns.
@@ -41,8 +44,18 @@ struct RowsArgs {
     int64_t N_FFT, b0, N_tau, M, N_s, N_f;
     int64_t rows;
     int Q, C, wait_test;
+    int bulk;                // rows of F are whole 16-byte pieces: they leave by bulk copies
     uint32_t row_bytes, off_ex, off_row, off_bar;
 };
+
+// A bulk copy shared -> global (16-byte pieces) as a group of its own, and the wait until the
+// thread's copies have read their source.
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_addr(src)), "r"(bytes)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_store_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
 __device__ __forceinline__ void group_sync(int grp) {
     asm volatile("bar.sync %0, 256;" ::"r"(grp + 1) : "memory");
@@ -128,6 +141,7 @@ segfft_rows_kernel(RowsArgs q) {
                 for (int r = 0; r < 16; ++r) ex[wr1 + r] = v[r];
             }
             if (c0 == 0) {
+                if (tid == 0) bulk_store_read();   // the row before has left its buffer
                 if (__syncthreads_or(!ok)) {
                     if (tid == 0) {
                         atomicOr(q.err, 1u);
@@ -198,12 +212,18 @@ segfft_rows_kernel(RowsArgs q) {
         if (zero) {
             for (int i = tid; i < (int)q.N_f; i += SR_THREADS) Fo[i] = make_float2(0.f, 0.f);
         } else if constexpr (!DIRECT) {
+            if (q.bulk) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncthreads();
-            for (int i = tid; i < (int)q.N_f; i += SR_THREADS) Fo[i] = row[i];
+            if (!q.bulk) {
+                for (int i = tid; i < (int)q.N_f; i += SR_THREADS) Fo[i] = row[i];
+            } else if (tid == 0) {
+                bulk_store(Fo, row, (uint32_t)q.N_f * 8u);
+            }
         }
         cur = s_next;
-        __syncthreads();   // the row buffer, the exchange buffers and s_next are free
+        __syncthreads();   // the row buffer (or its copy is under way), the exchange buffers and s_next are free
     }
+    if (tid == 0) bulk_store_read();
 }
 
 constexpr size_t SR_SMEM = 226 * 1024;
@@ -258,6 +278,7 @@ cc_status launch_segfft_rows(cc_plan* plan, int64_t n_t, const void* ab, float2*
     q.C = p.C4;
     q.wait_test = p.wait_test;
     if (q.rows > 0x7fffffff - 65536) return fail(CC_ERR_UNSUPPORTED, "too many segment transforms in one launch");
+    q.bulk = q.N_f % 2 == 0 && ((uintptr_t)F & 15) == 0;
     const bool bf16 = p.store == CC_STORE_BF16;
     void (*const kern)(RowsArgs) = bf16 ? (direct ? segfft_rows_kernel<true, true> : segfft_rows_kernel<true, false>)
                                         : (direct ? segfft_rows_kernel<false, true> : segfft_rows_kernel<false, false>);

@@ -32,6 +32,9 @@ CASES = {
     "Ns2050": (dict(n_samples=2050 * 7, T_sft=205.0, T_max=2050.0, T_short=2050.0), {}, cc.STORE_FP32),
     "one_coset": (dict(n_samples=480 * 9, T_sft=240.0, T_max=480.0, T_short=480.0), dict(), cc.STORE_FP32),
     "no_lag_Q1": (dict(n_samples=3600 * 5, T_sft=360.0, T_max=0.0, T_short=3600.0, n_det=1), {}, cc.STORE_FP32),
+    # an even number of bins: rows leave by bulk copies
+    "even_row": (dict(n_samples=3600 * 9, T_sft=360.0, T_max=3600.0, T_short=3600.0, f_band=0.10005), {}, cc.STORE_FP32),
+    "even_row_bf16": (dict(n_samples=3600 * 9, T_sft=360.0, T_max=3600.0, T_short=3600.0, f_band=0.10005), {}, cc.STORE_BF16),
     "long_row": (dict(n_samples=3600 * 3, T_sft=360.0, T_max=3600.0, T_short=3600.0), dict(mu_f=1e-3), cc.STORE_FP32),
     "many_cosets": (dict(n_samples=3600 * 3, T_sft=360.0, T_max=3600.0, T_short=3600.0, n_det=1),
                     dict(mu_f=5e-4), cc.STORE_FP32),
@@ -68,6 +71,8 @@ def test_segment_fft_rows(name):
         if name == "one_coset":
             assert plan.info["L"] < 4096 and p.N_FFT == 4096
             plan.set_tuning(transform_len=4096)
+        if name.startswith("even_row"):
+            assert p.N_f % 2 == 0
         F = plan.segment_fft(t, n_t).cpu().numpy()
         plan.check()
     err = np.abs(F - Fref).max()
