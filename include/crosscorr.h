@@ -254,14 +254,17 @@ cc_status crosscorr_search_noalloc(cc_plan* plan, const void* const* x_dev, cons
  *                     FUSED, else STAGED;
  *   CC_PATH_FUSED     one kernel per template batch: a thread-block cluster resamples
  *                     each segment into shared memory and transforms it on chip; needs
- *                     a few MB of workspace (FP32 storage, coset length <= 4096);
+ *                     a few MB of workspace (FP32 storage, coset length <= 4096).  Three
+ *                     and four detectors take the two-pass kernels where those serve the
+ *                     plan and the workspace holds at least one template of them;
  *   CC_PATH_TWO_PASS  a_r, b_r of a template batch written to HBM in the plan's
  *                     storage type (up to 24 GB of workspace), then every segment is
  *                     transformed on chip at the G >= 2 N_s frequencies that determine the
  *                     products of two segments, the products are summed there, and one
  *                     transform per template takes the sums to the output bins (Q <= 2,
  *                     R <= 1, not CC_PAIRS_CROSS_ONLY, coset length >= 64, output bins in the
- *                     lower half of each coset); a persistent kernel fed by TMA bulk copies
+ *                     lower half of each coset; CC_PATH_AUTO takes these kernels for wider
+ *                     bands too); a persistent kernel fed by TMA bulk copies
  *                     where rows are whole 16-byte pieces (see crosscorr_plan_check).
  *                     Segments longer than 4096 samples stored in BF16 are transformed at
  *                     the output bins instead;
@@ -342,7 +345,9 @@ cc_status crosscorr_plan_set_demod_form(cc_plan* plan, int form);
  *   x(b T_sft + j dt') = exp(-2 pi i f_h b T_sft) (-1)^j
  *                        sum_{m < n_prime} exp(2 pi i j m / n_prime) band[b][m] / T_sft
  * (Eqs. shifted-for-fft, long-time-series-het-corrected), zero in gaps.  Asynchronous on
- * `stream` (a small twiddle table is allocated stream-ordered).  1 <= n_prime <= 16384. */
+ * `stream` (a small twiddle table is allocated stream-ordered where n_prime is above 1536
+ * or has a prime factor above 5).
+ * 1 <= n_prime <= 16384. */
 cc_status crosscorr_sfts_to_series(const void* band_dev, const int64_t* block_sft_dev, int64_t n_blocks,
                                    int64_t n_prime, double T_sft, double f_h, void* x_dev, void* stream);
 

@@ -43,8 +43,11 @@
 //   * one CTA barrier per transform: the second pass's outputs that a last-pass butterfly needs
 //     come from one column of threads, which share a half-warp and exchange them in place.
 //
-// What bounds it (L = 4096): the FP32 pipe and the shared-memory exchanges of the two inner
-// passes, each about 1500 cycles per 4096-point transform and SM.
+// What bounds it (L = 4096): instruction issue (64 to 70 % of the slots with 16 warps per SM), the
+// FP32 pipe (54 %) and the shared-memory exchanges (55 %) together.  120-day band (N_s = 3600,
+// 2880 segments, two detectors), 72 templates at once, per template: 144 us; 151 with XOR-swizzled
+// exchanges, 161 with every sum compensated at every segment, 174 with three barriers a
+// transform, 640 at the output bins (8 transforms of 4096 points a row instead of 2).
 //
 // Waits are bounded (about one second): a wait that runs out sets bit 0 of the plan's error
 // word; the CTA agrees on it at the next barrier, waits for its copies in flight, frees its

@@ -9,7 +9,9 @@
 // C = 2 F splits into two F-point DFTs: c = 2 u takes a_f, c = 2 u + 1 takes a_f W_C^f.  Each
 // F-point DFT combines a_f +- a_(F-f) (half the products of the direct sum); its constants
 // are kernel parameters, read as immediate operands.  Bound by the write of Z (2 x the bytes
-// of the segment) for F up to about ten.
+// of the segment) for F up to about ten: 150 us per template of the 120-day band at a ten-hour lag
+// (F = 9, 0.93 GB read and written, 6.2 TB/s); the whole search 0.74 ms per template in FP32, 6.4
+// when every coset read and twiddled the whole segment.
 #include <algorithm>
 
 #include "corr.cuh"

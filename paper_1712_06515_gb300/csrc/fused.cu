@@ -99,7 +99,8 @@ bool fused_layout(const cc_plan* plan, int64_t n_t, FusedLayout* lay) {
 // of templates: a block computes KN_BLOCK consecutive delays of every detector, one a thread,
 // and writes the records whose four knots it holds.  The binary-orbit part of each delay is
 // computed once for all detectors (it depends on the source time only); the barycentric part
-// per detector.  Bound by the FP64 rate.
+// per detector.  Bound by the FP64 pipe (86 % busy): 25 us per template of the 120-day band with two
+// detectors, 33.5 with a fixed number of steps.
 constexpr int KN_BLOCK = 128, KN_OUT = KN_BLOCK - 3;
 
 __global__ void __launch_bounds__(KN_BLOCK)

@@ -59,7 +59,7 @@ static bool fused_supported(const cc_plan* plan) {
 
 // The two-pass kernels also serve plans whose output bins reach the upper half of their cosets
 // (f_band near 1/dt), which CC_PATH_TWO_PASS by name leaves to the others: 64 templates of a
-// one-day 1 Hz band take 0.2 ms on the lag grid, 7.8 ms on the cluster kernel.
+// one-day 1 Hz band take 0.25 ms on the lag grid, 7.8 ms on the cluster kernel.
 static int resolve_path(const cc_plan* plan) {
     if (plan->search_path != CC_PATH_AUTO) return plan->search_path;
     if (plan->Q <= 2 && lag_grid_supported(plan)) return CC_PATH_TWO_PASS;

@@ -15,8 +15,8 @@
 //
 // What bounds it: shared memory (65 % of its wavefronts) and issue, with the 16 warps per SM that
 // registers and 200 KB of buffers allow, and the barriers between a row's rounds.  20 days, three
-// templates (N_FFT = 32768, N_f = 12356): 433 us, 470 with plain stores of the row, 660 with a CTA
-// per coset; 510 MB leave.
+// templates (N_FFT = 32768, N_f = 12356): 433 us, 470 with plain stores of the row, about 650
+// with a CTA per coset; 510 MB leave.
 //
 // Waits on the mbarrier are bounded (about one second): a wait that runs out sets bit 0 of the
 // plan's error word, the CTA waits (bounded again) for the copy in flight and returns.

@@ -30,10 +30,11 @@
 //     thread -- live in tensor memory, read and written once per segment, the Kahan sums in
 //     registers.
 //
-// What bounds it: instruction issue (68 % of the slots, about 1150 instructions a warp and
-// transform, 16 warps per SM), the FP32 pipe (53 %) and the shared-memory exchanges (55 %); Z
-// leaves HBM at 1.7 TB/s.  The 120-day band at a ten-hour lag, per template: 684 us; 842 us with
-// padded buffers, two barriers a transform, twiddles read through L1 and one stage.
+// What bounds it: instruction issue (71 % of the slots, about 970 instructions a warp and
+// transform, 16 warps per SM), the FP32 pipe (59 %) and the shared-memory exchanges (58 %); Z
+// leaves HBM at 1.8 TB/s.  The 120-day band at a ten-hour lag, per template of two: 667 us; 684 with
+// XOR-swizzled exchanges, 842 with two more barriers a transform, twiddles read through L1 and
+// one stage.  (16 at once: 600.)
 //
 // Waits on the mbarriers are bounded (about one second of clock): a wait that runs out sets bit
 // 0 of the plan's device error word, every thread of the CTA agrees on it at the next barrier,
