@@ -386,7 +386,8 @@ cc_status crosscorr_plan_set_wait_test(cc_plan* plan, int on);
 /* The k largest rho over (template, bin) of a device float[n_t][N_f] array,
  * descending, ties by (template, bin) ascending; hits_host receives
  * min(k, n_t*N_f) records.  Synchronises the stream.  1 <= k <= 4096.
- * Its group maxima and candidate lists live in a plan-owned buffer of about 15 MB, allocated by the
+ * Its group maxima and candidate lists live in a plan-owned buffer of about 15 MB (its list in
+ * 50 KB of pinned host memory), allocated by the
  * first call on the plan (later calls allocate nothing) and separate from the search
  * workspace, so a search queued on another stream for the same plan is not disturbed;
  * two top-k calls on one plan must not run at the same time (one plan per thread). */

@@ -172,6 +172,7 @@ struct cc_plan {
     size_t ws_bytes = 0;
     // top-k candidate lists (crosscorr_rho_topk), allocated by its first call
     void* topk_ws = nullptr;
+    void* topk_host = nullptr;   // pinned host memory the selection writes its list to
 };
 
 namespace cc {

@@ -202,6 +202,7 @@ void crosscorr_plan_destroy(cc_plan* p) {
     if (p->learned_w) cudaFree(p->learned_w);
     if (p->learned_taps) cudaFree(p->learned_taps);
     if (p->topk_ws) cudaFree(p->topk_ws);
+    if (p->topk_host) cudaFreeHost(p->topk_host);
     delete p;
 }
 

@@ -139,7 +139,8 @@ topk_pass2(const float* __restrict__ cv, const long long* __restrict__ ci, long 
 //
 // What bounds it: the read of rho, then the one block's chain of latencies (24.7 M values,
 // k = 100: about 8 us to reread 119 groups, 3 us for the threshold, 2 us for the ranks).  The
-// whole call, with its copy and synchronisation, 73 us; 2140 us by the block lists alone.
+// whole call, with its synchronisation, 69 us (74 with a copy of the list); 2140 us by the block
+// lists alone.
 // ---------------------------------------------------------------------------
 constexpr int SEL_THREADS = 1024;
 constexpr int SEL_BLOCKS = 152;        // one per SM
@@ -147,8 +148,11 @@ constexpr int SEL_GROUPS = 16384;      // maxima
 constexpr int SEL_CAP = 8192;          // collected candidates
 constexpr int SEL_BATCH = 8;           // 16-byte loads a lane has in flight while it rereads
 
-struct SelHead {                       // followed by the hits' indices [k] and values [k]
-    unsigned count, err, done, pad;
+struct SelHead {                       // on the device: blocks done; the maxima follow
+    unsigned done, pad[3];
+};
+struct SelOut {                        // in pinned host memory, followed by the hits' indices [k] and values [k]
+    unsigned count, err, pad[2];
 };
 
 __device__ __forceinline__ unsigned sel_key(float v) {
@@ -178,7 +182,7 @@ __device__ __forceinline__ unsigned group_max(const float* __restrict__ rho, lon
 
 __global__ void __launch_bounds__(SEL_THREADS)
 topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups, int k, int aligned,
-            unsigned* __restrict__ maxima, SelHead* head, long long* __restrict__ out_i, float* __restrict__ out_v,
+            unsigned* __restrict__ maxima, SelHead* head, SelOut* out, long long* __restrict__ out_i, float* __restrict__ out_v,
             const unsigned* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ bool last;
@@ -313,8 +317,8 @@ topk_select(const float* __restrict__ rho, long long n, int gsize, int n_groups,
         }
     }
     if (tid == 0) {
-        head->count = (unsigned)m;
-        head->err = __ldcg(err);
+        out->count = (unsigned)m;
+        out->err = __ldcg(err);
     }
 }
 
@@ -361,25 +365,34 @@ extern "C" cc_status crosscorr_rho_topk(cc_plan* plan, const float* rho_dev, int
     const long long gsize = std::max<long long>(256, ((n + most - 1) / most + 127) / 128 * 128);
     const long long n_groups = (n + gsize - 1) / gsize;
     if (n_groups >= 2 * (long long)nk) {
+        // the list goes straight to pinned host memory (50 KB, allocated by the first call): a copy
+        // to pageable memory after the kernel cost 5 us
+        if (!plan->topk_host) {
+            const cudaError_t ea = cudaHostAlloc(&plan->topk_host, sizeof(SelOut) + (size_t)TOPK_MAX * 12,
+                                                 cudaHostAllocMapped | cudaHostAllocPortable);
+            if (ea != cudaSuccess) {
+                plan->topk_host = nullptr;
+                return cuda_fail(ea, "top-k result buffer");
+            }
+        }
         SelHead* head = (SelHead*)plan->topk_ws;
-        long long* oi = (long long*)(head + 1);
-        float* ov = (float*)(oi + nk);
-        unsigned* maxima = (unsigned*)((char*)(head + 1) + (size_t)TOPK_MAX * 12);
+        unsigned* maxima = (unsigned*)(head + 1);
+        SelOut* out = nullptr;
         const size_t sm = (size_t)SEL_CAP * sizeof(Cand) + SEL_GROUPS * sizeof(unsigned short);
         cudaError_t e = cudaFuncSetAttribute(topk_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&out, plan->topk_host, 0);
         if (e == cudaSuccess) e = cudaMemsetAsync(head, 0, sizeof(SelHead), st);
         if (e != cudaSuccess) return cuda_fail(e, "top-k selection set-up");
+        long long* oi = (long long*)(out + 1);
+        float* ov = (float*)(oi + nk);
         const int aligned = ((uintptr_t)rho_dev & 15) == 0;
         const int blocks = (int)std::min<long long>(SEL_BLOCKS, (n_groups + SEL_THREADS / 32 - 1) / (SEL_THREADS / 32));
-        topk_select<<<blocks, SEL_THREADS, sm, st>>>(rho_dev, n, (int)gsize, (int)n_groups, nk, aligned, maxima, head, oi, ov,
-                                                     plan->dp.err);
+        topk_select<<<blocks, SEL_THREADS, sm, st>>>(rho_dev, n, (int)gsize, (int)n_groups, nk, aligned, maxima, head, out, oi,
+                                                     ov, plan->dp.err);
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "topk launch");
-        std::vector<char> back(sizeof(SelHead) + (size_t)nk * 12);
-        e = cudaMemcpyAsync(back.data(), head, back.size(), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return cuda_fail(e, "topk copy");
-        const SelHead* h = (const SelHead*)back.data();
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "topk");
+        const SelOut* h = (const SelOut*)plan->topk_host;
         if (h->err) return crosscorr_plan_check(plan, stream);   // a failed bounded wait of the searches before
         if (h->count <= (unsigned)SEL_CAP) {
             const long long* hi = (const long long*)(h + 1);
