@@ -139,9 +139,9 @@ struct cc_plan {
     int search_path = CC_PATH_AUTO;           // crosscorr_plan_set_path
     cc_tuning tuning = {0, 0, 0};             // crosscorr_plan_set_tuning
     int kbar_span4 = 0;                       // largest transform position of a bin, 4096-point cosets
-    // two-pass search, lag grid: coset and pass twiddles [C][272] of the plan's grid and of one
-    // coset, roots of its transform length and of 4096 (plan-owned)
-    const float2 *corr_twk = nullptr, *corr_twk1 = nullptr, *corr_twL = nullptr, *corr_tw4096 = nullptr;
+    // two-pass search, where the lag grid serves the plan: coset and pass twiddles [C][272] of its
+    // grid, roots of its transform length and of 4096 (plan-owned)
+    const float2 *corr_twk = nullptr, *corr_twL = nullptr, *corr_tw4096 = nullptr;
     const float2 *corr_twp = nullptr, *corr_twp4096 = nullptr;   // last-pass powers (corr_powers)
     // staged segment FFT by rows (segfft_rows.cu; segments of up to 4096 samples, plan-owned):
     // last-pass powers [C4][4][256], output bin of each coset position [C4][2048], row counter

@@ -216,6 +216,7 @@ struct CorrLayout {
 };
 
 std::vector<float2> corr_powers(int64_t L, int64_t C) {
+    if (L < 16) return {};   // no pass of 16 points a thread
     const int64_t GT = L / 16, RL = L >= 512 ? L / 256 : L / 16, nb = 16 / RL, G = C * L;
     int np = 0;
     while ((1 << np) < RL) ++np;
@@ -244,10 +245,10 @@ bool two_pass_supported(const cc_plan* plan) {
 // Whether the lag grid serves the plan: the conditions of two_pass_supported but any output bins
 // (the last transform reaches all of them); with three or four detectors FP32 storage and at
 // least 256-point transforms (one activity bit per detector and template of a series group).
+// Asked at plan creation too, before the kernel parameters are filled.
 bool lag_grid_supported(const cc_plan* plan) {
-    const DevParams& p = plan->dp;
-    if (p.R > 1 || p.pair_mode == CC_PAIRS_CROSS_ONLY || p.L < 64 || p.L > 4096 || plan->N_f < 1) return false;
-    return p.Q <= 2 || (p.store == CC_STORE_FP32 && p.L >= 128);
+    if (plan->R > 1 || plan->cfg.pair_mode == CC_PAIRS_CROSS_ONLY || plan->L < 64 || plan->L > 4096 || plan->N_f < 1) return false;
+    return plan->Q <= 2 || (plan->cfg.store == CC_STORE_FP32 && plan->L >= 128);
 }
 
 static int sm_count() {
@@ -504,7 +505,7 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         a.scratch = scratch;
         a.ctr = ctr;
         a.err = p.err;
-        a.twk = y.C == 1 ? plan->corr_twk1 : plan->corr_twk;
+        a.twk = plan->corr_twk;
         a.twp = y.padded ? plan->corr_twp4096 : plan->corr_twp;
         a.N_s = p.N_s;
         a.M = (int)p.M;
@@ -534,7 +535,7 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         }
         q.U = U;
         q.h = y.C > 2 ? h : nullptr;
-        q.twL = y.L == CORR_POINTS ? plan->corr_tw4096 : plan->corr_twL;
+        q.twL = y.padded ? plan->corr_tw4096 : plan->corr_twL;
         q.norm = (const float4*)norm;
         q.D = D;
         q.M = p.M;

@@ -53,6 +53,9 @@ cudaError_t launch_corr_t(const CorrArgs& a, int sms, cudaStream_t st);
 // of a transform, butterfly i, power 2^n of W_G^(c + C b), G = C L, at ((c nb + i) np + n) L/16 + j.
 std::vector<float2> corr_powers(int64_t L, int64_t C);
 
+// Whether the lag grid serves the plan (corr.cu): its tables are made for such plans only.
+bool lag_grid_supported(const cc_plan* plan);
+
 // Work units per resident CTA slot (2 per SM), shared by the layout and the launch.
 constexpr int CORR_CTAS_PER_SM = 2;
 

@@ -454,34 +454,40 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
             bin = (int)k;
         }
     }
-    // The lag grid of the two-pass search (corr.cu): G = Cg x Lg points, the same split of the
-    // coset twiddles W_G^(c s) and the second pass's twiddles; [1] for one coset (c = 0).
-    const int64_t Lg = 2 * p->N_s <= 4096 ? 2 * L : 4096;
-    const int64_t Cg = p->N_s > 4096 ? 2 * ((p->N_s + 4095) / 4096) : 2 * p->N_s <= 4096 ? 1 : 2;
-    auto roots = [](int64_t n) {
-        std::vector<float2> v(n);
-        for (int64_t j = 0; j < n; ++j) {
-            const double ang = -2.0 * M_PI * (double)j / (double)n;
-            v[j] = make_float2((float)cos(ang), (float)sin(ang));
-        }
-        return v;
-    };
-    auto grid_twiddles = [](int64_t Cn) {
-        std::vector<float2> v((size_t)Cn * 272);
-        const uint64_t G = (uint64_t)Cn * 4096;
+    // The lag grid of the two-pass search (corr.cu), where it serves the plan: G = Cg x Lg points, the
+    // same split of the coset twiddles W_G^(c s) and the second pass's twiddles; the 4096-point
+    // tables beside them for a plan of shorter transforms that may be tuned to transform_len 4096.
+    std::vector<float2> gp, gp4, gk, gl, g4;
+    if (cc::lag_grid_supported(p)) {
+        const int64_t Lg = 2 * p->N_s <= 4096 ? 2 * L : 4096;
+        const int64_t Cg = p->N_s > 4096 ? 2 * ((p->N_s + 4095) / 4096) : 2 * p->N_s <= 4096 ? 1 : 2;
+        const bool pad = L < 4096 && C4 > 0;
+        auto roots = [](int64_t n) {
+            std::vector<float2> v(n);
+            for (int64_t j = 0; j < n; ++j) {
+                const double ang = -2.0 * M_PI * (double)j / (double)n;
+                v[j] = make_float2((float)cos(ang), (float)sin(ang));
+            }
+            return v;
+        };
+        gk.resize((size_t)Cg * 272);
+        const uint64_t G = (uint64_t)Cg * 4096;
         auto w = [&](uint64_t j) {
             const double ang = -2.0 * M_PI * (double)(j % G) / (double)G;
             return make_float2((float)cos(ang), (float)sin(ang));
         };
-        for (uint64_t c2 = 0; c2 < (uint64_t)Cn; ++c2)
+        for (uint64_t c2 = 0; c2 < (uint64_t)Cg; ++c2)
             for (uint64_t r = 0; r < 16; ++r) {
-                v[c2 * 272 + r] = w(256 * c2 * r);
-                for (uint64_t k = 0; k < 16; ++k) v[c2 * 272 + 16 + 16 * r + k] = w(16 * r * ((uint64_t)Cn * k + c2));
+                gk[c2 * 272 + r] = w(256 * c2 * r);
+                for (uint64_t k = 0; k < 16; ++k) gk[c2 * 272 + 16 + 16 * r + k] = w(16 * r * ((uint64_t)Cg * k + c2));
             }
-        return v;
-    };
-    const std::vector<float2> gp = cc::corr_powers(Lg, Cg), gp4 = cc::corr_powers(4096, 1);
-    const std::vector<float2> gk = grid_twiddles(Cg), gk1 = grid_twiddles(1), gl = roots(Lg), g4 = roots(4096);
+        gp = cc::corr_powers(Lg, Cg);
+        gl = roots(Lg);
+        if (pad) {
+            gp4 = cc::corr_powers(4096, 1);
+            g4 = roots(4096);
+        }
+    }
     // coset maps of the 4096-point decomposition (the same as the plan's when L = 4096)
     std::vector<int> off4, ck4, cm4;
     if (C4 > 0 && C4 != C) {
@@ -507,7 +513,6 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
         (!rtw.empty() && (st = upload(p, rtw.data(), rtw.size(), &p->rows_twp)) != CC_OK) ||
         (!rkm.empty() && (st = upload(p, rkm.data(), rkm.size(), &p->rows_kmap)) != CC_OK) ||
         (st = upload(p, gk.data(), gk.size(), &p->corr_twk)) != CC_OK ||
-        (st = upload(p, gk1.data(), gk1.size(), &p->corr_twk1)) != CC_OK ||
         (st = upload(p, gl.data(), gl.size(), &p->corr_twL)) != CC_OK ||
         (st = upload(p, gp.data(), gp.size(), &p->corr_twp)) != CC_OK ||
         (st = upload(p, gp4.data(), gp4.size(), &p->corr_twp4096)) != CC_OK ||

@@ -3,7 +3,10 @@ host-side argument validation rejects bad input before any CUDA call.  No
 compute calls: these run without a GPU."""
 import ctypes
 import os
+import platform
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -153,3 +156,17 @@ def test_entry_points_reject_null_plan(lib):
     assert lib.crosscorr_plan_kernel_time(None, ctypes.byref(ms), ctypes.byref(n)) == CC_ERR_INVALID
     lib.crosscorr_plan_destroy(None)
     assert lib.crosscorr_status_string(3) == b"CUDA error"
+
+
+@pytest.mark.skipif(platform.machine() != "x86_64", reason="calls a C++ function by the x86-64 convention")
+@pytest.mark.parametrize("points,cosets,entries", [(2, 1, 0), (8, 1, 0), (16, 1, 0), (32, 1, 16), (4096, 2, 2048)])
+def test_pass_tables_of_the_shortest_transforms(lib, points, cosets, entries):
+    """The pair kernel's table of last-pass powers is empty below 16 points (segments of at most
+    four samples ask for it at plan creation) instead of dividing by a radix of zero.  In a child
+    process: the division ends one on this machine."""
+    code = (f"import ctypes; f = ctypes.CDLL({_lib.LIBPATH!r})._ZN2cc11corr_powersEll; v = (ctypes.c_void_p * 3)(); "
+            f"f.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_int64]; f.restype = None; "
+            f"f(v, {points}, {cosets}); print(((v[1] or 0) - (v[0] or 0)) // 8)")
+    run = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True)
+    assert run.returncode == 0, run.returncode
+    assert int(run.stdout) == entries

@@ -121,3 +121,17 @@ def test_small_workspace(n_det):
 @pytest.mark.parametrize("tune", [dict(batch_templates=2), dict(chunk_waves=1), dict(chunk_waves=400), dict(transform_len=4096)])
 def test_splits(tune):
     run(600, 40, 5, {}, **tune)
+
+
+@pytest.mark.parametrize("n_s", [1, 2, 4, 5, 8, 32])
+def test_segments_below_the_lag_grid(n_s):
+    """The shortest segments (coset lengths 4 to 32) are no plans of the lag grid: its tables are
+    not made for them and the automatic path serves them."""
+    ds = synth.tiny(seed=83, n_samples=1500, T_sft=float(n_s), T_max=float(n_s), T_short=float(n_s), f_band=0.9, n_templates=3,
+                    duty=0.8, mean_lock_s=8.0 * n_s)
+    ref = oracle.rho(ds)
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        assert plan.search_path != cc.PATH_TWO_PASS
+        got = plan.search(torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV)).cpu().numpy()
+    for t in range(3):
+        assert np.abs(got[t] - ref[t]).max() <= 1e-4 * max(1.0, np.abs(ref[t]).max())
