@@ -63,7 +63,9 @@ def templates5(templates):
     import torch
     if templates.shape[-1] == 5:
         return templates
-    if templates.is_cuda and templates.dim() == 2 and templates.dtype == torch.float64 and templates.is_contiguous():
+    # the library's kernel reads rows of three doubles, on the current device
+    if (templates.is_cuda and templates.dim() == 2 and templates.shape[1] == 3 and templates.dtype == torch.float64
+            and templates.is_contiguous() and not templates.is_neg() and templates.get_device() == torch.cuda.current_device()):
         return _circular(templates, None)
     z = torch.zeros((templates.shape[0], 2), dtype=templates.dtype, device=templates.device)
     return torch.cat([templates, z], dim=1).contiguous()

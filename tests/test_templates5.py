@@ -1,0 +1,35 @@
+"""Template rows widened to (a_p, T_asc, P, e, omega): the library's kernel takes rows of three
+doubles only, every other width goes the way it went without that kernel."""
+import numpy as np
+import pytest
+
+import paper_1712_06515_gb300 as cc
+
+torch = pytest.importorskip("torch")
+
+
+class OnDevice(torch.Tensor):
+    """A host tensor that passes for a CUDA tensor."""
+    is_cuda = property(lambda self: True)
+
+
+@pytest.mark.parametrize("width", [1, 2, 4, 6])
+def test_other_widths_stay_off_the_kernel(width, monkeypatch):
+    def kernel(*args):
+        raise AssertionError("rows of another width than three given to the kernel")
+
+    monkeypatch.setattr(cc, "_circular", kernel)
+    t = torch.arange(5.0 * width, dtype=torch.float64).reshape(5, width)
+    got = cc.templates5(t.as_subclass(OnDevice)).as_subclass(torch.Tensor)
+    assert torch.equal(got, torch.cat([t, torch.zeros(5, 2, dtype=torch.float64)], dim=1))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,width", [(1, 3), (257, 3), (0, 3), (7, 1), (7, 2), (7, 4), (7, 5)])
+def test_widths_on_the_device(n, width):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    t = torch.from_numpy(np.random.default_rng(1).standard_normal((n, width)))
+    for v in (t.cuda(), t.t().contiguous().cuda().t()):     # rows, and columns in memory
+        got = cc.templates5(v).cpu()
+        assert torch.equal(got, t if width == 5 else torch.cat([t, torch.zeros(n, 2, dtype=torch.float64)], dim=1))
