@@ -66,18 +66,18 @@ def templates5(templates):
     # the library's kernel reads rows of three doubles, on the current device
     if (templates.is_cuda and templates.dim() == 2 and templates.shape[1] == 3 and templates.dtype == torch.float64
             and templates.is_contiguous() and not templates.is_neg() and templates.get_device() == torch.cuda.current_device()):
-        return _circular(templates, None)
+        return _circular(templates)
     z = torch.zeros((templates.shape[0], 2), dtype=templates.dtype, device=templates.device)
     return torch.cat([templates, z], dim=1).contiguous()
 
 
-def _circular(t3, stream):
-    """[n, 3] contiguous CUDA rows widened to [n, 5] by the library, on `stream`."""
+def _circular(t3):
+    """[n, 3] contiguous CUDA rows widened to [n, 5] by the library, on the current stream."""
     import torch
     lib = _lib.load()
     out = torch.empty((t3.shape[0], 5), dtype=torch.float64, device=t3.device)
     check("crosscorr_templates_circular", lib.crosscorr_templates_circular(_dptr(t3), t3.shape[0], _dptr(out),
-                                                                          _stream_handle(stream)))
+                                                                          _stream_handle(None)))
     return out
 
 
@@ -244,20 +244,25 @@ class CrossCorrPlan:
         arr = (c_void_p * self.Q)(*[_dptr(xi) for xi in xs])
         return arr, xs
 
-    def _templates(self, templates):
+    def _templates(self, templates, stream=None):
         """(n_t, device templates [n_t, 5]): rows (a_p, T_asc, P, e, omega); [n_t, 3]
-        circular rows are widened with e = omega = 0 (a device copy, ordered on the stream)."""
+        circular rows are widened with e = omega = 0: a device copy made on the call's stream and
+        allocated for it, so that neither the copy nor the reuse of its memory can run ahead of
+        the calls that read it."""
         import torch
         _check_tensor("templates", templates, torch.float64)
         if templates.dim() != 2 or templates.shape[1] not in (3, 5):
             raise ValueError("templates must be [n_t, 5] (a_p, T_asc, P, e, omega) or [n_t, 3] (circular)")
-        return templates.shape[0], templates5(templates)
+        if stream is None or templates.shape[1] == 5:
+            return templates.shape[0], templates5(templates)
+        with torch.cuda.stream(stream):
+            return templates.shape[0], templates5(templates)
 
     # -- the C ABI calls -------------------------------------------------------
     def resample(self, x, templates, ab=None, norm=None, stream=None):
         """Stage 1: a_r, b_r series [n_t, Q, 2, N_tau] and segment norms [n_t, Q, M, 4]."""
         import torch
-        n_t, templates = self._templates(templates)
+        n_t, templates = self._templates(templates, stream)
         xp, _ = self._xptrs(x)
         dev = templates.device
         if ab is None:
@@ -292,7 +297,7 @@ class CrossCorrPlan:
     def search(self, x, templates, rho=None, stream=None):
         """The whole path: rho [n_t, N_f] float32."""
         import torch
-        n_t, templates = self._templates(templates)
+        n_t, templates = self._templates(templates, stream)
         xp, _ = self._xptrs(x)
         if rho is None:
             rho = torch.empty((n_t, self.N_f), dtype=torch.float32, device=templates.device)
@@ -353,7 +358,7 @@ class CrossCorrPlan:
     def demod_search(self, templates, rho=None, stream=None):
         """Detector-frame (demodulation) rho [n_t, N_f] at the plan's output frequencies."""
         import torch
-        n_t, templates = self._templates(templates)
+        n_t, templates = self._templates(templates, stream)
         if rho is None:
             rho = torch.empty((n_t, self.N_f), dtype=torch.float32, device=templates.device)
         _check_tensor("rho", rho, torch.float32)

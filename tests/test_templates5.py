@@ -33,3 +33,31 @@ def test_widths_on_the_device(n, width):
     for v in (t.cuda(), t.t().contiguous().cuda().t()):     # rows, and columns in memory
         got = cc.templates5(v).cpu()
         assert torch.equal(got, t if width == 5 else torch.cat([t, torch.zeros(n, 2, dtype=torch.float64)], dim=1))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("method", ["search", "demod_search"])
+def test_widening_runs_on_the_calls_stream(method):
+    """A search on another stream than the current one, behind whose long queue the widening of
+    [n, 3] templates must not wait (the search would read rows not yet written)."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import synth
+    ds = synth.tiny(seed=5, n_templates=3)
+    x, tm = torch.from_numpy(ds.x64).cuda(), torch.from_numpy(ds.templates).cuda()
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        plan.demod_prepare(x)
+        want = getattr(plan, method)(x, tm) if method == "search" else plan.demod_search(tm)
+        rho = torch.zeros_like(want)
+        torch.cuda.synchronize()
+        side = torch.cuda.Stream()
+        torch.cuda._sleep(int(1e9))                         # half a second on the current stream
+        if method == "search":
+            plan.search(x, tm, rho, stream=side)
+        else:
+            plan.demod_search(tm, rho, stream=side)
+        side.synchronize()
+        with torch.cuda.stream(side):
+            got = rho.cpu()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want.cpu())
