@@ -140,8 +140,11 @@ struct cc_plan {
     cc_tuning tuning = {0, 0, 0};             // crosscorr_plan_set_tuning
     int kbar_span4 = 0;                       // largest transform position of a bin, 4096-point cosets
     // two-pass search, where the lag grid serves the plan: coset and pass twiddles [C][272] of its
-    // grid, roots of its transform length and of 4096 (plan-owned)
-    const float2 *corr_twk = nullptr, *corr_twL = nullptr, *corr_tw4096 = nullptr;
+    // grid; as two floats (twofloat.cuh) the roots of its transform length, of 4096 and of the plan's
+    // coset length, and the powers of the grid's and the output grid's root (plan-owned)
+    const float2* corr_twk = nullptr;
+    const float4 *corr_root = nullptr, *corr_root4096 = nullptr, *corr_rootL = nullptr;
+    const float4 *corr_glo = nullptr, *corr_ghi = nullptr, *corr_nlo = nullptr, *corr_nhi = nullptr;
     const float2 *corr_twp = nullptr, *corr_twp4096 = nullptr;   // last-pass powers (corr_powers)
     // staged segment FFT by rows (segfft_rows.cu; segments of up to 4096 samples, plan-owned):
     // last-pass powers [C4][4][256], output bin of each coset position [C4][2048], row counter

@@ -5,7 +5,7 @@
 //
 //   corr_lags_kernel   sums the partial rows of a template, inverse transform per coset to
 //                      lags, and the template's normalisation;
-//   corr_merge_kernel  the lag sequence from the cosets (more than two cosets only);
+//   corr_merge_kernel  the lag sequence from the cosets (more than one);
 //   corr_rho_kernel    one coset of the N_FFT-point output transform of the lag sequence,
 //                      normalised at the output bins.
 //
@@ -13,12 +13,22 @@
 //   rho_raw(k) = Re sum_(n = 0)^(2 N_s - 1) h(n) W_N^(k n),
 //   h(0) = a(0), h(n) = 2 a(n) [n < N_s] + conj(b(N_s - n)) [n >= 1]
 // (a(-l) = conj(a(l)) because A is real; a pair of consecutive segments carries the phase
-// W_N^(-k N_s) of their distance; b counts twice with every ordered pair).  Per template the
-// three take about 0.1 % of the operations of the segment transforms at the 120-day band.
+// W_N^(-k N_s) of their distance; b counts twice with every ordered pair).
+//
+// These three work on numbers of two floats (twofloat.cuh).  A and B hold the power of every
+// frequency of the series, in the searched band or not, and a transform spreads the rounding of
+// the loudest of them over all lags and from there over all output bins: in FP32 a line of three
+// times the noise outside the band left errors of 0.08 in rho, where sums at the output bins
+// leave 1e-5, because there the rounding is relative to the spectra's amplitude.  Bound by the
+// FP32 pipe (about twelve operations for one of FP64, whose rate here is 1/64) and, for few
+// templates, by latency.  A pass with them in two floats against FP32: 144 templates of the 120-day
+// band 40.6 against 40.3 ms, 4 templates of an hour 59 against 56 us.
 #include <algorithm>
 
 #include "corr.cuh"
 #include "segpair.cuh"
+#include "tma.cuh"
+#include "twofloat.cuh"
 
 namespace cc {
 
@@ -51,31 +61,53 @@ CC_CORR_INST_MULTI_FULL(extern)
 constexpr size_t TWO_PASS_WS_BUDGET = (size_t)24 << 30;   // a_r, b_r (and folded rows) of one template batch
 constexpr size_t MULTI_WS_BUDGET = (size_t)4 << 30;       // the same for three and four detectors (the fused path's plans)
 constexpr int LAG_THREADS = 256;
+constexpr int LAG_MAX_THREADS = 1024;   // the two-float transforms: a radix-4 butterfly a thread, at least LAG_THREADS
 constexpr int ROW_BLOCK = 32;        // partial rows summed by one block of corr_rows_kernel
 
 // What the kernels after corr_kernel need.
 struct LagArgs {
-    const float* raw;       // [n_t][n_rows][planes][G]
-    float2* U;              // [n_t][planes > 1 ? 2 : 1][C][L]: per coset the inverse transform of A and B
-    float2* h;              // [n_t][n_lags] (C > 2)
-    const float2* twL;      // exp(-2 pi i j / L)
+    const float* raw;       // [n_t][n_rows][planes][words][G]: partial sums (words 2: and what they round off)
+    ffc* U;                 // [n_t][planes > 1 ? 2 : 1][C][L]: per coset the inverse transform of A and B
+    ffc* h;                 // [n_t][n_lags] (C > 1)
+    const ffc* root;        // exp(-2 pi i j / L)
+    const ffc *g_lo, *g_hi; // powers of exp(-2 pi i / G) (C > 1), see ffc_power
     const float4* norm;     // [n_t][Q][M]
     double* D;              // [n_t] sqrt(2 / normalisation), 0 without weight
     int64_t M;
-    int L, log2L, C, planes, n_rows, n_lags, N_s, Q, R, pair_mode;
+    int L, log2L, C, planes, words, n_rows, n_lags, N_s, Q, R, pair_mode;
 };
 
-// Sum of ROW_BLOCK partial rows (few templates have many): out [n_t][gridDim.y][len].
+// One partial row's value at p, its second word at p + lo (lo = 0: none)
+__device__ __forceinline__ ff row_value(const float* __restrict__ p, size_t lo) {
+    return make_float2(__ldg(p), lo ? __ldg(p + lo) : 0.f);
+}
+
+// Sum of ROW_BLOCK partial rows (few templates have many): out [n_t][gridDim.y][planes][2][G].
 __global__ void __launch_bounds__(LAG_THREADS)
-corr_rows_kernel(const float* __restrict__ raw, int n_rows, int64_t len, float* __restrict__ out) {
+corr_rows_kernel(const float* __restrict__ raw, int n_rows, int planes, int words, int64_t G, float* __restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * LAG_THREADS + threadIdx.x, t = blockIdx.z;
-    if (i >= len) return;
+    if (i >= planes * G) return;
+    const int64_t pl = i / G, m = i - pl * G;
     const int r0 = blockIdx.y * ROW_BLOCK, r1 = min(n_rows, r0 + ROW_BLOCK);
-    const float* p = raw + (size_t)t * n_rows * len + i;
-    float s = 0.f, cp = 0.f;
+    const size_t stride = (size_t)planes * words * G;
+    const float* p = raw + (size_t)t * n_rows * stride + pl * words * G + m;
+    const size_t lo = words > 1 ? G : 0;
+    ff s = make_float2(0.f, 0.f);
 #pragma unroll 8
-    for (int r = r0; r < r1; ++r) kahan_add(s, cp, __ldg(p + (size_t)r * len));
-    out[((size_t)t * gridDim.y + blockIdx.y) * len + i] = s;
+    for (int r = r0; r < r1; ++r) s = ff_add(s, row_value(p + r * stride, lo));
+    float* const o = out + (((size_t)t * gridDim.y + blockIdx.y) * planes + pl) * 2 * G + m;
+    o[0] = s.x;
+    o[G] = s.y;
+}
+
+// The L roots of a block's transform into shared memory, under the loads of its input, and the
+// barrier before both are read.
+__device__ __forceinline__ void stage_roots(ffc* dst, const ffc* __restrict__ root, int L) {
+    for (int j = threadIdx.x; j < L; j += blockDim.x) cp_async<16>(dst + j, root + j);
+}
+__device__ __forceinline__ void roots_staged() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
 }
 
 __device__ __forceinline__ double norm_pair(float4 a, float4 b) {
@@ -83,17 +115,17 @@ __device__ __forceinline__ double norm_pair(float4 a, float4 b) {
 }
 
 // grid: x = coset c (x = C, y = 0: the normalisation factor of template z), y = A or B, z = template.
-__global__ void __launch_bounds__(LAG_THREADS)
+__global__ void __launch_bounds__(LAG_MAX_THREADS)
 corr_lags_kernel(const LagArgs q) {
-    extern __shared__ __align__(16) float2 buf[];
+    extern __shared__ __align__(16) ffc buf[];
     const int c = blockIdx.x, ser = blockIdx.y;
     const size_t t = blockIdx.z;
     if (c == q.C) {   // sum over the pair set of A_i A_j + B_i B_j + 2 C_i C_j
         if (ser) return;
-        __shared__ double red[LAG_THREADS / 32];
+        __shared__ double red[LAG_MAX_THREADS / 32];
         const float4* nt = q.norm + t * q.Q * q.M;
         double acc = 0.0;
-        for (int64_t idx = threadIdx.x; idx < q.Q * q.M; idx += LAG_THREADS) {
+        for (int64_t idx = threadIdx.x; idx < q.Q * q.M; idx += blockDim.x) {
             const int Y = (int)(idx / q.M);
             const int64_t K = idx - Y * q.M;
             const float4 nY = nt[Y * q.M + K];
@@ -109,59 +141,64 @@ corr_lags_kernel(const LagArgs q) {
         __syncthreads();
         if (threadIdx.x == 0) {
             double s = 0.0;
-            for (int w = 0; w < LAG_THREADS / 32; ++w) s += red[w];
+            for (int w = 0; w < (int)blockDim.x / 32; ++w) s += red[w];
             q.D[t] = s > 0.0 ? 1.4142135623730951 / sqrt(s) : 0.0;
         }
         return;
     }
-    const size_t G = (size_t)q.C * q.L;
-    const float* p0 = q.raw + t * q.n_rows * q.planes * G + (size_t)c * q.L;
+    const size_t G = (size_t)q.C * q.L, plane = q.words * G, stride = q.planes * plane, lo = q.words > 1 ? G : 0;
+    const float* p0 = q.raw + t * q.n_rows * stride + (size_t)c * q.L;
+    stage_roots(buf + 2 * q.L, q.root, q.L);
     // the inverse transform as the conjugate of the forward one of the conjugate
-    for (int m = threadIdx.x; m < q.L; m += LAG_THREADS) {
-        float re = 0.f, cr = 0.f, im = 0.f, ci = 0.f;
-        const float* p = p0 + m;
+    for (int m = threadIdx.x; m < q.L; m += blockDim.x) {
+        const float* p = p0 + m + (ser ? plane : 0);
+        ff re = make_float2(0.f, 0.f), im = re;
         if (ser == 0) {
-#pragma unroll 4
-            for (int r = 0; r < q.n_rows; ++r) kahan_add(re, cr, __ldg(p + (size_t)r * q.planes * G));
+#pragma unroll 8
+            for (int r = 0; r < q.n_rows; ++r) re = ff_add(re, row_value(p + r * stride, lo));
         } else {
 #pragma unroll 4
             for (int r = 0; r < q.n_rows; ++r) {
-                kahan_add(re, cr, __ldg(p + ((size_t)r * q.planes + 1) * G));
-                kahan_add(im, ci, __ldg(p + ((size_t)r * q.planes + 2) * G));
+                re = ff_add(re, row_value(p + r * stride, lo));
+                im = ff_add(im, row_value(p + r * stride + plane, lo));
             }
         }
-        buf[m] = make_float2(re, -im);
+        buf[m] = ffc_make(re, ff_neg(im));
     }
-    __syncthreads();
-    const float2* res = fft_stockham(buf, buf + q.L, q.L, q.log2L, q.twL);
-    const float sc = 1.0f / (float)G;
-    float2* o = q.U + ((t * (q.planes > 1 ? 2 : 1) + ser) * q.C + c) * q.L;
-    for (int m = threadIdx.x; m < q.L; m += LAG_THREADS) o[m] = make_float2(res[m].x * sc, -res[m].y * sc);
+    roots_staged();
+    const ffc* res = ffc_stockham(buf, buf + q.L, q.L, q.log2L, buf + 2 * q.L);
+    // times 1 / G = 1 / (C L): C is not a power of two for folded segments
+    const float inv_l = 1.0f / (float)q.L;
+    const ff inv_c = ff_from(1.0 / (double)q.C);
+    ffc* o = q.U + ((t * (q.planes > 1 ? 2 : 1) + ser) * q.C + c) * q.L;
+    for (int m = threadIdx.x; m < q.L; m += blockDim.x) {
+        const ffc v = ffc_scale2(ffc_conj(res[m]), inv_l);
+        o[m] = q.C == 1 ? v : ffc_make(ff_mul(ffc_re(v), inv_c), ff_mul(ffc_im(v), inv_c));
+    }
 }
 
 // sum_c W_G^(-c l) u_c(l mod L): the inverse transform at lag l from those of the cosets
-__device__ __forceinline__ float2 lag_value(const float2* __restrict__ u, int C, int L, int l) {
-    float2 v = __ldg(u + (l & (L - 1)));
-    for (int c = 1; c < C; ++c) {
-        const float2 w = unit_root(-(int64_t)c * l, (int64_t)C * L);
-        v = cadd(v, cmul(__ldg(u + (size_t)c * L + (l & (L - 1))), w));
+__device__ __forceinline__ ffc lag_value(const LagArgs& q, const ffc* __restrict__ u, int l) {
+    ffc v = __ldg(u + (l & (q.L - 1)));
+    for (int c = 1; c < q.C; ++c) {
+        const ffc w = ffc_conj(ffc_power(q.g_lo, q.g_hi, (uint64_t)c * (uint64_t)l % ((uint64_t)q.C * q.L)));
+        v = ffc_add(v, ffc_mul(__ldg(u + (size_t)c * q.L + (l & (q.L - 1))), w));
     }
     return v;
 }
 
-__device__ __forceinline__ float2 lag_h(const LagArgs& q, size_t t, int n) {
+__device__ __forceinline__ ffc lag_h(const LagArgs& q, size_t t, int n) {
     const int G = q.C * q.L;
-    const float2* u = q.U + t * (q.planes > 1 ? 2 : 1) * G;
-    float2 h = make_float2(0.f, 0.f);
+    const ffc* u = q.U + t * (q.planes > 1 ? 2 : 1) * G;
+    ffc h = make_float4(0.f, 0.f, 0.f, 0.f);
     if (n < q.N_s) {
-        const float2 a = lag_value(u, q.C, q.L, n);
-        h = n > 0 ? cscale(a, 2.f) : a;
+        const ffc a = lag_value(q, u, n);
+        h = n > 0 ? ffc_scale2(a, 2.f) : a;
     }
     if (q.planes > 1 && n > 0) {
         const int l = q.N_s - n;
-        const float2 b = lag_value(u + G, q.C, q.L, l < 0 ? l + G : l);
-        const float f = q.pair_mode == CC_PAIRS_ALL_ORDERED ? 2.f : 1.f;
-        h = make_float2(fmaf(f, b.x, h.x), fmaf(-f, b.y, h.y));
+        const ffc b = ffc_conj(lag_value(q, u + G, l < 0 ? l + G : l));
+        h = ffc_add(h, q.pair_mode == CC_PAIRS_ALL_ORDERED ? ffc_scale2(b, 2.f) : b);
     }
     return h;
 }
@@ -174,31 +211,36 @@ corr_merge_kernel(const LagArgs q) {
 }
 
 // Output bins b0 + c + C m (the plan's coset lists), one coset per block: position p takes
-// sum_f h(p + f L) W_N^((b0 + c)(p + f L)), an L-point transform gives the bins.
+// sum_f h(p + f L) W_N^((b0 + c)(p + f L)), an L-point transform gives the bins.  L and root are
+// the plan's; n_lo, n_hi: powers of exp(-2 pi i / N).
 // grid: x = coset, y = template.
-__global__ void __launch_bounds__(LAG_THREADS)
-corr_rho_kernel(const LagArgs q, int L, int log2L, const float2* __restrict__ twL, int64_t N_FFT, int64_t b0,
-                const int* __restrict__ off, const int* __restrict__ ck, const int* __restrict__ cm, int64_t N_f,
-                float* __restrict__ rho) {
-    extern __shared__ __align__(16) float2 buf[];
+__global__ void __launch_bounds__(LAG_MAX_THREADS)
+corr_rho_kernel(const LagArgs q, int L, int log2L, const ffc* __restrict__ root, const ffc* __restrict__ n_lo,
+                const ffc* __restrict__ n_hi, int64_t N_FFT, int64_t b0, const int* __restrict__ off,
+                const int* __restrict__ ck, const int* __restrict__ cm, int64_t N_f, float* __restrict__ rho) {
+    extern __shared__ __align__(16) ffc buf[];
     const int c = blockIdx.x;
     const size_t t = blockIdx.y;
-    const uint64_t N = (uint64_t)N_FFT, mask = N - 1;
+    stage_roots(buf + 2 * L, root, L);
+    const uint64_t mask = (uint64_t)N_FFT - 1;
     const uint64_t bc = ((uint64_t)b0 + (uint64_t)c) & mask;
-    for (int pos = threadIdx.x; pos < L; pos += LAG_THREADS) {
-        float2 acc = make_float2(0.f, 0.f);
+    for (int pos = threadIdx.x; pos < L; pos += blockDim.x) {
+        ffc acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
         for (int n = pos; n < q.n_lags; n += L) {
-            const float2 h = q.h ? __ldg(q.h + t * q.n_lags + n) : lag_h(q, t, n);
-            acc = cadd(acc, cmul(h, twiddle_N((bc * (uint64_t)n) & mask, N)));
+            const ffc h = q.h ? __ldg(q.h + t * q.n_lags + n) : lag_h(q, t, n);
+            acc = ffc_add(acc, ffc_mul(h, ffc_power(n_lo, n_hi, (bc * (uint64_t)n) & mask)));
         }
         buf[pos] = acc;
     }
-    __syncthreads();
-    const float2* res = fft_stockham(buf, buf + L, L, log2L, twL);
+    roots_staged();
+    const ffc* res = ffc_stockham(buf, buf + L, L, log2L, buf + 2 * L);
     const double sc = q.D[t];
     const int e = __ldg(off + c + 1);
-    for (int i = __ldg(off + c) + threadIdx.x; i < e; i += LAG_THREADS)
-        rho[t * N_f + __ldg(ck + i)] = sc > 0.0 ? (float)((double)res[__ldg(cm + i)].x * sc) : 0.f;
+    for (int i = __ldg(off + c) + threadIdx.x; i < e; i += blockDim.x) {
+        const ffc v = res[__ldg(cm + i)];
+        rho[t * N_f + __ldg(ck + i)] = sc > 0.0 ? (float)(((double)v.x + (double)v.y) * sc) : 0.f;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -326,9 +368,9 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     // compensated sums: only units of more than one plain run touch them
     const int64_t ctas = std::min<int64_t>(slots, per_chunk * a.n_chunks);
     y->scratch = a.chunk_len > CORR_FLUSH ? al256((size_t)ctas * (y->planes > 1 ? 96 : 32) * CORR_THREADS * sizeof(float)) : 0;
-    y->rows2 = al256(b * y->n_blocks * y->planes * y->G * sizeof(float));
-    y->U = al256(b * (y->planes > 1 ? 2 : 1) * y->G * sizeof(float2));
-    y->h = y->C > 2 ? al256(b * y->n_lags * sizeof(float2)) : 0;
+    y->rows2 = al256(b * y->n_blocks * y->planes * 2 * y->G * sizeof(float));
+    y->U = al256(b * (y->planes > 1 ? 2 : 1) * y->G * sizeof(ffc));
+    y->h = y->C > 1 ? al256(b * y->n_lags * sizeof(ffc)) : 0;
     y->kn = al256(b * plan->Q * knot_rows(plan) * sizeof(KnotRec));
     y->total = y->ab + y->z + y->norm + y->act + y->D + y->raw + y->scratch + y->rows2 + y->U + y->h + y->kn + 256;
 }
@@ -484,8 +526,8 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         float* raw = (float*)take(y.raw);
         float* scratch = (float*)take(y.scratch);
         float* rows2 = (float*)take(y.rows2);
-        float2* U = (float2*)take(y.U);
-        float2* h = (float2*)take(y.h);
+        ffc* U = (ffc*)take(y.U);
+        ffc* h = (ffc*)take(y.h);
         KnotRec* kn = (KnotRec*)take(y.kn);
         int* ctr = (int*)take(256);
         if ((s = launch_knots(plan, t_dev + t0, nb, kn, st, ctr)) != CC_OK) return s;
@@ -525,17 +567,20 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         LagArgs q;
         q.raw = raw;
         q.n_rows = y.n_rows;
+        q.words = 1;
         if (y.n_blocks) {
-            const int64_t len = y.planes * y.G;
-            corr_rows_kernel<<<dim3((unsigned)launch_blocks_for(len, LAG_THREADS), (unsigned)y.n_blocks, (unsigned)nb),
-                               LAG_THREADS, 0, st>>>(raw, y.n_rows, len, rows2);
+            corr_rows_kernel<<<dim3((unsigned)launch_blocks_for(y.planes * y.G, LAG_THREADS), (unsigned)y.n_blocks, (unsigned)nb),
+                               LAG_THREADS, 0, st>>>(raw, y.n_rows, y.planes, q.words, y.G, rows2);
             count_launch();
             q.raw = rows2;
             q.n_rows = y.n_blocks;
+            q.words = 2;
         }
         q.U = U;
-        q.h = y.C > 2 ? h : nullptr;
-        q.twL = y.padded ? plan->corr_tw4096 : plan->corr_twL;
+        q.h = y.C > 1 ? h : nullptr;
+        q.root = y.padded ? plan->corr_root4096 : plan->corr_root;
+        q.g_lo = plan->corr_glo;
+        q.g_hi = plan->corr_ghi;
         q.norm = (const float4*)norm;
         q.D = D;
         q.M = p.M;
@@ -549,19 +594,21 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         q.Q = p.Q;
         q.R = (int)p.R;
         q.pair_mode = p.pair_mode;
-        const size_t sm1 = (size_t)2 * y.L * sizeof(float2), sm2 = (size_t)2 * p.L * sizeof(float2);
-        const int big = (int)(2 * CORR_POINTS * sizeof(float2));
-        if ((sm1 > 48 * 1024 && (e = cudaFuncSetAttribute(corr_lags_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess) ||
-            (sm2 > 48 * 1024 && (e = cudaFuncSetAttribute(corr_rho_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess))
+        const size_t sm1 = (size_t)3 * y.L * sizeof(ffc), sm2 = (size_t)3 * p.L * sizeof(ffc);
+        const int thr1 = std::max(LAG_THREADS, y.L / 4), thr2 = std::max(LAG_THREADS, p.L / 4);
+        const int big = (int)(3 * CORR_POINTS * sizeof(ffc));
+        if ((sm1 > 32 * 1024 && (e = cudaFuncSetAttribute(corr_lags_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess) ||
+            (sm2 > 32 * 1024 && (e = cudaFuncSetAttribute(corr_rho_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big)) != cudaSuccess))
             return cuda_fail(e, "lag kernels smem attribute");
-        corr_lags_kernel<<<dim3((unsigned)(y.C + 1), y.planes > 1 ? 2u : 1u, (unsigned)nb), LAG_THREADS, sm1, st>>>(q);
+        corr_lags_kernel<<<dim3((unsigned)(y.C + 1), y.planes > 1 ? 2u : 1u, (unsigned)nb), thr1, sm1, st>>>(q);
         count_launch();
-        if (y.C > 2) {
+        if (y.C > 1) {
             corr_merge_kernel<<<dim3((unsigned)launch_blocks_for(y.n_lags, LAG_THREADS), (unsigned)nb), LAG_THREADS, 0, st>>>(q);
             count_launch();
         }
-        corr_rho_kernel<<<dim3((unsigned)p.C, (unsigned)nb), LAG_THREADS, sm2, st>>>(
-            q, p.L, p.log2L, p.twL, p.N_FFT, p.b0, p.coset_off, p.coset_k, p.coset_m, p.N_f, rho + t0 * plan->N_f);
+        corr_rho_kernel<<<dim3((unsigned)p.C, (unsigned)nb), thr2, sm2, st>>>(
+            q, p.L, p.log2L, plan->corr_rootL, plan->corr_nlo, plan->corr_nhi, p.N_FFT, p.b0, p.coset_off, p.coset_k, p.coset_m,
+            p.N_f, rho + t0 * plan->N_f);
         count_launch();
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "lag kernels launch");
     }

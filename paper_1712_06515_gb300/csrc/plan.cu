@@ -16,6 +16,7 @@
 
 #include "common.cuh"
 #include "corr.cuh"
+#include "twofloat.cuh"
 
 namespace {
 thread_local std::string g_last_error;
@@ -457,16 +458,20 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
     // The lag grid of the two-pass search (corr.cu), where it serves the plan: G = Cg x Lg points, the
     // same split of the coset twiddles W_G^(c s) and the second pass's twiddles; the 4096-point
     // tables beside them for a plan of shorter transforms that may be tuned to transform_len 4096.
-    std::vector<float2> gp, gp4, gk, gl, g4;
+    // As two floats: the roots of the transforms after the pair kernel, and the powers of the grid's and
+    // of the output grid's root, the first 4096 and every 4096th.
+    std::vector<float2> gp, gp4, gk;
+    std::vector<float4> root, root4, rootL, glo, ghi, nlo, nhi;
     if (cc::lag_grid_supported(p)) {
         const int64_t Lg = 2 * p->N_s <= 4096 ? 2 * L : 4096;
         const int64_t Cg = p->N_s > 4096 ? 2 * ((p->N_s + 4095) / 4096) : 2 * p->N_s <= 4096 ? 1 : 2;
         const bool pad = L < 4096 && C4 > 0;
-        auto roots = [](int64_t n) {
-            std::vector<float2> v(n);
+        auto powers = [](int64_t order, int64_t step, int64_t n) {   // exp(-2 pi i step j / order), j < n
+            std::vector<float4> v((size_t)n);
             for (int64_t j = 0; j < n; ++j) {
-                const double ang = -2.0 * M_PI * (double)j / (double)n;
-                v[j] = make_float2((float)cos(ang), (float)sin(ang));
+                const double ang = -2.0 * M_PI * (double)(step * j % order) / (double)order;
+                const float2 c2 = cc::ff_from(cos(ang)), s2 = cc::ff_from(sin(ang));
+                v[(size_t)j] = make_float4(c2.x, c2.y, s2.x, s2.y);
             }
             return v;
         };
@@ -482,11 +487,18 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
                 for (uint64_t k = 0; k < 16; ++k) gk[c2 * 272 + 16 + 16 * r + k] = w(16 * r * ((uint64_t)Cg * k + c2));
             }
         gp = cc::corr_powers(Lg, Cg);
-        gl = roots(Lg);
+        root = powers(Lg, 1, Lg);
+        if (L != Lg) rootL = powers(L, 1, L);
         if (pad) {
             gp4 = cc::corr_powers(4096, 1);
-            g4 = roots(4096);
+            if (Lg != 4096) root4 = powers(4096, 1, 4096);
         }
+        if (Cg > 1) {
+            glo = powers(Cg * 4096, 1, 4096);
+            ghi = powers(Cg, 1, Cg);
+        }
+        nlo = powers(N, 1, std::min<int64_t>(N, 4096));
+        nhi = powers(N, 4096, std::max<int64_t>(1, N / 4096));
     }
     // coset maps of the 4096-point decomposition (the same as the plan's when L = 4096)
     std::vector<int> off4, ck4, cm4;
@@ -512,11 +524,16 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
         (st = upload(p, twk.data(), twk.size(), &dp.twk)) != CC_OK ||
         (!rtw.empty() && (st = upload(p, rtw.data(), rtw.size(), &p->rows_twp)) != CC_OK) ||
         (!rkm.empty() && (st = upload(p, rkm.data(), rkm.size(), &p->rows_kmap)) != CC_OK) ||
-        (st = upload(p, gk.data(), gk.size(), &p->corr_twk)) != CC_OK ||
-        (st = upload(p, gl.data(), gl.size(), &p->corr_twL)) != CC_OK ||
-        (st = upload(p, gp.data(), gp.size(), &p->corr_twp)) != CC_OK ||
-        (st = upload(p, gp4.data(), gp4.size(), &p->corr_twp4096)) != CC_OK ||
-        (st = upload(p, g4.data(), g4.size(), &p->corr_tw4096)) != CC_OK ||
+        (!root.empty() && ((st = upload(p, gk.data(), gk.size(), &p->corr_twk)) != CC_OK ||
+                           (st = upload(p, gp.data(), gp.size(), &p->corr_twp)) != CC_OK ||
+                           (st = upload(p, root.data(), root.size(), &p->corr_root)) != CC_OK ||
+                           (st = upload(p, nlo.data(), nlo.size(), &p->corr_nlo)) != CC_OK ||
+                           (st = upload(p, nhi.data(), nhi.size(), &p->corr_nhi)) != CC_OK)) ||
+        (!gp4.empty() && (st = upload(p, gp4.data(), gp4.size(), &p->corr_twp4096)) != CC_OK) ||
+        (!rootL.empty() && (st = upload(p, rootL.data(), rootL.size(), &p->corr_rootL)) != CC_OK) ||
+        (!root4.empty() && (st = upload(p, root4.data(), root4.size(), &p->corr_root4096)) != CC_OK) ||
+        (!glo.empty() && ((st = upload(p, glo.data(), glo.size(), &p->corr_glo)) != CC_OK ||
+                          (st = upload(p, ghi.data(), ghi.size(), &p->corr_ghi)) != CC_OK)) ||
         (!off4.empty() && ((st = upload(p, off4.data(), off4.size(), &dp.coset4_off)) != CC_OK ||
                            (st = upload(p, ck4.data(), ck4.size(), &dp.coset4_k)) != CC_OK ||
                            (st = upload(p, cm4.data(), cm4.size(), &dp.coset4_m)) != CC_OK)) ||
@@ -525,6 +542,8 @@ cc_status crosscorr_plan(const cc_config* cfg, const cc_detector* dets, cc_plan*
         return st;
     }
 
+    if (!p->corr_rootL) p->corr_rootL = p->corr_root;
+    if (!p->corr_root4096) p->corr_root4096 = p->corr_root;
     dp.Q = p->Q;
     dp.D = c.D;
     dp.pair_mode = c.pair_mode;

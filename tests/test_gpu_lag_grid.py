@@ -135,3 +135,31 @@ def test_segments_below_the_lag_grid(n_s):
         got = plan.search(torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV)).cpu().numpy()
     for t in range(3):
         assert np.abs(got[t] - ref[t]).max() <= 1e-4 * max(1.0, np.abs(ref[t]).max())
+
+
+def line_ds(freq, amp, n_s, m, n_det=2, pair_mode=0, f_band=0.1, n_t=2):
+    """Noise of unit level and a line of `amp` times that at `freq` cycles a sample in the detector
+    frame, seen by templates of no orbit from the barycentre itself: the line keeps its frequency
+    (the samples go in as FP32 values on both sides)."""
+    tm = np.stack([np.zeros(n_t), np.full(n_t, 1.13e9), np.full(n_t, 68023.7)], 1)
+    ds = synth.tiny(seed=91, n_samples=n_s * m, T_sft=n_s / 2.0 if n_s % 2 == 0 else float(n_s), T_short=float(n_s), T_max=float(n_s), f_band=f_band, templates=tm, n_det=n_det,
+                    pair_mode=pair_mode, duty=0.8, mean_lock_s=3.0 * n_s, zero_roemer=True, sigma_jitter=0.0)
+    line = amp * np.exp(2j * np.pi * ((freq * np.arange(n_s * m)) % 1.0))
+    ds.x = (ds.x + np.where(ds.x != 0, line, 0)).astype(np.complex64).astype(np.complex128)
+    return ds
+
+
+@pytest.mark.parametrize("amp", [3.0, 10.0])
+@pytest.mark.parametrize("n_s,m,n_det,mode", [(128, 160, 2, 0), (600, 64, 2, 0), (600, 64, 2, 2), (3000, 24, 2, 0), (3000, 24, 2, 2), (4098, 12, 2, 0), (9000, 8, 2, 0),
+                                              (600, 40, 3, 0), (3000, 12, 4, 0)])
+def test_line_outside_the_band(n_s, m, n_det, mode, amp):
+    """A line far outside the searched band, louder than the noise, leaves rho in the band at the
+    FP32 bar: the transforms between the sums at all frequencies and the output bins carry more
+    than FP32 (there the line's rounding would reach every bin, 1e-2 to 1 in rho at these levels)."""
+    ds = line_ds(0.43, amp, n_s, m, n_det, mode)
+    ref = oracle.rho(ds)
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        got = plan.search(torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV)).cpu().numpy()
+        plan.check()
+    for t in range(2):
+        assert np.abs(got[t] - ref[t]).max() <= 1e-4 * max(1.0, np.abs(ref[t]).max())
