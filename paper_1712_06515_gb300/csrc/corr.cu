@@ -66,7 +66,7 @@ constexpr int ROW_BLOCK = 32;        // partial rows summed by one block of corr
 
 // What the kernels after corr_kernel need.
 struct LagArgs {
-    const float* raw;       // [n_t][n_rows][planes][words][G]: partial sums (words 2: and what they round off)
+    const float* raw;       // [n_t][n_rows][planes][2][G]: partial sums and what they round off
     ffc* U;                 // [n_t][planes > 1 ? 2 : 1][C][L]: per coset the inverse transform of A and B
     ffc* h;                 // [n_t][n_lags] (C > 1)
     const ffc* root;        // exp(-2 pi i j / L)
@@ -74,30 +74,37 @@ struct LagArgs {
     const float4* norm;     // [n_t][Q][M]
     double* D;              // [n_t] sqrt(2 / normalisation), 0 without weight
     int64_t M;
-    int L, log2L, C, planes, words, n_rows, n_lags, N_s, Q, R, pair_mode;
+    int L, log2L, C, planes, n_rows, n_lags, N_s, Q, R, pair_mode;
 };
 
-// One partial row's value at p, its second word at p + lo (lo = 0: none)
-__device__ __forceinline__ ff row_value(const float* __restrict__ p, size_t lo) {
-    return make_float2(__ldg(p), lo ? __ldg(p + lo) : 0.f);
-}
+// One partial row's value at p, its second word G further on
+__device__ __forceinline__ ff row_value(const float* __restrict__ p, size_t G) { return make_float2(__ldg(p), __ldg(p + G)); }
 
-// Sum of ROW_BLOCK partial rows (few templates have many): out [n_t][gridDim.y][planes][2][G].
+// Sum of ROW_BLOCK partial rows (few templates have many): out [n_t][gridDim.y][planes][2][G], four
+// neighbouring values a thread.
 __global__ void __launch_bounds__(LAG_THREADS)
-corr_rows_kernel(const float* __restrict__ raw, int n_rows, int planes, int words, int64_t G, float* __restrict__ out) {
-    const int64_t i = (int64_t)blockIdx.x * LAG_THREADS + threadIdx.x, t = blockIdx.z;
+corr_rows_kernel(const float* __restrict__ raw, int n_rows, int planes, int G, float* __restrict__ out) {
+    const int i = 4 * (blockIdx.x * LAG_THREADS + threadIdx.x);
+    const size_t t = blockIdx.z;
     if (i >= planes * G) return;
-    const int64_t pl = i / G, m = i - pl * G;
+    const int pl = i / G, m = i - pl * G;
     const int r0 = blockIdx.y * ROW_BLOCK, r1 = min(n_rows, r0 + ROW_BLOCK);
-    const size_t stride = (size_t)planes * words * G;
-    const float* p = raw + (size_t)t * n_rows * stride + pl * words * G + m;
-    const size_t lo = words > 1 ? G : 0;
-    ff s = make_float2(0.f, 0.f);
-#pragma unroll 8
-    for (int r = r0; r < r1; ++r) s = ff_add(s, row_value(p + r * stride, lo));
-    float* const o = out + (((size_t)t * gridDim.y + blockIdx.y) * planes + pl) * 2 * G + m;
-    o[0] = s.x;
-    o[G] = s.y;
+    const size_t stride = (size_t)planes * 2 * G;
+    const float* p = raw + t * n_rows * stride + (size_t)pl * 2 * G + m;
+    ff s[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int r = r0; r < r1; ++r) {
+        const float4 h = __ldg((const float4*)(p + r * stride)), l = __ldg((const float4*)(p + r * stride + G));
+        s[0] = ff_add(s[0], make_float2(h.x, l.x));
+        s[1] = ff_add(s[1], make_float2(h.y, l.y));
+        s[2] = ff_add(s[2], make_float2(h.z, l.z));
+        s[3] = ff_add(s[3], make_float2(h.w, l.w));
+    }
+    float* const o = out + ((t * gridDim.y + blockIdx.y) * planes + pl) * 2 * (size_t)G + m;
+    *(float4*)o = make_float4(s[0].x, s[1].x, s[2].x, s[3].x);
+    *(float4*)(o + G) = make_float4(s[0].y, s[1].y, s[2].y, s[3].y);
 }
 
 // The L roots of a block's transform into shared memory, under the loads of its input, and the
@@ -146,7 +153,7 @@ corr_lags_kernel(const LagArgs q) {
         }
         return;
     }
-    const size_t G = (size_t)q.C * q.L, plane = q.words * G, stride = q.planes * plane, lo = q.words > 1 ? G : 0;
+    const size_t G = (size_t)q.C * q.L, plane = 2 * G, stride = q.planes * plane;
     const float* p0 = q.raw + t * q.n_rows * stride + (size_t)c * q.L;
     stage_roots(buf + 2 * q.L, q.root, q.L);
     // the inverse transform as the conjugate of the forward one of the conjugate
@@ -155,12 +162,12 @@ corr_lags_kernel(const LagArgs q) {
         ff re = make_float2(0.f, 0.f), im = re;
         if (ser == 0) {
 #pragma unroll 8
-            for (int r = 0; r < q.n_rows; ++r) re = ff_add(re, row_value(p + r * stride, lo));
+            for (int r = 0; r < q.n_rows; ++r) re = ff_add(re, row_value(p + r * stride, G));
         } else {
 #pragma unroll 4
             for (int r = 0; r < q.n_rows; ++r) {
-                re = ff_add(re, row_value(p + r * stride, lo));
-                im = ff_add(im, row_value(p + r * stride + plane, lo));
+                re = ff_add(re, row_value(p + r * stride, G));
+                im = ff_add(im, row_value(p + r * stride + plane, G));
             }
         }
         buf[m] = ffc_make(re, ff_neg(im));
@@ -254,7 +261,7 @@ struct CorrLayout {
     int64_t G, t_pad;
     CorrArgs a;
     // workspace pieces of a batch, bytes
-    size_t ab, z, norm, act, D, raw, scratch, rows2, U, h, kn, total;
+    size_t ab, z, norm, act, D, raw, rows2, U, h, kn, total;
 };
 
 std::vector<float2> corr_powers(int64_t L, int64_t C) {
@@ -331,11 +338,15 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     a.off_bar = (uint32_t)o;
     a.smem = (uint32_t)(o + 16);
     // Chunks of segments: units are equal, handed out one by one to two CTAs per SM, each
-    // rereads its first segment's predecessor (R = 1) and writes one row (about the traffic of
-    // another segment): the count with the least ceil(units / slots) (length + overhead); with
-    // cc_tuning.chunk_waves, that many units per slot, at most M / (4 R + 1) chunks.
+    // rereads its first segment's predecessor (R = 1) and writes one row (98 KB with a lag, written
+    // and read again: about the time of four segments): the count with the least
+    // ceil(units / slots) (length + overhead); with cc_tuning.chunk_waves, that many units per
+    // slot, at most M / (4 R + 1) chunks.
     const int64_t slots = (int64_t)CORR_CTAS_PER_SM * sm_count();
     const int64_t per_chunk = (2 * n_t + y->T - 1) / y->T * y->C;
+    // rows beyond ROW_BLOCK are summed first (a launch, about three segments' time) where the blocks
+    // of corr_lags_kernel do not fill the chip
+    const bool pre_sum = n_t * y->C * (y->planes > 1 ? 2 : 1) < sm_count();
     const int64_t minch = (p.M + CORR_MAX_CHUNK - 1) / CORR_MAX_CHUNK;
     const int64_t maxch = std::max<int64_t>(minch, p.M);
     int64_t nch = minch;
@@ -346,8 +357,7 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
         int64_t best = -1;
         for (int64_t n = minch; n <= most; n += 1 + n / 16) {
             const int64_t len = (p.M + n - 1) / n, waves = (per_chunk * ((p.M + len - 1) / len) + slots - 1) / slots;
-            // more rows than a block of corr_rows_kernel takes cost that launch, about three segments' time
-            const int64_t cost = waves * (len + p.R + 1) + (2 * n > ROW_BLOCK ? 3 : 0);
+            const int64_t cost = waves * (len + p.R + (y->planes > 1 ? 4 : 2)) + (2 * n > ROW_BLOCK && pre_sum ? 3 : 0);
             if (best < 0 || cost < best) {
                 best = cost;
                 nch = n;
@@ -357,22 +367,19 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     a.chunk_len = (int)((p.M + nch - 1) / nch);
     a.n_chunks = (int)((p.M + a.chunk_len - 1) / a.chunk_len);
     y->n_rows = 2 * a.n_chunks;
-    y->n_blocks = y->n_rows > ROW_BLOCK ? (y->n_rows + ROW_BLOCK - 1) / ROW_BLOCK : 0;
+    y->n_blocks = y->n_rows > ROW_BLOCK && pre_sum ? (y->n_rows + ROW_BLOCK - 1) / ROW_BLOCK : 0;
     const size_t b = (size_t)n_t;
     y->ab = al256(b * plan->Q * 2 * plan->N_tau * (plan->cfg.store == CC_STORE_BF16 ? 4 : 8));
     y->z = y->folded ? al256(b * plan->Q * 2 * plan->M * y->G * esz) : 0;
     y->norm = al256(b * plan->Q * plan->M * sizeof(float4));
     y->act = al256((size_t)plan->Q * plan->M * y->t_pad);
     y->D = al256(b * sizeof(double));
-    y->raw = al256(b * y->n_rows * y->planes * y->G * sizeof(float));
-    // compensated sums: only units of more than one plain run touch them
-    const int64_t ctas = std::min<int64_t>(slots, per_chunk * a.n_chunks);
-    y->scratch = a.chunk_len > CORR_FLUSH ? al256((size_t)ctas * (y->planes > 1 ? 96 : 32) * CORR_THREADS * sizeof(float)) : 0;
+    y->raw = al256(b * y->n_rows * y->planes * 2 * y->G * sizeof(float));
     y->rows2 = al256(b * y->n_blocks * y->planes * 2 * y->G * sizeof(float));
     y->U = al256(b * (y->planes > 1 ? 2 : 1) * y->G * sizeof(ffc));
     y->h = y->C > 1 ? al256(b * y->n_lags * sizeof(ffc)) : 0;
     y->kn = al256(b * plan->Q * knot_rows(plan) * sizeof(KnotRec));
-    y->total = y->ab + y->z + y->norm + y->act + y->D + y->raw + y->scratch + y->rows2 + y->U + y->h + y->kn + 256;
+    y->total = y->ab + y->z + y->norm + y->act + y->D + y->raw + y->rows2 + y->U + y->h + y->kn + 256;
 }
 
 // Templates per batch: as many as the budget of a_r, b_r and folded rows holds.
@@ -524,7 +531,6 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         uint8_t* act = (uint8_t*)take(y.act);
         double* D = (double*)take(y.D);
         float* raw = (float*)take(y.raw);
-        float* scratch = (float*)take(y.scratch);
         float* rows2 = (float*)take(y.rows2);
         ffc* U = (ffc*)take(y.U);
         ffc* h = (ffc*)take(y.h);
@@ -544,7 +550,6 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         a.src = y.folded ? z : ab;
         a.act = act;
         a.raw = raw;
-        a.scratch = scratch;
         a.ctr = ctr;
         a.err = p.err;
         a.twk = plan->corr_twk;
@@ -567,14 +572,12 @@ cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, 
         LagArgs q;
         q.raw = raw;
         q.n_rows = y.n_rows;
-        q.words = 1;
         if (y.n_blocks) {
-            corr_rows_kernel<<<dim3((unsigned)launch_blocks_for(y.planes * y.G, LAG_THREADS), (unsigned)y.n_blocks, (unsigned)nb),
-                               LAG_THREADS, 0, st>>>(raw, y.n_rows, y.planes, q.words, y.G, rows2);
+            corr_rows_kernel<<<dim3((unsigned)launch_blocks_for(y.planes * y.G, 4 * LAG_THREADS), (unsigned)y.n_blocks, (unsigned)nb),
+                               LAG_THREADS, 0, st>>>(raw, y.n_rows, y.planes, (int)y.G, rows2);
             count_launch();
             q.raw = rows2;
             q.n_rows = y.n_blocks;
-            q.words = 2;
         }
         q.U = U;
         q.h = y.C > 1 ? h : nullptr;

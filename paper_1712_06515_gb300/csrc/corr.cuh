@@ -9,7 +9,6 @@ namespace cc {
 
 constexpr int CORR_THREADS = 256;
 constexpr int CORR_MAX_CHUNK = 1023;    // segments of a chunk (its activity words, and one before, are kept on chip)
-constexpr int CORR_FLUSH = 16;          // segments of a plain FP32 run of the sums
 constexpr int CORR_POINTS = 4096;   // points of one CTA's transforms: 4096 / L of L points each
 
 // T transforms a CTA: elements of an exchange buffer (T = 1: padded), activity bits of a detector
@@ -22,8 +21,7 @@ __host__ __device__ constexpr int corr_act_bytes(int T) { return T == 1 ? 1 : 4;
 struct CorrArgs {
     const void* src;        // a_r, b_r [n_t][Q][2][N_tau], or folded rows Z [n_t][Q][2][M][C][4096]
     const uint8_t* act;     // [Q][M][t_pad]: the detector has weight in (segment, template)
-    float* raw;             // [n_t][2 n_chunks][planes][C][L] partial sums (planes: A, and Re B, Im B with a lag)
-    float* scratch;         // [CTAs][48 or 16 sums][2][256] compensated sums of a CTA's unit
+    float* raw;             // [n_t][2 n_chunks][planes][2][C][L] partial sums and what they round off (planes: A, and Re B, Im B with a lag)
     int* ctr;               // unit counter, zero at launch
     unsigned* err;          // the plan's device error word
     const float2* twk;      // [C][272] coset and second-pass twiddles on the grid of G = C L points

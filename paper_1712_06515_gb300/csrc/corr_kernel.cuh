@@ -13,8 +13,9 @@
 // detectors, the kernel accumulates over segments, per template and weight,
 //   A(j) = sum_K sum_(X<Y) Re(conj(T_YK) T_XK)   (|S_K|^2 with every ordered pair), real,
 //   B(j) = sum_K conj(S_K) S_(K-1)     (R = 1), complex,
-// each in FP32: at most CORR_FLUSH segments plainly, those sums compensated (a run of that
-// length rounds to a twentieth of what the transforms' own rounding leaves in its terms).
+// each compensated at every segment, and left as two floats: the value and what it rounds off
+// (the sums after it carry those, corr.cu; a line just outside the band leaves in rho what sums
+// at the output bins leave there, five times that with plain runs of 16 segments).
 //
 // A CTA of 256 threads holds 4096 points, 16 per thread: T = 4096 / L transforms of L
 // points, each one (template, weight) series (L = 4096: one).  G = L for N_s <= 2048
@@ -29,13 +30,11 @@
 //   * the rows of the next (detector, segment) arrive by cp.async.bulk (TMA) on an mbarrier
 //     under the current transform's later passes (16-byte rows; otherwise by 8- or 4-byte
 //     cp.async);
-//   * the running sums, S_(K-1) and detector 0's spectrum -- 112 words per thread -- live in
-//     tensor memory, 32 columns per group of four bins, read and written by tcgen05.ld/st once
-//     per segment: registers hold only the transform (16 points), so two CTAs of 128 registers
-//     fit an SM.  MULTI (three or four detectors) keeps the sum of the earlier detectors in
-//     registers; without a lag so are the sums (16 words) and detector 0's spectrum;
-//   * the compensated sums of a unit sit in global memory (L2), a slot per CTA, touched every
-//     CORR_FLUSH segments;
+//   * the running sums, their compensations and S_(K-1) -- 128 words per thread -- live in
+//     tensor memory, 32 columns per group of four bins (8 without a lag), read and written by
+//     tcgen05.ld/st once per segment: registers hold only the transform (16 points) and detector
+//     0's spectrum (MULTI, three or four detectors: the sum of the earlier ones), so two CTAs of
+//     128 registers fit an SM;
 //   * twiddles as in the staged kernel: the coset factor of sample s = t + 256 r is split
 //     between a factor per r (first pass) and the table of the second and the powers of the
 //     last pass.  The coset's tables (10 KB) are kept in shared memory: read through L1, whose
@@ -45,9 +44,9 @@
 //
 // What bounds it (L = 4096): instruction issue (64 to 70 % of the slots with 16 warps per SM), the
 // FP32 pipe (54 %) and the shared-memory exchanges (55 %) together.  120-day band (N_s = 3600,
-// 2880 segments, two detectors), 72 templates at once, per template: 144 us; 151 with XOR-swizzled
-// exchanges, 161 with every sum compensated at every segment, 174 with three barriers a
-// transform, 640 at the output bins (8 transforms of 4096 points a row instead of 2).
+// 2880 segments, two detectors), 72 templates at once, per template: 151 us; 158 with XOR-swizzled
+// exchanges, 181 with three barriers a transform, 640 at the output bins (8 transforms of 4096
+// points a row instead of 2).  (Plain FP32 runs of 16 segments take 144 us and lose precision.)
 //
 // Waits are bounded (about one second): a wait that runs out sets bit 0 of the plan's error
 // word; the CTA agrees on it at the next barrier, waits for its copies in flight, frees its
@@ -105,6 +104,14 @@ __device__ __forceinline__ void twiddle_powers(float2 (&x)[16], const float2 (&w
     }
 }
 
+// Compensated sums of two FP32 values in paired operations (the same rounding as kahan_add
+// on each): y = v - c, t = s + y, c = (t - s) - y.
+__device__ __forceinline__ void kahan2(float2& s, float2& c, float2 v) {
+    const float2 y = csub(v, c), t = cadd(s, y);
+    c = csub(csub(t, s), y);
+    s = t;
+}
+
 // The TA activity bytes (0 or 1) at p, aligned to TA, of which the first `valid` count, as bits.
 template <int TA>
 __device__ __forceinline__ uint32_t act_bits(const uint8_t* p, int valid) {
@@ -120,10 +127,9 @@ __global__ void __launch_bounds__(CORR_THREADS, CORR_CTAS_PER_SM)
 corr_kernel(const CorrArgs q) {
     using S = CorrShape<LT>;
     constexpr int L = S::L, T = S::T, GT = S::GT, RL = S::RL, NSL = S::NSL, BPT = S::BPT, TA = S::TA, NP = S::NP;
-    // tensor-memory words per group of four bins: A [4], B [4] re im, S of the segment before
-    // [4], detector 0's spectrum [4] (F0T)
-    constexpr bool F0T = LAG && !MULTI;
-    constexpr int W = 32, OF = 20;
+    // tensor-memory words per group of four bins: A [4], its compensations [4]; LAG: per bin B re im,
+    // its compensations, S of the segment before
+    constexpr int W = LAG ? 32 : 8;
     constexpr uint32_t COLS = 8 * W;                 // two warps of a lane quarter, four groups each
     constexpr uint32_t ESZ = BF16 ? 4 : 8;
     constexpr int PLANES = LAG ? 3 : 1;
@@ -157,7 +163,7 @@ corr_kernel(const CorrArgs q) {
     const int C = q.C, M = q.M;
     const size_t act_x = (size_t)M * q.t_pad;        // bytes of one detector's activity
 
-    if (LAG && warp == 0) tmem_alloc(&s_tmem, COLS);
+    if (warp == 0) tmem_alloc(&s_tmem, COLS);
     if (tid == 0) {
         mbar_init(bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -171,7 +177,7 @@ corr_kernel(const CorrArgs q) {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tm_base = LAG ? s_tmem : 0u;
+    const uint32_t tm_base = s_tmem;
     const uint32_t tm = tm_base + ((uint32_t)(warp & 3) << 21) + (uint32_t)(warp >> 2) * (COLS / 2);
     const uint32_t own_bit = T > 1 ? 1u << (g >> 1) : 1u;
     uint32_t phase = 0;
@@ -266,63 +272,13 @@ corr_kernel(const CorrArgs q) {
             }
         };
 
-        float sA[16];           // !LAG: the sums
-        if constexpr (LAG) {    // zero sums
+        {   // zero sums
             float z[W];
 #pragma unroll
             for (int i = 0; i < W; ++i) z[i] = 0.f;
 #pragma unroll
             for (int gi = 0; gi < 4; ++gi) tmem_st(tm + gi * W, z);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) sA[e] = 0.f;
         }
-        bool flushed = false;   // the unit's compensated sums hold something
-        int run = 0;            // segments in the plain sums
-        // the plain sums into the compensated ones; the last time the totals go to the row buffer
-        float* const acc = q.scratch + (size_t)blockIdx.x * (LAG ? 96 : 32) * CORR_THREADS + tid;
-        float* const fl = (float*)ex;
-        constexpr int FP = CORR_POINTS + CORR_POINTS / 16;
-        auto put = [&](bool final, int e, int n, int pl, float val) {   // sum n of the thread: element e, plane pl
-            float* const p = acc + (size_t)2 * n * CORR_THREADS;
-            float sum = val, comp = 0.f;
-            if (flushed) {
-                sum = p[0];
-                comp = p[CORR_THREADS];
-                kahan_add(sum, comp, val);
-            }
-            if (final) {
-                const int b = e / RL, m = g * L + (S::PASS2 ? 16 * (i0 + RL * b) + k : j + GT * b) + NSL * (e % RL);
-                fl[pl * FP + m + (m >> 4)] = sum;
-            } else {
-                p[0] = sum;
-                p[CORR_THREADS] = comp;
-            }
-        };
-        auto flush = [&](bool final) {
-            if constexpr (LAG) {
-                tmem_wait_st();
-#pragma unroll 1
-                for (int gi = 0; gi < 4; ++gi) {
-                    float z[W];
-                    tmem_ld(z, tm + gi * W);
-#pragma unroll
-                    for (int n = 0; n < 12; ++n) {
-                        put(final, 4 * gi + (n < 4 ? n : (n - 4) >> 1), gi * 12 + n, n < 4 ? 0 : 1 + ((n - 4) & 1), z[n]);
-                        z[n] = 0.f;
-                    }
-                    if (!final) tmem_st(tm + gi * W, z);
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    put(final, e, e, 0, sA[e]);
-                    sA[e] = 0.f;
-                }
-            }
-            flushed = true;
-            run = 0;
-        };
         if (!(q.wait_test && first_unit)) issue_after(Kl, -1);
         first_unit = false;
         bool prev_zero = true;
@@ -335,16 +291,10 @@ corr_kernel(const CorrArgs q) {
                 continue;
             }
             const bool acc_on = !LAG || K >= Ka;
-            if (acc_on && ++run > CORR_FLUSH) {
-                flush(false);
-                run = 1;
-            }
-            float2 v[16], f0[16];   // f0 (unless F0T): detector 0's spectrum, MULTI: the earlier ones' sum
-            bool have = false;      // an earlier detector's spectrum is kept
-            if constexpr (!F0T) {
+            float2 v[16], f0[16];   // f0: detector 0's spectrum, MULTI: the earlier ones' sum
+            bool have = false;      // f0 holds something
 #pragma unroll
-                for (int e = 0; e < 16; ++e) f0[e] = make_float2(0.f, 0.f);
-            }
+            for (int e = 0; e < 16; ++e) f0[e] = make_float2(0.f, 0.f);
 #pragma unroll 1
             for (int X = 0; X < q.Q; ++X) {
                 const uint32_t xbits = (bits >> (X * SH)) & ((1u << SH) - 1u);
@@ -433,98 +383,117 @@ corr_kernel(const CorrArgs q) {
                 if constexpr (MULTI) {
                     // this detector's pairs with the earlier ones, then their sum
                     if (have && acc_on && !q.all_ordered) {
-                        if constexpr (LAG) {
-                            tmem_wait_st();
+                        tmem_wait_st();
 #pragma unroll
-                            for (int gi = 0; gi < 4; ++gi) {
-                                float z[8];
-                                tmem_ld(z, tm + gi * W);
+                        for (int gi = 0; gi < 4; ++gi) {
+                            float z[8];
+                            tmem_ld(z, tm + gi * W);
 #pragma unroll
-                                for (int i = 0; i < 4; ++i)
-                                    z[i] = fmaf(v[4 * gi + i].x, f0[4 * gi + i].x, fmaf(v[4 * gi + i].y, f0[4 * gi + i].y, z[i]));
-                                tmem_st(tm + gi * W, z);
+                            for (int h = 0; h < 2; ++h) {
+                                const int e = 4 * gi + 2 * h;
+                                float2 s = make_float2(z[2 * h], z[2 * h + 1]), cp = make_float2(z[4 + 2 * h], z[5 + 2 * h]);
+                                kahan2(s, cp, make_float2(redot(v[e], f0[e]), redot(v[e + 1], f0[e + 1])));
+                                z[2 * h] = s.x;
+                                z[2 * h + 1] = s.y;
+                                z[4 + 2 * h] = cp.x;
+                                z[5 + 2 * h] = cp.y;
                             }
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) sA[e] = fmaf(v[e].x, f0[e].x, fmaf(v[e].y, f0[e].y, sA[e]));
+                            tmem_st(tm + gi * W, z);
                         }
                     }
                     have = true;
 #pragma unroll
                     for (int e = 0; e < 16; ++e) f0[e] = cadd(f0[e], v[e]);
                 } else if (X + 1 < q.Q && (bits >> SH) != 0) {   // the second detector pairs with this one
-                    if constexpr (F0T) {
 #pragma unroll
-                        for (int gi = 0; gi < 4; ++gi) {
-                            float z[8];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                z[2 * i] = v[4 * gi + i].x;
-                                z[2 * i + 1] = v[4 * gi + i].y;
-                            }
-                            tmem_st(tm + gi * W + OF, z);
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) f0[e] = v[e];
-                    }
+                    for (int e = 0; e < 16; ++e) f0[e] = v[e];
                     have = true;
                 }
             }
             if (failed) break;
             // pair terms of segment K
-            if constexpr (LAG) {
+            const bool same = acc_on && (q.all_ordered || (!MULTI && have));   // terms of A
+            if (LAG || same) {
                 tmem_wait_st();
 #pragma unroll
                 for (int gi = 0; gi < 4; ++gi) {
                     float z[W];
                     tmem_ld(z, tm + gi * W);
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int e = 4 * gi + i;
-                        float2 Sk = MULTI ? f0[e] : v[e];
-                        if (!MULTI && have) {
-                            const float2 f = F0T ? make_float2(z[OF + 2 * i], z[OF + 2 * i + 1]) : f0[e];
-                            Sk = cadd(f, v[e]);
-                            if (acc_on && !q.all_ordered) z[i] = fmaf(v[e].x, f.x, fmaf(v[e].y, f.y, z[i]));
+                    for (int h = 0; h < 2; ++h) {
+                        const int e = 4 * gi + 2 * h;
+                        float2 Sk[2];
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) Sk[i] = MULTI ? f0[e + i] : cadd(f0[e + i], v[e + i]);
+                        if (same) {
+                            const float2 d = q.all_ordered ? make_float2(redot(Sk[0], Sk[0]), redot(Sk[1], Sk[1]))
+                                                           : make_float2(redot(v[e], f0[e]), redot(v[e + 1], f0[e + 1]));
+                            float2 s = make_float2(z[2 * h], z[2 * h + 1]), cp = make_float2(z[4 + 2 * h], z[5 + 2 * h]);
+                            kahan2(s, cp, d);
+                            z[2 * h] = s.x;
+                            z[2 * h + 1] = s.y;
+                            z[4 + 2 * h] = cp.x;
+                            z[5 + 2 * h] = cp.y;
                         }
-                        if (acc_on && q.all_ordered) z[i] = fmaf(Sk.x, Sk.x, fmaf(Sk.y, Sk.y, z[i]));
-                        float* const B = z + 4 + 2 * i;
-                        float* const P = z + 12 + 2 * i;
-                        if (acc_on && !prev_zero) {
-                            B[0] = fmaf(Sk.x, P[0], fmaf(Sk.y, P[1], B[0]));
-                            B[1] = fmaf(Sk.x, P[1], fmaf(-Sk.y, P[0], B[1]));
+                        if constexpr (LAG) {
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                float* const B = z + 8 + 6 * (2 * h + i);
+                                if (acc_on && !prev_zero) {
+                                    const float2 d = make_float2(redot(Sk[i], make_float2(B[4], B[5])),
+                                                                 fmaf(Sk[i].x, B[5], -Sk[i].y * B[4]));
+                                    float2 s = make_float2(B[0], B[1]), cp = make_float2(B[2], B[3]);
+                                    kahan2(s, cp, d);
+                                    B[0] = s.x;
+                                    B[1] = s.y;
+                                    B[2] = cp.x;
+                                    B[3] = cp.y;
+                                }
+                                B[4] = Sk[i].x;
+                                B[5] = Sk[i].y;
+                            }
                         }
-                        P[0] = Sk.x;
-                        P[1] = Sk.y;
                     }
                     tmem_st(tm + gi * W, z);
                 }
-            } else if (q.all_ordered) {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const float2 Sk = MULTI ? f0[e] : cadd(f0[e], v[e]);
-                    sA[e] = fmaf(Sk.x, Sk.x, fmaf(Sk.y, Sk.y, sA[e]));
-                }
-            } else if (!MULTI && have) {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) sA[e] = fmaf(v[e].x, f0[e].x, fmaf(v[e].y, f0[e].y, sA[e]));
             }
             prev_zero = false;
         }
         if (failed) break;
-        // the unit's sums to its row, through the exchange buffers (padded) for whole lines
-        __syncthreads();   // every thread has left the last transform's buffers
-        flush(true);
-        __syncthreads();
+        // the unit's sums to its row, through the exchange buffers (padded) for whole lines: the
+        // values, then what they round off
+        float* const fl = (float*)ex;
+        constexpr int FP = CORR_POINTS + CORR_POINTS / 16;
+        tmem_wait_st();
+#pragma unroll 1
+        for (int part = 0; part < 2; ++part) {
+            __syncthreads();   // every thread has left the last transform's buffers (read the part before)
 #pragma unroll
-        for (int pl = 0; pl < PLANES; ++pl)
-            for (int o = tid; o < CORR_POINTS; o += CORR_THREADS) {
-                const int so = sg * T + o / L, to = so >> 1;
-                if (to < q.n_t)
-                    q.raw[((((size_t)to * 2 * q.n_chunks + (size_t)(so & 1) * q.n_chunks + chunk) * PLANES + pl) * C + c) * L + o % L] =
-                        fl[pl * FP + o + (o >> 4)];
+            for (int gi = 0; gi < 4; ++gi) {
+                float z[W];
+                tmem_ld(z, tm + gi * W);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int e = 4 * gi + i, b = e / RL;
+                    const int m = g * L + (S::PASS2 ? 16 * (i0 + RL * b) + k : j + GT * b) + NSL * (e % RL), o = m + (m >> 4);
+                    fl[o] = part ? -z[4 + i] : z[i];
+                    if constexpr (LAG) {
+                        const float* const B = z + 8 + 6 * i;
+                        fl[FP + o] = part ? -B[2] : B[0];
+                        fl[2 * FP + o] = part ? -B[3] : B[1];
+                    }
+                }
             }
+            __syncthreads();
+#pragma unroll
+            for (int pl = 0; pl < PLANES; ++pl)
+                for (int o = tid; o < CORR_POINTS; o += CORR_THREADS) {
+                    const int so = sg * T + o / L, to = so >> 1;
+                    if (to < q.n_t)
+                        q.raw[((((size_t)to * 2 * q.n_chunks + (size_t)(so & 1) * q.n_chunks + chunk) * 2 * PLANES + 2 * pl + part) * C + c) * L + o % L] =
+                            fl[pl * FP + o + (o >> 4)];
+                }
+        }
         __syncthreads();   // the next unit's first pass rewrites the buffers
     }
     if (failed && tid == 0) {
@@ -532,7 +501,7 @@ corr_kernel(const CorrArgs q) {
         mbar_wait(bar, phase ^ 1);   // the copy still in flight, bounded
     }
     __syncthreads();
-    if (LAG && warp == 0) tmem_free(tm_base, COLS);
+    if (warp == 0) tmem_free(tm_base, COLS);
 }
 
 template <int LT, bool BF16, bool LAG, bool HALF, bool MULTI>

@@ -163,3 +163,22 @@ def test_line_outside_the_band(n_s, m, n_det, mode, amp):
         plan.check()
     for t in range(2):
         assert np.abs(got[t] - ref[t]).max() <= 1e-4 * max(1.0, np.abs(ref[t]).max())
+
+
+@pytest.mark.parametrize("n_s,m,amp", [(600, 256, 3.0), (128, 1000, 1.0)])
+def test_line_beside_the_band(n_s, m, amp):
+    """A line just outside the band leaks into it, so the rounding of the sums at its frequency is
+    seen there: with sums compensated at every segment and kept as two floats the error is that of
+    sums at the output bins (the one-pass kernel) and no more than half as much again; plain FP32
+    runs of 16 segments left twice as much.  Chunks of 50 segments and more, equal templates."""
+    ds = line_ds(0.26, amp, n_s, m, f_band=0.5, n_t=64)
+    ref = oracle.rho(ds, templates=ds.templates[:1])[0]
+    x, tm = torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV)
+    rms = {}
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        plan.set_tuning(chunk_waves=1)
+        for path in (cc.PATH_TWO_PASS, cc.PATH_FUSED):
+            plan.set_path(path)
+            rms[path] = np.sqrt(((plan.search(x, tm)[0].cpu().numpy() - ref) ** 2).mean())
+        plan.check()
+    assert rms[cc.PATH_TWO_PASS] <= 1.5 * rms[cc.PATH_FUSED]
