@@ -44,8 +44,8 @@
 //
 // What bounds it (L = 4096): instruction issue (64 to 70 % of the slots with 16 warps per SM), the
 // FP32 pipe (54 %) and the shared-memory exchanges (55 %) together.  120-day band (N_s = 3600,
-// 2880 segments, two detectors), 72 templates at once, per template: 151 us; 158 with XOR-swizzled
-// exchanges, 181 with three barriers a transform, 640 at the output bins (8 transforms of 4096
+// 2880 segments, two detectors), 72 templates at once, per template: 151 us; 161 with XOR-swizzled
+// exchanges, 174 with three barriers a transform, 640 at the output bins (8 transforms of 4096
 // points a row instead of 2).  (Plain FP32 runs of 16 segments take 144 us and lose precision.)
 //
 // Waits are bounded (about one second): a wait that runs out sets bit 0 of the plan's error
