@@ -496,11 +496,15 @@ corr_kernel(const CorrArgs q) {
         }
         __syncthreads();   // the next unit's first pass rewrites the buffers
     }
+    // a failed wait leaves stores under way: every warp's are complete before tensor memory is freed
+    tmem_wait_st();
     if (failed && tid == 0) {
         atomicOr(q.err, 1u);
         mbar_wait(bar, phase ^ 1);   // the copy still in flight, bounded
     }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0) tmem_free(tm_base, COLS);
 }
 

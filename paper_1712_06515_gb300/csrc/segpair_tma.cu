@@ -284,6 +284,8 @@ segpair_tma_kernel(const PairArgs q) {
         for (int i = tid; i < nbc; i += TT_THREADS) out[__ldg(q.coset_k + o + i)] = accm[__ldg(q.coset_m + o + i)];
         // the next unit's first pass rewrites the buffer: the unit fetch's barrier orders it
     }
+    // a failed wait leaves stores under way: every warp's are complete before tensor memory is freed
+    tmem_wait_st();
     if (failed && tid == 0) {
         atomicOr(q.err, 1u);
         for (int s = 0; s < 2; ++s)   // copies still in flight, bounded
@@ -291,6 +293,7 @@ segpair_tma_kernel(const PairArgs q) {
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0) tmem_free(tm_base, COLS);
 }
 

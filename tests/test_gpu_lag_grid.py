@@ -182,3 +182,26 @@ def test_line_beside_the_band(n_s, m, amp):
             rms[path] = np.sqrt(((plan.search(x, tm)[0].cpu().numpy() - ref) ** 2).mean())
         plan.check()
     assert rms[cc.PATH_TWO_PASS] <= 1.5 * rms[cc.PATH_FUSED]
+
+
+@pytest.mark.parametrize("n_det,n_s,T_max", [(2, 128, 128.0), (2, 128, 0.0), (2, 3000, 3000.0), (3, 256, 256.0), (4, 2052, 0.0)])
+def test_failed_waits_leave_the_kernel_usable(n_det, n_s, T_max):
+    """Searches whose first bounded wait runs out report it, three times in a row, and the next
+    search gives the bits of the one before them: a CTA that gives up has its tensor-memory stores
+    behind it before it frees the memory."""
+    ds = synth.tiny(seed=97, n_samples=n_s * 12, T_sft=n_s / 4.0, T_short=float(n_s), T_max=T_max, f_band=0.1, n_templates=2, n_det=n_det,
+                    duty=0.8, mean_lock_s=3.0 * n_s)
+    x, tm = torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV)
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        good = plan.search(x, tm).cpu()
+        plan.check()
+        for _ in range(3):
+            plan.set_wait_test(True)
+            plan.search(x, tm)
+            with pytest.raises(cc.CrossCorrError) as e:
+                plan.check()
+            assert e.value.status == 4
+        plan.set_wait_test(False)
+        again = plan.search(x, tm).cpu()
+        plan.check()
+    assert torch.equal(again, good)
