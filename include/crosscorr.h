@@ -286,7 +286,9 @@ cc_status crosscorr_plan_search_path(const cc_plan* plan, int* path);
  * allocates nothing, which makes crosscorr_search capturable in a CUDA graph.  Plans
  * whose searches run one after another on one stream may share one workspace.
  * crosscorr_plan_workspace_size gives the bytes a search of n_t templates needs on the
- * path crosscorr_search takes, with the plan's current tuning. */
+ * path crosscorr_search takes, with the plan's current tuning.  On the two-pass path a
+ * buffer of those bytes also holds every search of fewer templates, although some of them
+ * alone would be given more (they are split into fewer segment chunks there). */
 cc_status crosscorr_plan_set_workspace(cc_plan* plan, void* ws_dev, size_t ws_bytes);
 cc_status crosscorr_plan_workspace_size(const cc_plan* plan, int64_t n_t, size_t* bytes);
 

@@ -306,8 +306,12 @@ static int sm_count() {
     return sms;
 }
 
-// Grid, shared memory, chunk split and workspace of a batch of n_t templates.
-static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
+// The fewest segment chunks a search can be split into.
+static int64_t least_chunks(const cc_plan* plan) { return (plan->M + CORR_MAX_CHUNK - 1) / CORR_MAX_CHUNK; }
+
+// Grid, shared memory, chunk split (of at most max_chunks chunks, where the kernel can do with as
+// few) and workspace of a batch of n_t templates.
+static void corr_layout(const cc_plan* plan, int64_t n_t, int64_t max_chunks, CorrLayout* y) {
     const DevParams& p = plan->dp;
     const bool padded = plan->tuning.transform_len == CORR_POINTS && p.L < CORR_POINTS;
     y->padded = padded;
@@ -347,7 +351,7 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     // rows beyond ROW_BLOCK are summed first (a launch, about three segments' time) where the blocks
     // of corr_lags_kernel do not fill the chip
     const bool pre_sum = n_t * y->C * (y->planes > 1 ? 2 : 1) < sm_count();
-    const int64_t minch = (p.M + CORR_MAX_CHUNK - 1) / CORR_MAX_CHUNK;
+    const int64_t minch = least_chunks(plan);
     const int64_t maxch = std::max<int64_t>(minch, p.M);
     int64_t nch = minch;
     if (plan->tuning.chunk_waves > 0) {
@@ -364,10 +368,10 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
             }
         }
     }
+    nch = std::max(minch, std::min(nch, max_chunks));
     a.chunk_len = (int)((p.M + nch - 1) / nch);
     a.n_chunks = (int)((p.M + a.chunk_len - 1) / a.chunk_len);
     y->n_rows = 2 * a.n_chunks;
-    y->n_blocks = y->n_rows > ROW_BLOCK && pre_sum ? (y->n_rows + ROW_BLOCK - 1) / ROW_BLOCK : 0;
     const size_t b = (size_t)n_t;
     y->ab = al256(b * plan->Q * 2 * plan->N_tau * (plan->cfg.store == CC_STORE_BF16 ? 4 : 8));
     y->z = y->folded ? al256(b * plan->Q * 2 * plan->M * y->G * esz) : 0;
@@ -375,7 +379,10 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
     y->act = al256((size_t)plan->Q * plan->M * y->t_pad);
     y->D = al256(b * sizeof(double));
     y->raw = al256(b * y->n_rows * y->planes * 2 * y->G * sizeof(float));
-    y->rows2 = al256(b * y->n_blocks * y->planes * 2 * y->G * sizeof(float));
+    // (held for any batch of that many rows, so that the bytes of a chunk split grow with the batch)
+    const int blocks = y->n_rows > ROW_BLOCK ? (y->n_rows + ROW_BLOCK - 1) / ROW_BLOCK : 0;
+    y->n_blocks = pre_sum ? blocks : 0;
+    y->rows2 = al256(b * blocks * y->planes * 2 * y->G * sizeof(float));
     y->U = al256(b * (y->planes > 1 ? 2 : 1) * y->G * sizeof(ffc));
     y->h = y->C > 1 ? al256(b * y->n_lags * sizeof(ffc)) : 0;
     y->kn = al256(b * plan->Q * knot_rows(plan) * sizeof(KnotRec));
@@ -384,11 +391,13 @@ static void corr_layout(const cc_plan* plan, int64_t n_t, CorrLayout* y) {
 
 // Templates per batch: as many as the budget of a_r, b_r and folded rows holds.
 static int64_t two_pass_batch(const cc_plan* plan, int64_t n_t) {
-    const size_t per = (size_t)plan->Q * 2 * plan->N_tau * (plan->cfg.store == CC_STORE_BF16 ? 4 : 8) +
-                       (plan->N_s > CORR_POINTS ? (size_t)plan->Q * 2 * plan->M * 2 * fold_count(plan) * CORR_POINTS * 8
-                                                : 0);
-    const int64_t b = plan->tuning.batch_templates > 0 ? plan->tuning.batch_templates
-                                                       : (int64_t)std::max<size_t>(1, (plan->Q > 2 ? MULTI_WS_BUDGET : TWO_PASS_WS_BUDGET) / per);
+    const size_t ab = (size_t)plan->Q * 2 * plan->N_tau * (plan->cfg.store == CC_STORE_BF16 ? 4 : 8);
+    const size_t z = segpair_tma_supported(plan) ? segpair_tma_fold_bytes(plan)
+                     : plan->N_s > CORR_POINTS   ? (size_t)plan->Q * 2 * plan->M * 2 * fold_count(plan) * CORR_POINTS * 8
+                                                 : 0;
+    const int64_t b = plan->tuning.batch_templates > 0
+                          ? plan->tuning.batch_templates
+                          : (int64_t)std::max<size_t>(1, (plan->Q > 2 ? MULTI_WS_BUDGET : TWO_PASS_WS_BUDGET) / (ab + z));
     return std::max<int64_t>(1, std::min<int64_t>({b, n_t, 65535}));
 }
 
@@ -399,21 +408,18 @@ struct FoldedLayout {
     size_t ab, z, norm, D, raw, kn, total;
 };
 
-static void folded_chunks(const cc_plan* plan, int64_t n_t, FoldedLayout* y) {
-    const int64_t nch = segpair_tma_chunks(plan, n_t);
+static void folded_chunks(const cc_plan* plan, int64_t n_t, int64_t max_chunks, FoldedLayout* y) {
+    const int64_t nch = std::max<int64_t>(least_chunks(plan), std::min<int64_t>(segpair_tma_chunks(plan, n_t), max_chunks));
     y->chunk_len = (plan->M + nch - 1) / nch;
     y->n_chunks = (int)((plan->M + y->chunk_len - 1) / y->chunk_len);
 }
 
-static void folded_layout(const cc_plan* plan, int64_t n_t, FoldedLayout* y) {
-    const size_t ab = (size_t)plan->Q * 2 * plan->N_tau * 4, z = segpair_tma_fold_bytes(plan);
-    const int64_t want = plan->tuning.batch_templates > 0 ? plan->tuning.batch_templates
-                                                          : (int64_t)std::max<size_t>(1, TWO_PASS_WS_BUDGET / (ab + z));
-    y->batch = std::max<int64_t>(1, std::min<int64_t>({want, n_t, 65535}));
-    folded_chunks(plan, y->batch, y);
-    const size_t b = (size_t)y->batch;
-    y->ab = al256(ab * b);
-    y->z = al256(z * b);
+static void folded_layout(const cc_plan* plan, int64_t batch, int64_t max_chunks, FoldedLayout* y) {
+    y->batch = batch;
+    folded_chunks(plan, batch, max_chunks, y);
+    const size_t b = (size_t)batch;
+    y->ab = al256((size_t)plan->Q * 2 * plan->N_tau * 4 * b);
+    y->z = al256(segpair_tma_fold_bytes(plan) * b);
     y->norm = al256(b * plan->Q * plan->M * sizeof(float4));
     y->D = al256(b * sizeof(double));
     y->raw = al256(b * 2 * y->n_chunks * plan->N_f * sizeof(float));
@@ -421,11 +427,70 @@ static void folded_layout(const cc_plan* plan, int64_t n_t, FoldedLayout* y) {
     y->total = y->ab + y->z + y->norm + y->D + y->raw + y->kn + al256((size_t)plan->dp.C4 * sizeof(int));
 }
 
+// How a search is split: templates per batch and the largest number of segment chunks.
+struct Split {
+    int64_t batch, chunks;
+};
+
+static size_t split_bytes(const cc_plan* plan, int64_t n_t, Split f) {
+    if (segpair_tma_supported(plan)) {
+        FoldedLayout y;
+        folded_layout(plan, f.batch, f.chunks, &y);
+        return y.total;
+    }
+    CorrLayout y;
+    corr_layout(plan, f.batch, f.chunks, &y);
+    size_t bytes = y.total;
+    if (n_t % f.batch) {   // the last batch may split its segments into more chunks
+        corr_layout(plan, n_t % f.batch, f.chunks, &y);
+        bytes = std::max(bytes, y.total);
+    }
+    return bytes;
+}
+
+// The split of a search of n_t templates: the fastest one, or, with less memory than that takes,
+// fewer chunks (the partial rows of a search of few templates can be most of its bytes); batch 0:
+// does not fit.  With the fewest chunks the bytes grow with the templates, so memory that holds
+// n of them in some split holds any smaller number.
+static Split fit_split(const cc_plan* plan, int64_t n_t, size_t avail) {
+    Split f{two_pass_batch(plan, n_t), plan->M};
+    if (split_bytes(plan, n_t, f) <= avail) return f;
+    const int64_t least = least_chunks(plan);
+    while (f.chunks > least) {
+        f.chunks = std::max(least, f.chunks * 3 / 4);
+        if (split_bytes(plan, n_t, f) <= avail) return f;
+    }
+    return Split{0, least};
+}
+
+// The split to search n_t templates with, and its workspace: the plan's own memory grows to the
+// fastest split's; the caller's, and the plan's while its stream is captured (when nothing can be
+// allocated), is taken as it is.
+static cc_status claim_split(cc_plan* plan, int64_t n_t, cudaStream_t st, Split* f) {
+    *f = fit_split(plan, n_t, SIZE_MAX);
+    const size_t need = split_bytes(plan, n_t, *f);
+    if (plan->ws_bytes >= need) return CC_OK;
+    bool fixed = plan->ws_external;
+    if (!fixed && plan->ws_bytes > 0) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        fixed = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusActive;
+    }
+    if (fixed) {
+        const Split g = fit_split(plan, n_t, plan->ws_bytes);
+        if (g.batch > 0) {
+            *f = g;
+            return CC_OK;
+        }
+    }
+    return ensure_workspace(plan, need);
+}
+
 static cc_status search_folded_bf16(cc_plan* plan, const cc_template* t_dev, int64_t n_t, float* rho, cudaStream_t st) {
-    FoldedLayout y;
-    folded_layout(plan, n_t, &y);
-    cc_status s = ensure_workspace(plan, y.total);
+    Split f;
+    cc_status s = claim_split(plan, n_t, st, &f);
     if (s != CC_OK) return s;
+    FoldedLayout y;
+    folded_layout(plan, f.batch, f.chunks, &y);
     char* w = (char*)plan->ws;
     void* ab = w;
     void* z = w += y.ab;
@@ -437,7 +502,7 @@ static cc_status search_folded_bf16(cc_plan* plan, const cc_template* t_dev, int
     for (int64_t t0 = 0; t0 < n_t; t0 += y.batch) {
         const int64_t nb = std::min(y.batch, n_t - t0);
         FoldedLayout b = y;
-        folded_chunks(plan, nb, &b);   // chunking for this batch size (workspace sized for the largest)
+        folded_chunks(plan, nb, f.chunks, &b);   // chunking for this batch size (workspace sized for the largest)
         if (b.n_chunks > y.n_chunks) b = y;
         if ((s = launch_knots(plan, t_dev + t0, nb, kn, st)) != CC_OK) return s;
         if ((s = launch_resample(plan, t_dev + t0, nb, ab, norm, st, kn, knot_rows(plan))) != CC_OK) return s;
@@ -455,21 +520,7 @@ static cc_status search_folded_bf16(cc_plan* plan, const cc_template* t_dev, int
 }
 
 size_t two_pass_workspace_bytes(const cc_plan* plan, int64_t n_t) {
-    if (n_t < 1) return 0;
-    if (segpair_tma_supported(plan)) {
-        FoldedLayout y;
-        folded_layout(plan, n_t, &y);
-        return y.total;
-    }
-    const int64_t b = two_pass_batch(plan, n_t);
-    CorrLayout y;
-    corr_layout(plan, b, &y);
-    size_t bytes = y.total;
-    if (n_t % b) {   // the last batch may split its segments into more chunks
-        corr_layout(plan, n_t % b, &y);
-        bytes = std::max(bytes, y.total);
-    }
-    return bytes;
+    return n_t < 1 ? 0 : split_bytes(plan, n_t, fit_split(plan, n_t, SIZE_MAX));
 }
 
 template <bool BF16, bool LAG>
@@ -509,14 +560,14 @@ static cudaError_t launch_corr(const CorrLayout& y, cudaStream_t st) {
 cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, float* rho, cudaStream_t st) {
     if (segpair_tma_supported(plan)) return search_folded_bf16(plan, t_dev, n_t, rho, st);
     const DevParams& p = plan->dp;
-    const int64_t batch = two_pass_batch(plan, n_t);
-    cc_status s = ensure_workspace(plan, two_pass_workspace_bytes(plan, n_t));
+    Split f;
+    cc_status s = claim_split(plan, n_t, st, &f);
     if (s != CC_OK) return s;
     cudaError_t e;
-    for (int64_t t0 = 0; t0 < n_t; t0 += batch) {
-        const int64_t nb = std::min(batch, n_t - t0);
+    for (int64_t t0 = 0; t0 < n_t; t0 += f.batch) {
+        const int64_t nb = std::min(f.batch, n_t - t0);
         CorrLayout y;
-        corr_layout(plan, nb, &y);
+        corr_layout(plan, nb, f.chunks, &y);
         const int64_t units = (2 * nb + y.T - 1) / y.T * y.C * y.a.n_chunks;
         if (units > 0x7fffffff) return fail(CC_ERR_UNSUPPORTED, "too many work units in one launch");
         char* w = (char*)plan->ws;

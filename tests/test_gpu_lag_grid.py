@@ -205,3 +205,39 @@ def test_failed_waits_leave_the_kernel_usable(n_det, n_s, T_max):
         again = plan.search(x, tm).cpu()
         plan.check()
     assert torch.equal(again, good)
+
+
+@pytest.mark.parametrize("n_s,m,n_det,store,most,fewer", [
+    (1200, 6, 2, 0, 26, (25, 17, 1)), (3000, 20, 2, 1, 26, (25, 23)), (9000, 10, 2, 0, 13, (12, 1)),
+    (8192, 20, 2, 1, 9, (8, 1))])
+def test_fewer_templates_in_a_larger_searchs_workspace(n_s, m, n_det, store, most, fewer):
+    """A caller's buffer of the bytes stated for a number of templates serves every smaller number
+    (whose fastest split may take more), and the plan's own memory, grown by the larger search,
+    serves the smaller one while its stream is captured."""
+    ds = synth.tiny(seed=101, n_samples=n_s * m, T_sft=n_s / 4.0, T_short=float(n_s), T_max=float(n_s), f_band=0.1, n_templates=most,
+                    n_det=n_det, duty=0.8, mean_lock_s=2.0 * n_s)
+    ref = oracle.rho(ds, templates=ds.templates[:3])
+    x, tm = torch.from_numpy(ds.x64).to(DEV), cc.templates5(torch.from_numpy(ds.templates).to(DEV))
+    tol = 1e-2 if store else 1e-4
+    with cc.CrossCorrPlan(ds.cfg, ds.dets, store=store) as plan:
+        size = plan.workspace_size(most)
+        if n_s != 8192:
+            assert plan.workspace_size(fewer[0]) > size    # its fastest split takes more
+        plan.set_workspace(torch.empty(size, dtype=torch.uint8, device=DEV))
+        for n in (most,) + tuple(fewer):
+            rho = torch.empty((n, plan.N_f), dtype=torch.float32, device=DEV)
+            plan.search(x, tm[:n], rho)
+            plan.check()
+            for t in range(min(n, 3)):
+                assert np.abs(rho[t].cpu().numpy() - ref[t]).max() <= tol * max(1.0, np.abs(ref[t]).max()), (n, t)
+        plan.set_workspace(None)
+        plan.search(x, tm)
+        for n in fewer:
+            rho = torch.zeros((n, plan.N_f), dtype=torch.float32, device=DEV)
+            torch.cuda.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                plan.search(x, tm[:n], rho)
+            g.replay()
+            plan.check()
+            assert np.abs(rho[0].cpu().numpy() - ref[0]).max() <= tol * max(1.0, np.abs(ref[0]).max()), n
