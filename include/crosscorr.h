@@ -256,7 +256,9 @@ cc_status crosscorr_search_noalloc(cc_plan* plan, const void* const* x_dev, cons
  *                     each segment into shared memory and transforms it on chip; needs
  *                     a few MB of workspace (FP32 storage, coset length <= 4096).  Three
  *                     and four detectors take the two-pass kernels where those serve the
- *                     plan and the workspace holds at least one template of them;
+ *                     plan and the workspace holds at least one template of them (a caller's
+ *                     as it is; the plan's own grows to at most about 4 GB of resampled
+ *                     series, as it does for the wider bands of CC_PATH_AUTO below);
  *   CC_PATH_TWO_PASS  a_r, b_r of a template batch written to HBM in the plan's
  *                     storage type (up to 24 GB of workspace), then every segment is
  *                     transformed on chip at the G >= 2 N_s frequencies that determine the

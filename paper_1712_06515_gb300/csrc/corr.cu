@@ -59,7 +59,7 @@ CC_CORR_INST_MULTI(extern, 4096)
 CC_CORR_INST_MULTI_FULL(extern)
 
 constexpr size_t TWO_PASS_WS_BUDGET = (size_t)24 << 30;   // a_r, b_r (and folded rows) of one template batch
-constexpr size_t MULTI_WS_BUDGET = (size_t)4 << 30;       // the same for three and four detectors (the fused path's plans)
+constexpr size_t SHARED_WS_BUDGET = (size_t)4 << 30;      // the same for plans that the cluster or stage kernels serve too
 constexpr int LAG_THREADS = 256;
 constexpr int LAG_MAX_THREADS = 1024;   // the two-float transforms: a radix-4 butterfly a thread, at least LAG_THREADS
 constexpr int ROW_BLOCK = 32;        // partial rows summed by one block of corr_rows_kernel
@@ -397,7 +397,7 @@ static int64_t two_pass_batch(const cc_plan* plan, int64_t n_t) {
                                                  : 0;
     const int64_t b = plan->tuning.batch_templates > 0
                           ? plan->tuning.batch_templates
-                          : (int64_t)std::max<size_t>(1, (plan->Q > 2 ? MULTI_WS_BUDGET : TWO_PASS_WS_BUDGET) / (ab + z));
+                          : (int64_t)std::max<size_t>(1, (two_pass_supported(plan) ? TWO_PASS_WS_BUDGET : SHARED_WS_BUDGET) / (ab + z));
     return std::max<int64_t>(1, std::min<int64_t>({b, n_t, 65535}));
 }
 
@@ -449,9 +449,12 @@ static size_t split_bytes(const cc_plan* plan, int64_t n_t, Split f) {
 }
 
 // The split of a search of n_t templates: the fastest one, or, with less memory than that takes,
-// fewer chunks (the partial rows of a search of few templates can be most of its bytes); batch 0:
-// does not fit.  With the fewest chunks the bytes grow with the templates, so memory that holds
-// n of them in some split holds any smaller number.
+// fewer chunks (the partial rows of a search of few templates can be most of its bytes).  With the
+// fewest chunks the bytes grow with the templates, so memory that holds n of them in some split
+// holds any smaller number.  Plans that other kernels serve in little memory (more than two
+// detectors, bands over both coset halves) then take fewer templates at once, down to one: the
+// cluster kernel needs a few MB for any search, at 20 to 30 times the time on large ones.  batch 0:
+// does not fit.
 static Split fit_split(const cc_plan* plan, int64_t n_t, size_t avail) {
     Split f{two_pass_batch(plan, n_t), plan->M};
     if (split_bytes(plan, n_t, f) <= avail) return f;
@@ -460,7 +463,12 @@ static Split fit_split(const cc_plan* plan, int64_t n_t, size_t avail) {
         f.chunks = std::max(least, f.chunks * 3 / 4);
         if (split_bytes(plan, n_t, f) <= avail) return f;
     }
-    return Split{0, least};
+    int64_t fits = 0, over = f.batch;
+    while (!two_pass_supported(plan) && over - fits > 1) {
+        f.batch = fits + (over - fits) / 2;
+        (split_bytes(plan, f.batch, f) <= avail ? fits : over) = f.batch;
+    }
+    return Split{fits, least};
 }
 
 // The split to search n_t templates with, and its workspace: the plan's own memory grows to the
@@ -473,16 +481,22 @@ static cc_status claim_split(cc_plan* plan, int64_t n_t, cudaStream_t st, Split*
     bool fixed = plan->ws_external;
     if (!fixed && plan->ws_bytes > 0) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        fixed = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusActive;
+        if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+        fixed = cap == cudaStreamCaptureStatusActive;
     }
-    if (fixed) {
-        const Split g = fit_split(plan, n_t, plan->ws_bytes);
-        if (g.batch > 0) {
-            *f = g;
-            return CC_OK;
-        }
-    }
-    return ensure_workspace(plan, need);
+    if (!fixed) return ensure_workspace(plan, need);
+    const Split g = fit_split(plan, n_t, plan->ws_bytes);
+    if (g.batch < 1)
+        return fail(CC_ERR_OOM, "workspace of " + std::to_string(plan->ws_bytes) + " bytes; this call needs " + std::to_string(need));
+    *f = g;
+    return CC_OK;
+}
+
+// Whether the two-pass kernels can search n_t templates of a plan that other kernels serve too, with
+// the memory they need claimed.
+bool two_pass_claim(cc_plan* plan, int64_t n_t, cudaStream_t st) {
+    Split f;
+    return claim_split(plan, n_t, st, &f) == CC_OK;
 }
 
 static cc_status search_folded_bf16(cc_plan* plan, const cc_template* t_dev, int64_t n_t, float* rho, cudaStream_t st) {

@@ -15,6 +15,7 @@ size_t pair_workspace_bytes(const cc_plan* plan, int64_t n_t);
 bool two_pass_supported(const cc_plan* plan);
 bool lag_grid_supported(const cc_plan* plan);
 size_t two_pass_workspace_bytes(const cc_plan* plan, int64_t n_t);
+bool two_pass_claim(cc_plan* plan, int64_t n_t, cudaStream_t st);
 cc_status search_two_pass(cc_plan* plan, const cc_template* t_dev, int64_t n_t, float* rho, cudaStream_t st);
 
 constexpr size_t STAGED_WS_BUDGET = (size_t)6 << 30;
@@ -143,11 +144,9 @@ extern "C" cc_status crosscorr_search(cc_plan* plan, const void* const* x_dev, c
     const bool wide = path == CC_PATH_TWO_PASS && plan->search_path == CC_PATH_AUTO && !two_pass_supported(plan);
     if (path == CC_PATH_TWO_PASS && !wide) return search_two_pass(plan, t_dev, n_t, rho_dev, st);
     if (wide || (path == CC_PATH_FUSED && fused_on_lag_grid(plan))) {
-        // a workspace that cannot hold a batch (the caller's, or no memory for the plan's own)
+        // a workspace that cannot hold one template (the caller's, or no memory for the plan's own)
         // leaves the search to the cluster or the stage kernels
-        const size_t need = two_pass_workspace_bytes(plan, n_t);
-        if (plan->ws_external ? plan->ws_bytes >= need : ensure_workspace(plan, need) == CC_OK)
-            return search_two_pass(plan, t_dev, n_t, rho_dev, st);
+        if (two_pass_claim(plan, n_t, st)) return search_two_pass(plan, t_dev, n_t, rho_dev, st);
         if (wide) path = fused_supported(plan) ? CC_PATH_FUSED : CC_PATH_STAGED;
     }
     FusedLayout lay;

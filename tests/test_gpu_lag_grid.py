@@ -208,7 +208,7 @@ def test_failed_waits_leave_the_kernel_usable(n_det, n_s, T_max):
 
 
 @pytest.mark.parametrize("n_s,m,n_det,store,most,fewer", [
-    (1200, 6, 2, 0, 26, (25, 17, 1)), (3000, 20, 2, 1, 26, (25, 23)), (9000, 10, 2, 0, 13, (12, 1)),
+    (1200, 6, 2, 0, 26, (25, 17, 1)), (600, 100, 3, 0, 9, (8, 5, 1)), (3000, 20, 2, 1, 26, (25, 23)), (9000, 10, 2, 0, 13, (12, 1)),
     (8192, 20, 2, 1, 9, (8, 1))])
 def test_fewer_templates_in_a_larger_searchs_workspace(n_s, m, n_det, store, most, fewer):
     """A caller's buffer of the bytes stated for a number of templates serves every smaller number
@@ -241,3 +241,52 @@ def test_fewer_templates_in_a_larger_searchs_workspace(n_s, m, n_det, store, mos
             g.replay()
             plan.check()
             assert np.abs(rho[0].cpu().numpy() - ref[0]).max() <= tol * max(1.0, np.abs(ref[0]).max()), n
+
+
+def small_workspace(ds, n_t):
+    """Bytes that hold the cluster kernel's search of a plan but not one template of the lag grid."""
+    two = synth.SearchConfig(**dict(vars(ds.cfg), n_det=2))     # by name: three detectors may take the lag grid
+    with cc.CrossCorrPlan(two, ds.dets[:2]) as plan:
+        plan.set_path(cc.PATH_FUSED)
+        small = 3 * plan.workspace_size(n_t)
+        assert small < ds.cfg.n_det * 2 * plan.N_tau * 8
+    return small
+
+
+@pytest.mark.parametrize("n_det,n_s,T_max,mode,learned", [
+    (3, 256, 256.0, 0, False), (4, 256, 256.0, 0, False), (3, 256, 256.0, 2, False), (4, 1024, 1024.0, 2, False), (4, 256, 0.0, 0, False),
+    (3, 256, 256.0, 0, True), (4, 1024, 1024.0, 2, True)])
+def test_cluster_kernel_of_three_and_four_detectors(n_det, n_s, T_max, mode, learned):
+    """What a workspace too small for the lag grid leaves the search to: the cluster kernel, against
+    the oracle, and for the learned taps against the lag grid's rho."""
+    n_t = 3
+    ds = synth.tiny(seed=103, n_samples=n_s * 60, T_sft=n_s / 2.0, T_short=float(n_s), T_max=T_max, f_band=0.5 if learned else 0.1,
+                    n_templates=n_t, n_det=n_det, pair_mode=mode, duty=0.8, mean_lock_s=3.0 * n_s)
+    x, tm = torch.from_numpy(ds.x64).to(DEV), torch.from_numpy(ds.templates).to(DEV)
+    with cc.CrossCorrPlan(ds.cfg, ds.dets, interp=cc.INTERP_LEARNED if learned else cc.INTERP_EXACT) as plan:
+        ref = plan.search(x, tm).cpu().numpy() if learned else oracle.rho(ds)
+        plan.set_workspace(torch.empty(small_workspace(ds, n_t), dtype=torch.uint8, device=DEV))
+        got = plan.search(x, tm).cpu().numpy()
+        plan.check()
+    for t in range(n_t):
+        assert np.abs(got[t] - ref[t]).max() <= 1e-4 * max(1.0, np.abs(ref[t]).max())
+
+
+@pytest.mark.parametrize("n_det,f_band", [(3, 0.1), (2, 1.0)])
+def test_batches_cut_to_the_workspace(n_det, f_band):
+    """Plans that the cluster kernel serves too still take the lag grid in a caller's workspace of two
+    templates: in batches, each of several launches, where the cluster kernel has two for all."""
+    ds = synth.tiny(seed=107, n_samples=240 * 40, T_sft=240.0, T_max=0.0, T_short=240.0, f_band=f_band, duty=0.8, mean_lock_s=2400.0, n_det=n_det,
+                    n_templates=7)
+    ref = oracle.rho(ds)
+    x, tm = torch.from_numpy(ds.x64).to(DEV), cc.templates5(torch.from_numpy(ds.templates).to(DEV))
+    lib = cc.load()
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        plan.set_workspace(torch.empty(plan.workspace_size(2), dtype=torch.uint8, device=DEV))
+        n0 = lib.crosscorr_kernel_launches()
+        got = plan.search(x, tm).cpu().numpy()
+        launches = lib.crosscorr_kernel_launches() - n0
+        plan.check()
+    assert launches >= 4 * 4      # four batches of knots, resampling, products and at least one transform
+    for t in range(7):
+        assert np.abs(got[t] - ref[t]).max() <= 1e-4 * max(1.0, np.abs(ref[t]).max())
