@@ -68,8 +68,9 @@ __device__ __forceinline__ float2 sinc_pairs(const SincTab<DT>& tb, const float2
         O.x = fmaf(h, o.x, O.x);
         O.y = fmaf(h, o.y, O.y);
     }
+    // (a sample that falls on one of the series is that one, whatever lies beside it: not 0 x inf)
     const float2 x0 = xc[0];
-    return make_float2(fmaf(s, fmaf(delta, E.x, O.x), sc * x0.x), fmaf(s, fmaf(delta, E.y, O.y), sc * x0.y));
+    return delta == 0.f ? x0 : make_float2(fmaf(s, fmaf(delta, E.x, O.x), sc * x0.x), fmaf(s, fmaf(delta, E.y, O.y), sc * x0.y));
 }
 
 // sinc_taps (common.cuh) with the half width at compile time for DT > 0, value for value: its

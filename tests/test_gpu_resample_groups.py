@@ -101,3 +101,21 @@ def test_long_bf16_segments(n_s, m, n_t, D, learned):
     assert float(far.mean()) <= 1e-4
     assert float((a16 != r32).mean()) <= 1e-2
     assert float(np.abs(n16 - n32).max()) <= 4e-5 * float(np.abs(n32).max())
+
+
+@pytest.mark.parametrize("D", [5, 8, 16])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_whole_samples_ignore_their_neighbours(D, bad):
+    """Source samples that fall on detector samples (no orbit, data from the barycentre) are those
+    samples: one that is not finite stays alone."""
+    tm = np.array([[0.0, synth.T_ASC_O1, synth.SCO_X1_P]])
+    ds = synth.tiny(seed=79, n_samples=2400, T_sft=200.0, T_max=600.0, T_short=600.0, D=D, f_band=0.1, templates=tm, duty=1.0,
+                    zero_roemer=True)
+    x = ds.x64.copy()
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        want = plan.resample(torch.from_numpy(x).to(DEV), torch.from_numpy(tm).to(DEV))[0].cpu().numpy()
+        x[:, 1000] = bad
+        got = plan.resample(torch.from_numpy(x).to(DEV), torch.from_numpy(tm).to(DEV))[0].cpu().numpy()
+    assert not np.isfinite(got[..., 1000]).any()
+    keep = np.arange(want.shape[-1]) != 1000
+    assert np.isfinite(want).all() and np.array_equal(got[..., keep], want[..., keep])
