@@ -338,6 +338,35 @@ __device__ __forceinline__ void warp_pass(const float2* src, float2* dst, const 
     }
 }
 
+// exp(-2 pi i e / n), 0 <= e < n < 2^21, to the last place: 2 pi e / n = (pi / 2) (k + r / n) with
+// integers k and |r| <= n / 2, the angle phi = (pi / 2) r / n and the leading terms of the sine's and
+// the cosine's series in two floats each, the rest of the series (below 0.016) in one.  The error
+// is the final rounding and 4e-9 more, as of FP64 values rounded; an angle rounded to FP32 left up
+// to 1.3e-7 (four times as much on the mean), which every pass of the transform took up.
+__device__ __forceinline__ float2 exact_root(int e, int n) {
+    const int k = (8 * e + n) / (2 * n), r = 4 * e - k * n;
+    const float fn = (float)n, fr = (float)r, x = __fdiv_rn(fr, fn), xl = __fdividef(__fmaf_rn(-x, fn, fr), fn);
+    const float h = __fmul_rn(x, 1.57079637f);
+    const float l = __fmaf_rn(x, 1.57079637f, -h) + __fmaf_rn(x, -4.37113883e-8f, xl * 1.57079637f);   // phi = h + l
+    const float t = __fmul_rn(h, h), tl = __fmaf_rn(h, h, -t) + 2.f * h * l;                          // phi^2
+    // cos: 1 - t / 2 + t^2 (1/4! - t/6! + ...)
+    float c = fmaf(fmaf(fmaf(fmaf(1.f / 479001600.f, t, -1.f / 3628800.f), t, 1.f / 40320.f), t, -1.f / 720.f), t, 1.f / 24.f);
+    const float u = 0.5f * t, c0 = __fsub_rn(1.f, u);
+    c = __fadd_rn(c0, fmaf(c, t * t, __fsub_rn(__fsub_rn(1.f, c0), u) - 0.5f * tl));
+    // sin: h - phi^3 / 6 + (l + phi^5 (1/5! - t/7! + ...))
+    const float p3 = __fmul_rn(h, t), p3l = __fmaf_rn(h, t, -p3) + __fmaf_rn(h, tl, l * t);
+    const float b = __fmul_rn(p3, -0.166666672f), bl = __fmaf_rn(p3, -0.166666672f, -b) + __fmaf_rn(p3, 4.96705355e-9f, p3l * -0.166666672f);
+    float s = fmaf(fmaf(fmaf(-1.f / 39916800.f, t, 1.f / 362880.f), t, -1.f / 5040.f), t, 1.f / 120.f);
+    const float s0 = __fadd_rn(h, b);
+    s = __fadd_rn(s0, fmaf(s, p3 * t, __fadd_rn(__fsub_rn(h, s0), b) + (l + bl)));
+    switch (k & 3) {
+        case 0: return make_float2(c, -s);
+        case 1: return make_float2(-s, -c);
+        case 2: return make_float2(-c, s);
+        default: return make_float2(s, c);
+    }
+}
+
 // N' up to 1536: a CTA takes `chunk` consecutive T_sft blocks, its warps one block after the
 // other from a shared counter (locked SFTs and gaps come in runs of hours: the CTAs' sizes
 // differ, and more CTAs than fit at once even that out).  Per warp three N'-point shared
@@ -346,7 +375,7 @@ __device__ __forceinline__ void warp_pass(const float2* src, float2* dst, const 
 // series.  The forward twiddles exp(-2 pi i e / N') and the blocks' phase factors are formed
 // once per CTA.  Only warp-level synchronisation after that.
 // What bounds it: instruction issue (60 %) and the shared-memory passes with 20 warps per SM; the
-// traffic alone would take 20 us.  28800 blocks of N' = 360, 60 % of them locked: 40.7 us; 44.8 with
+// traffic alone would take 20 us.  28800 blocks of N' = 360, 60 % of them locked: 41.0 us; 44.8 with
 // 8-byte copies and a 64-bit remainder per twiddle, 57.6 with a global block counter.
 __global__ void __launch_bounds__(SS_THREADS)
 sft_fft_warp_kernel(const float2* __restrict__ band, const int64_t* __restrict__ block_sft, int64_t n_blocks,
@@ -372,10 +401,10 @@ sft_fft_warp_kernel(const float2* __restrict__ band, const int64_t* __restrict__
         sincospif(2.0f * c, &sn, &cs);
         s_rot[i] = make_float2(cs * scale, -sn * scale);
     }
-    for (int e = threadIdx.x; e < n_prime; e += blockDim.x) {   // exp(-2 pi i e / N'), the angle within half a turn
-        float sn, cs;
-        sincospif(-2.0f * (float)(2 * e > n_prime ? e - n_prime : e) / (float)n_prime, &sn, &cs);
-        twf[e] = make_float2(cs, sn);
+    for (int e = threadIdx.x; 2 * e <= n_prime; e += blockDim.x) {
+        const float2 w = exact_root(e, n_prime);
+        if (e > 0) twf[n_prime - e] = make_float2(w.x, -w.y);
+        twf[e] = w;
     }
     __syncthreads();
     auto grab = [&]() -> int {

@@ -80,3 +80,19 @@ def test_sfts_to_series_repeatable():
     a = cc.sfts_to_series(band, bsd, 360.0, 150.0).cpu().numpy()
     b = cc.sfts_to_series(band, bsd, 360.0, 150.0).cpu().numpy()
     assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [20, 24, 25, 27, 36, 40, 45, 72])
+def test_twiddles_to_the_last_place(n):
+    """One nonzero bin of an N' = R1 R2 in two passes: the first gives ones, the first output of each
+    butterfly of the second is a twiddle alone, so those samples are the roots exp(2 pi i j m / N')
+    as the kernel holds them (f_h = 0, T_sft = 1).  Rounded from more precise values each part is
+    within 2^-25, allowed a fifth more; an angle rounded to FP32 leaves up to three times that."""
+    few = min(r for r in range(2, 10) if n % r == 0 and n // r in (2, 3, 4, 5, 8, 9) and r in (2, 3, 4, 5, 8, 9))
+    m, j = np.meshgrid(np.arange(few), np.arange(few), indexing="ij")
+    band = torch.zeros(few, n, dtype=torch.complex64)
+    band[torch.arange(few), torch.arange(few)] = 1.0
+    x = cc.sfts_to_series(band.to(DEV), torch.arange(few, device=DEV), 1.0, 0.0).cpu().numpy().reshape(few, n)[:, :few]
+    want = (-1.0) ** j * np.exp(2j * np.pi * ((m * j) % n) / n)
+    err = np.maximum(np.abs(x.real - want.real), np.abs(x.imag - want.imag))
+    assert err.max() <= 1.2 * 2.0 ** -25, err.max()
