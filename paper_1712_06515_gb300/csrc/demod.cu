@@ -11,7 +11,8 @@
 //     time order built by the prepare call), the signal's bin position and phase as
 //     linear functions of the output bin; one thread per (template, output bin) then
 //     walks the SFTs in time order, forms
-//     y_K = sum_m (-1)^m sinc(kappa_Km) z_Km exp(-i Phi_K) (= Xi_K z_K exp(-i Phi_K)) and
+//     y_K = sum_m (-1)^m sinc(kappa_Km) z_Km exp(-i Phi_K) (= Xi_K z_K exp(-i Phi_K); here and in
+//     Xi_K with every sinc times pi / 4, which cancels in rho) and
 //     sums Gamma_KL 2 Re(conj(y_K) y_L) over every earlier SFT L within T_max, with the
 //     normalisation sum (Xi_K Xi_L Gamma_KL)^2 alongside; rho = raw / sqrt(2 den).  Two
 //     forms of that sum: the method's pair loop (demod_pair_kernel, one term per pair,
@@ -248,19 +249,22 @@ struct SftIn {
     float2 z0, z1;
 };
 
-// The two sinc weights of kappa = -f and 1 - f, f = h + 1/2: with
-// g(h) = sin(pi f) / (pi f (1 - f)) = cos(pi h) / (pi (1/4 - h^2)), an entire even function,
-// sinc(f) = g (1 - f) and sinc(1 - f) = g f.  g as a polynomial in h^2 by Chebyshev fit on
-// |h| <= 1/2 (largest error 4e-12).
+// The two sinc weights of kappa = -f and 1 - f, f = h + 1/2, times pi / 4: with
+// g(h) = cos(pi h) / (1 - 4 h^2), an entire even function, sinc(f) = (4 / pi) g (1/2 - h) and
+// sinc(1 - f) = (4 / pi) g (1/2 + h); the common factor cancels in rho.  g = 1 + u P(u), u = h^2, P of
+// degree four by least squares at Chebyshev nodes, one coefficient after the other rounded to FP32
+// and the rest fitted again: 2.5e-10 from g on |h| <= 1/2.  In FP32 the sincs are within 9e-8 (a
+// series for one and a quotient for the other: 1.4e-7).
 __device__ __forceinline__ float2 sinc_weights(float h) {
     const float u = h * h;
-    float g = -0.000581711926f;
-    g = fmaf(g, u, 0.00805632297f);
-    g = fmaf(g, u, -0.0728914161f);
-    g = fmaf(g, u, 0.406804216f);
-    g = fmaf(g, u, -1.19022713f);
-    g = fmaf(g, u, 1.27323954f);
-    return make_float2(g * (0.5f - h), g * (0.5f + h));
+    float g = -0.000398144301f;
+    g = fmaf(g, u, 0.00628934102f);
+    g = fmaf(g, u, -0.0572400875f);
+    g = fmaf(g, u, 0.319502473f);
+    g = fmaf(g, u, -0.934802175f);
+    g = fmaf(g, u, 1.f);
+    const float k = 0.5f * g;
+    return make_float2(fmaf(-h, g, k), fmaf(h, g, k));
 }
 
 // The demodulated bin y (the two-bin sinc interpolation, rotated by the heterodyne phase) and
@@ -307,8 +311,8 @@ __device__ __forceinline__ void rec_fetch(SftIn& q, const SepRec& r, float df, f
 // s_(l - R_s); a jump over empty blocks, and every 4 (R_s + 1) steps, sums the window
 // exactly.  Records and control words reach shared memory by cp.async, SG at a time, one group
 // ahead; SFT i + 1's bins load while SFT i is summed.  What bounds it: instruction issue (66 %
-// active with the twelve warps whose rings fit an SM, 115 instructions per SFT and 32 bins): 16
-// templates on 120 days 32.1 ms, 44.9 with one bin a thread.
+// active with the twelve warps whose rings fit an SM, about 110 instructions per SFT and 32 bins): 16
+// templates on 120 days 28.8 ms, 44.9 with one bin a thread.
 constexpr int SB = 2, SG = 16;
 
 template <bool RING>

@@ -5,6 +5,8 @@ mid-time, the pair set against its closed-form count, unit variance in noise (th
 of N), h0^2 scaling, the argmax on the injection, and the invariances."""
 import dataclasses
 import math
+import os
+import re
 
 import numpy as np
 import pytest
@@ -183,3 +185,27 @@ def test_separable_rearrangement_equals_pair_loop(kw):
         sep = np.where(den > 0, raw / np.sqrt(2.0 * den), 0.0)
         ref = demod.demod_rho(ds, tmpl)
         np.testing.assert_allclose(sep, ref, rtol=0, atol=1e-9 * max(1.0, np.abs(ref).max()))
+
+
+def test_sinc_weights_polynomial():
+    """The two-bin interpolation's weights as the kernel evaluates them (FP32, the coefficients of its
+    source, pi / 4 of the sincs): within one FP32 step below one, where a series for one and a
+    quotient for the other are within 1.4e-7."""
+    src = open(os.path.join(os.path.dirname(oracle.__file__), "..", "paper_1712_06515_gb300", "csrc", "demod.cu")).read()
+    body = src[src.index("float2 sinc_weights(float h)"):]
+    body = body[:body.index("\n}")]
+    coef = [np.float32(c) for c in re.findall(r"(?:g = |g, u, )(-?[\d.]+)f", body)]
+
+    def fma(a, b, c):   # the product of two FP32 values is exact in FP64
+        return (a.astype(np.float64) * np.asarray(b, np.float64) + np.asarray(c, np.float64)).astype(np.float32)
+
+    h = np.linspace(-0.5, 0.5, 200001).astype(np.float32)
+    u = h * h
+    g = np.full_like(u, coef[0])
+    for c in coef[1:]:
+        g = fma(g, u, c)
+    norm = 4.0 / np.pi if coef[-1] == 1.0 else 1.0     # (g = 4 / pi at h = 0: the sincs themselves)
+    k = np.float32(0.5) * g
+    f = h.astype(np.float64) + 0.5
+    got = np.stack([fma(-h, g, k), fma(h, g, k)]).astype(np.float64) * norm
+    assert np.abs(got - np.stack([np.sinc(f), np.sinc(1.0 - f)])).max() <= 2.0 ** -23
