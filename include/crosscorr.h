@@ -300,7 +300,8 @@ typedef struct {
                                  (0: as many as 24 GB of resampled series hold) */
     int32_t chunk_waves;      /* fused and two-pass: split each template's segments into
                                  chunks until the launch has about this many CTA waves
-                                 (0: 4 for fused, 40 for two-pass) */
+                                 (0: 4 for fused; two-pass takes the split of least time,
+                                 by the units' length and the rows they leave) */
     int32_t transform_len;    /* two-pass, segments of at most 1024 samples: 0 takes the
                                  shortest transform (the power of two of at least twice the
                                  segment), 4096 one 4096-point transform per segment

@@ -263,19 +263,6 @@ __device__ __forceinline__ int64_t floor_div(int64_t a, int64_t b) {
     return (q * b > a) ? q - 1 : q;
 }
 
-// Linear interpolation of an FP64 table at time t (end intervals extrapolate);
-// inv_dt = 1 / table spacing.
-__device__ __forceinline__ double table_lerp(const double* tab, double t0, double inv_dt, int64_t n,
-                                             double t) {
-    double u = (t - t0) * inv_dt;
-    double fi = floor(u);
-    int64_t i = (int64_t)fi;
-    i = i < 0 ? 0 : (i > n - 2 ? n - 2 : i);
-    double f = u - (double)i;
-    double v0 = __ldg(tab + i), v1 = __ldg(tab + i + 1);
-    return v0 + f * (v1 - v0);
-}
-
 // Orbit of one template in the form the timing code uses (times relative to t0).
 struct Orbit {
     double a_p, tasc_rel, invP, e;

@@ -456,7 +456,7 @@ static size_t split_bytes(const cc_plan* plan, int64_t n_t, Split f) {
 // cluster kernel needs a few MB for any search, at 20 to 30 times the time on large ones.  batch 0:
 // does not fit.
 static Split fit_split(const cc_plan* plan, int64_t n_t, size_t avail) {
-    Split f{two_pass_batch(plan, n_t), plan->M};
+    Split f{two_pass_batch(plan, n_t), plan->M};   // as many chunks as pay
     if (split_bytes(plan, n_t, f) <= avail) return f;
     const int64_t least = least_chunks(plan);
     while (f.chunks > least) {
@@ -475,7 +475,7 @@ static Split fit_split(const cc_plan* plan, int64_t n_t, size_t avail) {
 // fastest split's; the caller's, and the plan's while its stream is captured (when nothing can be
 // allocated), is taken as it is.
 static cc_status claim_split(cc_plan* plan, int64_t n_t, cudaStream_t st, Split* f) {
-    *f = fit_split(plan, n_t, SIZE_MAX);
+    *f = Split{two_pass_batch(plan, n_t), plan->M};
     const size_t need = split_bytes(plan, n_t, *f);
     if (plan->ws_bytes >= need) return CC_OK;
     bool fixed = plan->ws_external;
@@ -534,7 +534,7 @@ static cc_status search_folded_bf16(cc_plan* plan, const cc_template* t_dev, int
 }
 
 size_t two_pass_workspace_bytes(const cc_plan* plan, int64_t n_t) {
-    return n_t < 1 ? 0 : split_bytes(plan, n_t, fit_split(plan, n_t, SIZE_MAX));
+    return n_t < 1 ? 0 : split_bytes(plan, n_t, Split{two_pass_batch(plan, n_t), plan->M});
 }
 
 template <bool BF16, bool LAG>

@@ -335,7 +335,9 @@ cc_status launch_resample_group(cc_plan* plan, int64_t n_t, void* ab, float* nor
     static const int groups[] = {12, 6, 3, 2, 1, 0}, groups8[] = {8, 4, 2, 1, 0};
     const int* gp = warps == 12 ? groups : warps == 8 ? groups8 : groups8 + 1;
     if (warps == 12) ++gp;
-    while (gp[1] && (gp[0] >= 2 * n_t || p.M * p.Q * ((n_t + gp[0] - 1) / gp[0]) < 304)) ++gp;
+    int dev = 0, sms = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    while (gp[1] && (gp[0] >= 2 * n_t || p.M * p.Q * ((n_t + gp[0] - 1) / gp[0]) < 2 * sms)) ++gp;
     const int tg = gp[0];
     const int64_t most = bf16 ? RG_TILE_BF16 : RG_TILE, tiles = (p.N_s + most - 1) / most;
     const int tile = (int)(((p.N_s + tiles - 1) / tiles + 31) & ~(int64_t)31);
