@@ -253,7 +253,7 @@ class CrossCorrPlan:
         _check_tensor("templates", templates, torch.float64)
         if templates.dim() != 2 or templates.shape[1] not in (3, 5):
             raise ValueError("templates must be [n_t, 5] (a_p, T_asc, P, e, omega) or [n_t, 3] (circular)")
-        if stream is None or templates.shape[1] == 5:
+        if not isinstance(stream, torch.cuda.Stream) or templates.shape[1] == 5:
             return templates.shape[0], templates5(templates)
         with torch.cuda.stream(stream):
             return templates.shape[0], templates5(templates)

@@ -36,6 +36,22 @@ def test_widths_on_the_device(n, width):
 
 
 @pytest.mark.gpu
+def test_any_object_with_a_stream_handle():
+    """The calls take whatever carries a stream handle, not only torch's streams."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import types
+
+    import synth
+    ds = synth.tiny(seed=5, n_templates=3)
+    x, tm = torch.from_numpy(ds.x64).cuda(), torch.from_numpy(ds.templates).cuda()
+    with cc.CrossCorrPlan(ds.cfg, ds.dets) as plan:
+        want = plan.search(x, tm).cpu()
+        here = types.SimpleNamespace(cuda_stream=torch.cuda.current_stream().cuda_stream)
+        assert torch.equal(plan.search(x, tm, stream=here).cpu(), want)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("method", ["search", "demod_search"])
 def test_widening_runs_on_the_calls_stream(method):
     """A search on another stream than the current one, behind whose long queue the widening of
